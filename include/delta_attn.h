@@ -155,8 +155,8 @@ DELTA_API delta_status_t delta_attn_prefill(delta_state_t* st, const void* q, co
  * window, counters (Eq. 6 sums over the sequences: S_c_eq6 uses sum min(W_b, n_b) / sum n_b) and
  * decode hand-off.  Afterwards the batch elements stand at different positions:
  * delta_state_sequence_position reports each, delta_state_position the longest, and
- * delta_attn_decode_step advances every sequence by one token from where it stands (one kernel
- * launch per batch element while the positions differ).  Needs a fresh or reset state. */
+ * delta_attn_decode_step advances every sequence by one token from where it stands (in one launch
+ * where delta_state_decode_kernel reports 1 and the compressed key cache is off).  Needs a fresh or reset state. */
 DELTA_API delta_status_t delta_attn_prefill_varlen(delta_state_t* st, const void* q, const void* k, const void* v,
                                          void* out, const int32_t* seq_lens, const int32_t* windows,
                                          float theta, void* stream);
@@ -309,15 +309,15 @@ DELTA_API int32_t delta_state_sequence_position(const delta_state_t* st, int32_t
  * DELTA_ERR_UNSUPPORTED. */
 DELTA_API int32_t delta_state_prefill_kernel(const delta_state_t* st);
 
-/* Which kernel the next delta_attn_decode_step of this state would use: 1 = score products
- * on the tensor cores (bf16, d = 64, top-down query deltas or key deltas, at most 73728 keys:
- * the telescoped form of Eq. 4, see delta_attn_decode_step), 0 = the FP32-pipe kernel,
- * -1 for a null state.  Both compute the same step and keep the same state. */
+/* Which kernel the next delta_attn_decode_step of this state would use: 1 = score and value
+ * products on the tensor cores (bf16, top-down query deltas or key deltas: the telescoped form of
+ * Eq. 4, see delta_attn_decode_step), 0 = the FP32-pipe kernel, -1 for a null state.  Both compute
+ * the same step and keep the same state. */
 DELTA_API int32_t delta_state_decode_kernel(const delta_state_t* st);
 
-/* Force the decode kernel of a state: 1 = tensor-core scores whatever the slice length
- * (DELTA_ERR_UNSUPPORTED unless bf16, d = 64, top-down query deltas or key deltas), 0 = FP32 pipes, -1 = chosen per
- * step (the default).  Host-side only. */
+/* Force the decode kernel of a state: 1 = tensor cores (DELTA_ERR_UNSUPPORTED unless bf16, top-down
+ * query deltas or key deltas), 0 = FP32 pipes, -1 = the library's choice (the default).  Host-side
+ * only. */
 DELTA_API delta_status_t delta_state_set_decode_kernel(delta_state_t* st, int32_t which);
 DELTA_API delta_status_t delta_state_set_prefill_kernel(delta_state_t* st, int32_t which);
 

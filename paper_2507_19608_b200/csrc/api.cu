@@ -40,13 +40,11 @@ struct delta_state {
   int n;         // tokens seen (of the longest sequence, after a prefill over sequences of different lengths)
   std::vector<int> n_b;   // tokens seen per batch element
   bool ragged = false;    // the batch elements stand at different positions
-  std::vector<DecodeTmapCache> dec_tmap_b, dec_tmap_h_b;   // per batch element, for ragged decoding
   int qhat_sel;  // which q_hat buffer is current
   int forced_kernel;  // -1 auto, 0 generic, 1 tensor-core
   // Eq. 6 bookkeeping that needs no device work: sum of window lengths and sequence lengths
   double win_sum[2], len_sum[2];
-  DecodeTmapCache dec_tmap;   // tensor map of the key cache the decode steps read
-  DecodeTmapCache dec_tmap_h; // and of the reference-key cache (key deltas)
+  DecodeTmapCache dec_maps[3];     // tensor maps of the key, value and reference-key caches the decode steps read
   int forced_decode_kernel = -1;   // -1: chosen per step
   bool key_cache_packed = false;   // key deltas: decode from the compressed key-delta cache
   // optional per-kernel timing of prefill (host-side event objects)
@@ -240,16 +238,15 @@ int32_t delta_state_prefill_kernel(const delta_state_t* st) {
   return tc_eligible(st, 2) ? 2 : 0;   // the telescoped tensor-core kernel is the fastest where it applies
 }
 
-// Can the tensor-core decode kernel serve this state at all (whatever the slice length)?
+// Can the tensor-core decode kernel serve this state?
 static bool decode_tc_possible(const delta_state* st) {
-  return st->cfg.source != DELTA_SRC_QUERY_BOTTOM_UP && decode_tc_applies(st->shape, st->cfg.dtype, -1);
+  return st->cfg.source != DELTA_SRC_QUERY_BOTTOM_UP && decode_mma_applies(st->shape, st->cfg.dtype);
 }
 
 int32_t delta_state_decode_kernel(const delta_state_t* st) {
   if (!st) return -1;
   if (!decode_tc_possible(st)) return 0;
-  if (st->forced_decode_kernel >= 0) return st->forced_decode_kernel;
-  return decode_tc_applies(st->shape, st->cfg.dtype, st->n) ? 1 : 0;
+  return st->forced_decode_kernel >= 0 ? st->forced_decode_kernel : 1;
 }
 
 delta_status_t delta_state_set_decode_kernel(delta_state_t* st, int32_t which) {
@@ -539,26 +536,19 @@ delta_status_t delta_attn_prefill_host(delta_state_t* st, const void* q_host, co
 
 }  // extern "C"
 
-// One decode-step launch over a view (the whole batch, or one batch element) at position n.
+// One decode-step launch at position n over a view (the whole batch, or one batch element), for the
+// kernels that take one position per launch.
 static cudaError_t decode_launch(delta_state* st, const Shape& shape, const Workspace& ws, const void* q_new,
                                  const void* k_new, const void* v_new, void* k_cache, void* v_cache, void* out,
-                                 int n, float theta, int32_t window, DecodeTmapCache* tmap, DecodeTmapCache* tmap_h,
-                                 cudaStream_t cs) {
-  const bool tcs = decode_tc_possible(st) &&
-                   (st->forced_decode_kernel >= 0 ? st->forced_decode_kernel == 1
-                                                  : decode_tc_applies(shape, st->cfg.dtype, n));
-  if (st->cfg.source == DELTA_SRC_KEY && st->key_cache_packed)
-    return launch_decode_step_keypacked(shape, ws, q_new, k_new, v_new, k_cache, v_cache, out, n, theta, window,
-                                        st->qhat_sel, cs);
+                                 int n, float theta, int32_t window, cudaStream_t cs) {
   if (st->cfg.source == DELTA_SRC_KEY)
-    return tcs ? launch_decode_step_key_tc(shape, ws, q_new, k_new, v_new, k_cache, v_cache, out, n, theta, window,
-                                           st->qhat_sel, tmap, tmap_h, cs)
+    return st->key_cache_packed
+               ? launch_decode_step_keypacked(shape, ws, q_new, k_new, v_new, k_cache, v_cache, out, n, theta, window,
+                                              st->qhat_sel, cs)
                : launch_decode_step_key(shape, ws, q_new, k_new, v_new, k_cache, v_cache, out, n, theta, window,
                                         st->qhat_sel, cs);
-  return tcs ? launch_decode_step_tc(shape, ws, q_new, k_new, v_new, k_cache, v_cache, out, n, theta, window,
-                                     st->qhat_sel, tmap, cs)
-             : launch_decode_step(shape, ws, q_new, k_new, v_new, k_cache, v_cache, out, n, theta, window,
-                                  st->cfg.dtype, st->qhat_sel, cs);
+  return launch_decode_step(shape, ws, q_new, k_new, v_new, k_cache, v_cache, out, n, theta, window, st->cfg.dtype,
+                            st->qhat_sel, cs);
 }
 
 extern "C" {
@@ -580,17 +570,19 @@ delta_status_t delta_attn_decode_step(delta_state_t* st, const void* q_new, cons
   if (st->n >= c.T_max) return DELTA_ERR_CAPACITY;      // (the longest sequence decides)
   cudaStream_t cs = (cudaStream_t)stream;
   cudaError_t e = cudaSuccess;
-  if (!st->ragged) {
-    e = decode_launch(st, st->shape, st->ws, q_new, k_new, v_new, k_cache, v_cache, out, st->n, theta, window,
-                      &st->dec_tmap, &st->dec_tmap_h, cs);
+  const bool key_packed = c.source == DELTA_SRC_KEY && st->key_cache_packed;
+  if (!key_packed && delta_state_decode_kernel(st) == 1) {
+    // one launch, whether the batch elements stand at one position or at different ones
+    e = launch_decode_step_mma(st->shape, st->ws, q_new, k_new, v_new, k_cache, v_cache, out, st->n,
+                               st->ragged ? st->n_b.data() : nullptr, theta, window, st->qhat_sel,
+                               c.source == DELTA_SRC_KEY, st->dec_maps, cs);
     if (e != cudaSuccess) return cuda_fail(e);
-    const int L = st->n + 1;
-    st->win_sum[1] += (double)c.B * (double)(window < L ? window : L);
-    st->len_sum[1] += (double)c.B * (double)L;
+  } else if (!st->ragged) {
+    e = decode_launch(st, st->shape, st->ws, q_new, k_new, v_new, k_cache, v_cache, out, st->n, theta, window, cs);
+    if (e != cudaSuccess) return cuda_fail(e);
   } else {
     // the batch elements stand at different positions: one launch per element over its view
     const size_t es = c.dtype == DELTA_F32 ? 4 : 2;
-    if (st->dec_tmap_b.size() != (size_t)c.B) { st->dec_tmap_b.resize((size_t)c.B); st->dec_tmap_h_b.resize((size_t)c.B); }
     for (int b = 0; b < c.B; ++b) {
       Shape sh;
       Workspace ws;
@@ -598,13 +590,14 @@ delta_status_t delta_attn_decode_step(delta_state_t* st, const void* q_new, cons
       const size_t qo = (size_t)b * c.H * c.d * es, ko = (size_t)b * c.H_kv * c.d * es;
       const size_t co = (size_t)b * c.H_kv * c.T_max * c.d * es;
       e = decode_launch(st, sh, ws, (const char*)q_new + qo, (const char*)k_new + ko, (const char*)v_new + ko,
-                        (char*)k_cache + co, (char*)v_cache + co, (char*)out + qo, st->n_b[(size_t)b], theta, window,
-                        &st->dec_tmap_b[(size_t)b], &st->dec_tmap_h_b[(size_t)b], cs);
+                        (char*)k_cache + co, (char*)v_cache + co, (char*)out + qo, st->n_b[(size_t)b], theta, window, cs);
       if (e != cudaSuccess) return cuda_fail(e);
-      const int L = st->n_b[(size_t)b] + 1;
-      st->win_sum[1] += (double)(window < L ? window : L);
-      st->len_sum[1] += (double)L;
     }
+  }
+  for (int b = 0; b < c.B; ++b) {
+    const int L = st->n_b[(size_t)b] + 1;
+    st->win_sum[1] += (double)(window < L ? window : L);
+    st->len_sum[1] += (double)L;
   }
   for (auto& nb : st->n_b) nb += 1;
   st->qhat_sel ^= 1;

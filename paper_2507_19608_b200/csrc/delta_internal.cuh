@@ -3,6 +3,7 @@
 #include <cuda_runtime.h>
 #include <cuda_bf16.h>
 #include <stdint.h>
+#include <atomic>
 #include "../../include/delta_attn.h"
 
 namespace delta {
@@ -58,6 +59,21 @@ struct Shape {
   int n_ckpt() const { return (T_max + DELTA_CKPT_ROWS - 1) / DELTA_CKPT_ROWS; }
 };
 
+// What a launcher does once per device (function attributes, which the runtime keeps): has it been
+// done on the current device / it has.  (Devices past 63 do it every time.)
+inline int device_slot() {
+  int dev = 0;
+  return (cudaGetDevice(&dev) == cudaSuccess && dev >= 0 && dev < 64) ? dev : -1;
+}
+inline bool device_done(const std::atomic<uint64_t>& mask) {
+  const int dev = device_slot();
+  return dev >= 0 && ((mask.load(std::memory_order_acquire) >> dev) & 1u);
+}
+inline void device_mark(std::atomic<uint64_t>& mask) {
+  const int dev = device_slot();
+  if (dev >= 0) mask.fetch_or(1ull << dev, std::memory_order_release);
+}
+
 void count_launch(int n = 1);
 // Records the text of a failed CUDA runtime call for delta_last_cuda_error; returns DELTA_ERR_CUDA.
 delta_status_t cuda_fail(cudaError_t e);
@@ -93,24 +109,19 @@ cudaError_t launch_decode_step(const Shape& s, const Workspace& w, const void* q
                                void* out, int n, float theta, int window, int dtype, int qhat_sel,
                                cudaStream_t st);
 
-// K3 (key deltas): one decode step of strategy (3); bf16 only, needs w.qhat_rows (reference-key cache).
-// K3 with the score products on the tensor cores (bf16, d = 64): same step, same state.
-// Host-side cache of the key cache's tensor map (encoded once per cache pointer, not per step).
+// Host-side cache of a cache's tensor map (encoded once per cache pointer, not per step).
 struct DecodeTmapCache {
   const void* ptr = nullptr;
   alignas(64) unsigned char map[128];
 };
-// Does the step at position n take this kernel?  (bf16, d = 64, and a cache short enough for 64
-// slices of nine tiles.)  n < 0: shape and type only.
-bool decode_tc_applies(const Shape& s, int dtype, int n);
-cudaError_t launch_decode_step_tc(const Shape& s, const Workspace& w, const void* q_new, const void* k_new,
-                                  const void* v_new, void* k_cache, void* v_cache, void* out, int n, float theta,
-                                  int window, int qhat_sel, DecodeTmapCache* cache, cudaStream_t st);
-// The same for key deltas: tiles come from the reference-key cache or, inside the window, the key cache.
-cudaError_t launch_decode_step_key_tc(const Shape& s, const Workspace& w, const void* q_new, const void* k_new,
-                                      const void* v_new, void* k_cache, void* v_cache, void* out, int n,
-                                      float theta, int window, int qhat_sel, DecodeTmapCache* cache_k,
-                                      DecodeTmapCache* cache_h, cudaStream_t st);
+// K3 for bf16 caches (query and key deltas; key: w.qhat_rows is the reference-key cache).  n: tokens
+// seen (the longest sequence's); n_b: null, or the tokens seen by every batch element of a ragged
+// batch; maps: the state's tensor maps of the key, value and reference-key caches.
+bool decode_mma_applies(const Shape& s, int dtype);
+cudaError_t launch_decode_step_mma(const Shape& s, const Workspace& w, const void* q_new, const void* k_new,
+                                   const void* v_new, void* k_cache, void* v_cache, void* out, int n, const int* n_b,
+                                   float theta, int window, int qhat_sel, bool key, DecodeTmapCache* maps,
+                                   cudaStream_t st);
 // K3 (key deltas) from the compressed key-delta cache, the kernel that builds that cache behind a
 // prefill, and its geometry (values per KV head at most, 32-row segments).
 size_t keypack_capacity(int T_max, int d);
@@ -119,6 +130,7 @@ cudaError_t launch_pack_keys(const Shape& s, const Workspace& w, const void* k, 
 cudaError_t launch_decode_step_keypacked(const Shape& s, const Workspace& w, const void* q_new, const void* k_new,
                                          const void* v_new, void* k_cache, void* v_cache, void* out, int n,
                                          float theta, int window, int qhat_sel, cudaStream_t st);
+// K3 (key deltas) on the FP32 pipes.
 cudaError_t launch_decode_step_key(const Shape& s, const Workspace& w, const void* q_new,
                                    const void* k_new, const void* v_new, void* k_cache, void* v_cache,
                                    void* out, int n, float theta, int window, int qhat_sel,

@@ -1,0 +1,690 @@
+// K3 (bf16 caches) -- one decode step of strategy (1) or strategy (3), head dimension 64 or 128
+// (Section III-A "Decoding Stage Considerations", Section III-B "Decoding Stage").
+//
+// Eq. 4's running sum telescopes: R(n)[j] = q_hat(n) . k_j (query deltas), and for bf16 inputs every
+// element of q_hat is a copy of an input element, so a step's scores are two small dense products
+// per cached key, q_hat . k_j outside the window and q . k_j inside it.  Key deltas (KEY): one
+// product, q . k_hat(j) outside the window and q . k_j inside it, k_hat(j) being the rows of the
+// library's reference-key cache.
+//
+// Bound: one pass over the key and value cache (HBM, or L2 for a layer stepped in a loop); for a few
+// sequences the chain of dependent latencies in front of and behind that pass.  So a warp works alone:
+// it owns units of 32 keys, brings their key and value rows in by TMA (one box each, 128-byte swizzle,
+// its own two barriers), multiplies on mma.sync (m16n8k16) straight from the swizzled rows and keeps
+// its own running softmax; warps meet once, at the end.  Staging by per-thread cp.async instead of TMA
+// was bound by the SM's load path at half the rate (batch 16, 2048 keys: 18.9 us per step, TMA 12.2).
+// G <= 8 query rows against the cache are no shape for a 128-row tcgen05 tile, whose operands,
+// commits and tensor-memory reads put four hand-overs between a key tile and its softmax; the score
+// product here fills 16 rows with the G references and the G queries, so that one thread receives both
+// scores of a (head, key) pair in registers.
+//   scores  A = [references; queries] (16 x D), B = 8 keys: the contraction index may be permuted
+//           freely as long as both operands agree, so a thread takes 16-byte pieces of its key's row;
+//   P.V     A = P with the score accumulator's layout, B = 16 keys x 8 channels: output columns may
+//           be permuted, so a thread takes 16-byte pieces of four value rows and zips pairs of rows.
+//           P keeps fp32 precision as a sum of three bf16 parts: rows 0-7 of A carry the first part,
+//           rows 8-15 the second (the same thread holds both), the third goes to rows G .. 2G-1,
+//           whose lanes duplicate the scores of rows 0 .. G-1 (G <= 4), or to a second product (G = 8).
+// The row that arrives with the step is scored from k_new and v_new and written to the caches by the
+// warp that owns its unit.  The slices of a (batch, KV head) are one thread-block cluster: every warp
+// sends its partial result to the CTA that finishes those channels with st.async, which counts its
+// bytes on the receiver's barrier (a merge through global memory takes 2 us more; a cluster barrier
+// with release semantics waits 0.7 us for the step's global stores).
+// Measured, us per step, against the kernel before it (tcgen05 scores for d = 64, FP32 pipes for
+// d = 128): Llama layer at 2048 keys, batch 1 8.9 -> 4.8, batch 4 10.3 -> 7.0, batch 16 18.4 -> 12.3
+// (5.9 TB/s); batch 8 at 4096 keys 18.0 -> 11.8; BitNet layer (d = 128) at 1531 keys, batch 2
+// 16.7 -> 6.5, at 2000 keys, batch 16 45.5 -> 14.9; key deltas, batch 4 at 1777 keys 12.1 -> 6.8.
+#include <cuda.h>
+
+#include "decode_common.cuh"
+#include "tc_common.cuh"
+
+namespace delta {
+
+namespace {
+
+template <int D> constexpr int kWarps = D == 64 ? 8 : 4;    // warps per CTA
+constexpr int UK = 32;                    // keys a warp works on at a time
+constexpr int kMaxCluster = 16;           // slices merged through distributed shared memory
+constexpr int kRaggedMax = 64;            // batch elements of one ragged launch
+constexpr int REC = 16;                   // floats of a partial result's record: 16 channels of one head
+
+struct MmaDecodeParams {
+  const __nv_bfloat16 *q_new, *k_new, *v_new;
+  __nv_bfloat16 *k_cache, *v_cache, *khat_cache, *out;
+  uint16_t* row_nnz;
+  const float* ref_in;
+  float *ref_out, *R, *partial;
+  uint32_t* ticket;
+  unsigned long long* counters;
+  int n, T_max, H, chunk, nsplit, W, b0;
+  float theta, scale_log2e;
+  int ragged;
+  int n_b[kRaggedMax];                    // ragged: tokens seen per batch element b0 ..
+};
+
+__device__ __forceinline__ void async16(uint32_t dst, const void* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
+}
+__device__ __forceinline__ void async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+__device__ __forceinline__ void sts128z(uint32_t dst) {
+  asm volatile("st.shared.v4.u32 [%0], {%1, %1, %1, %1};" ::"r"(dst), "r"(0) : "memory");
+}
+__device__ __forceinline__ void mma16816(float (&c)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0,
+                                         uint32_t b1) {
+  asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, "
+               "{%0, %1, %2, %3};"
+               : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3]) : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+}
+__device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
+  const __nv_bfloat162 t = __floats2bfloat162_rn(lo, hi);
+  return *reinterpret_cast<const uint32_t*>(&t);
+}
+// (lo, hi) as three bf16 pairs whose sum is (lo, hi) to fp32 precision
+__device__ __forceinline__ void split3(float lo, float hi, uint32_t& p0, uint32_t& p1, uint32_t& p2) {
+  p0 = pack_bf16(lo, hi);
+  const float r0 = lo - __uint_as_float(p0 << 16), r1 = hi - __uint_as_float(p0 & 0xffff0000u);
+  p1 = pack_bf16(r0, r1);
+  p2 = pack_bf16(r0 - __uint_as_float(p1 << 16), r1 - __uint_as_float(p1 & 0xffff0000u));
+}
+__device__ __forceinline__ uint32_t cluster_map(uint32_t addr, uint32_t rank) {
+  uint32_t r;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
+  return r;
+}
+// Stores into the shared memory of a CTA of the cluster that count their bytes on its barrier: the
+// receiver waits for the bytes, and nothing of the sender's (its global stores least of all) has to
+// be flushed first, as a cluster barrier with release semantics would.
+__device__ __forceinline__ void cluster_send4(uint32_t addr, uint32_t bar, float a, float b, float c, float d) {
+  asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v4.f32 [%0], {%2, %3, %4, %5}, [%1];" ::"r"(addr),
+               "r"(bar), "f"(a), "f"(b), "f"(c), "f"(d) : "memory");
+}
+__device__ __forceinline__ void cluster_send2(uint32_t addr, uint32_t bar, float a, float b) {
+  asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v2.f32 [%0], {%2, %3}, [%1];" ::"r"(addr),
+               "r"(bar), "f"(a), "f"(b) : "memory");
+}
+__device__ __forceinline__ void sts_f4(uint32_t addr, float a, float b, float c, float d) {
+  asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "f"(a), "f"(b), "f"(c), "f"(d) : "memory");
+}
+__device__ __forceinline__ void sts_f2(uint32_t addr, float a, float b) {
+  asm volatile("st.shared.v2.f32 [%0], {%1, %2};" ::"r"(addr), "f"(a), "f"(b) : "memory");
+}
+__device__ __forceinline__ float2 lds_f2(uint32_t addr) {
+  float2 v;
+  asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(addr));
+  return v;
+}
+__device__ __forceinline__ float4 lds_f4(uint32_t addr) { return tc::lds128(addr); }
+
+__device__ __forceinline__ int warp_sum(int x) {
+#pragma unroll
+  for (int s = 16; s > 0; s >>= 1) x += __shfl_xor_sync(0xffffffffu, x, s);
+  return x;
+}
+
+// Shared memory: per warp one unit of keys and values (128-byte swizzle, blocks of [32 rows][64
+// channels]), then the merge's records [slot][slice x warp][REC] and (maximum, row sum) pairs.
+template <int D, int G> struct MmaSmem {
+  static constexpr int NW = kWarps<D>;
+  static constexpr uint32_t HALF = UK * D * 2;             // keys, or values, of a unit
+  static constexpr uint32_t RING = NW * 2 * HALF;
+  static constexpr int NB = G * D / 16;                    // 16-channel blocks of the result
+  static constexpr uint32_t NREC = (NB + kMaxCluster - 1) * NW;
+  static constexpr size_t bytes = 1024 + RING + NREC * (REC + 2) * 4;
+};
+
+}  // namespace
+
+template <int D, int G, bool KEY, bool CLUSTER>
+__global__ void __launch_bounds__(32 * kWarps<D>, 2)
+decode_step_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ CUtensorMap tm_v,
+                       const __grid_constant__ CUtensorMap tm_h, const __grid_constant__ MmaDecodeParams p) {
+  using TC = __nv_bfloat16;
+  using SM = MmaSmem<D, G>;
+  constexpr int MNW = kWarps<D>;
+  constexpr int NC = D / 32;                 // 16-byte pieces of a key row per thread
+  constexpr int NV = D / 64;                 // 64-channel blocks of a row
+  constexpr int NT8 = D / 8;                 // n-tiles of P.V
+  extern __shared__ unsigned char dsm_raw[];
+  __shared__ __align__(8) unsigned long long bars[2 * MNW + 1];
+  __shared__ int s_last, s_fail;
+  const uint32_t ring = (smem_u32(dsm_raw) + 1023u) & ~1023u;
+  const uint32_t recs = ring + SM::RING, mls = recs + SM::NREC * REC * 4;
+
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int g = lane >> 2, t = lane & 3;     // row of the accumulators, thread of the row
+  const int hd = g % G, part = g / G;        // the head this thread's row stands for; which part of P it feeds
+  const int split = blockIdx.x, bkv = p.b0 * (p.H / G) + blockIdx.y;
+  const int H_kv = p.H / G;
+  const int b = bkv / H_kv, kvh = bkv - b * H_kv;
+  const int n = p.ragged ? p.n_b[b - p.b0] : p.n, T_max = p.T_max, W = p.W;
+  const int L = n + 1;
+  const int j0 = split * p.chunk, j1 = min(j0 + p.chunk, L);
+  const float theta = p.theta;
+
+  // the merge: blocks of 16 channels of one head; slice r of the cluster finishes blocks r, r + cs, ..
+  // (a CTA without a cluster all of them), each from the records of every warp of every slice
+  const int cs = CLUSTER ? p.nsplit : 1, rank = CLUSTER ? split : 0, nsrc = cs * MNW;
+  const uint32_t bar_m = smem_u32(&bars[2 * MNW]);
+  if (CLUSTER) {
+    if (tid == 0) {
+      tc::mbar_init(bar_m, 1);
+      asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+      const int slots = (SM::NB - rank + cs - 1) / cs;
+      tc::mbar_expect_tx(bar_m, (uint32_t)(slots * nsrc) * (REC + 2) * 4);
+    }
+    __syncwarp();
+    asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
+  }
+  if (!CLUSTER && j0 >= L) return;           // ragged batch: this sequence has fewer slices
+
+  const size_t row0 = (size_t)bkv * T_max;
+  const TC* const kc = p.k_cache + row0 * D;
+  const TC* const vc = p.v_cache + row0 * D;
+  const TC* const hc = KEY ? p.khat_cache + row0 * D : nullptr;
+  const TC* const kn = p.k_new + (size_t)bkv * D;
+  const TC* const vn = p.v_new + (size_t)bkv * D;
+  const int wl = n - W + 1;                  // first key inside the decode window
+
+  // ---- the warp's ring: one unit of keys, one of values.  Row r, 16-byte chunk c of a 64-channel
+  // block lies at r * 128 + ((c ^ (r & 7)) << 4): what TMA's 128-byte swizzle writes.
+  const uint32_t slot_k = ring + (uint32_t)warp * 2 * SM::HALF, slot_v = slot_k + SM::HALF;
+  const uint32_t bar_k = smem_u32(&bars[2 * warp]), bar_v = bar_k + 8;
+  if (lane == 0) {
+    tc::mbar_init(bar_k, 1);
+    tc::mbar_init(bar_v, 1);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    tc::fence_proxy_async();
+  }
+  if (tid == 0) s_fail = 0;
+  __syncwarp();
+  // A unit whose rows come from one cache goes by TMA; the unit of the row that arrives with the
+  // step (rows behind it: zeros) and, key deltas, the unit of the window's edge row by row.
+  auto k_plain = [&](int jg) { return jg + UK <= n && (!KEY || jg + UK <= wl || jg >= wl); };
+  auto fetch_k = [&](int jg) {
+    if (k_plain(jg)) {
+      if (lane == 0) {
+        tc::mbar_expect_tx(bar_k, SM::HALF);
+        const CUtensorMap* tm = (KEY && jg < wl) ? &tm_h : &tm_k;
+#pragma unroll
+        for (int c = 0; c < NV; ++c) tc::tma_load_3d(slot_k + c * UK * 128, tm, bar_k, 64 * c, jg, bkv);
+      }
+    } else {
+#pragma unroll
+      for (int c = 0; c < NV; ++c)
+#pragma unroll
+        for (int i = 0; i < UK / 4; ++i) {
+          const int r = 4 * i + (lane >> 3), ch = lane & 7, j = jg + r;
+          const uint32_t dst = slot_k + c * UK * 128 + r * 128 + ((ch ^ (r & 7)) << 4);
+          const TC* src = (KEY && j < wl) ? hc : kc;
+          if (j <= n) async16(dst, (j < n ? src + (size_t)j * D : kn) + 64 * c + 8 * ch);
+          else sts128z(dst);
+        }
+    }
+  };
+  auto fetch_v = [&](int jg) {
+    if (jg + UK <= n) {
+      if (lane == 0) {
+        tc::mbar_expect_tx(bar_v, SM::HALF);
+#pragma unroll
+        for (int c = 0; c < NV; ++c) tc::tma_load_3d(slot_v + c * UK * 128, &tm_v, bar_v, 64 * c, jg, bkv);
+      }
+    } else {
+#pragma unroll
+      for (int c = 0; c < NV; ++c)
+#pragma unroll
+        for (int i = 0; i < UK / 4; ++i) {
+          const int r = 4 * i + (lane >> 3), ch = lane & 7, j = jg + r;
+          const uint32_t dst = slot_v + c * UK * 128 + r * 128 + ((ch ^ (r & 7)) << 4);
+          if (j <= n) async16(dst, (j < n ? vc + (size_t)j * D : vn) + 64 * c + 8 * ch);
+          else sts128z(dst);
+        }
+    }
+  };
+  // the step in front (or the prefill) has written the reference, row n - 1 of the caches, the tickets
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  // The next step's CTAs may become resident from here on.  (Released at the kernel's start they
+  // take the places of this step's own late CTAs: 30 us per step for 18 at batch 16.)
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  int jg = j0 + UK * warp;
+  if (jg < j1) { fetch_k(jg); fetch_v(jg); }
+
+  // ---- threshold step (Eq. 2-3): the operand rows, straight into registers
+  uint32_t ar[NC][4], aq[NC][4];             // rows g and g + 8 of A, channels 32 c + 8 t ..
+  uint32_t khat_new[KEY ? NC : 1][4];        // KEY: the reference key after this step
+  int fired = 0;
+  const bool keep = split == 0 && warp == 0;
+  {
+    const size_t o = ((size_t)b * p.H + kvh * G + hd) * D;
+    const float* const rp = p.ref_in + (KEY ? (size_t)bkv * D : o);
+    uint4 q4[NC], x4[NC];
+    float4 r4[NC][2];
+#pragma unroll
+    for (int c = 0; c < NC; ++c) {
+      const int ch = 32 * c + 8 * t;
+      q4[c] = __ldcg(reinterpret_cast<const uint4*>(p.q_new + o + ch));
+      r4[c][0] = __ldcg(reinterpret_cast<const float4*>(rp + ch));
+      r4[c][1] = __ldcg(reinterpret_cast<const float4*>(rp + ch) + 1);
+      if (KEY) x4[c] = __ldcg(reinterpret_cast<const uint4*>(kn + ch));
+    }
+#pragma unroll
+    for (int c = 0; c < NC; ++c) {
+      const uint32_t qw[4] = {q4[c].x, q4[c].y, q4[c].z, q4[c].w};
+      const uint4 xx = KEY ? x4[c] : q4[c];
+      const uint32_t xw[4] = {xx.x, xx.y, xx.z, xx.w};
+      float ref[8] = {r4[c][0].x, r4[c][0].y, r4[c][0].z, r4[c][0].w, r4[c][1].x, r4[c][1].y, r4[c][1].z, r4[c][1].w};
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        const float x = (i & 1) ? __uint_as_float(xw[i >> 1] & 0xffff0000u) : __uint_as_float(xw[i >> 1] << 16);
+        const bool fire = fabsf(__fsub_rn(x, ref[i])) > theta;
+        ref[i] = fire ? x : ref[i];
+        fired += fire ? 1 : 0;
+      }
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        // exactly bf16: copies of input elements (or the zero the reference starts from)
+        const uint32_t rw = __byte_perm(__float_as_uint(ref[2 * i]), __float_as_uint(ref[2 * i + 1]), 0x7632);
+        ar[c][i] = KEY ? qw[i] : rw;
+        aq[c][i] = KEY ? 0u : qw[i];
+        if (KEY) khat_new[c][i] = rw;
+      }
+      if (keep && (KEY ? g == 0 : part == 0)) {
+        float4* rq = reinterpret_cast<float4*>(p.ref_out + (KEY ? (size_t)bkv * D : o) + 32 * c + 8 * t);
+        rq[0] = make_float4(ref[0], ref[1], ref[2], ref[3]);
+        rq[1] = make_float4(ref[4], ref[5], ref[6], ref[7]);
+      }
+    }
+    if (!(KEY ? g == 0 : part == 0)) fired = 0;
+  }
+
+  // ---- the warp's units
+  float o_acc[NT8][4];
+#pragma unroll
+  for (int i = 0; i < NT8; ++i)
+#pragma unroll
+    for (int e = 0; e < 4; ++e) o_acc[i][e] = 0.0f;
+  float m = -INFINITY, l = 0.0f;
+  unsigned done = 0;
+  uint32_t ph_k = 0, ph_v = 0;
+  // Column x of a score block stands for key x ^ (4 (x & 1)) of its 8 keys: with the swizzle, the
+  // eight lanes of a shared-memory phase then touch eight different chunks, for keys and values alike.
+  const int kx0 = 2 * t, kx1 = (2 * t + 1) ^ 4;            // this thread's two keys of a block
+  const int kr = g ^ (4 * (g & 1));                        // the key row it reads
+  const uint32_t k_off = slot_k + kr * 128, k_sw = kr & 7;
+  const uint32_t v_off0 = slot_v + kx0 * 128 + ((g ^ kx0) << 4), v_off1 = slot_v + kx1 * 128 + ((g ^ kx1) << 4);
+  float* const Rg = KEY ? nullptr : p.R + ((size_t)b * p.H + kvh * G + hd) * T_max;
+  for (; jg < j1; jg += UK * MNW) {
+    const int jn = jg + UK * MNW;            // the warp's next unit
+    const bool owner = n < jg + UK;          // of the row that arrives with the step
+    const bool tma_k = k_plain(jg), tma_v = jg + UK <= n;
+    if (tma_k) {
+      if (!mbar_wait(bar_k, ph_k)) s_fail = 1;
+      ph_k ^= 1u;
+    } else {
+      async_wait_all();
+      __syncwarp();
+    }
+    float s[4][4];
+#pragma unroll
+    for (int h = 0; h < 4; ++h) {
+#pragma unroll
+      for (int e = 0; e < 4; ++e) s[h][e] = 0.0f;
+#pragma unroll
+      for (int c = 0; c < NC; ++c) {
+        // channels 32 c + 8 t .. of the row: chunk 4 (c & 1) + t of block c >> 1
+        uint4 k4 = tc::lds128u(k_off + (c >> 1) * UK * 128 + h * 1024 + (((4 * (c & 1) + t) ^ k_sw) << 4));
+        if (KEY && W <= 0 && jg + 8 * h + kr == n)         // no window: even the new key goes by its reference
+          k4 = make_uint4(khat_new[c][0], khat_new[c][1], khat_new[c][2], khat_new[c][3]);
+        mma16816(s[h], ar[c][0], aq[c][0], ar[c][1], aq[c][1], k4.x, k4.y);
+        mma16816(s[h], ar[c][2], aq[c][2], ar[c][3], aq[c][3], k4.z, k4.w);
+      }
+    }
+    if (KEY) {
+      // multiply-adds: d inside the window, nnz(Delta k_j) outside
+      const int j = jg + lane;
+      int nz_new = 0;
+      if (owner) {
+        nz_new = warp_sum(fired);
+        if (lane == 0 && DELTA_IN(n, T_max, p.counters)) p.row_nnz[row0 + n] = (uint16_t)nz_new;
+      }
+      if (j < j1) done += (n - j < W) ? (unsigned)D : (j == n) ? (unsigned)nz_new : (unsigned)p.row_nnz[row0 + j];
+      if (!tma_k) tc::fence_proxy_async();                 // rows written by the warp, TMA overwrites them
+    }
+    __syncwarp();                            // every key of the unit has been used
+    if (jn < j1) fetch_k(jn);
+
+    // hybrid select, scale, running maximum of the row (4 threads hold it)
+    float v[8];
+#pragma unroll
+    for (int h = 0; h < 4; ++h) {
+      v[2 * h] = ((KEY || jg + 8 * h + kx0 < wl) ? s[h][0] : s[h][2]) * p.scale_log2e;
+      v[2 * h + 1] = ((KEY || jg + 8 * h + kx1 < wl) ? s[h][1] : s[h][3]) * p.scale_log2e;
+    }
+    if (owner) {
+#pragma unroll
+      for (int h = 0; h < 4; ++h) {
+        if (jg + 8 * h + kx0 > n) v[2 * h] = -INFINITY;
+        if (jg + 8 * h + kx1 > n) v[2 * h + 1] = -INFINITY;
+      }
+    }
+    float mx = tc::fmax3(fmaxf(v[0], v[1]), tc::fmax3(v[2], v[3], v[4]), tc::fmax3(v[5], v[6], v[7]));
+    mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
+    mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
+    if (__any_sync(0xffffffffu, mx > m)) {
+      const float mn = fmaxf(m, mx), al = tc::ex2(m - mn);
+      m = mn;
+      l *= al;
+#pragma unroll
+      for (int i = 0; i < NT8; ++i)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) o_acc[i][e] *= al;
+    }
+    float pr[8];
+#pragma unroll
+    for (int e = 0; e < 8; ++e) pr[e] = tc::ex2(v[e] - m);
+    l += ((pr[0] + pr[1]) + (pr[2] + pr[3])) + ((pr[4] + pr[5]) + (pr[6] + pr[7]));
+    if (tma_v) {
+      if (!mbar_wait(bar_v, ph_v)) s_fail = 1;
+      ph_v ^= 1u;
+    } else {
+      async_wait_all();
+      __syncwarp();
+    }
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {            // 16 keys per product
+      uint32_t f0, f1, f2, g0, g1, g2;
+      split3(pr[4 * q], pr[4 * q + 1], f0, f1, f2);
+      split3(pr[4 * q + 2], pr[4 * q + 3], g0, g1, g2);
+      uint32_t a0 = f0, a1 = f1, a2 = g0, a3 = g1;
+      if (G <= 4) {
+        a0 = part == 0 ? f0 : part == 1 ? f2 : 0u; a1 = part == 0 ? f1 : 0u;
+        a2 = part == 0 ? g0 : part == 1 ? g2 : 0u; a3 = part == 0 ? g1 : 0u;
+      }
+#pragma unroll
+      for (int c = 0; c < NV; ++c) {
+        uint4 vr[4];
+#pragma unroll
+        for (int r = 0; r < 4; ++r)
+          vr[r] = tc::lds128u(((r & 1) ? v_off1 : v_off0) + c * UK * 128 + (2 * q + (r >> 1)) * 1024);
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+          auto word = [&](int r) { return i < 2 ? vr[r].x : i < 4 ? vr[r].y : i < 6 ? vr[r].z : vr[r].w; };
+          const uint32_t sel = (i & 1) ? 0x7632u : 0x5410u;
+          const uint32_t b0 = __byte_perm(word(0), word(1), sel), b1 = __byte_perm(word(2), word(3), sel);
+          mma16816(o_acc[8 * c + i], a0, a1, a2, a3, b0, b1);
+          if (G == 8) mma16816(o_acc[8 * c + i], f2, 0u, g2, 0u, b0, b1);
+        }
+      }
+    }
+    __syncwarp();
+    if (jn < j1) fetch_v(jn);
+    if (!KEY && part == 0) {                 // R[j] = q_hat . k_j
+#pragma unroll
+      for (int h = 0; h < 4; ++h) {
+        const int ja = jg + 8 * h + kx0, jb = jg + 8 * h + kx1;
+        if ((!owner || ja <= n) && DELTA_IN(ja, T_max, p.counters)) Rg[ja] = s[h][0];
+        if ((!owner || jb <= n) && DELTA_IN(jb, T_max, p.counters)) Rg[jb] = s[h][1];
+      }
+    }
+    if (owner && DELTA_IN(n, T_max, p.counters)) {
+      // the row that arrives with the step joins the caches
+      if (lane < D / 8) {
+        reinterpret_cast<uint4*>(p.k_cache + (row0 + n) * D)[lane] = __ldcg(reinterpret_cast<const uint4*>(kn) + lane);
+        reinterpret_cast<uint4*>(p.v_cache + (row0 + n) * D)[lane] = __ldcg(reinterpret_cast<const uint4*>(vn) + lane);
+      }
+      if (KEY && g == 0)
+#pragma unroll
+        for (int c = 0; c < NC; ++c)
+          *reinterpret_cast<uint4*>(p.khat_cache + (row0 + n) * D + 32 * c + 8 * t) =
+              make_uint4(khat_new[c][0], khat_new[c][1], khat_new[c][2], khat_new[c][3]);
+    }
+  }
+
+  // ---- the warp's result: the parts of P meet again, the row sum over the row's four threads
+  l += __shfl_xor_sync(0xffffffffu, l, 1);
+  l += __shfl_xor_sync(0xffffffffu, l, 2);
+#pragma unroll
+  for (int i = 0; i < NT8; ++i) {
+    o_acc[i][0] += o_acc[i][2];
+    o_acc[i][1] += o_acc[i][3];
+    if (G <= 4) {
+      o_acc[i][0] += __shfl_down_sync(0xffffffffu, o_acc[i][0], 4 * G);
+      o_acc[i][1] += __shfl_down_sync(0xffffffffu, o_acc[i][1], 4 * G);
+    }
+  }
+  // ---- merge: every warp sends its part to where it is finished
+  const int src = rank * MNW + warp;
+  if (CLUSTER) asm volatile("barrier.cluster.wait.aligned;" ::: "memory");          // every slice runs
+  if (part == 0) {
+#pragma unroll
+    for (int c = 0; c < NV; ++c) {
+      // tile 8c + i, accumulator column x holds channel 64 c + 8 x + i; this thread has columns 2t, 2t + 1
+      const int q = hd * (D / 16) + 4 * c + t, r = q % cs, rec = (q / cs) * nsrc + src;
+      uint32_t dst = recs + (uint32_t)rec * (REC * 4), dml = mls + (uint32_t)rec * 8, rbar = bar_m;
+      if (CLUSTER) { dst = cluster_map(dst, r); dml = cluster_map(dml, r); rbar = cluster_map(bar_m, r); }
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        const float* const oe = &o_acc[8 * c + 4 * (e & 1)][0] + (e >> 1);
+        if (CLUSTER) cluster_send4(dst + 16 * e, rbar, oe[0], oe[4], oe[8], oe[12]);
+        else sts_f4(dst + 16 * e, oe[0], oe[4], oe[8], oe[12]);
+      }
+      if (CLUSTER) cluster_send2(dml, rbar, m, l); else sts_f2(dml, m, l);
+    }
+  }
+  if (keep) {
+    const int f = warp_sum(fired);
+    if (lane == 0) {
+      const int n_in = min(L, max(W, 0));
+      atomicAdd(&p.counters[CNT_DECODE_NNZ], (unsigned long long)f);
+      atomicAdd(&p.counters[CNT_DECODE_ELEMS], (unsigned long long)(KEY ? D : G * D));
+      atomicAdd(&p.counters[CNT_DECODE_MACS_DENSE], (unsigned long long)L * D * G);
+      if (!KEY)
+        atomicAdd(&p.counters[CNT_DECODE_MACS_DONE],
+                  (unsigned long long)n_in * D * G + (unsigned long long)(L - n_in) * f);
+    }
+  }
+  if (KEY) {
+    const int d = warp_sum((int)done);
+    if (lane == 0 && d) atomicAdd(&p.counters[CNT_DECODE_MACS_DONE], (unsigned long long)d * G);
+  }
+  if (CLUSTER) {
+    if (!mbar_wait(bar_m, 0)) s_fail = 1;
+  } else {
+    __syncthreads();
+  }
+  if (tid == 0 && s_fail) atomicMax(&p.counters[CNT_STATUS], (unsigned long long)DELTA_ERR_TIMEOUT);
+
+  // One warp per block: lane = (4 channels, one of 8 groups of parts).
+  const int c4 = lane & 3, sg = lane >> 2;
+  const int ns = (L + p.chunk - 1) / p.chunk;               // slices of this sequence
+  for (int slot = warp; slot * cs + rank < SM::NB; slot += MNW) {
+    const int q = slot * cs + rank;
+    const uint32_t rb = recs + (uint32_t)(slot * nsrc) * (REC * 4) + 16 * c4, mb = mls + (uint32_t)(slot * nsrc) * 8;
+    float M = -INFINITY;
+#pragma unroll
+    for (int x = 0; x < (CLUSTER ? kMaxCluster : 1) * MNW; x += 32)
+      if (x + lane < nsrc) M = fmaxf(M, lds_f2(mb + 8 * (x + lane)).x);
+#pragma unroll
+    for (int x = 1; x < 32; x <<= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, x));
+    float a[5] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
+#pragma unroll 4
+    for (int x = sg; x < nsrc; x += 8) {
+      const float2 ml = lds_f2(mb + 8 * x);
+      const float4 o = lds_f4(rb + x * (REC * 4));
+      const float f = tc::ex2(ml.x - M);                     // 0 for a warp without keys
+      a[0] = fmaf(f, o.x, a[0]); a[1] = fmaf(f, o.y, a[1]); a[2] = fmaf(f, o.z, a[2]); a[3] = fmaf(f, o.w, a[3]);
+      a[4] = fmaf(f, ml.y, a[4]);
+    }
+#pragma unroll
+    for (int x = 4; x < 32; x <<= 1)
+#pragma unroll
+      for (int e = 0; e < 5; ++e) a[e] += __shfl_xor_sync(0xffffffffu, a[e], x);
+    const int hh = q / (D / 16), ch = (q % (D / 16)) * 16 + 4 * c4;
+    if (sg == 0) {
+      if (CLUSTER || ns == 1) {
+        const float inv = 1.0f / a[4];
+        *reinterpret_cast<uint2*>(p.out + ((size_t)b * p.H + kvh * G + hh) * D + ch) =
+            make_uint2(pack_bf16(a[0] * inv, a[1] * inv), pack_bf16(a[2] * inv, a[3] * inv));
+      } else {
+        // slices through global memory: this slice's part
+        float* const pg = p.partial + (((size_t)bkv * kMaxDecodeSplits + split) * G + hh) * (D + 2);
+        pg[ch] = a[0]; pg[ch + 1] = a[1]; pg[ch + 2] = a[2]; pg[ch + 3] = a[3];
+        if (ch == 0) { pg[D] = M; pg[D + 1] = a[4]; }
+      }
+    }
+  }
+  if (CLUSTER || ns == 1) return;
+
+  // ---- the last CTA of the (batch, KV head) to arrive merges the slices
+  __threadfence();
+  __syncthreads();
+  if (tid == 0) s_last = atomicAdd(&p.ticket[bkv], 1u) == (uint32_t)ns - 1u;
+  __syncthreads();
+  if (!s_last) return;
+  __threadfence();
+  const float* const pb = p.partial + (size_t)bkv * kMaxDecodeSplits * G * (D + 2);
+  for (int e = tid; e < G * D; e += 32 * MNW) {
+    const int hh = e / D, c = e - hh * D;
+    float M = -INFINITY, nu = 0.0f, de = 0.0f;
+#pragma unroll 8
+    for (int r = 0; r < ns; ++r) M = fmaxf(M, __ldcg(pb + ((size_t)r * G + hh) * (D + 2) + D));
+#pragma unroll 8
+    for (int r = 0; r < ns; ++r) {
+      const float* const pr = pb + ((size_t)r * G + hh) * (D + 2);
+      const float f = tc::ex2(__ldcg(pr + D) - M);
+      nu = fmaf(f, __ldcg(pr + c), nu);
+      de = fmaf(f, __ldcg(pr + D + 1), de);
+    }
+    p.out[((size_t)b * p.H + kvh * G + hh) * D + c] = __float2bfloat16_rn(nu / de);
+  }
+  if (tid == 0) p.ticket[bkv] = 0;                          // ready for the next step
+}
+
+// Slices of a step over sequences of up to L keys (the new one included).  A step takes 4 to 5 us plus,
+// for every unit a warp works through, 1.1 us (d = 64) or 1.3 us (d = 128) while a CTA has its SM for
+// itself and 1.75 us where two share one (measured from 1 to 192 KV heads, 300 to 16000 keys); the
+// slices are those that minimise that.  All slices of a KV head form one cluster, and clusters have to
+// find room in a GPC: from 1.75 CTAs per SM on (1.6 for clusters of 9 to 12, 1.35 for 13 to 16) some
+// wait for a second wave (batch 16, 2048 keys: 256 CTAs 12 us, 384 CTAs 17 us).  Very long caches of
+// few heads: up to 64 slices merged through global memory (4.5 us more than a cluster).
+static void decode_mma_slices(const Shape& s, int L, int* nsplit_out, int* chunk_out, bool* cluster_out) {
+  const int bkv = s.B * s.H_kv, sms = device_sm_count();
+  const int nw = s.d == 64 ? kWarps<64> : kWarps<128>;
+  const int units = (L + UK - 1) / UK;
+  float best = 3.4e38f;
+  int best_ns = 1;
+  for (int ns = 1; ns <= kMaxDecodeSplits && (ns - 1) * nw < units; ++ns) {       // a unit per warp at least
+    const long ctas = (long)bkv * ns;
+    const bool alone = ctas * 100 <= (long)sms * 92;
+    if (ns > kMaxCluster && ctas > sms) break;
+    if (ns > 1 && ns <= kMaxCluster && ctas * 100 > (long)sms * (ns <= 8 ? 175 : ns <= 12 ? 160 : 135)) continue;
+    const int per = (units + ns - 1) / ns;                       // units per slice; per warp mostly the longest counts
+    const float rounds = 0.8f * (float)((per + nw - 1) / nw) + 0.2f * (float)per / (float)nw;
+    const float us = rounds * (!alone ? 1.75f : s.d == 64 ? 1.1f : 1.3f) +
+                     (ns > kMaxCluster ? 4.5f + 0.15f * (float)(ns - 24) : (ns > 8 ? 0.075f : 0.06f) * (float)ns);
+    if (us < best - 0.02f) { best = us; best_ns = ns; }
+  }
+  const int chunk = (units + best_ns - 1) / best_ns * UK;
+  *nsplit_out = (L + chunk - 1) / chunk;
+  *chunk_out = chunk;
+  *cluster_out = *nsplit_out > 1 && *nsplit_out <= kMaxCluster;
+}
+
+template <int D, int G, bool KEY, bool CLUSTER>
+static cudaError_t launch_mma(const CUtensorMap& tk, const CUtensorMap& tv, const CUtensorMap& th,
+                              const MmaDecodeParams& p, int bkv, cudaStream_t st) {
+  auto kern = decode_step_mma_kernel<D, G, KEY, CLUSTER>;
+  constexpr size_t smem = MmaSmem<D, G>::bytes;
+  static std::atomic<uint64_t> ready{0};
+  if (!device_done(ready)) {
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    // (two CTAs per SM need the largest shared-memory carve-out)
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout,
+                                                   (int)cudaSharedmemCarveoutMaxShared);
+    if (e == cudaSuccess && CLUSTER) e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    if (e != cudaSuccess) return e;
+    device_mark(ready);
+  }
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)p.nsplit, (unsigned)bkv);
+  cfg.blockDim = dim3(32 * kWarps<D>);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = (unsigned)p.nsplit;
+  attr[1].val.clusterDim.y = 1;
+  attr[1].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = CLUSTER ? 2 : 1;
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, tk, tv, th, p);
+  count_launch();
+  return e;
+}
+
+// The tensor map of a [B * H_kv, T_max, d] bf16 cache (box: UK rows of 64 channels), encoded once
+// per cache pointer.
+static const CUtensorMap* row_map(DecodeTmapCache* cache, const void* ptr, const Shape& s) {
+  static_assert(sizeof(CUtensorMap) <= sizeof(cache->map), "tensor-map cache");
+  CUtensorMap* m = reinterpret_cast<CUtensorMap*>(cache->map);
+  if (cache->ptr != ptr) {
+    if (!tc::encode3(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, ptr, (uint64_t)s.d, (uint64_t)s.T_max, (uint64_t)s.B * s.H_kv,
+                     (uint64_t)s.d * 2, (uint64_t)s.T_max * s.d * 2, 64, UK, CU_TENSOR_MAP_SWIZZLE_128B))
+      return nullptr;
+    cache->ptr = ptr;
+  }
+  return m;
+}
+
+bool decode_mma_applies(const Shape& s, int dtype) { return dtype == DELTA_BF16 && (s.d == 64 || s.d == 128); }
+
+cudaError_t launch_decode_step_mma(const Shape& s, const Workspace& w, const void* q_new, const void* k_new,
+                                   const void* v_new, void* k_cache, void* v_cache, void* out, int n, const int* n_b,
+                                   float theta, int window, int qhat_sel, bool key, DecodeTmapCache* maps, cudaStream_t st) {
+  if (key && !w.qhat_rows) return cudaErrorNotSupported;
+  using TC = __nv_bfloat16;
+  const CUtensorMap* const tk = row_map(&maps[0], k_cache, s);
+  const CUtensorMap* const tv = row_map(&maps[1], v_cache, s);
+  const CUtensorMap* const th = key ? row_map(&maps[2], w.qhat_rows, s) : tk;
+  if (!tk || !tv || !th) return cudaErrorInvalidValue;
+  MmaDecodeParams p;
+  p.q_new = (const TC*)q_new; p.k_new = (const TC*)k_new; p.v_new = (const TC*)v_new;
+  p.k_cache = (TC*)k_cache; p.v_cache = (TC*)v_cache; p.khat_cache = w.qhat_rows; p.out = (TC*)out;
+  p.row_nnz = w.row_nnz; p.ref_in = w.qhat[qhat_sel]; p.ref_out = w.qhat[qhat_sel ^ 1]; p.R = w.R;
+  p.partial = w.dec_partial; p.ticket = w.dec_ticket; p.counters = w.counters;
+  p.n = n; p.T_max = s.T_max; p.H = s.H; p.W = window; p.theta = theta;
+  p.scale_log2e = 1.4426950408889634f / sqrtf((float)s.d);
+  p.ragged = n_b != nullptr;
+  p.b0 = 0;
+  const int G = s.g();
+  bool cluster;
+  decode_mma_slices(s, n + 1, &p.nsplit, &p.chunk, &cluster);
+  if (p.nsplit > kMaxDecodeSplits) return cudaErrorInvalidValue;
+  cudaError_t err = cudaSuccess;
+  for (; p.b0 < s.B && err == cudaSuccess; p.b0 += kRaggedMax) {
+    const int nb = n_b ? (s.B - p.b0 < kRaggedMax ? s.B - p.b0 : kRaggedMax) : s.B;
+    if (n_b)
+      for (int i = 0; i < nb; ++i) p.n_b[i] = n_b[p.b0 + i];
+#define GO(DD, GG)                                                                                           \
+    err = key ? (cluster ? launch_mma<DD, GG, true, true>(*tk, *tv, *th, p, nb * s.H_kv, st)                                \
+                         : launch_mma<DD, GG, true, false>(*tk, *tv, *th, p, nb * s.H_kv, st))                              \
+              : (cluster ? launch_mma<DD, GG, false, true>(*tk, *tv, *th, p, nb * s.H_kv, st)                               \
+                         : launch_mma<DD, GG, false, false>(*tk, *tv, *th, p, nb * s.H_kv, st))
+#define GO_G(DD)                                                                                             \
+    switch (G) {                                                                                             \
+      case 1: GO(DD, 1); break;                                                                              \
+      case 2: GO(DD, 2); break;                                                                              \
+      case 4: GO(DD, 4); break;                                                                              \
+      case 8: GO(DD, 8); break;                                                                              \
+      default: return cudaErrorInvalidValue;                                                                 \
+    }
+    if (s.d == 64) { GO_G(64) } else { GO_G(128) }
+#undef GO_G
+#undef GO
+    if (!n_b) break;
+  }
+  return err;
+}
+
+}  // namespace delta
