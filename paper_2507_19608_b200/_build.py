@@ -5,11 +5,14 @@ from __future__ import annotations
 import os
 import shutil
 import subprocess
+import sysconfig
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libdelta_attn.so")
 LIB_DEBUG = os.path.join(HERE, "libdelta_attn_dbg.so")      # the same sources with -DDELTA_DEBUG_BOUNDS
+CALLS = os.path.join(HERE, "_calls.so")                      # CPython entry points over the library
+CALLS_SOURCE = "py_calls.cpp"
 SOURCES = ["api.cu", "k1_delta_construct.cu", "k2_hybrid_attn_generic.cu", "k2_hybrid_attn_tc.cu", "k2_hybrid_attn_tcq.cu",
            "k3_decode_step.cu", "k3_decode_step_mma.cu", "k3_decode_step_key.cu", "k3_decode_step_keypacked.cu", "decode_noalloc.cu"]
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
@@ -28,10 +31,24 @@ def _stale(lib: str) -> bool:
     if not os.path.exists(lib):
         return True
     t = os.path.getmtime(lib)
-    deps = [os.path.join(CSRC, f) for f in os.listdir(CSRC)]
+    deps = [os.path.join(CSRC, f) for f in os.listdir(CSRC) if f != CALLS_SOURCE]
     deps.append(os.path.join(os.path.dirname(HERE), "include", "delta_attn.h"))
     deps.append(os.path.abspath(__file__))
     return any(os.path.getmtime(d) > t for d in deps)
+
+
+def build_calls(force: bool = False) -> str:
+    """Compile the CPython entry points (g++, no CUDA) if missing or older than their source."""
+    src = os.path.join(CSRC, CALLS_SOURCE)
+    if not force and os.path.exists(CALLS) and os.path.getmtime(CALLS) >= os.path.getmtime(src):
+        return CALLS
+    cmd = [os.environ.get("CXX") or shutil.which("g++") or "g++", "-O2", "-std=c++17", "-shared", "-fPIC",
+           "-fvisibility=hidden", "-I", sysconfig.get_paths()["include"], "-o", CALLS + ".tmp", src]
+    r = subprocess.run(cmd, capture_output=True, text=True)
+    if r.returncode != 0:
+        raise RuntimeError("g++ failed:\n" + r.stdout + r.stderr)
+    os.replace(CALLS + ".tmp", CALLS)
+    return CALLS
 
 
 def build(force: bool = False, verbose: bool = False, debug_bounds: bool = False) -> str:
@@ -56,4 +73,5 @@ def build(force: bool = False, verbose: bool = False, debug_bounds: bool = False
 
 if __name__ == "__main__":
     import sys
+    print(build_calls(force="--force" in sys.argv))
     print(build(force="--force" in sys.argv, verbose="-v" in sys.argv, debug_bounds="--debug-bounds" in sys.argv))

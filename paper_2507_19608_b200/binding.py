@@ -8,6 +8,8 @@ or loaded, importing this module raises.
 from __future__ import annotations
 
 import ctypes as C
+import importlib.machinery
+import importlib.util
 import os
 
 from . import _build
@@ -139,11 +141,34 @@ def _ptr(t):
     raise TypeError(type(t))
 
 
+def _torch_streams():
+    """(current device, raw stream of a device): torch's own lookups behind current_stream(), whose
+    Stream object costs 3.4 us a call."""
+    import torch
+    torch.cuda.current_stream()          # brings CUDA up
+    return torch._C._cuda_getDevice, torch._C._cuda_getCurrentRawStream
+
+
+_lookup = None
+
+
 def _stream(stream):
     if stream is None:
-        import torch
-        return torch.cuda.current_stream().cuda_stream
+        global _lookup
+        if _lookup is None:
+            _lookup = _torch_streams()
+        return _lookup[1](_lookup[0]())
     return int(getattr(stream, "cuda_stream", stream))
+
+
+def _load_calls():
+    """The CPython entry points of the two calls on a serving loop's path (csrc/py_calls.cpp)."""
+    loader = importlib.machinery.ExtensionFileLoader("_calls", _build.build_calls())
+    mod = importlib.util.module_from_spec(importlib.util.spec_from_loader("_calls", loader))
+    loader.exec_module(mod)
+    address = lambda f: C.cast(f, C.c_void_p).value      # noqa: E731
+    mod.setup(address(lib.delta_attn_decode_step), address(lib.delta_attn_prefill), _ptr, _stream, _check, _torch_streams)
+    return mod
 
 
 def make_config(B, H, H_kv, d, T_max, dtype="bf16", source=DELTA_SRC_QUERY,
@@ -163,9 +188,11 @@ class DeltaState:
 
     def __init__(self, cfg: delta_config_t, handle, workspace):
         self.cfg, self.handle, self.workspace = cfg, handle, workspace
+        self.raw = handle.value        # the handle as an integer, for the native entry points
+        self.views = {}                # (array, address) -> tensor over the workspace
 
     def __del__(self):
-        h, self.handle = getattr(self, "handle", None), None
+        h, self.handle, self.raw = getattr(self, "handle", None), None, 0
         if h and lib is not None:      # module globals are gone while the interpreter shuts down
             lib.delta_state_destroy(h)
 
@@ -183,12 +210,14 @@ def delta_state_init(cfg: delta_config_t, device="cuda", stream=None, workspace=
 
 
 def delta_state_reset(st: DeltaState, stream=None):
-    _check(lib.delta_state_reset(st.handle, _stream(stream)), "delta_state_reset")
+    # (host-side only: the library does not use the stream)
+    _check(lib.delta_state_reset(st.handle, None if stream is None else _stream(stream)), "delta_state_reset")
 
 
-def delta_attn_prefill(st: DeltaState, q, k, v, out, T, H, H_kv, d, theta, window, stream=None):
-    _check(lib.delta_attn_prefill(st.handle, _ptr(q), _ptr(k), _ptr(v), _ptr(out), T, H, H_kv, d,
-                                  theta, window, _stream(stream)), "delta_attn_prefill")
+_calls = _load_calls()
+
+# delta_attn_prefill(st, q, k, v, out, T, H, H_kv, d, theta, window, stream=None)
+delta_attn_prefill = _calls.delta_attn_prefill
 
 
 def delta_attn_prefill_varlen(st: DeltaState, q, k, v, out, seq_lens, windows, theta, stream=None):
@@ -218,11 +247,8 @@ def delta_attn_prefill_host(st: DeltaState, q_host, k_host, v_host, out_host, st
                                        window, _stream(stream)), "delta_attn_prefill_host")
 
 
-def delta_attn_decode_step(st: DeltaState, q_new, k_new, v_new, k_cache, v_cache, out, theta, window,
-                           stream=None):
-    _check(lib.delta_attn_decode_step(st.handle, _ptr(q_new), _ptr(k_new), _ptr(v_new),
-                                      _ptr(k_cache), _ptr(v_cache), _ptr(out), theta, window,
-                                      _stream(stream)), "delta_attn_decode_step")
+# delta_attn_decode_step(st, q_new, k_new, v_new, k_cache, v_cache, out, theta, window, stream=None)
+delta_attn_decode_step = _calls.delta_attn_decode_step
 
 
 def delta_attn_decode_step_noalloc(q_new, k_new, v_new, k_cache, v_cache, out, qhat_in, qhat_out, R,
@@ -308,6 +334,9 @@ def delta_state_view(st: DeltaState, what: int):
     import torch
     p, n = C.c_void_p(), C.c_size_t(0)
     _check(lib.delta_state_view(st.handle, what, C.byref(p), C.byref(n)), "delta_state_view")
+    t = st.views.get((what, p.value))
+    if t is not None:
+        return t.detach()               # another tensor over the same memory
     off = p.value - st.workspace.data_ptr()
     raw = st.workspace[off:off + n.value]
     c = st.cfg
@@ -317,4 +346,5 @@ def delta_state_view(st: DeltaState, what: int):
               DELTA_VIEW_IDX: (c.B, c.H, c.T_max, c.d), DELTA_VIEW_QHAT_TILE: (c.B, c.H, nt, c.d),
               DELTA_VIEW_QHAT: (c.B, c.H, c.d), DELTA_VIEW_R: (c.B, c.H, c.T_max),
               DELTA_VIEW_COUNTERS: (n.value // 8,)}
-    return raw.view(getattr(torch, _VIEW_DTYPES[what])).view(shapes[what])
+    t = st.views[(what, p.value)] = raw.view(getattr(torch, _VIEW_DTYPES[what])).view(shapes[what])
+    return t.detach()
