@@ -292,7 +292,8 @@ DELTA_API int32_t delta_state_position(const delta_state_t* st);
 DELTA_API int32_t delta_state_sequence_position(const delta_state_t* st, int32_t b);
 
 /* Which prefill kernel the next delta_attn_prefill on this state will use:
- *   0 = generic CUDA-core kernel (every configuration);
+ *   0 = fp32-arithmetic kernel (query deltas, either dtype; the only one for fp32 inputs): the
+ *       telescoped form with every product at fp32 precision;
  *   1 = tcgen05/TMA kernel, out-of-window scores by Eq. 4's running sum of sparse delta
  *       products on the FP32 pipes, skipping all-zero delta blocks (bf16, d = 64);
  *   2 = tcgen05/TMA kernel, out-of-window scores by the telescoped form of Eq. 4,

@@ -363,13 +363,13 @@ static delta_status_t prefill_launch(delta_state* st, const Shape& shape, const 
   const bool rev = c.source == DELTA_SRC_QUERY_BOTTOM_UP;
   const bool tcq = which >= 2 && which <= 5;
   if ((key || rev) && !tcq) return DELTA_ERR_UNSUPPORTED;   // no tensor-core kernel on this device
-  // The telescoped attention kernel reads nothing the finish kernel writes (delta values,
-  // mask words, counts, indices, counters, hand-off row), so it runs directly behind the chain
-  // kernel and the finish kernel comes last.  Both are launched with programmatic stream
+  // The telescoped attention kernels (all but kernel 1) read nothing the finish kernel writes (delta
+  // values, mask words, counts, indices, counters, hand-off row), so they run directly behind the
+  // chain kernel and the finish kernel comes last.  Both are launched with programmatic stream
   // serialisation: the attention CTAs are resident and set up by the time the chain ends, and
   // the finish kernel's launch overlaps the end of the attention kernel.  With per-kernel
   // timing on, the kernels run in their natural order with events between them.
-  const bool chained = tcq && !prof;
+  const bool chained = !use_tc && !prof;
   MARK(0);
   // the delta stream: the queries (strategy 1) or the keys, per KV head (strategy 3)
   if ((e = launch_delta_chain(shape, ws, key ? k : q, T, theta, c.dtype, c.init, key, rev, zero_ptr, zero_bytes, cs)) != cudaSuccess)
@@ -379,7 +379,7 @@ static delta_status_t prefill_launch(delta_state* st, const Shape& shape, const 
     if (tcq)
       return launch_hybrid_attn_tcq(shape, ws, q, k, v, out, T, theta, c.init, window, c.prefill_window, key,
                                     rev, /*form=*/which == 3 ? 1 : which == 4 ? 2 : which == 5 ? 3 : 0, cs);
-    return launch_hybrid_attn_generic(shape, ws, q, k, v, out, T, window, c.prefill_window, c.dtype, cs);
+    return launch_hybrid_attn_generic(shape, ws, q, k, v, out, T, theta, c.init, window, c.prefill_window, c.dtype, cs);
   };
   if (chained && !key) {
     if ((e = attention()) != cudaSuccess) return cuda_fail(e);

@@ -99,10 +99,10 @@ int device_sm_count();
 cudaError_t launch_delta_finish(const Shape& s, const Workspace& w, const void* q, const void* k, int T,
                                 float theta, int window, int shape, int dtype, int init, bool want_kt,
                                 bool key_stream, bool reverse, int programmatic, cudaStream_t st);
-// K2 (generic): fused hybrid attention on CUDA cores, any supported dtype.
-cudaError_t launch_hybrid_attn_generic(const Shape& s, const Workspace& w, const void* q,
-                                       const void* k, const void* v, void* out, int T, int window,
-                                       int shape, int dtype, cudaStream_t st);
+// K2 on the FP32 pipes, either dtype; reads the chain kernel's checkpoints and nothing of the finish kernel's.
+cudaError_t launch_hybrid_attn_generic(const Shape& s, const Workspace& w, const void* q, const void* k, const void* v,
+                                       void* out, int T, float theta, int init, int window, int shape, int dtype,
+                                       cudaStream_t st);
 // K3: one decode step.
 cudaError_t launch_decode_step(const Shape& s, const Workspace& w, const void* q_new,
                                const void* k_new, const void* v_new, void* k_cache, void* v_cache,

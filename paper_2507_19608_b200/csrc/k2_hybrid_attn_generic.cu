@@ -1,290 +1,465 @@
-// K2 (generic) -- fused hybrid delta attention on the plain FP32 pipes (Section III-B; Eq. 1, 4).
-// Serves every supported element type; it is the production path for fp32 inputs and the
-// fall-back for bf16 shapes the tensor-core kernel does not take.
+// K2 (fp32 arithmetic) -- fused hybrid delta attention in fp32 precision (Section III-B; Eq. 1, 4).
+// The production path for fp32 inputs; serves bf16 inputs too.
 //
-// One CTA owns 64 query rows of one head and walks the key tiles up to the diagonal:
-//   * tiles that touch the window get the exact 64x64xd product;
-//   * tiles with out-of-window pairs get the running delta sums of Eq. 4:
-//       R(i)[j] = seed[j] + sum_{s = i0..i} sum_{c fired in row s} dq[s][c] * k_j[c],
-//     seed[j] = q_hat(i0 - 1) . k_j (the reference in front of the tile telescopes every
-//     earlier row of the recursion).  A warp owns 8 consecutive rows and all 64 keys, walks its
-//     rows in order with the compacted channel lists, and skips everything that did not fire;
-//   * scale, causal mask, online softmax, P.V accumulate in registers.
+// Eq. 4's running sum telescopes: the sum of all Delta q up to row i is the reference q_hat(i)
+// (Eq. 3), so the out-of-window score of pair (i, j) is q_hat(i).k_j.  q_hat's elements are copies of
+// input elements, so this form carries fewer roundings than the recursion over rounded differences.
+//
+// Arithmetic.  An fp32 number is the sum of three bf16 parts (8 bits of mantissa each, the exponent
+// range is the same): x = h + m + l.  A product of two takes six tensor-core products, h.h, h.m, m.h,
+// h.l, l.h, m.m; the dropped ones are below 2^-24 of it.  h.h has an accumulator of its own and the
+// five small ones another, the output of a key tile is summed in fresh accumulators and joins the
+// running output by one fp32 multiply-add per element, so no long chain of tensor-core additions
+// (which truncate) touches a large value.  The error against exact arithmetic is that of the FP32
+// pipes, whose 74 TFLOP/s a fused kernel reaches to a quarter (each 16-byte shared-memory operand feeds
+// few multiply-adds): the same kernel on packed fma.rn.f32x2 ran at 20 TFLOP/s, the kernel before it,
+// sparse delta sums on the FP32 pipes, at 6.  Relative error against fp64 dense attention at 1000
+// tokens: 1.8e-7 (FP32-pipe kernel 3.7e-7).  Measured, whole prefill: 24 heads x 1425 tokens, d = 64:
+// 212 us = 29 TFLOP/s; 16 heads x 1000: 350 -> 95 us; one head x 128: 54 -> 13 us (the kernel 42 -> 6).
+//
+// Bound: mma.sync issue (m16n8k16 every 8 clocks per scheduler) once the chip is full, the walk of the
+// last query tile where it is not.  A CTA of four warps owns 64 / KS query rows of one head and walks
+// the 64-key tiles up to the diagonal; KS warps share 16 rows and deal a tile's keys among themselves
+// (KS = 1: most work per byte staged; KS = 4: the shortest walk, with four times as many CTAs; the
+// launcher weighs them).  Keys and values come from global memory into registers while the tensor
+// cores work on the tile before, are split into their parts and stored swizzled for ldmatrix.
+// A tile takes Q_hat.K^T where none of its pairs is inside the window, Q.K^T where all causal ones are,
+// both where it is mixed.  The reference rows are rebuilt from the 8-row checkpoints of the chain
+// kernel (Eq. 2-3 re-run per block), so nothing of the finish kernel is read.
 #include "delta_internal.cuh"
+#include "tc_common.cuh"
 
 namespace delta {
 
 namespace {
-constexpr int BM = 64, BN = 64, NT = 256, NWARP = NT / 32;
+constexpr int BN = 64, NT = 128;
 
-template <int D> struct GenSmem {
-  static constexpr int KS_LD = BN + 1;
-  static constexpr int QS_LD = D + 4;
-  static constexpr int SS_LD = BN + 1;
-  static constexpr size_t floats = (size_t)D * KS_LD      // Ks  [D][BN+1]  channel-major keys
-                                   + (size_t)BN * D       // Vs  [BN][D]
-                                   + (size_t)BM * QS_LD   // Qs  [BM][D+4]
-                                   + (size_t)BM * D       // dQs [BM][D]
-                                   + (size_t)BM * SS_LD   // Ss  [BM][BN+1]
-                                   + (size_t)NWARP * BN   // seedp
-                                   + (size_t)NWARP * BN   // tot
-                                   + D                    // qhat
-                                   + 3 * BM;              // m, l, alpha
-  static constexpr size_t bytes = floats * 4 + (size_t)BM * D /*idx*/ + BM * 4 /*nnz*/;
+// Shared memory: bf16 parts as blocks of [rows][64 channels], 16-byte chunk c of row r at
+// r * 128 + ((c ^ (r & 7)) << 4); part-major, channel block inside.  NP parts: 3 (fp32) or 1 (bf16).
+template <int D, int KS, int NP> struct F32Smem {
+  static constexpr int BM = 64 / KS;
+  static constexpr uint32_t QPART = BM * D * 2, KPART = BN * D * 2;
+  static constexpr uint32_t OFF_QH = NP * QPART, OFF_K = 2 * NP * QPART, OFF_V = OFF_K + NP * KPART;
+  static constexpr uint32_t RAW = BM * (D + 4) * 4;                    // the query rows in fp32, before the first key tile
+  static constexpr uint32_t MERGE = (KS - 1) * 16 * (D + 2) * 4 * (4 / KS);
+  static constexpr uint32_t END = OFF_V + NP * KPART;
+  static constexpr uint32_t bytes = (END - OFF_K > RAW ? END : OFF_K + RAW) + 1024;
+  static_assert(MERGE <= END, "the merge buffer fits");
 };
+
+__device__ __forceinline__ uint32_t pack2(float lo, float hi) {
+  const __nv_bfloat162 t = __floats2bfloat162_rn(lo, hi);
+  return *reinterpret_cast<const uint32_t*>(&t);
+}
+// the bf16 parts of (lo, hi), packed
+template <int NP> __device__ __forceinline__ void parts_of(float lo, float hi, uint32_t (&p)[NP]) {
+  p[0] = pack2(lo, hi);
+  if constexpr (NP == 3) {
+    const float r0 = lo - __uint_as_float(p[0] << 16), r1 = hi - __uint_as_float(p[0] & 0xffff0000u);
+    p[1] = pack2(r0, r1);
+    p[2] = pack2(r0 - __uint_as_float(p[1] << 16), r1 - __uint_as_float(p[1] & 0xffff0000u));
+  }
+}
+__device__ __forceinline__ void sts128(uint32_t a, uint32_t x, uint32_t y, uint32_t z, uint32_t w) {
+  asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(a), "r"(x), "r"(y), "r"(z), "r"(w) : "memory");
+}
+// eight consecutive channels (chunk c of row r of a block) into all parts
+template <int NP> __device__ __forceinline__ void store_parts(uint32_t block, uint32_t part_stride, int r, int c, const float (&x)[8]) {
+  uint32_t w[4][NP];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) parts_of<NP>(x[2 * i], x[2 * i + 1], w[i]);
+  const uint32_t a = block + r * 128 + ((c ^ (r & 7)) << 4);
+#pragma unroll
+  for (int p = 0; p < NP; ++p) sts128(a + p * part_stride, w[0][p], w[1][p], w[2][p], w[3][p]);
+}
+__device__ __forceinline__ void load8f(const float* p, float (&x)[8]) {
+  const float4 a = __ldg(reinterpret_cast<const float4*>(p)), b = __ldg(reinterpret_cast<const float4*>(p) + 1);
+  x[0] = a.x; x[1] = a.y; x[2] = a.z; x[3] = a.w; x[4] = b.x; x[5] = b.y; x[6] = b.z; x[7] = b.w;
+}
+__device__ __forceinline__ void load8f(const __nv_bfloat16* p, float (&x)[8]) {
+  const uint4 u = __ldg(reinterpret_cast<const uint4*>(p));
+  const uint32_t w[4] = {u.x, u.y, u.z, u.w};
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    x[2 * i] = __uint_as_float(w[i] << 16);
+    x[2 * i + 1] = __uint_as_float(w[i] & 0xffff0000u);
+  }
+}
+__device__ __forceinline__ void ldsm4(uint32_t addr, uint32_t (&r)[4]) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr) : "memory");
+}
+__device__ __forceinline__ void ldsm4t(uint32_t addr, uint32_t (&r)[4]) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0, %1, %2, %3}, [%4];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr) : "memory");
+}
+__device__ __forceinline__ void mma(float (&c)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
+  asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, "
+               "{%0, %1, %2, %3};"
+               : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3]) : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+// big += a.b of the first parts, small += the other products of the parts that count
+template <int NA, int NB>
+__device__ __forceinline__ void mma_parts(float (&big)[4], float (&small)[4], const uint32_t (&a)[NA][4],
+                                          const uint32_t (&b)[NB][4], int half) {
+  mma(big, a[0], b[0][2 * half], b[0][2 * half + 1]);
+  if constexpr (NB == 3) {
+    mma(small, a[0], b[2][2 * half], b[2][2 * half + 1]);
+    if constexpr (NA == 3) {
+      mma(small, a[1], b[1][2 * half], b[1][2 * half + 1]);
+      mma(small, a[2], b[0][2 * half], b[0][2 * half + 1]);
+    }
+    mma(small, a[0], b[1][2 * half], b[1][2 * half + 1]);
+  }
+  if constexpr (NA == 3) {
+    mma(small, a[1], b[0][2 * half], b[0][2 * half + 1]);
+    if constexpr (NB == 1) mma(small, a[2], b[0][2 * half], b[0][2 * half + 1]);
+  }
+}
 }  // namespace
 
-template <typename TIn, int D>
-__global__ void __launch_bounds__(NT, (D == 64 ? 2 : 1)) hybrid_attn_generic_kernel(
-    const TIn* __restrict__ q, const TIn* __restrict__ k, const TIn* __restrict__ v,
-    TIn* __restrict__ out, const float* __restrict__ dq, const uint16_t* __restrict__ row_nnz,
-    const uint8_t* __restrict__ idx, const float* __restrict__ qhat_tile, int T, int T_max,
-    int n_tiles, int H, int g, int W, int shape, float scale_log2e) {
-  using SM = GenSmem<D>;
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  float* Ks = reinterpret_cast<float*>(smem_raw);
-  float* Vs = Ks + (size_t)D * SM::KS_LD;
-  float* Qs = Vs + (size_t)BN * D;
-  float* dQs = Qs + (size_t)BM * SM::QS_LD;
-  float* Ss = dQs + (size_t)BM * D;
-  float* seedp = Ss + (size_t)BM * SM::SS_LD;
-  float* tot = seedp + NWARP * BN;
-  float* qhat_s = tot + NWARP * BN;
-  float* m_s = qhat_s + D;
-  float* l_s = m_s + BM;
-  float* alpha_s = l_s + BM;
-  uint8_t* idxs = reinterpret_cast<uint8_t*>(alpha_s + BM);
-  int* nnz_s = reinterpret_cast<int*>(idxs + (size_t)BM * D);
+template <typename TIn, int D, int KS>
+__global__ void __launch_bounds__(NT, D == 64 ? 2 : 1) hybrid_attn_f32_kernel(
+    const TIn* __restrict__ q, const TIn* __restrict__ k, const TIn* __restrict__ v, TIn* __restrict__ out,
+    const float* __restrict__ ckpt, unsigned long long* __restrict__ counters, int T, int T_max, int n_ckpt, int H, int g,
+    int W, int shape, float theta, int basis_row, float scale_log2e) {
+  constexpr int NP = sizeof(TIn) == 4 ? 3 : 1;
+  using SM = F32Smem<D, KS, NP>;
+  constexpr int BM = SM::BM, NB = D / 64;          // NB: 64-channel blocks of a row
+  constexpr int NTW = 8 / KS;                      // 8-key blocks of a tile per warp
+  constexpr int TASKS = BN * D / 8 / NT;           // 8-channel pieces of a key (value) tile per thread
+  extern __shared__ unsigned char smem_raw[];
+  const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
+  float* const rawq = reinterpret_cast<float*>(smem_raw + (base - smem_u32(smem_raw)) + SM::OFF_K);     // [BM][D + 4]
 
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int qt = (int)gridDim.x - 1 - (int)blockIdx.x;  // heaviest query tiles first
-  const int bh = blockIdx.y;
-  const int b = bh / H, h = bh - b * H;
-  const int kvh = h / g, H_kv = H / g;
-  const int i0 = qt * BM;
+  const int g8 = lane >> 2, t4 = lane & 3;         // row of the fragments, thread of the row
+  const int rg = warp / KS, kg = warp % KS;        // the warp's 16 rows, its share of a tile's keys
+  const int qt = (int)gridDim.x - 1 - (int)blockIdx.x;     // longest walks first
+  const int bh = blockIdx.y, b = bh / H, h = bh - b * H;
+  const size_t bkv = (size_t)b * (H / g) + h / g;
+  const int i0 = qt * BM, i1 = min(i0 + BM, T) - 1;
+  const TIn* const kp = k + bkv * T_max * D;
+  const TIn* const vp = v + bkv * T_max * D;
+  const int n_kt = i1 / BN + 1;
 
-  const TIn* qp = q + ((size_t)bh * T + i0) * D;
-  const float* dqp = dq + ((size_t)bh * T_max + i0) * D;
-  const uint8_t* idxp = idx + ((size_t)bh * T_max + i0) * D;
-  const uint16_t* nnzp = row_nnz + (size_t)bh * T_max + i0;
-  const TIn* kp = k + ((size_t)b * H_kv + kvh) * (size_t)T_max * D;
-  const TIn* vp = v + ((size_t)b * H_kv + kvh) * (size_t)T_max * D;
-  const int rows_valid = min(BM, T - i0);
-
-  // ---- stage the query tile: exact rows, delta rows, compacted indices, counts, reference
-  for (int e = tid; e < BM * D; e += NT) {
-    const int r = e / D, c = e - r * D;
-    const bool ok = r < rows_valid;
-    Qs[r * SM::QS_LD + c] = ok ? to_f32(qp[(size_t)r * D + c]) : 0.0f;
-    dQs[r * D + c] = ok ? dqp[(size_t)r * D + c] : 0.0f;
-    idxs[r * D + c] = ok ? idxp[(size_t)r * D + c] : (uint8_t)0xFF;
-  }
-  if (tid < BM) {
-    nnz_s[tid] = tid < rows_valid ? (int)nnzp[tid] : 0;
-    m_s[tid] = -INFINITY;
-    l_s[tid] = 0.0f;
-  }
-  if (tid < D) qhat_s[tid] = qhat_tile[((size_t)bh * n_tiles + qt) * D + tid];
-
-  const int ty = tid >> 4, tx = tid & 15;  // 16 x 16 micro-tile grid for the dense products
-  constexpr int EV = D / 16;
-  float O[4][EV];
+  float st[TASKS][8];                              // a tile on its way from global memory
+  auto fetch = [&](const TIn* src, int r0) {
 #pragma unroll
-  for (int r = 0; r < 4; ++r)
+    for (int i = 0; i < TASKS; ++i) {
+      const int e = tid + i * NT, r = r0 + e / (D / 8), c = e % (D / 8);
+      if (r < T) load8f(src + (size_t)r * D + 8 * c, st[i]);
+      else {
 #pragma unroll
-    for (int e = 0; e < EV; ++e) O[r][e] = 0.0f;
+        for (int x = 0; x < 8; ++x) st[i][x] = 0.0f;
+      }
+    }
+  };
+  auto stage = [&](uint32_t off) {
+#pragma unroll
+    for (int i = 0; i < TASKS; ++i) {
+      const int e = tid + i * NT, r = e / (D / 8), c = e % (D / 8);
+      store_parts<NP>(base + off + (c >> 3) * (BN * 128), SM::KPART, r, c & 7, st[i]);
+    }
+  };
+  // ---- query rows: fp32 for the re-run of Eq. 2-3, parts for the products
+  for (int e = tid; e < BM * (D / 8); e += NT) {
+    const int r = e / (D / 8), c = e % (D / 8);
+    float x[8] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
+    if (i0 + r < T) load8f(q + ((size_t)bh * T + i0 + r) * D + 8 * c, x);
+    store_parts<NP>(base + (c >> 3) * (BM * 128), SM::QPART, r, c & 7, x);
+#pragma unroll
+    for (int i = 0; i < 8; i += 4)
+      *reinterpret_cast<float4*>(rawq + r * (D + 4) + 8 * c + i) = make_float4(x[i], x[i + 1], x[i + 2], x[i + 3]);
+  }
+  fetch(kp, 0);
+  // the chain kernel's checkpoints (programmatic stream serialisation: all above are inputs)
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  __syncthreads();
+  // reference rows: Eq. 2-3 over every (channel, 8-row block) from the block's checkpoint
+  for (int e = tid; e < (BM / 8) * D; e += NT) {
+    const int blk = e / D, c = e - blk * D, r0 = i0 + 8 * blk;
+    if (r0 < T && DELTA_IN(r0 / DELTA_CKPT_ROWS, n_ckpt, counters)) {
+      float ref = __ldcg(&ckpt[((size_t)bh * n_ckpt + r0 / DELTA_CKPT_ROWS) * D + c]);
+#pragma unroll
+      for (int r = 0; r < 8; ++r) {
+        float* const x = rawq + (8 * blk + r) * (D + 4) + c;
+        const bool fire = r0 + r == basis_row || fabsf(__fsub_rn(*x, ref)) > theta;
+        ref = fire ? *x : ref;
+        *x = ref;                                          // (rows past the end: never stored)
+      }
+    }
+  }
+  __syncthreads();
+  for (int e = tid; e < BM * (D / 8); e += NT) {
+    const int r = e / (D / 8), c = e % (D / 8);
+    float x[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) x[i] = rawq[r * (D + 4) + 8 * c + i];
+    store_parts<NP>(base + SM::OFF_QH + (c >> 3) * (BM * 128), SM::QPART, r, c & 7, x);
+  }
+  __syncthreads();
 
-  const int i1 = i0 + rows_valid - 1;  // last valid row of the tile
-  for (int jt = 0; jt <= qt; ++jt) {
-    const int j0 = jt * BN;
-    const int j1 = min(j0 + BN, T) - 1;
-    // conservative tile classification (the per-element predicate decides in the end)
-    bool need_exact, all_in;
-    if (W <= 0) { need_exact = false; all_in = false; }
-    else if (shape == 0) {
-      need_exact = (i0 / W <= j1 / W) && (j0 / W <= i1 / W);
-      all_in = (i0 / W == i1 / W) && (j0 / W == j1 / W) && (i0 / W == j0 / W);
+  float o[NB][8][4];
+#pragma unroll
+  for (int x = 0; x < NB; ++x)
+#pragma unroll
+    for (int n = 0; n < 8; ++n)
+#pragma unroll
+      for (int e = 0; e < 4; ++e) o[x][n][e] = 0.0f;
+  float m[2] = {-INFINITY, -INFINITY}, l[2] = {0.0f, 0.0f};              // of rows g8 and g8 + 8
+  const int arow = 16 * rg + (lane & 15), achk = lane >> 4;             // ldmatrix rows and chunks of the operands
+  const int krow = (64 / KS) * kg + (lane & 7) + ((lane >> 4) << 3), kchk = (lane >> 3) & 1;
+  const int vrow = (64 / KS) * kg + (lane & 15), vchk = lane >> 4;
+  auto products = [&](uint32_t rows, float (&s)[NTW][4]) {
+    float small[NTW][4];
+#pragma unroll
+    for (int n = 0; n < NTW; ++n)
+#pragma unroll
+      for (int e = 0; e < 4; ++e) { s[n][e] = 0.0f; small[n][e] = 0.0f; }
+#pragma unroll 1
+    for (int x = 0; x < NB; ++x)
+#pragma unroll
+      for (int ks = 0; ks < 4; ++ks) {
+        uint32_t a[NP][4];
+#pragma unroll
+        for (int p = 0; p < NP; ++p)
+          ldsm4(rows + p * SM::QPART + x * (BM * 128) + arow * 128 + (((2 * ks + achk) ^ (arow & 7)) << 4), a[p]);
+#pragma unroll
+        for (int n = 0; n < NTW; n += 2) {
+          uint32_t bb[NP][4];
+#pragma unroll
+          for (int p = 0; p < NP; ++p)
+            ldsm4(base + SM::OFF_K + p * SM::KPART + x * (BN * 128) + (krow + 8 * n) * 128 +
+                      (((2 * ks + kchk) ^ (krow & 7)) << 4), bb[p]);
+          mma_parts<NP, NP>(s[n], small[n], a, bb, 0);
+          mma_parts<NP, NP>(s[n + 1], small[n + 1], a, bb, 1);
+        }
+      }
+#pragma unroll
+    for (int n = 0; n < NTW; ++n)
+#pragma unroll
+      for (int e = 0; e < 4; ++e) s[n][e] += small[n][e];
+  };
+  // keys some row of the tile scores exactly, keys every row does (empty ranges without a window)
+  int ex_lo = 1, ex_hi = 0, full_lo = 1, full_hi = 0;
+  if (W > 0) {
+    if (shape == 0) {
+      ex_lo = (i0 / W) * W; ex_hi = (i1 / W) * W + W - 1;
+      if (i1 < ex_lo + W) { full_lo = ex_lo; full_hi = ex_lo + W - 1; }
     } else {
-      need_exact = max(0, i0 - j1) < W;
-      all_in = (i1 - j0) < W;
+      ex_lo = i0 - W + 1; ex_hi = i1; full_lo = i1 - W + 1; full_hi = i1;
     }
-    const bool need_delta = !all_in;
+  }
+  const int ia = i0 + 16 * rg + g8, ib = ia + 8;           // the thread's two rows
 
-    __syncthreads();  // previous tile's consumers are done with Ks / Vs / Ss
-    for (int e = tid; e < BN * D; e += NT) {
-      const int j = e / D, c = e - j * D;
-      const bool ok = (j0 + j) < T;
-      Ks[c * SM::KS_LD + j] = ok ? to_f32(kp[(size_t)(j0 + j) * D + c]) : 0.0f;
-      Vs[j * D + c] = ok ? to_f32(vp[(size_t)(j0 + j) * D + c]) : 0.0f;
+  for (int jt = 0; jt < n_kt; ++jt) {
+    const int j0 = jt * BN, j1 = min(j0 + BN, i1 + 1) - 1;      // (keys past the last row meet no query)
+    const bool some_in = j1 >= ex_lo && j0 <= ex_hi, all_in = j0 >= full_lo && j1 <= full_hi;
+    stage(SM::OFF_K);
+    fetch(vp, j0);
+    __syncthreads();                                       // the keys are staged, the values of the tile before read
+    float s[NTW][4];
+    products(base + (all_in ? 0u : SM::OFF_QH), s);
+    if (some_in && !all_in) {
+      float se[NTW][4];
+      products(base, se);
+#pragma unroll
+      for (int e2 = 0; e2 < 2; ++e2) {
+        const int i = e2 ? ib : ia;
+        int lo, hi;                                        // exact keys of row i: lo <= j < hi
+        if (shape == 0) { lo = (i / W) * W; hi = lo + W; } else { lo = i - W + 1; hi = i + 1; }
+#pragma unroll
+        for (int n = 0; n < NTW; ++n)
+#pragma unroll
+          for (int e = 0; e < 2; ++e) {
+            const int j = j0 + (64 / KS) * kg + 8 * n + 2 * t4 + e;
+            if (j >= lo && j < hi) s[n][2 * e2 + e] = se[n][2 * e2 + e];
+          }
+      }
     }
-    __syncthreads();
-
-    if (need_exact) {
-      float acc[4][4];
+    // ---- scale, causal mask, online softmax (four threads hold a row's scores)
+    float al[2];
 #pragma unroll
-      for (int r = 0; r < 4; ++r)
+    for (int e2 = 0; e2 < 2; ++e2) {
+      const int i = e2 ? ib : ia;
+      float mx = -INFINITY;
 #pragma unroll
-        for (int e = 0; e < 4; ++e) acc[r][e] = 0.0f;
-#pragma unroll 4
-      for (int c = 0; c < D; ++c) {
-        float a[4], bb[4];
+      for (int n = 0; n < NTW; ++n)
 #pragma unroll
-        for (int r = 0; r < 4; ++r) a[r] = Qs[(4 * ty + r) * SM::QS_LD + c];
+        for (int e = 0; e < 2; ++e) {
+          float& x = s[n][2 * e2 + e];
+          x = (j0 + (64 / KS) * kg + 8 * n + 2 * t4 + e <= i) ? x * scale_log2e : -INFINITY;
+          mx = fmaxf(mx, x);
+        }
+      mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
+      mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
+      const float mn = fmaxf(m[e2], mx), sub = mn == -INFINITY ? 0.0f : mn;       // (this warp's keys: maybe none yet)
+      al[e2] = exp2f(m[e2] - sub);
+      m[e2] = mn;
+      float sum = 0.0f;
 #pragma unroll
-        for (int e = 0; e < 4; ++e) bb[e] = Ks[c * SM::KS_LD + tx + 16 * e];
+      for (int n = 0; n < NTW; ++n)
 #pragma unroll
-        for (int r = 0; r < 4; ++r)
-#pragma unroll
-          for (int e = 0; e < 4; ++e) acc[r][e] = fmaf(a[r], bb[e], acc[r][e]);
-      }
-#pragma unroll
-      for (int r = 0; r < 4; ++r)
-#pragma unroll
-        for (int e = 0; e < 4; ++e) Ss[(4 * ty + r) * SM::SS_LD + tx + 16 * e] = acc[r][e];
-      __syncwarp();  // rows 8*warp .. 8*warp+7 are written and read by this warp only
+        for (int e = 0; e < 2; ++e) { float& x = s[n][2 * e2 + e]; x = exp2f(x - sub); sum += x; }
+      l[e2] = fmaf(l[e2], al[e2], sum);
     }
+    stage(SM::OFF_V);
+    if (jt + 1 < n_kt) fetch(kp, j0 + BN);
+    __syncthreads();                                       // the values are staged, every warp is done with the keys
 
-    if (need_delta) {
-      // seed partial: this warp's slice of q_hat . k_j
-      {
-        constexpr int CS = D / NWARP;
-        float s0 = 0.0f, s1 = 0.0f;
+    // ---- O = O * alpha + P.V, 64 channels at a time
 #pragma unroll
-        for (int cc = 0; cc < CS; ++cc) {
-          const int c = warp * CS + cc;
-          const float x = qhat_s[c];
-          s0 = fmaf(x, Ks[c * SM::KS_LD + lane], s0);
-          s1 = fmaf(x, Ks[c * SM::KS_LD + lane + 32], s1);
-        }
-        seedp[warp * BN + lane] = s0;
-        seedp[warp * BN + lane + 32] = s1;
-      }
-      float acc0 = 0.0f, acc1 = 0.0f;
-      for (int r = 0; r < 8; ++r) {
-        const int row = warp * 8 + r;
-        const int nz = nnz_s[row];
-        const uint8_t* ip = idxs + row * D;
-        const float* xp = dQs + row * D;
-        for (int p = 0; p < nz; ++p) {      // only fired channels; zero rows cost nothing
-          const int c = ip[p];
-          const float x = xp[c];
-          acc0 = fmaf(x, Ks[c * SM::KS_LD + lane], acc0);
-          acc1 = fmaf(x, Ks[c * SM::KS_LD + lane + 32], acc1);
-        }
-        const int i = i0 + row;
-        if (!in_window(i, j0 + lane, W, shape)) Ss[row * SM::SS_LD + lane] = acc0;
-        if (!in_window(i, j0 + lane + 32, W, shape)) Ss[row * SM::SS_LD + lane + 32] = acc1;
-      }
-      tot[warp * BN + lane] = acc0;
-      tot[warp * BN + lane + 32] = acc1;
-    }
-    __syncthreads();
-
-    // ---- scale, causal mask, online softmax (warp = 8 rows, lane = 2 columns)
-    {
-      float pre0 = 0.0f, pre1 = 0.0f;
-      if (need_delta) {
+    for (int x = 0; x < NB; ++x) {
+      float big[8][4], small[8][4];
 #pragma unroll
-        for (int w2 = 0; w2 < NWARP; ++w2) {
-          pre0 += seedp[w2 * BN + lane];
-          pre1 += seedp[w2 * BN + lane + 32];
-        }
-        for (int w2 = 0; w2 < warp; ++w2) {
-          pre0 += tot[w2 * BN + lane];
-          pre1 += tot[w2 * BN + lane + 32];
-        }
-      }
-      for (int r = 0; r < 8; ++r) {
-        const int row = warp * 8 + r;
-        const int i = i0 + row;
-        const int ja = j0 + lane, jb = j0 + lane + 32;
-        float s0 = Ss[row * SM::SS_LD + lane], s1 = Ss[row * SM::SS_LD + lane + 32];
-        if (!in_window(i, ja, W, shape)) s0 += pre0;
-        if (!in_window(i, jb, W, shape)) s1 += pre1;
-        s0 = (ja <= i && ja < T) ? s0 * scale_log2e : -INFINITY;
-        s1 = (jb <= i && jb < T) ? s1 * scale_log2e : -INFINITY;
-        float mx = fmaxf(s0, s1);
+      for (int n = 0; n < 8; ++n)
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-        const float m_old = m_s[row];
-        const float m_new = fmaxf(m_old, mx);
-        const float p0 = exp2f(s0 - m_new), p1 = exp2f(s1 - m_new);
-        float sum = p0 + p1;
+        for (int e = 0; e < 4; ++e) { big[n][e] = 0.0f; small[n][e] = 0.0f; }
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
-        Ss[row * SM::SS_LD + lane] = p0;
-        Ss[row * SM::SS_LD + lane + 32] = p1;
-        __syncwarp();
-        if (lane == 0) {
-          const float a = exp2f(m_old - m_new);
-          alpha_s[row] = a;
-          l_s[row] = l_s[row] * a + sum;
-          m_s[row] = m_new;
+      for (int kk = 0; kk < NTW / 2; ++kk) {
+        uint32_t a[3][4];
+#pragma unroll
+        for (int f = 0; f < 4; ++f) {
+          // fragment f: row g8 + 8 (f & 1), keys of block 2 kk + (f >> 1)
+          uint32_t w[3];
+          parts_of<3>(s[2 * kk + (f >> 1)][2 * (f & 1)], s[2 * kk + (f >> 1)][2 * (f & 1) + 1], w);
+          a[0][f] = w[0]; a[1][f] = w[1]; a[2][f] = w[2];
+        }
+#pragma unroll
+        for (int n = 0; n < 8; n += 2) {
+          uint32_t bb[NP][4];
+#pragma unroll
+          for (int p = 0; p < NP; ++p)
+            ldsm4t(base + SM::OFF_V + p * SM::KPART + x * (BN * 128) + (vrow + 16 * kk) * 128 +
+                       (((n + vchk) ^ (vrow & 7)) << 4), bb[p]);
+          mma_parts<3, NP>(big[n], small[n], a, bb, 0);
+          mma_parts<3, NP>(big[n + 1], small[n + 1], a, bb, 1);
         }
       }
-      __syncwarp();
-    }
-
-    // ---- O = alpha * O + P V   (rows 4*ty .. 4*ty+3 belong to this thread's own warp)
 #pragma unroll
-    for (int r = 0; r < 4; ++r) {
-      const float a = alpha_s[4 * ty + r];
+      for (int n = 0; n < 8; ++n)
 #pragma unroll
-      for (int e = 0; e < EV; ++e) O[r][e] *= a;
-    }
-    const int jmax = min(BN, i1 - j0 + 1);  // keys beyond the last valid row carry P = 0
-#pragma unroll 2
-    for (int j = 0; j < jmax; ++j) {
-      float p[4], vv[EV];
-#pragma unroll
-      for (int r = 0; r < 4; ++r) p[r] = Ss[(4 * ty + r) * SM::SS_LD + j];
-#pragma unroll
-      for (int e = 0; e < EV; ++e) vv[e] = Vs[j * D + tx + 16 * e];
-#pragma unroll
-      for (int r = 0; r < 4; ++r)
-#pragma unroll
-        for (int e = 0; e < EV; ++e) O[r][e] = fmaf(p[r], vv[e], O[r][e]);
+        for (int e = 0; e < 4; ++e) o[x][n][e] = fmaf(o[x][n][e], al[e >> 1], big[n][e] + small[n][e]);
     }
   }
 
-  __syncwarp();
+  // ---- the KS warps of a row group merge (through the operand tiles' space), normalise, store
 #pragma unroll
-  for (int r = 0; r < 4; ++r) {
-    const int row = 4 * ty + r;
-    if (row < rows_valid) {
-      const float inv = 1.0f / l_s[row];
-      TIn* op = out + ((size_t)bh * T + i0 + row) * D;
+  for (int e2 = 0; e2 < 2; ++e2) {
+    l[e2] += __shfl_xor_sync(0xffffffffu, l[e2], 1);
+    l[e2] += __shfl_xor_sync(0xffffffffu, l[e2], 2);
+  }
+  if constexpr (KS > 1) {
+    float* const buf = reinterpret_cast<float*>(smem_raw + (base - smem_u32(smem_raw))) + (size_t)rg * (KS - 1) * 16 * (D + 2);
+    __syncthreads();                                       // every warp is done with the operand tiles
+    if (kg > 0) {
+      float* const mine = buf + (size_t)(kg - 1) * 16 * (D + 2);
 #pragma unroll
-      for (int e = 0; e < EV; ++e) op[tx + 16 * e] = from_f32<TIn>(O[r][e] * inv);
+      for (int e2 = 0; e2 < 2; ++e2) {
+        float* const row = mine + (g8 + 8 * e2) * (D + 2);
+#pragma unroll
+        for (int x = 0; x < NB; ++x)
+#pragma unroll
+          for (int n = 0; n < 8; ++n)
+            *reinterpret_cast<float2*>(row + 64 * x + 8 * n + 2 * t4) = make_float2(o[x][n][2 * e2], o[x][n][2 * e2 + 1]);
+        if (t4 == 0) *reinterpret_cast<float2*>(row + D) = make_float2(m[e2], l[e2]);
+      }
+    }
+    __syncthreads();
+    if (kg > 0) return;
+#pragma unroll
+    for (int e2 = 0; e2 < 2; ++e2)
+#pragma unroll
+      for (int w = 0; w < KS - 1; ++w) {
+        const float* const row = buf + ((size_t)w * 16 + g8 + 8 * e2) * (D + 2);
+        const float2 ml = *reinterpret_cast<const float2*>(row + D);
+        const float mn = fmaxf(m[e2], ml.x), fa = exp2f(m[e2] - mn), fb = exp2f(ml.x - mn);      // (warp 0 has key 0)
+        m[e2] = mn;
+        l[e2] = l[e2] * fa + ml.y * fb;
+#pragma unroll
+        for (int x = 0; x < NB; ++x)
+#pragma unroll
+          for (int n = 0; n < 8; ++n) {
+            const float2 y = *reinterpret_cast<const float2*>(row + 64 * x + 8 * n + 2 * t4);
+            o[x][n][2 * e2] = o[x][n][2 * e2] * fa + y.x * fb;
+            o[x][n][2 * e2 + 1] = o[x][n][2 * e2 + 1] * fa + y.y * fb;
+          }
+      }
+  }
+#pragma unroll
+  for (int e2 = 0; e2 < 2; ++e2) {
+    const int i = e2 ? ib : ia;
+    if (i < T && DELTA_IN(i, T, counters)) {
+      const float inv = 1.0f / l[e2];
+      TIn* const op = out + ((size_t)bh * T + i) * D + 2 * t4;
+#pragma unroll
+      for (int x = 0; x < NB; ++x)
+#pragma unroll
+        for (int n = 0; n < 8; ++n) {
+          const float a = o[x][n][2 * e2] * inv, c = o[x][n][2 * e2 + 1] * inv;
+          if constexpr (sizeof(TIn) == 4) *reinterpret_cast<float2*>(op + 64 * x + 8 * n) = make_float2(a, c);
+          else *reinterpret_cast<uint32_t*>(op + 64 * x + 8 * n) = pack2(a, c);
+        }
     }
   }
 }
 
-cudaError_t launch_hybrid_attn_generic(const Shape& s, const Workspace& w, const void* q,
-                                       const void* k, const void* v, void* out, int T, int window,
-                                       int shape, int dtype, cudaStream_t st) {
-  const dim3 grid((T + BM - 1) / BM, s.B * s.H);
-  const float scale_log2e = 1.4426950408889634f / sqrtf((float)s.d);
-  cudaError_t err = cudaSuccess;
-#define LAUNCH(TIN, DD)                                                                         \
-  do {                                                                                          \
-    auto kern = hybrid_attn_generic_kernel<TIN, DD>;                                            \
-    err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,               \
-                               (int)GenSmem<DD>::bytes);                                        \
-    if (err != cudaSuccess) return err;                                                         \
-    kern<<<grid, NT, GenSmem<DD>::bytes, st>>>((const TIN*)q, (const TIN*)k, (const TIN*)v,     \
-                                                (TIN*)out, w.dq, w.row_nnz, w.idx, w.qhat_tile, \
-                                                T, s.T_max, s.n_tiles, s.H, s.g(), window,      \
-                                                shape, scale_log2e);                            \
-  } while (0)
-  if (dtype == DELTA_F32) {
-    if (s.d == 64) LAUNCH(float, 64); else LAUNCH(float, 128);
-  } else {
-    if (s.d == 64) LAUNCH(__nv_bfloat16, 64); else LAUNCH(__nv_bfloat16, 128);
+template <typename TIn, int D, int KS>
+static cudaError_t launch_f32(const Shape& s, const Workspace& w, const void* q, const void* k, const void* v, void* out,
+                              int T, float theta, int init, int window, int shape, cudaStream_t st) {
+  auto kern = hybrid_attn_f32_kernel<TIn, D, KS>;
+  constexpr size_t smem = F32Smem<D, KS, sizeof(TIn) == 4 ? 3 : 1>::bytes;
+  static std::atomic<uint64_t> ready{0};
+  if (!device_done(ready)) {
+    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    device_mark(ready);
   }
-#undef LAUNCH
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)((T + 64 / KS - 1) / (64 / KS)), (unsigned)(s.B * s.H));
+  cfg.blockDim = dim3(NT);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  const cudaError_t e =
+      cudaLaunchKernelEx(&cfg, kern, (const TIn*)q, (const TIn*)k, (const TIn*)v, (TIn*)out, (const float*)w.ckpt, w.counters,
+                         T, s.T_max, s.n_ckpt(), s.H, s.g(), window, shape, theta, init == DELTA_INIT_BASIS_EXACT ? 0 : -1,
+                         1.4426950408889634f / sqrtf((float)s.d));
   count_launch();
-  return cudaGetLastError();
+  return e;
+}
+
+cudaError_t launch_hybrid_attn_generic(const Shape& s, const Workspace& w, const void* q, const void* k, const void* v,
+                                       void* out, int T, float theta, int init, int window, int shape, int dtype,
+                                       cudaStream_t st) {
+  // Warps per row group.  A key tile of 64 costs 3.3 / 2.2 / 1.4 us where a CTA walks alone and takes
+  // 4.0 / 2.2 / 1.6 us of an SM where the chip is full (KS = 1 / 2 / 4; d = 64, 1 to 256 heads of 128 to
+  // 4000 tokens); every halving of the rows doubles the tiles.  The longest walk bounds a small
+  // grid, the sum of all tiles, with half a walk for the uneven end, a large one.
+  int ks = 1;
+  float best = 3.4e38f;
+  for (int c = 0; c < 3; ++c) {
+    constexpr float alone[3] = {3.3f, 2.2f, 1.4f}, full[3] = {4.0f, 2.2f, 1.6f};
+    const float walk = (float)((T + BN - 1) / BN), tiles = 0.5f * walk * (walk + 1.0f) * (float)(1 << c) * (float)(s.B * s.H);
+    const float us = fmaxf(walk * alone[c], tiles / (float)device_sm_count() * full[c] + 0.5f * walk * alone[c]);
+    if (us < best) { best = us; ks = 1 << c; }
+  }
+#define GO(TIN, DD)                                                                                            \
+  return ks == 4   ? launch_f32<TIN, DD, 4>(s, w, q, k, v, out, T, theta, init, window, shape, st)            \
+         : ks == 2 ? launch_f32<TIN, DD, 2>(s, w, q, k, v, out, T, theta, init, window, shape, st)            \
+                    : launch_f32<TIN, DD, 1>(s, w, q, k, v, out, T, theta, init, window, shape, st)
+  if (dtype == DELTA_F32) {
+    if (s.d == 64) { GO(float, 64); } else { GO(float, 128); }
+  } else {
+    if (s.d == 64) { GO(__nv_bfloat16, 64); } else { GO(__nv_bfloat16, 128); }
+  }
+#undef GO
 }
 
 }  // namespace delta
