@@ -542,11 +542,8 @@ static cudaError_t decode_launch(delta_state* st, const Shape& shape, const Work
                                  const void* k_new, const void* v_new, void* k_cache, void* v_cache, void* out,
                                  int n, float theta, int32_t window, cudaStream_t cs) {
   if (st->cfg.source == DELTA_SRC_KEY)
-    return st->key_cache_packed
-               ? launch_decode_step_keypacked(shape, ws, q_new, k_new, v_new, k_cache, v_cache, out, n, theta, window,
-                                              st->qhat_sel, cs)
-               : launch_decode_step_key(shape, ws, q_new, k_new, v_new, k_cache, v_cache, out, n, theta, window,
-                                        st->qhat_sel, cs);
+    return launch_decode_step_key(shape, ws, q_new, k_new, v_new, k_cache, v_cache, out, n, theta, window, st->qhat_sel,
+                                  cs);
   return launch_decode_step(shape, ws, q_new, k_new, v_new, k_cache, v_cache, out, n, theta, window, st->cfg.dtype,
                             st->qhat_sel, cs);
 }
@@ -571,11 +568,11 @@ delta_status_t delta_attn_decode_step(delta_state_t* st, const void* q_new, cons
   cudaStream_t cs = (cudaStream_t)stream;
   cudaError_t e = cudaSuccess;
   const bool key_packed = c.source == DELTA_SRC_KEY && st->key_cache_packed;
-  if (!key_packed && delta_state_decode_kernel(st) == 1) {
+  if (key_packed || delta_state_decode_kernel(st) == 1) {
     // one launch, whether the batch elements stand at one position or at different ones
     e = launch_decode_step_mma(st->shape, st->ws, q_new, k_new, v_new, k_cache, v_cache, out, st->n,
                                st->ragged ? st->n_b.data() : nullptr, theta, window, st->qhat_sel,
-                               c.source == DELTA_SRC_KEY, st->dec_maps, cs);
+                               c.source == DELTA_SRC_KEY, key_packed, st->dec_maps, cs);
     if (e != cudaSuccess) return cuda_fail(e);
   } else if (!st->ragged) {
     e = decode_launch(st, st->shape, st->ws, q_new, k_new, v_new, k_cache, v_cache, out, st->n, theta, window, cs);

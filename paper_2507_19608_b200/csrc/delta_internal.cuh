@@ -120,16 +120,13 @@ struct DecodeTmapCache {
 bool decode_mma_applies(const Shape& s, int dtype);
 cudaError_t launch_decode_step_mma(const Shape& s, const Workspace& w, const void* q_new, const void* k_new,
                                    const void* v_new, void* k_cache, void* v_cache, void* out, int n, const int* n_b,
-                                   float theta, int window, int qhat_sel, bool key, DecodeTmapCache* maps,
+                                   float theta, int window, int qhat_sel, bool key, bool packed, DecodeTmapCache* maps,
                                    cudaStream_t st);
-// K3 (key deltas) from the compressed key-delta cache, the kernel that builds that cache behind a
-// prefill, and its geometry (values per KV head at most, 32-row segments).
+// The compressed key-delta cache (packed = true above decodes from it): the kernel that builds it
+// behind a prefill, and its geometry (values per KV head at most, 32-row segments).
 size_t keypack_capacity(int T_max, int d);
 int keypack_segments(int T_max);
 cudaError_t launch_pack_keys(const Shape& s, const Workspace& w, const void* k, int T, cudaStream_t st);
-cudaError_t launch_decode_step_keypacked(const Shape& s, const Workspace& w, const void* q_new, const void* k_new,
-                                         const void* v_new, void* k_cache, void* v_cache, void* out, int n,
-                                         float theta, int window, int qhat_sel, cudaStream_t st);
 // K3 (key deltas) on the FP32 pipes.
 cudaError_t launch_decode_step_key(const Shape& s, const Workspace& w, const void* q_new,
                                    const void* k_new, const void* v_new, void* k_cache, void* v_cache,

@@ -52,6 +52,11 @@ struct MmaDecodeParams {
   const __nv_bfloat16 *q_new, *k_new, *v_new;
   __nv_bfloat16 *k_cache, *v_cache, *khat_cache, *out;
   uint16_t* row_nnz;
+  // the compressed key-delta cache (MODE 2)
+  uint32_t *mask, *kp_mask, *seg_off, *used;
+  uint16_t *kp_nnz, *vals, *base;
+  size_t cap;
+  int nseg_max;
   const float* ref_in;
   float *ref_out, *R, *partial;
   uint32_t* ticket;
@@ -115,6 +120,17 @@ __device__ __forceinline__ float2 lds_f2(uint32_t addr) {
 }
 __device__ __forceinline__ float4 lds_f4(uint32_t addr) { return tc::lds128(addr); }
 
+__device__ __forceinline__ uint32_t lds_u32(uint32_t a) {
+  uint32_t v;
+  asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(a));
+  return v;
+}
+__device__ __forceinline__ uint32_t lds_u16(uint32_t a) {
+  uint32_t v;
+  asm volatile("ld.shared.u16 %0, [%1];" : "=r"(v) : "r"(a));
+  return v;
+}
+__device__ __forceinline__ void sts_u32(uint32_t a, uint32_t v) { asm volatile("st.shared.u32 [%0], %1;" ::"r"(a), "r"(v) : "memory"); }
 __device__ __forceinline__ int warp_sum(int x) {
 #pragma unroll
   for (int s = 16; s > 0; s >>= 1) x += __shfl_xor_sync(0xffffffffu, x, s);
@@ -123,23 +139,30 @@ __device__ __forceinline__ int warp_sum(int x) {
 
 // Shared memory: per warp one unit of keys and values (128-byte swizzle, blocks of [32 rows][64
 // channels]), then the merge's records [slot][slice x warp][REC] and (maximum, row sum) pairs.
-template <int D, int G> struct MmaSmem {
+// PACKED: per warp also the encoding of one 32-row segment: values, mask words, the reference in front.
+template <int D, int G, bool PACKED> struct MmaSmem {
   static constexpr int NW = kWarps<D>;
+  static constexpr uint32_t VALS = UK * D * 2 + 16, MASKS = UK * (D / 32) * 4, PACK = PACKED ? VALS + MASKS + D * 2 : 0;
   static constexpr uint32_t HALF = UK * D * 2;             // keys, or values, of a unit
   static constexpr uint32_t RING = NW * 2 * HALF;
   static constexpr int NB = G * D / 16;                    // 16-channel blocks of the result
-  static constexpr uint32_t NREC = (NB + kMaxCluster - 1) * NW;
-  static constexpr size_t bytes = 1024 + RING + NREC * (REC + 2) * 4;
+  // records of a CTA of a cluster of cs
+  __host__ __device__ static constexpr uint32_t nrec(int cs) { return (uint32_t)((NB + cs - 1) / cs * cs) * NW; }
+  static constexpr size_t bytes(int cs) { return 1024 + RING + nrec(cs) * (REC + 2) * 4 + NW * PACK; }
 };
 
 }  // namespace
 
-template <int D, int G, bool KEY, bool CLUSTER>
+// MODE 0: query deltas; 1: key deltas, dense reference-key rows; 2: key deltas from the compressed
+// key-delta cache (k1_pack_keys.cu has its layout): a unit is one segment of the
+// encoding, whose rows the warp rebuilds into its key slot.
+template <int D, int G, int MODE, bool CLUSTER>
 __global__ void __launch_bounds__(32 * kWarps<D>, 2)
 decode_step_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ CUtensorMap tm_v,
                        const __grid_constant__ CUtensorMap tm_h, const __grid_constant__ MmaDecodeParams p) {
   using TC = __nv_bfloat16;
-  using SM = MmaSmem<D, G>;
+  constexpr bool KEY = MODE != 0, PACKED = MODE == 2;
+  using SM = MmaSmem<D, G, PACKED>;
   constexpr int MNW = kWarps<D>;
   constexpr int NC = D / 32;                 // 16-byte pieces of a key row per thread
   constexpr int NV = D / 64;                 // 64-channel blocks of a row
@@ -148,7 +171,7 @@ decode_step_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_co
   __shared__ __align__(8) unsigned long long bars[2 * MNW + 1];
   __shared__ int s_last, s_fail;
   const uint32_t ring = (smem_u32(dsm_raw) + 1023u) & ~1023u;
-  const uint32_t recs = ring + SM::RING, mls = recs + SM::NREC * REC * 4;
+  const uint32_t recs = ring + SM::RING, mls = recs + SM::nrec(CLUSTER ? p.nsplit : 1) * REC * 4;
 
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int g = lane >> 2, t = lane & 3;     // row of the accumulators, thread of the row
@@ -180,7 +203,7 @@ decode_step_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_co
   const size_t row0 = (size_t)bkv * T_max;
   const TC* const kc = p.k_cache + row0 * D;
   const TC* const vc = p.v_cache + row0 * D;
-  const TC* const hc = KEY ? p.khat_cache + row0 * D : nullptr;
+  const TC* const hc = MODE == 1 ? p.khat_cache + row0 * D : nullptr;
   const TC* const kn = p.k_new + (size_t)bkv * D;
   const TC* const vn = p.v_new + (size_t)bkv * D;
   const int wl = n - W + 1;                  // first key inside the decode window
@@ -200,11 +223,27 @@ decode_step_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_co
   // A unit whose rows come from one cache goes by TMA; the unit of the row that arrives with the
   // step (rows behind it: zeros) and, key deltas, the unit of the window's edge row by row.
   auto k_plain = [&](int jg) { return jg + UK <= n && (!KEY || jg + UK <= wl || jg >= wl); };
+  const uint32_t pack_s = mls + SM::nrec(CLUSTER ? p.nsplit : 1) * 8 + (uint32_t)warp * SM::PACK;       // values, mask words, base
+  const uint32_t* const so = PACKED ? p.seg_off + (size_t)bkv * (p.nseg_max + 1) : nullptr;
+  auto from_pack = [&](int jg) { return PACKED && jg < wl && jg < n; };          // some row is a cached reference row
   auto fetch_k = [&](int jg) {
-    if (k_plain(jg)) {
+    if (from_pack(jg)) {
+      // (the entry behind the last cached segment is being rewritten by this step's owner where the new
+      // row extends or follows that segment: old and new value both bound the cached values)
+      if (lane == 0) {
+        const int sg = jg / UK;
+        const uint32_t v0 = __ldcg(so + sg), v1 = __ldcg(so + sg + 1);
+        const uint32_t vb = min((v1 - v0 + 7u) & ~7u, (uint32_t)UK * D) * 2u;
+        tc::mbar_expect_tx(bar_k, vb + SM::MASKS + D * 2);
+        if (vb) bulk_load(pack_s, p.vals + (size_t)bkv * p.cap + v0, vb, bar_k);
+        bulk_load(pack_s + SM::VALS, p.kp_mask + ((size_t)bkv * p.nseg_max * UK + jg) * (D / 32), SM::MASKS, bar_k);
+        bulk_load(pack_s + SM::VALS + SM::MASKS, p.base + ((size_t)bkv * p.nseg_max + sg) * D, D * 2, bar_k);
+      }
+      // (the original keys of a mixed unit's window rows follow when the rows are rebuilt)
+    } else if (k_plain(jg)) {
       if (lane == 0) {
         tc::mbar_expect_tx(bar_k, SM::HALF);
-        const CUtensorMap* tm = (KEY && jg < wl) ? &tm_h : &tm_k;
+        const CUtensorMap* tm = (MODE == 1 && jg < wl) ? &tm_h : &tm_k;
 #pragma unroll
         for (int c = 0; c < NV; ++c) tc::tma_load_3d(slot_k + c * UK * 128, tm, bar_k, 64 * c, jg, bkv);
       }
@@ -215,7 +254,7 @@ decode_step_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_co
         for (int i = 0; i < UK / 4; ++i) {
           const int r = 4 * i + (lane >> 3), ch = lane & 7, j = jg + r;
           const uint32_t dst = slot_k + c * UK * 128 + r * 128 + ((ch ^ (r & 7)) << 4);
-          const TC* src = (KEY && j < wl) ? hc : kc;
+          const TC* src = (MODE == 1 && j < wl) ? hc : kc;
           if (j <= n) async16(dst, (j < n ? src + (size_t)j * D : kn) + 64 * c + 8 * ch);
           else sts128z(dst);
         }
@@ -240,18 +279,27 @@ decode_step_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_co
         }
     }
   };
+  // Reference-key rows and their encoding are the library's own: all but the row (segment) the step in
+  // front may be writing is final before this kernel can start, since that step releases it only
+  // behind its own wait, and is requested ahead of the wait.  (Key and value rows are the caller's.)
+  int jg = j0 + UK * warp;
+  const bool early_k = KEY && jg < j1 && jg + UK <= min(n - 1, wl);
+  if (early_k) fetch_k(jg);
   // the step in front (or the prefill) has written the reference, row n - 1 of the caches, the tickets
   asm volatile("griddepcontrol.wait;" ::: "memory");
   // The next step's CTAs may become resident from here on.  (Released at the kernel's start they
   // take the places of this step's own late CTAs: 30 us per step for 18 at batch 16.)
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  int jg = j0 + UK * warp;
-  if (jg < j1) { fetch_k(jg); fetch_v(jg); }
+  if (jg < j1) {
+    if (!early_k) fetch_k(jg);
+    fetch_v(jg);
+  }
 
   // ---- threshold step (Eq. 2-3): the operand rows, straight into registers
   uint32_t ar[NC][4], aq[NC][4];             // rows g and g + 8 of A, channels 32 c + 8 t ..
   uint32_t khat_new[KEY ? NC : 1][4];        // KEY: the reference key after this step
   int fired = 0;
+  uint32_t fbits = 0;                        // PACKED: which of this thread's channels fired, 8 per piece
   const bool keep = split == 0 && warp == 0;
   {
     const size_t o = ((size_t)b * p.H + kvh * G + hd) * D;
@@ -278,6 +326,7 @@ decode_step_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_co
         const bool fire = fabsf(__fsub_rn(x, ref[i])) > theta;
         ref[i] = fire ? x : ref[i];
         fired += fire ? 1 : 0;
+        if (PACKED) fbits |= (fire ? 1u : 0u) << (8 * c + i);
       }
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
@@ -312,11 +361,103 @@ decode_step_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_co
   const uint32_t k_off = slot_k + kr * 128, k_sw = kr & 7;
   const uint32_t v_off0 = slot_v + kx0 * 128 + ((g ^ kx0) << 4), v_off1 = slot_v + kx1 * 128 + ((g ^ kx1) << 4);
   float* const Rg = KEY ? nullptr : p.R + ((size_t)b * p.H + kvh * G + hd) * T_max;
+  // Rows jg .. jg + 31 of the reference-key stream from their encoding, into the key slot: lane = two
+  // channels (of a 64-channel block), walking the rows; the window's rows and the new one are keys.
+  auto rebuild = [&](int jg) {
+    constexpr int NWD = D / 32;
+    const int last = min(UK, min(n, wl) - jg);             // rows that are cached references
+    const int hi = lane >> 4, sh = 2 * (lane & 15);        // this lane's channels: bits sh, sh + 1 of word 2 c + hi
+    const uint32_t lt = (1u << sh) - 1u;
+#pragma unroll
+    for (int c = 0; c < NV; ++c) {
+      uint32_t cur = lds_u32(pack_s + SM::VALS + SM::MASKS + 128 * c + 4 * lane), at = pack_s;
+      const uint32_t dst = slot_k + c * UK * 128 + 4 * (lane & 3);
+#pragma unroll 8
+      for (int r = 0; r < last; ++r) {
+        uint32_t w[NWD], below = 0, total = 0;
+#pragma unroll
+        for (int i = 0; i < NWD; ++i) {
+          w[i] = lds_u32(pack_s + SM::VALS + 4 * (r * NWD + i));
+          if (i == 2 * c) below = total + (hi ? (uint32_t)__popc(w[i]) : 0u);
+          total += __popc(w[i]);
+        }
+        const uint32_t mine = hi ? w[2 * c + 1] : w[2 * c];
+        const uint32_t a = at + 2 * (below + __popc(mine & lt)), f = mine >> sh;
+        // (a channel that has not fired reads some value of the pool and drops it: no branch, and the
+        // loads of eight rows are in flight together)
+        const uint32_t x0 = lds_u16(a), x1 = lds_u16(a + 2 * (f & 1u));
+        cur = (f & 1u) ? __byte_perm(cur, x0, 0x3254) : cur;
+        cur = (f & 2u) ? __byte_perm(cur, x1, 0x5410) : cur;
+        sts_u32(dst + r * 128 + (((lane >> 2) ^ (r & 7)) << 4), cur);
+        at += 2 * total;
+      }
+#pragma unroll 1
+      for (int e = last * 8 + lane; e < UK * 8; e += 32) {
+        const int r = e >> 3, ch = e & 7, j = jg + r;
+        const uint32_t dst = slot_k + c * UK * 128 + r * 128 + ((ch ^ (r & 7)) << 4);
+        if (j <= n) async16(dst, (j < n ? kc + (size_t)j * D : kn) + 64 * c + 8 * ch);
+        else sts128z(dst);
+      }
+    }
+    async_wait_all();
+    __syncwarp();
+  };
+  // The new row joins the encoding (the warp that owns its unit): values behind the pool's end (on a
+  // multiple of 8 where it opens a segment), mask words, count, offsets, the segment's base.
+  auto append = [&](int nz) {
+    const int sg = n / UK;
+    const bool opens = (n % UK) == 0;
+    const uint32_t pool = __ldcg(p.used + bkv), pos = opens ? (pool + 7u) & ~7u : pool;
+    uint16_t* const vg = p.vals + (size_t)bkv * p.cap;
+    uint32_t at = pos;
+#pragma unroll
+    for (int c = 0; c < NC; ++c) {
+      // word c: thread t of row 0 holds its bits 8 t .. 8 t + 7
+      uint32_t byte = (fbits >> (8 * c)) & 0xffu;
+      uint32_t word = byte << (8 * t);
+      word |= __shfl_xor_sync(0xffffffffu, word, 1);
+      word |= __shfl_xor_sync(0xffffffffu, word, 2);
+      if (g == 0) {
+        uint32_t rank = at + __popc(word & ((1u << (8 * t)) - 1u));
+#pragma unroll
+        for (int e = 0; e < 8; ++e)
+          if ((byte >> e) & 1u) {
+            // (a fired channel's new reference is the key value itself)
+            if (DELTA_IN(rank, p.cap, p.counters)) vg[rank] = (uint16_t)(khat_new[c][e >> 1] >> (16 * (e & 1)));
+            ++rank;
+          }
+        if (t == 0) {
+          p.mask[(row0 + n) * NC + c] = word;
+          p.kp_mask[((size_t)bkv * p.nseg_max * UK + n) * NC + c] = word;
+        }
+        if (opens) {
+          const float4* const rp = reinterpret_cast<const float4*>(p.ref_in + (size_t)bkv * D + 32 * c + 8 * t);
+          const float4 r0 = __ldcg(rp), r1 = __ldcg(rp + 1);
+          const float rr[8] = {r0.x, r0.y, r0.z, r0.w, r1.x, r1.y, r1.z, r1.w};
+#pragma unroll
+          for (int e = 0; e < 8; ++e)                     // exactly bf16
+            p.base[((size_t)bkv * p.nseg_max + sg) * D + 32 * c + 8 * t + e] = (uint16_t)(__float_as_uint(rr[e]) >> 16);
+        }
+      }
+      at += __popc(__shfl_sync(0xffffffffu, word, 0));
+    }
+    if (lane == 0 && DELTA_IN(sg + 1, p.nseg_max + 1, p.counters)) {
+      uint32_t* const sw = p.seg_off + (size_t)bkv * (p.nseg_max + 1);
+      if (opens) sw[sg] = pos;
+      sw[sg + 1] = pos + (uint32_t)nz;
+      p.used[bkv] = pos + (uint32_t)nz;
+      p.kp_nnz[(size_t)bkv * p.nseg_max * UK + n] = (uint16_t)nz;
+    }
+  };
   for (; jg < j1; jg += UK * MNW) {
     const int jn = jg + UK * MNW;            // the warp's next unit
     const bool owner = n < jg + UK;          // of the row that arrives with the step
-    const bool tma_k = k_plain(jg), tma_v = jg + UK <= n;
-    if (tma_k) {
+    const bool packed = from_pack(jg), tma_k = !packed && k_plain(jg), tma_v = jg + UK <= n;
+    if (packed) {
+      if (!mbar_wait(bar_k, ph_k)) s_fail = 1;
+      ph_k ^= 1u;
+      rebuild(jg);
+    } else if (tma_k) {
       if (!mbar_wait(bar_k, ph_k)) s_fail = 1;
       ph_k ^= 1u;
     } else {
@@ -338,10 +479,10 @@ decode_step_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_co
         mma16816(s[h], ar[c][2], aq[c][2], ar[c][3], aq[c][3], k4.z, k4.w);
       }
     }
+    int nz_new = 0;
     if (KEY) {
       // multiply-adds: d inside the window, nnz(Delta k_j) outside
       const int j = jg + lane;
-      int nz_new = 0;
       if (owner) {
         nz_new = warp_sum(fired);
         if (lane == 0 && DELTA_IN(n, T_max, p.counters)) p.row_nnz[row0 + n] = (uint16_t)nz_new;
@@ -431,7 +572,8 @@ decode_step_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_co
         reinterpret_cast<uint4*>(p.k_cache + (row0 + n) * D)[lane] = __ldcg(reinterpret_cast<const uint4*>(kn) + lane);
         reinterpret_cast<uint4*>(p.v_cache + (row0 + n) * D)[lane] = __ldcg(reinterpret_cast<const uint4*>(vn) + lane);
       }
-      if (KEY && g == 0)
+      if constexpr (PACKED) append(nz_new);
+      if (MODE == 1 && g == 0)
 #pragma unroll
         for (int c = 0; c < NC; ++c)
           *reinterpret_cast<uint4*>(p.khat_cache + (row0 + n) * D + 32 * c + 8 * t) =
@@ -565,8 +707,9 @@ decode_step_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_co
 // slices are those that minimise that.  All slices of a KV head form one cluster, and clusters have to
 // find room in a GPC: from 1.75 CTAs per SM on (1.6 for clusters of 9 to 12, 1.35 for 13 to 16) some
 // wait for a second wave (batch 16, 2048 keys: 256 CTAs 12 us, 384 CTAs 17 us).  Very long caches of
-// few heads: up to 64 slices merged through global memory (4.5 us more than a cluster).
-static void decode_mma_slices(const Shape& s, int L, int* nsplit_out, int* chunk_out, bool* cluster_out) {
+// few heads: up to 64 slices merged through global memory (4.5 us more than a cluster).  The compressed
+// key cache: 2.5 us more per unit, for the rebuilding.
+static void decode_mma_slices(const Shape& s, int L, bool packed, int* nsplit_out, int* chunk_out, bool* cluster_out) {
   const int bkv = s.B * s.H_kv, sms = device_sm_count();
   const int nw = s.d == 64 ? kWarps<64> : kWarps<128>;
   const int units = (L + UK - 1) / UK;
@@ -579,7 +722,7 @@ static void decode_mma_slices(const Shape& s, int L, int* nsplit_out, int* chunk
     if (ns > 1 && ns <= kMaxCluster && ctas * 100 > (long)sms * (ns <= 8 ? 175 : ns <= 12 ? 160 : 135)) continue;
     const int per = (units + ns - 1) / ns;                       // units per slice; per warp mostly the longest counts
     const float rounds = 0.8f * (float)((per + nw - 1) / nw) + 0.2f * (float)per / (float)nw;
-    const float us = rounds * (!alone ? 1.75f : s.d == 64 ? 1.1f : 1.3f) +
+    const float us = rounds * ((!alone ? 1.75f : s.d == 64 ? 1.1f : 1.3f) + (packed ? 2.5f : 0.0f)) +
                      (ns > kMaxCluster ? 4.5f + 0.15f * (float)(ns - 24) : (ns > 8 ? 0.075f : 0.06f) * (float)ns);
     if (us < best - 0.02f) { best = us; best_ns = ns; }
   }
@@ -589,14 +732,15 @@ static void decode_mma_slices(const Shape& s, int L, int* nsplit_out, int* chunk
   *cluster_out = *nsplit_out > 1 && *nsplit_out <= kMaxCluster;
 }
 
-template <int D, int G, bool KEY, bool CLUSTER>
+template <int D, int G, int MODE, bool CLUSTER>
 static cudaError_t launch_mma(const CUtensorMap& tk, const CUtensorMap& tv, const CUtensorMap& th,
                               const MmaDecodeParams& p, int bkv, cudaStream_t st) {
-  auto kern = decode_step_mma_kernel<D, G, KEY, CLUSTER>;
-  constexpr size_t smem = MmaSmem<D, G>::bytes;
+  auto kern = decode_step_mma_kernel<D, G, MODE, CLUSTER>;
+  using SM = MmaSmem<D, G, MODE == 2>;
+  const size_t smem = SM::bytes(CLUSTER ? p.nsplit : 1);
   static std::atomic<uint64_t> ready{0};
   if (!device_done(ready)) {
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SM::bytes(kMaxCluster - 1));
     // (two CTAs per SM need the largest shared-memory carve-out)
     if (e == cudaSuccess) e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout,
                                                    (int)cudaSharedmemCarveoutMaxShared);
@@ -641,8 +785,8 @@ bool decode_mma_applies(const Shape& s, int dtype) { return dtype == DELTA_BF16 
 
 cudaError_t launch_decode_step_mma(const Shape& s, const Workspace& w, const void* q_new, const void* k_new,
                                    const void* v_new, void* k_cache, void* v_cache, void* out, int n, const int* n_b,
-                                   float theta, int window, int qhat_sel, bool key, DecodeTmapCache* maps, cudaStream_t st) {
-  if (key && !w.qhat_rows) return cudaErrorNotSupported;
+                                   float theta, int window, int qhat_sel, bool key, bool packed, DecodeTmapCache* maps, cudaStream_t st) {
+  if ((key && !w.qhat_rows) || (packed && (!key || !w.kp_vals))) return cudaErrorNotSupported;
   using TC = __nv_bfloat16;
   const CUtensorMap* const tk = row_map(&maps[0], k_cache, s);
   const CUtensorMap* const tv = row_map(&maps[1], v_cache, s);
@@ -655,22 +799,25 @@ cudaError_t launch_decode_step_mma(const Shape& s, const Workspace& w, const voi
   p.partial = w.dec_partial; p.ticket = w.dec_ticket; p.counters = w.counters;
   p.n = n; p.T_max = s.T_max; p.H = s.H; p.W = window; p.theta = theta;
   p.scale_log2e = 1.4426950408889634f / sqrtf((float)s.d);
+  p.mask = w.mask; p.kp_mask = w.kp_mask; p.seg_off = w.kp_segoff; p.used = w.kp_used;
+  p.kp_nnz = w.kp_nnz; p.vals = w.kp_vals; p.base = w.kp_base;
+  p.cap = keypack_capacity(s.T_max, s.d); p.nseg_max = keypack_segments(s.T_max);
   p.ragged = n_b != nullptr;
   p.b0 = 0;
   const int G = s.g();
   bool cluster;
-  decode_mma_slices(s, n + 1, &p.nsplit, &p.chunk, &cluster);
+  decode_mma_slices(s, n + 1, packed, &p.nsplit, &p.chunk, &cluster);
   if (p.nsplit > kMaxDecodeSplits) return cudaErrorInvalidValue;
   cudaError_t err = cudaSuccess;
   for (; p.b0 < s.B && err == cudaSuccess; p.b0 += kRaggedMax) {
     const int nb = n_b ? (s.B - p.b0 < kRaggedMax ? s.B - p.b0 : kRaggedMax) : s.B;
     if (n_b)
       for (int i = 0; i < nb; ++i) p.n_b[i] = n_b[p.b0 + i];
+#define GO_M(DD, GG, M)                                                                                      \
+    err = cluster ? launch_mma<DD, GG, M, true>(*tk, *tv, *th, p, nb * s.H_kv, st)                           \
+                  : launch_mma<DD, GG, M, false>(*tk, *tv, *th, p, nb * s.H_kv, st)
 #define GO(DD, GG)                                                                                           \
-    err = key ? (cluster ? launch_mma<DD, GG, true, true>(*tk, *tv, *th, p, nb * s.H_kv, st)                                \
-                         : launch_mma<DD, GG, true, false>(*tk, *tv, *th, p, nb * s.H_kv, st))                              \
-              : (cluster ? launch_mma<DD, GG, false, true>(*tk, *tv, *th, p, nb * s.H_kv, st)                               \
-                         : launch_mma<DD, GG, false, false>(*tk, *tv, *th, p, nb * s.H_kv, st))
+    if (packed) { GO_M(DD, GG, 2); } else if (key) { GO_M(DD, GG, 1); } else { GO_M(DD, GG, 0); }
 #define GO_G(DD)                                                                                             \
     switch (G) {                                                                                             \
       case 1: GO(DD, 1); break;                                                                              \
@@ -682,6 +829,7 @@ cudaError_t launch_decode_step_mma(const Shape& s, const Workspace& w, const voi
     if (s.d == 64) { GO_G(64) } else { GO_G(128) }
 #undef GO_G
 #undef GO
+#undef GO_M
     if (!n_b) break;
   }
   return err;
