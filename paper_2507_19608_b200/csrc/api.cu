@@ -340,10 +340,10 @@ static void view_of(const delta_state* st, int b, Shape* sh, Workspace* w) {
   }
 }
 
-// The three kernels of a prefill over one view (the whole batch, or one batch element).
+// The three kernels of a prefill over a uniform batch or a group of sequences of different lengths.
 static delta_status_t prefill_launch(delta_state* st, const Shape& shape, const Workspace& ws, const void* q,
-                                     const void* k, const void* v, void* out, int32_t T, float theta,
-                                     int32_t window, cudaStream_t cs, bool prof) {
+                                     const void* k, const void* v, void* out, const SeqBatch& seqs, float theta,
+                                     cudaStream_t cs, bool prof) {
   const delta_config_t& c = st->cfg;
   cudaError_t e;
   // a pending reset: the chain kernel clears the span, less the front of qhat[0] that the chain
@@ -372,31 +372,31 @@ static delta_status_t prefill_launch(delta_state* st, const Shape& shape, const 
   const bool chained = !use_tc && !prof;
   MARK(0);
   // the delta stream: the queries (strategy 1) or the keys, per KV head (strategy 3)
-  if ((e = launch_delta_chain(shape, ws, key ? k : q, T, theta, c.dtype, c.init, key, rev, zero_ptr, zero_bytes, cs)) != cudaSuccess)
+  if ((e = launch_delta_chain(shape, ws, key ? k : q, seqs, theta, c.dtype, c.init, key, rev, zero_ptr, zero_bytes, cs)) != cudaSuccess)
     return cuda_fail(e);
   auto attention = [&]() -> cudaError_t {
-    if (use_tc) return launch_hybrid_attn_tc(shape, ws, q, k, v, out, T, window, c.prefill_window, cs);
+    if (use_tc) return launch_hybrid_attn_tc(shape, ws, q, k, v, out, seqs.s[0].T, seqs.s[0].W, c.prefill_window, cs);
     if (tcq)
-      return launch_hybrid_attn_tcq(shape, ws, q, k, v, out, T, theta, c.init, window, c.prefill_window, key,
+      return launch_hybrid_attn_tcq(shape, ws, q, k, v, out, seqs, theta, c.init, c.prefill_window, key,
                                     rev, /*form=*/which == 3 ? 1 : which == 4 ? 2 : which == 5 ? 3 : 0, cs);
-    return launch_hybrid_attn_generic(shape, ws, q, k, v, out, T, theta, c.init, window, c.prefill_window, c.dtype, cs);
+    return launch_hybrid_attn_generic(shape, ws, q, k, v, out, seqs, theta, c.init, c.prefill_window, c.dtype, cs);
   };
   if (chained && !key) {
     if ((e = attention()) != cudaSuccess) return cuda_fail(e);
     // (released by the attention CTAs once the chain is complete: it runs beside their last wave)
-    if ((e = launch_delta_finish(shape, ws, q, k, T, theta, window, c.prefill_window, c.dtype, c.init,
+    if ((e = launch_delta_finish(shape, ws, q, k, seqs, theta, c.prefill_window, c.dtype, c.init,
                                  use_tc, key, rev, 2, cs)) != cudaSuccess)
       return cuda_fail(e);
   } else if (chained) {
     // key deltas: the finish kernel writes the reference-key rows the attention kernel streams,
     // so it comes first (both programmatically serialised behind the kernel in front)
-    if ((e = launch_delta_finish(shape, ws, q, k, T, theta, window, c.prefill_window, c.dtype, c.init,
+    if ((e = launch_delta_finish(shape, ws, q, k, seqs, theta, c.prefill_window, c.dtype, c.init,
                                  use_tc, key, rev, 1, cs)) != cudaSuccess)
       return cuda_fail(e);
     if ((e = attention()) != cudaSuccess) return cuda_fail(e);
   } else {
     MARK(1);
-    if ((e = launch_delta_finish(shape, ws, q, k, T, theta, window, c.prefill_window, c.dtype, c.init,
+    if ((e = launch_delta_finish(shape, ws, q, k, seqs, theta, c.prefill_window, c.dtype, c.init,
                                  use_tc, key, rev, 0, cs)) != cudaSuccess)
       return cuda_fail(e);
     MARK(2);
@@ -404,7 +404,19 @@ static delta_status_t prefill_launch(delta_state* st, const Shape& shape, const 
   }
   MARK(3);
   // key deltas with the compressed cache: encode the key stream behind everything it is built from
-  if (key && st->key_cache_packed && (e = launch_pack_keys(shape, ws, k, T, cs)) != cudaSuccess) return cuda_fail(e);
+  if (key && st->key_cache_packed) {
+    if (!seqs.ragged) {
+      if ((e = launch_pack_keys(shape, ws, k, seqs.s[0].T, cs)) != cudaSuccess) return cuda_fail(e);
+    } else {
+      for (int i = 0; i < seqs.n; ++i) {
+        Shape sh;
+        Workspace w1;
+        view_of(st, seqs.s[i].b, &sh, &w1);
+        const size_t kv = (size_t)seqs.s[i].b * c.H_kv * c.T_max * c.d * 2;
+        if ((e = launch_pack_keys(sh, w1, (const char*)k + kv, seqs.s[i].T, cs)) != cudaSuccess) return cuda_fail(e);
+      }
+    }
+  }
   MARK(4);
 #undef MARK
   return DELTA_OK;
@@ -426,7 +438,10 @@ delta_status_t delta_attn_prefill(delta_state_t* st, const void* q, const void* 
   if (T > c.T_max) return DELTA_ERR_CAPACITY;
   if (st->n != 0) return DELTA_ERR_STATE;
   const bool prof = st->profiling;
-  s = prefill_launch(st, st->shape, st->ws, q, k, v, out, T, theta, window, (cudaStream_t)stream, prof);
+  SeqBatch seqs;
+  seqs.n = 1; seqs.T_longest = T; seqs.ragged = false;
+  seqs.s[0] = Seq{T, window, 0, 0};
+  s = prefill_launch(st, st->shape, st->ws, q, k, v, out, seqs, theta, (cudaStream_t)stream, prof);
   if (s != DELTA_OK) return s;
   st->profiled = prof;
   st->n = T;
@@ -451,26 +466,46 @@ delta_status_t delta_attn_prefill_varlen(delta_state_t* st, const void* q, const
     if (seq_lens[b] > c.T_max) return DELTA_ERR_CAPACITY;
   }
   if (st->n != 0) return DELTA_ERR_STATE;
+  // groups of kSeqMax sequences, three launches each; the kernel with the FP32 delta path, whose launch
+  // covers sequences of one length: a launch per sequence over its view
+  const bool one_by_one = delta_state_prefill_kernel(st) == 1;
   const size_t es = c.dtype == DELTA_F32 ? 4 : 2;
   size_t q_off = 0;     // elements in front of sequence b in the packed query / output arrays
   int t_longest = 0;
   bool same = true;
+  SeqBatch seqs;
+  seqs.n = 0; seqs.T_longest = 0; seqs.ragged = true;
   for (int b = 0; b < c.B; ++b) {
-    Shape sh;
-    Workspace ws;
-    view_of(st, b, &sh, &ws);
     const int T = seq_lens[b];
-    const size_t kv_off = (size_t)b * c.H_kv * c.T_max * c.d * es;
-    delta_status_t s = prefill_launch(st, sh, ws, (const char*)q + q_off * es, (const char*)k + kv_off,
-                                      (const char*)v + kv_off, (char*)out + q_off * es, T, theta, windows[b],
-                                      (cudaStream_t)stream, false);
-    if (s != DELTA_OK) return s;
+    if (one_by_one) {
+      Shape sh;
+      Workspace ws;
+      view_of(st, b, &sh, &ws);
+      const size_t kv_off = (size_t)b * c.H_kv * c.T_max * c.d * es;
+      SeqBatch one;
+      one.n = 1; one.T_longest = T; one.ragged = false;
+      one.s[0] = Seq{T, windows[b], 0, 0};
+      const delta_status_t s = prefill_launch(st, sh, ws, (const char*)q + q_off * es, (const char*)k + kv_off,
+                                              (const char*)v + kv_off, (char*)out + q_off * es, one, theta,
+                                              (cudaStream_t)stream, false);
+      if (s != DELTA_OK) return s;
+    } else {
+      seqs.s[seqs.n++] = Seq{T, windows[b], b, q_off};
+      seqs.T_longest = T > seqs.T_longest ? T : seqs.T_longest;
+      if (seqs.n == kSeqMax || b + 1 == c.B) {
+        const delta_status_t s = prefill_launch(st, st->shape, st->ws, q, k, v, out, seqs, theta, (cudaStream_t)stream, false);
+        if (s != DELTA_OK) return s;
+        seqs.n = 0; seqs.T_longest = 0;
+      }
+    }
     q_off += (size_t)c.H * T * c.d;
-    st->n_b[(size_t)b] = T;
-    st->win_sum[0] += (double)(windows[b] < T ? windows[b] : T);
-    st->len_sum[0] += (double)T;
     t_longest = T > t_longest ? T : t_longest;
     same = same && T == seq_lens[0];
+  }
+  for (int b = 0; b < c.B; ++b) {
+    st->n_b[(size_t)b] = seq_lens[b];
+    st->win_sum[0] += (double)(windows[b] < seq_lens[b] ? windows[b] : seq_lens[b]);
+    st->len_sum[0] += (double)seq_lens[b];
   }
   st->profiled = false;
   st->n = t_longest;

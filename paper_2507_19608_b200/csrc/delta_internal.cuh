@@ -59,6 +59,22 @@ struct Shape {
   int n_ckpt() const { return (T_max + DELTA_CKPT_ROWS - 1) / DELTA_CKPT_ROWS; }
 };
 
+// What a prefill kernel knows of one sequence.  A uniform batch is one entry whose heads are all
+// B * H heads; a ragged batch has an entry per batch element, up to kSeqMax in one launch: its heads
+// are the element's own, q_off the elements in front of it in the packed query and output arrays.
+constexpr int kSeqMax = 16;
+struct Seq {
+  int T, W, b;
+  size_t q_off;
+};
+template <int N> struct SeqList { Seq s[N]; };
+// The sequences of a launch: n = 1 (uniform, covering the whole batch) or a ragged group.
+struct SeqBatch {
+  int n, T_longest;
+  bool ragged;
+  Seq s[kSeqMax];
+};
+
 // What a launcher does once per device (function attributes, which the runtime keeps): has it been
 // done on the current device / it has.  (Devices past 63 do it every time.)
 inline int device_slot() {
@@ -84,8 +100,9 @@ delta_status_t cuda_fail(cudaError_t e);
 // reverse: rows are taken from T-1 down to 0 (strategy 2; query stream only).
 // zero_ptr, zero_bytes: a span (16-byte aligned, a multiple of 16 bytes) that the kernel's first
 // CTA clears before anything else: the deferred clearing of a state reset (none if null).
-cudaError_t launch_delta_chain(const Shape& s, const Workspace& w, const void* q, int T, float theta, int dtype,
-                               int init, bool key_stream, bool reverse, void* zero_ptr, size_t zero_bytes,
+// x: the packed queries or the key cache.
+cudaError_t launch_delta_chain(const Shape& s, const Workspace& w, const void* x, const SeqBatch& seqs, float theta,
+                               int dtype, int init, bool key_stream, bool reverse, void* zero_ptr, size_t zero_bytes,
                                cudaStream_t st);
 // K1b: row-parallel finish: delta values, mask words and (key stream) reference rows from the
 // 8-row checkpoints; counts, compacted indices, Eq. 6 counters, the decode hand-off row
@@ -96,12 +113,12 @@ int device_sm_count();
 // of the kernel in front; the kernel waits for that kernel's completion itself); 2 = the same, but
 // the kernel does not wait: the kernel in front releases it once the chain kernel's results are
 // complete (query deltas behind the telescoped attention kernel); 0 = an ordinary launch.
-cudaError_t launch_delta_finish(const Shape& s, const Workspace& w, const void* q, const void* k, int T,
-                                float theta, int window, int shape, int dtype, int init, bool want_kt,
+cudaError_t launch_delta_finish(const Shape& s, const Workspace& w, const void* q, const void* k, const SeqBatch& seqs,
+                                float theta, int shape, int dtype, int init, bool want_kt,
                                 bool key_stream, bool reverse, int programmatic, cudaStream_t st);
 // K2 on the FP32 pipes, either dtype; reads the chain kernel's checkpoints and nothing of the finish kernel's.
 cudaError_t launch_hybrid_attn_generic(const Shape& s, const Workspace& w, const void* q, const void* k, const void* v,
-                                       void* out, int T, float theta, int init, int window, int shape, int dtype,
+                                       void* out, const SeqBatch& seqs, float theta, int init, int shape, int dtype,
                                        cudaStream_t st);
 // K3: one decode step.
 cudaError_t launch_decode_step(const Shape& s, const Workspace& w, const void* q_new,

@@ -386,13 +386,15 @@ __device__ __forceinline__ void chain_stage_rev(const TIn* rows, int t0, int nro
 
 }  // namespace
 
-template <typename TIn, int D>
+template <typename TIn, int D, int N>
 __global__ void __launch_bounds__(D + 32) delta_chain_rows_kernel(
-    const TIn* __restrict__ q, float* __restrict__ qhat_tile, float* __restrict__ qhat_out,
-    float* __restrict__ ckpt, unsigned long long* __restrict__ counters, int T, int n_tiles, int n_ckpt,
-    float theta, int basis_exact, int src_rows, int reverse, uint4* zero_ptr, unsigned zero_n16) {
-  // q: the stream that becomes the delta matrix, [heads][src_rows][D] with rows 0..T-1 read
-  // (queries: src_rows = T; keys in the KV-cache layout: src_rows = T_max)
+    const TIn* __restrict__ x, const __grid_constant__ SeqList<N> seqs, float* __restrict__ qhat_tile,
+    float* __restrict__ qhat_out, float* __restrict__ ckpt, unsigned long long* __restrict__ counters, int n_tiles,
+    int n_ckpt, float theta, int basis_exact, int heads, int key_rows, int reverse, uint4* zero_ptr, unsigned zero_n16) {
+  // x: the stream that becomes the delta matrix: packed queries, a sequence's [heads][T][D] behind one
+  // another (key_rows = 0), or keys in the KV-cache layout [heads][key_rows][D], rows 0..T-1 read
+  const Seq& sq = seqs.s[N == 1 ? 0 : blockIdx.y];
+  const int T = sq.T, src_rows = key_rows ? key_rows : T;
   constexpr int NW = D / 32;                       // chain warps
   constexpr uint32_t ROW_BYTES = D * sizeof(TIn);
   constexpr uint32_t STAGE_BYTES = RROWS * ROW_BYTES;
@@ -400,12 +402,13 @@ __global__ void __launch_bounds__(D + 32) delta_chain_rows_kernel(
   __shared__ __align__(8) unsigned long long bars[2 * RSTAGES];   // full[RSTAGES], empty[RSTAGES]
   __shared__ int s_fail;
 
-  const int bh = blockIdx.x;
+  const int bh = sq.b * heads + (int)blockIdx.x;   // head of the workspace arrays
+  const TIn* const q = key_rows ? x + (size_t)bh * src_rows * D : x + sq.q_off + (size_t)blockIdx.x * T * D;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const uint32_t full0 = smem_u32(&bars[0]), empty0 = smem_u32(&bars[RSTAGES]);
   const int n_chunks = (T + RROWS - 1) / RROWS;
   // the deferred clearing of a state reset (see the table kernel)
-  if (zero_ptr && blockIdx.x == 0)
+  if (zero_ptr && blockIdx.x == 0 && blockIdx.y == 0)
     for (unsigned i = tid; i < zero_n16; i += blockDim.x) zero_ptr[i] = make_uint4(0u, 0u, 0u, 0u);
 
   if (tid == 0) {
@@ -425,7 +428,7 @@ __global__ void __launch_bounds__(D + 32) delta_chain_rows_kernel(
   if (warp == NW) {
     // ---- producer: keeps up to RSTAGES stages of query rows in flight
     if (lane == 0) {
-      const unsigned char* src = reinterpret_cast<const unsigned char*>(q) + (size_t)bh * src_rows * ROW_BYTES;
+      const unsigned char* src = reinterpret_cast<const unsigned char*>(q);
       const uint32_t ring0 = smem_u32(ring);
       for (int i = 0; i < n_chunks; ++i) {
         const int s = i % RSTAGES;
@@ -475,34 +478,41 @@ __global__ void __launch_bounds__(D + 32) delta_chain_rows_kernel(
 }
 
 
-static cudaError_t launch_delta_chain_rows(const Shape& s, const Workspace& w, const void* q, int T, float theta,
-                                          int dtype, int init, bool key_stream, bool reverse, void* zero_ptr,
-                                          size_t zero_bytes, cudaStream_t st) {
-  if (key_stream && reverse) return cudaErrorNotSupported;
-  const int grid = s.B * (key_stream ? s.H_kv : s.H);
-  const int src_rows = key_stream ? s.T_max : T;
-  const int basis = (init == DELTA_INIT_BASIS_EXACT) ? 1 : 0;
-  cudaError_t err = cudaSuccess;
-#define LAUNCH(TIN, DD)                                                                          \
-  do {                                                                                           \
-    auto kern = delta_chain_rows_kernel<TIN, DD>;                                                     \
-    const size_t smem = (size_t)RSTAGES * RROWS * DD * sizeof(TIN);                                      \
-    if (smem > 48 * 1024) {                                                                      \
-      err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);  \
-      if (err != cudaSuccess) return err;                                                        \
-    }                                                                                            \
-    kern<<<grid, DD + 32, smem, st>>>((const TIN*)q, w.qhat_tile, w.qhat[0], w.ckpt, w.counters, T, s.n_tiles, \
-                                      s.n_ckpt(), theta, basis, src_rows, reverse ? 1 : 0,       \
-                                      (uint4*)zero_ptr, (unsigned)(zero_bytes / 16));            \
-  } while (0)
-  if (dtype == DELTA_F32) {
-    if (s.d == 64) LAUNCH(float, 64); else LAUNCH(float, 128);
-  } else {
-    if (s.d == 64) LAUNCH(__nv_bfloat16, 64); else LAUNCH(__nv_bfloat16, 128);
+template <typename TIn, int D, int N>
+static cudaError_t launch_rows(const Shape& s, const Workspace& w, const void* x, const SeqBatch& seqs, float theta, int init,
+                               bool key_stream, bool reverse, void* zero_ptr, size_t zero_bytes, cudaStream_t st) {
+  auto kern = delta_chain_rows_kernel<TIn, D, N>;
+  constexpr size_t smem = (size_t)RSTAGES * RROWS * D * sizeof(TIn);
+  static std::atomic<uint64_t> ready{0};
+  if (smem > 48 * 1024 && !device_done(ready)) {
+    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    device_mark(ready);
   }
-#undef LAUNCH
+  SeqList<N> list;
+  for (int i = 0; i < N; ++i) list.s[i] = seqs.s[i < seqs.n ? i : 0];
+  const int heads = key_stream ? s.H_kv : s.H;
+  const dim3 grid((unsigned)(seqs.ragged ? heads : s.B * heads), (unsigned)seqs.n);
+  kern<<<grid, D + 32, smem, st>>>((const TIn*)x, list, w.qhat_tile, w.qhat[0], w.ckpt, w.counters, s.n_tiles, s.n_ckpt(),
+                                   theta, init == DELTA_INIT_BASIS_EXACT ? 1 : 0, heads, key_stream ? s.T_max : 0,
+                                   reverse ? 1 : 0, (uint4*)zero_ptr, (unsigned)(zero_bytes / 16));
   count_launch();
-  return err != cudaSuccess ? err : cudaGetLastError();
+  return cudaGetLastError();
+}
+
+static cudaError_t launch_delta_chain_rows(const Shape& s, const Workspace& w, const void* x, const SeqBatch& seqs,
+                                           float theta, int dtype, int init, bool key_stream, bool reverse, void* zero_ptr,
+                                           size_t zero_bytes, cudaStream_t st) {
+#define GO(TIN, DD)                                                                                              \
+  return seqs.ragged                                                                                             \
+             ? launch_rows<TIN, DD, kSeqMax>(s, w, x, seqs, theta, init, key_stream, reverse, zero_ptr, zero_bytes, st) \
+             : launch_rows<TIN, DD, 1>(s, w, x, seqs, theta, init, key_stream, reverse, zero_ptr, zero_bytes, st)
+  if (dtype == DELTA_F32) {
+    if (s.d == 64) { GO(float, 64); } else { GO(float, 128); }
+  } else {
+    if (s.d == 64) { GO(__nv_bfloat16, 64); } else { GO(__nv_bfloat16, 128); }
+  }
+#undef GO
 }
 
 // SMs of the current device (queried once per device).
@@ -517,16 +527,18 @@ int device_sm_count() {
   return cached[dev];
 }
 
-cudaError_t launch_delta_chain(const Shape& s, const Workspace& w, const void* q, int T, float theta, int dtype,
-                               int init, bool key_stream, bool reverse, void* zero_ptr, size_t zero_bytes,
+cudaError_t launch_delta_chain(const Shape& s, const Workspace& w, const void* x, const SeqBatch& seqs, float theta,
+                               int dtype, int init, bool key_stream, bool reverse, void* zero_ptr, size_t zero_bytes,
                                cudaStream_t st) {
   if (key_stream && reverse) return cudaErrorNotSupported;
   if (((uintptr_t)zero_ptr | zero_bytes) & 15u) return cudaErrorInvalidValue;
-  // the table kernel while every one of its CTAs (head x 32 channels) has an SM of its own
+  // the table kernel while every one of its CTAs (head x 32 channels) has an SM of its own (one
+  // tensor map: not for a ragged group)
   const long ctas = (long)s.B * (key_stream ? s.H_kv : s.H) * (s.d / CH);
-  if (ctas <= device_sm_count())
-    return launch_delta_chain_tables(s, w, q, T, theta, dtype, init, key_stream, reverse, zero_ptr, zero_bytes, st);
-  return launch_delta_chain_rows(s, w, q, T, theta, dtype, init, key_stream, reverse, zero_ptr, zero_bytes, st);
+  if (!seqs.ragged && ctas <= device_sm_count())
+    return launch_delta_chain_tables(s, w, x, seqs.s[0].T, theta, dtype, init, key_stream, reverse, zero_ptr, zero_bytes,
+                                     st);
+  return launch_delta_chain_rows(s, w, x, seqs, theta, dtype, init, key_stream, reverse, zero_ptr, zero_bytes, st);
 }
 
 // ---------------------------------------------------------------------------------------
@@ -535,21 +547,102 @@ cudaError_t launch_delta_chain(const Shape& s, const Workspace& w, const void* q
 //       indices, counters of Eq. 6 (d multiply-adds per in-window causal pair,
 //       nnz(Delta q_i) per out-of-window pair, against d per causal pair of dense attention).
 //   [n_idx_blocks, ...): one block per (batch, KV head, 64 keys): hand-off row
-//       R(T-1)[j] = q_hat(T-1).k_j for the heads of the group, and the channel-major fp32 key
-//       copy when kt != nullptr.
-template <typename TIn, int D>
-__global__ void __launch_bounds__(256, 5) delta_finish_kernel(
+//       R(T-1)[j] = q_hat(T-1).k_j for the heads of the group.
+namespace {
+__device__ __forceinline__ float2 load_pair(const float* p) { return *reinterpret_cast<const float2*>(p); }
+__device__ __forceinline__ float2 load_pair(const __nv_bfloat16* p) {
+  const uint32_t u = *reinterpret_cast<const uint32_t*>(p);
+  return make_float2(__uint_as_float(u << 16), __uint_as_float(u & 0xffff0000u));
+}
+__device__ __forceinline__ void load_eight(const float* p, float (&x)[8]) {
+  const float4 a = *reinterpret_cast<const float4*>(p), b = *reinterpret_cast<const float4*>(p + 4);
+  x[0] = a.x; x[1] = a.y; x[2] = a.z; x[3] = a.w; x[4] = b.x; x[5] = b.y; x[6] = b.z; x[7] = b.w;
+}
+__device__ __forceinline__ void load_eight(const __nv_bfloat16* p, float (&x)[8]) {
+  const uint4 u = *reinterpret_cast<const uint4*>(p);
+  const uint32_t w[4] = {u.x, u.y, u.z, u.w};
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    x[2 * i] = __uint_as_float(w[i] << 16);
+    x[2 * i + 1] = __uint_as_float(w[i] & 0xffff0000u);
+  }
+}
+// bit i of the low half to bit 2i
+__device__ __forceinline__ uint32_t spread16(uint32_t x) {
+  x &= 0xffffu;
+  x = (x | (x << 8)) & 0x00ff00ffu;
+  x = (x | (x << 4)) & 0x0f0f0f0fu;
+  x = (x | (x << 2)) & 0x33333333u;
+  return (x | (x << 1)) & 0x55555555u;
+}
+
+// Eq. 2-3 over the 8 rows of a block from its checkpoint (ck): delta values (dqp), reference rows (refp,
+// key deltas), fired channels ascending (srow, 8 x D bytes in shared memory, 0xFF where none), and in
+// lanes r and r + 8, .. the mask words of row r.  Lane = channels 2 lane, 2 lane + 1 of 64 at a time.
+// REV: strategy (2), rows from the top.  FULL: the block has all 8 rows and no un-thresholded basis row.
+template <typename TIn, int D, bool REV, bool FULL>
+__device__ __forceinline__ void finish_rows(const TIn* __restrict__ q, const float* __restrict__ ck, float* __restrict__ dqp,
+                                            __nv_bfloat16* __restrict__ refp, uint8_t* srow, int rbase, int T, float theta,
+                                            int basis_exact, uint32_t (&mw)[D / 32]) {
+  const int lane = threadIdx.x & 31;
+  const uint32_t lt = (1u << lane) - 1u;
+  int before[8];                                   // fired channels of the row in front of these 64
+#pragma unroll
+  for (int rr = 0; rr < 8; ++rr) before[rr] = 0;
+#pragma unroll
+  for (int c2 = 0; c2 < D / 64; ++c2) {
+    const int c = 64 * c2 + 2 * lane;
+    float2 ref = __ldcg(reinterpret_cast<const float2*>(ck + c));
+    const TIn* const qp = q + (size_t)rbase * D + c;
+    float2 v[8];
+#pragma unroll
+    for (int r = 0; r < 8; ++r) v[r] = (FULL || rbase + r < T) ? load_pair(qp + r * D) : make_float2(0.0f, 0.0f);
+    uint32_t even = 0, odd = 0;                    // of the lane's row
+#pragma unroll
+    for (int rr = 0; rr < 8; ++rr) {
+      const int r = REV ? 7 - rr : rr;
+      const bool live = FULL || rbase + r < T;
+      const bool basis = !FULL && basis_exact && rbase + r == (REV ? T - 1 : 0);
+      const float d0 = basis ? v[r].x : __fsub_rn(v[r].x, ref.x), d1 = basis ? v[r].y : __fsub_rn(v[r].y, ref.y);
+      const bool f0 = live && (basis || fabsf(d0) > theta), f1 = live && (basis || fabsf(d1) > theta);
+      ref.x = f0 ? v[r].x : ref.x;
+      ref.y = f1 ? v[r].y : ref.y;
+      if (live) {
+        *reinterpret_cast<float2*>(dqp + r * D + c) = make_float2(f0 ? d0 : 0.0f, f1 ? d1 : 0.0f);
+        if (refp)                                  // exactly bf16
+          *reinterpret_cast<uint32_t*>(refp + r * D + c) = __byte_perm(__float_as_uint(ref.x), __float_as_uint(ref.y), 0x7632);
+      }
+      const uint32_t be = __ballot_sync(0xffffffffu, f0), bo = __ballot_sync(0xffffffffu, f1);
+      uint8_t* const at = srow + r * D + before[r] + __popc(be & lt) + __popc(bo & lt);
+      if (f0) at[0] = (uint8_t)c;
+      if (f1) at[f0 ? 1 : 0] = (uint8_t)(c + 1);
+      if (c2 + 1 < D / 64) before[r] += __popc(be) + __popc(bo);
+      if ((lane & 7) == r) { even = be; odd = bo; }
+    }
+    mw[2 * c2] = spread16(even) | (spread16(odd) << 1);
+    mw[2 * c2 + 1] = spread16(even >> 16) | (spread16(odd >> 16) << 1);
+  }
+}
+}  // namespace
+
+template <typename TIn, int D, int N>
+__global__ void __launch_bounds__(256, D == 64 ? 5 : 4) delta_finish_kernel(
+    const __grid_constant__ SeqList<N> seqs,
     uint32_t* __restrict__ mask, uint16_t* __restrict__ row_nnz,
     uint32_t* __restrict__ tile_nnz, uint8_t* __restrict__ idx,
     unsigned long long* __restrict__ counters, const TIn* __restrict__ k,
-    const float* __restrict__ qhat, float* __restrict__ R, float* __restrict__ kt, int T,
-    int T_max, int n_tiles, int BH, int H, int g, int W, int shape, int n_idx_blocks, int kt_ld,
-    int key_stream, const TIn* __restrict__ q, int src_rows, float* __restrict__ dq,
+    const float* __restrict__ qhat, float* __restrict__ R,
+    int T_max, int n_tiles, int heads, int seq_heads, int seq_kv, int H, int g, int shape,
+    int key_stream, const TIn* __restrict__ x, float* __restrict__ dq,
     __nv_bfloat16* __restrict__ ref_rows, const float* __restrict__ ckpt, int n_ckpt, float theta,
     int basis_exact, int reverse, int wait_front) {
-  // q: the stream the chain kernel ran over, [heads][src_rows][D]; ref_rows (key deltas): the
-  // reference after every row, the cache of reference keys
+  // x: the stream the chain kernel ran over (see there); ref_rows (key deltas): the reference after
+  // every row, the cache of reference keys.  heads: heads of the delta stream per batch element;
+  // seq_heads, seq_kv: heads of the stream, KV heads that one entry of seqs stands for.
   constexpr int NW = D / 32;
+  const Seq& sq = seqs.s[N == 1 ? 0 : blockIdx.y];
+  const int T = sq.T, W = sq.W, src_rows = key_stream ? T_max : T;
+  const int tiles_used = (T + DELTA_TILE_ROWS - 1) / DELTA_TILE_ROWS, n_idx_blocks = seq_heads * tiles_used;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   // Launched with programmatic stream serialisation.  wait_front: the results of everything
   // in front are visible from here on (no effect in an ordinary launch).  Without it (query
@@ -563,108 +656,70 @@ __global__ void __launch_bounds__(256, 5) delta_finish_kernel(
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   if ((int)blockIdx.x < n_idx_blocks) {
     // ---- one block per (batch, head, 64-row tile); warp w serves rows 8w .. 8w+7
-    __shared__ unsigned long long s_red[3][8];
-    const int tiles_used = (T + DELTA_TILE_ROWS - 1) / DELTA_TILE_ROWS;
-    const int bh = blockIdx.x / tiles_used, tile = blockIdx.x - bh * tiles_used;
+    __shared__ uint32_t s_red[3][8];
+    const int hl = blockIdx.x / tiles_used, tile = blockIdx.x - hl * tiles_used;
+    const int bh = sq.b * heads + hl;                // head of the workspace arrays
+    const TIn* const q = key_stream ? x + (size_t)bh * T_max * D : x + sq.q_off + (size_t)hl * T * D;
     const int t0 = tile * DELTA_TILE_ROWS;
     const int rows = min(DELTA_TILE_ROWS, T - t0);
     const int r_mine = warp * 8 + (lane & 7);        // lanes 0..7 hold one row each
+    // The chain kernel left only the reference in front of every 8-row block.  The warp re-runs
+    // Eq. 2-3 over its 8 rows, lane = two neighbouring channels, 64 channels at a time: delta values
+    // (a row leaves as one 256-byte store), reference rows (key deltas), two ballots per row (even and
+    // odd channels), the rank of every fired channel in its row.
+    __shared__ __align__(16) uint8_t s_idx[8][8 * D];
+    uint8_t* const srow = s_idx[warp];
+    const int rbase = t0 + warp * 8, my_rows = min(8, rows - warp * 8);
     uint32_t mw[NW];
-    {
-      // The chain kernel left only the reference in front of every 8-row block.  The warp
-      // re-runs Eq. 2-3 over its 8 rows (lane = channel of a mask word): delta values, reference
-      // rows (key deltas), and one ballot per row for the mask word.
-      const int rbase = t0 + warp * 8;
 #pragma unroll
-      for (int w2 = 0; w2 < NW; ++w2) {
-        const int c = w2 * 32 + lane;
-        uint32_t word_mine = 0;
-        if (rbase < T && DELTA_IN(rbase / DELTA_CKPT_ROWS, n_ckpt, counters) && DELTA_IN(rbase + 7 < T ? rbase + 7 : T - 1, src_rows, counters) &&
-            DELTA_IN(T - 1, T_max, counters)) {
-          float ref = __ldcg(&ckpt[((size_t)bh * n_ckpt + rbase / DELTA_CKPT_ROWS) * D + c]);
-          float x[8];
+    for (int w2 = 0; w2 < NW; ++w2) mw[w2] = 0u;
+    if (rbase < T && DELTA_IN(rbase / DELTA_CKPT_ROWS, n_ckpt, counters) &&
+        DELTA_IN(rbase + 7 < T ? rbase + 7 : T - 1, src_rows, counters) && DELTA_IN(T - 1, T_max, counters)) {
 #pragma unroll
-          for (int r = 0; r < 8; ++r)
-            x[r] = (rbase + r < T) ? to_f32(q[((size_t)bh * src_rows + rbase + r) * D + c]) : 0.0f;
-#pragma unroll
-          for (int rr = 0; rr < 8; ++rr) {
-            const int r = reverse ? 7 - rr : rr;         // strategy (2) takes the rows from the top
-            const bool live = rbase + r < T;
-            bool fire;
-            float delta;
-            if (rbase + r == (reverse ? T - 1 : 0) && basis_exact) {
-              fire = true;                               // the basis vector is kept whole
-              delta = x[r];
-            } else {
-              const float diff = __fsub_rn(x[r], ref);
-              fire = fabsf(diff) > theta;
-              delta = fire ? diff : 0.0f;
-            }
-            fire = fire && live;
-            if (live) {
-              dq[((size_t)bh * T_max + rbase + r) * D + c] = delta;
-              ref = fire ? x[r] : ref;
-              if (ref_rows) ref_rows[((size_t)bh * T_max + rbase + r) * D + c] = __float2bfloat16_rn(ref);
-            }
-            const uint32_t word = __ballot_sync(0xffffffffu, fire);
-            if ((lane & 7) == r) word_mine = word;
-          }
-        }
-        mw[w2] = word_mine;
-        if (lane < 8 && r_mine < rows) mask[((size_t)bh * T_max + t0 + r_mine) * NW + w2] = word_mine;
-      }
+      for (int e = lane; e < 8 * D / 16; e += 32)
+        reinterpret_cast<uint4*>(srow)[e] = make_uint4(0xffffffffu, 0xffffffffu, 0xffffffffu, 0xffffffffu);
+      __syncwarp();
+      const bool plain = rbase + 8 <= T && !(basis_exact && (reverse ? rbase + 8 == T : rbase == 0));
+#define ROWS(REV, FULL)                                                                                          \
+  finish_rows<TIn, D, REV, FULL>(q, ckpt + ((size_t)bh * n_ckpt + rbase / DELTA_CKPT_ROWS) * D,                  \
+                                 dq + ((size_t)bh * T_max + rbase) * D,                                          \
+                                 ref_rows ? ref_rows + ((size_t)bh * T_max + rbase) * D : nullptr, srow, rbase, T, theta, \
+                                 basis_exact, mw)
+      if (reverse) { if (plain) ROWS(true, true); else ROWS(true, false); }
+      else { if (plain) ROWS(false, true); else ROWS(false, false); }
+#undef ROWS
     }
-    unsigned long long done = 0, dense = 0, tsum = 0;
+    if (lane < 8 && r_mine < rows) {
+      uint32_t* const mp = mask + ((size_t)bh * T_max + t0 + r_mine) * NW;
+      if constexpr (NW == 2) *reinterpret_cast<uint2*>(mp) = make_uint2(mw[0], mw[1]);
+      else *reinterpret_cast<uint4*>(mp) = make_uint4(mw[0], mw[1], mw[2], mw[3]);
+    }
+    // Eq. 6 (32 bits hold a warp's eight rows: 8 x 65536 keys x 128 channels x 8 heads)
+    uint32_t done = 0, dense = 0, tsum = 0;
     if (lane < 8 && r_mine < rows && DELTA_IN(t0 + r_mine, T_max, counters)) {
-      int nnz = 0;
+      uint32_t nnz = 0;
 #pragma unroll
       for (int w2 = 0; w2 < NW; ++w2) nnz += __popc(mw[w2]);
       row_nnz[(size_t)bh * T_max + t0 + r_mine] = (uint16_t)nnz;
-      tsum = (unsigned long long)nnz;
+      tsum = nnz;
       const int i = t0 + r_mine;
       if (!key_stream) {
         // query deltas: row i meets i + 1 keys, nnz multiply-adds per out-of-window key
-        const int n_in = in_window_count(i, W, shape);
-        done = (unsigned long long)n_in * D + (unsigned long long)(i + 1 - n_in) * nnz;
-        dense = (unsigned long long)(i + 1) * D;
+        const uint32_t n_in = (uint32_t)in_window_count(i, W, shape);
+        done = n_in * D + ((uint32_t)(i + 1) - n_in) * nnz;
+        dense = (uint32_t)(i + 1) * D;
       } else {
         // key deltas: key i meets the T - i queries behind it, for each of the g query heads
-        const int n_q = T - i;
-        const int n_in = in_window_col_count(i, T, W, shape);
-        done = (unsigned long long)g * ((unsigned long long)n_in * D + (unsigned long long)(n_q - n_in) * nnz);
-        dense = (unsigned long long)g * n_q * D;
+        const uint32_t n_q = (uint32_t)(T - i), n_in = (uint32_t)in_window_col_count(i, T, W, shape);
+        done = (uint32_t)g * (n_in * D + (n_q - n_in) * nnz);
+        dense = (uint32_t)g * n_q * D;
       }
     }
-    for (int o = 4; o > 0; o >>= 1) {
-      tsum += __shfl_down_sync(0xffffffffu, tsum, o);
-      done += __shfl_down_sync(0xffffffffu, done, o);
-      dense += __shfl_down_sync(0xffffffffu, dense, o);
-    }
+    tsum = __reduce_add_sync(0xffffffffu, tsum);
+    done = __reduce_add_sync(0xffffffffu, done);
+    dense = __reduce_add_sync(0xffffffffu, dense);
     if (lane == 0) { s_red[0][warp] = tsum; s_red[1][warp] = done; s_red[2][warp] = dense; }
-    // compacted indices: lane = channel within each mask word; the warp's 8 rows are assembled
-    // in shared memory and leave as 16-byte stores (8 consecutive rows are contiguous)
-    __shared__ __align__(16) uint8_t s_idx[8][8 * D];
-    uint8_t* srow = s_idx[warp];
-    const int my_rows = min(8, rows - warp * 8);
-    for (int r = 0; r < my_rows; ++r) {
-      uint32_t m[NW];
-      int nnz = 0;
-#pragma unroll
-      for (int w2 = 0; w2 < NW; ++w2) {
-        m[w2] = __shfl_sync(0xffffffffu, mw[w2], r);
-        nnz += __popc(m[w2]);
-      }
-      int basep = 0;
-#pragma unroll
-      for (int w2 = 0; w2 < NW; ++w2) {
-        if ((m[w2] >> lane) & 1u)
-          srow[r * D + basep + __popc(m[w2] & ((1u << lane) - 1u))] = (uint8_t)(w2 * 32 + lane);
-        basep += __popc(m[w2]);
-      }
-#pragma unroll
-      for (int pp = lane; pp < D; pp += 32)
-        if (pp >= nnz) srow[r * D + pp] = 0xFF;
-    }
+    // the compacted indices leave as 16-byte stores (8 consecutive rows are contiguous)
     __syncwarp();
     {
       uint4* dst = reinterpret_cast<uint4*>(idx + ((size_t)bh * T_max + t0 + warp * 8) * D);
@@ -685,68 +740,59 @@ __global__ void __launch_bounds__(256, 5) delta_finish_kernel(
     return;
   }
 
-  // ---- key pass: 64 keys of one (batch, KV head)
-  __shared__ float tile[D][65];
-  __shared__ float qh[8][D];
+  // ---- key pass: 64 keys of one (batch, KV head): R(T-1)[j] = q_hat(T-1).k_j, D / 8 lanes per key
+  __shared__ __align__(16) float qh[8][D];
   const int kblocks = (T + 63) / 64;
-  const int item = (int)blockIdx.x - n_idx_blocks;
-  const int bkv = item / kblocks, j0 = (item - bkv * kblocks) * 64;
-  const int H_kv = H / g;
+  const int item = (int)blockIdx.x - n_idx_blocks, kv_l = item / kblocks, j0 = (item - kv_l * kblocks) * 64;
+  if (key_stream || kv_l >= seq_kv) return;          // (a shorter sequence of a ragged group)
+  const int H_kv = H / g, bkv = sq.b * H_kv + kv_l;
   const int b = bkv / H_kv, kvh = bkv - b * H_kv;
-  const TIn* kp = k + (size_t)bkv * T_max * D;
-  {
-    constexpr int VEC = 16 / sizeof(TIn);            // elements per 16-byte load
-    constexpr int CPR = D / VEC;                     // 16-byte chunks per key row
-    for (int e = tid; e < 64 * CPR; e += 256) {
-      const int j = e / CPR, c = (e - j * CPR) * VEC;
-      TIn vals[VEC];
-      if (j0 + j < T) {
-        *reinterpret_cast<uint4*>(vals) = *reinterpret_cast<const uint4*>(kp + (size_t)(j0 + j) * D + c);
-#pragma unroll
-        for (int i = 0; i < VEC; ++i) tile[c + i][j] = to_f32(vals[i]);
-      } else {
-#pragma unroll
-        for (int i = 0; i < VEC; ++i) tile[c + i][j] = 0.0f;
-      }
-    }
-  }
-  for (int e = tid; e < g * D; e += 256) {
-    const int hh = e / D, c = e - hh * D;
-    qh[hh][c] = __ldcg(&qhat[((size_t)b * H + kvh * g + hh) * D + c]);
-  }
+  for (int e = tid; e < g * D; e += 256) qh[e / D][e % D] = __ldcg(&qhat[((size_t)b * H + kvh * g) * D + e]);
   __syncthreads();
-  if (kt != nullptr) {
-    float* op = kt + (size_t)bkv * D * kt_ld;
-    for (int e = tid; e < 64 * D; e += 256) {
-      const int c = e >> 6, j = e & 63;
-      if (j0 + j < kt_ld) op[(size_t)c * kt_ld + j0 + j] = tile[c][j];
-    }
-  }
-  {
-    const int j = tid & 63;
-    for (int hh = tid >> 6; hh < g; hh += 4) {
-      float acc = 0.0f;
-#pragma unroll 8
-      for (int c = 0; c < D; ++c) acc = fmaf(qh[hh][c], tile[c][j], acc);
-      if (j0 + j < T && DELTA_IN(j0 + j, T_max, counters)) R[((size_t)b * H + kvh * g + hh) * T_max + j0 + j] = acc;
+  constexpr int LPK = D / 8, KPW = 32 / LPK;         // lanes per key, keys per warp and pass
+  const int sub = lane / LPK, c0 = (lane % LPK) * 8;
+#pragma unroll
+  for (int i = 0; i < 8 / KPW; ++i) {
+    const int j = j0 + 8 * warp + i * KPW + sub;
+    float kv[8];
+    load_eight(k + ((size_t)bkv * T_max + min(j, T - 1)) * D + c0, kv);
+    for (int hh = 0; hh < g; ++hh) {
+      const float4 a = *reinterpret_cast<const float4*>(&qh[hh][c0]), c = *reinterpret_cast<const float4*>(&qh[hh][c0 + 4]);
+      float acc = a.x * kv[0];
+      acc = fmaf(a.y, kv[1], acc); acc = fmaf(a.z, kv[2], acc); acc = fmaf(a.w, kv[3], acc);
+      acc = fmaf(c.x, kv[4], acc); acc = fmaf(c.y, kv[5], acc); acc = fmaf(c.z, kv[6], acc); acc = fmaf(c.w, kv[7], acc);
+#pragma unroll
+      for (int o = LPK / 2; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+      if (lane % LPK == 0 && j < T && DELTA_IN(j, T_max, counters)) R[((size_t)b * H + kvh * g + hh) * T_max + j] = acc;
     }
   }
 }
 
-cudaError_t launch_delta_finish(const Shape& s, const Workspace& w, const void* q, const void* k, int T,
-                                float theta, int window, int shape, int dtype, int init, bool want_kt,
-                                bool key_stream, bool reverse, int programmatic, cudaStream_t st) {
+// The channel-major fp32 copy of the keys that the tensor-core kernel with the FP32 delta path reads.
+template <typename TIn, int D>
+__global__ void __launch_bounds__(256) key_copy_kernel(const TIn* __restrict__ k, float* __restrict__ kt, int T, int T_max, int kt_ld) {
+  __shared__ float tile[D][65];
+  const int bkv = blockIdx.y, j0 = blockIdx.x * 64;
+  for (int e = threadIdx.x; e < 64 * D; e += 256) {
+    const int j = e / D, c = e % D;
+    tile[c][j] = j0 + j < T ? to_f32(k[((size_t)bkv * T_max + j0 + j) * D + c]) : 0.0f;
+  }
+  __syncthreads();
+  for (int e = threadIdx.x; e < 64 * D; e += 256)
+    if (j0 + (e & 63) < kt_ld) kt[((size_t)bkv * D + (e >> 6)) * kt_ld + j0 + (e & 63)] = tile[e >> 6][e & 63];
+}
+
+template <typename TIn, int D, int N>
+static cudaError_t launch_finish(const Shape& s, const Workspace& w, const void* q, const void* k, const SeqBatch& seqs,
+                                 float theta, int shape, int init, bool want_kt, bool key_stream, bool reverse,
+                                 int programmatic, cudaStream_t st) {
   // programmatic: 0 = ordinary launch, 1 = programmatic serialisation, 2 = the same and the kernel
   // does not wait for the kernel in front (see the kernel)
   // key deltas: the index/counter pass runs over the KV heads and there is no hand-off row
-  const int BH = s.B * (key_stream ? s.H_kv : s.H);
-  const int tiles_used = (T + DELTA_TILE_ROWS - 1) / DELTA_TILE_ROWS;
-  const int n_idx_blocks = BH * tiles_used;
-  const int n_key_blocks = key_stream ? 0 : s.B * s.H_kv * ((T + 63) / 64);
-  const int kt_ld = (s.T_max + 3) / 4 * 4;
-  float* kt = (want_kt && w.kt) ? w.kt : nullptr;
+  const int heads = key_stream ? s.H_kv : s.H, nb = seqs.ragged ? 1 : s.B;
+  const int tiles = (seqs.T_longest + DELTA_TILE_ROWS - 1) / DELTA_TILE_ROWS;
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)(n_idx_blocks + n_key_blocks));
+  cfg.gridDim = dim3((unsigned)(nb * (heads * tiles + (key_stream ? 0 : s.H_kv * tiles))), (unsigned)seqs.n);
   cfg.blockDim = dim3(256);
   cfg.stream = st;
   cudaLaunchAttribute attr[1];
@@ -754,22 +800,37 @@ cudaError_t launch_delta_finish(const Shape& s, const Workspace& w, const void* 
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = programmatic ? 1 : 0;
-  cudaError_t err = cudaSuccess;
-#define LAUNCH(TIN, DD)                                                                          \
-  err = cudaLaunchKernelEx(&cfg, delta_finish_kernel<TIN, DD>,                                   \
-      w.mask, w.row_nnz, w.tile_nnz, w.idx, w.counters, (const TIN*)k, (const float*)w.qhat[0], w.R, kt, T,    \
-      s.T_max, s.n_tiles, BH, s.H, s.g(), window, shape, n_idx_blocks, kt_ld, key_stream ? 1 : 0,   \
-      key_stream ? (const TIN*)k : (const TIN*)q, key_stream ? s.T_max : T, w.dq,                 \
-      key_stream ? w.qhat_rows : (__nv_bfloat16*)nullptr, (const float*)w.ckpt, s.n_ckpt(), theta, \
-      init == DELTA_INIT_BASIS_EXACT ? 1 : 0, reverse ? 1 : 0, programmatic == 2 ? 0 : 1)
-  if (dtype == DELTA_F32) {
-    if (s.d == 64) LAUNCH(float, 64); else LAUNCH(float, 128);
-  } else {
-    if (s.d == 64) LAUNCH(__nv_bfloat16, 64); else LAUNCH(__nv_bfloat16, 128);
-  }
-#undef LAUNCH
+  SeqList<N> list;
+  for (int i = 0; i < N; ++i) list.s[i] = seqs.s[i < seqs.n ? i : 0];
+  const cudaError_t err = cudaLaunchKernelEx(
+      &cfg, delta_finish_kernel<TIn, D, N>, list, w.mask, w.row_nnz, w.tile_nnz, w.idx, w.counters, (const TIn*)k,
+      (const float*)w.qhat[0], w.R, s.T_max, s.n_tiles, heads, nb * heads, nb * s.H_kv,
+      s.H, s.g(), shape, key_stream ? 1 : 0, (const TIn*)(key_stream ? k : q), w.dq,
+      key_stream ? w.qhat_rows : (__nv_bfloat16*)nullptr, (const float*)w.ckpt, s.n_ckpt(), theta,
+      init == DELTA_INIT_BASIS_EXACT ? 1 : 0, reverse ? 1 : 0, programmatic == 2 ? 0 : 1);
   count_launch();
+  if (err == cudaSuccess && want_kt && w.kt) {       // (uniform batches only)
+    key_copy_kernel<TIn, D><<<dim3((unsigned)((seqs.T_longest + 63) / 64), (unsigned)(s.B * s.H_kv)), 256, 0, st>>>(
+        (const TIn*)k, w.kt, seqs.T_longest, s.T_max, (s.T_max + 3) / 4 * 4);
+    count_launch();
+  }
   return err != cudaSuccess ? err : cudaGetLastError();
+}
+
+cudaError_t launch_delta_finish(const Shape& s, const Workspace& w, const void* q, const void* k, const SeqBatch& seqs,
+                                float theta, int shape, int dtype, int init, bool want_kt, bool key_stream, bool reverse,
+                                int programmatic, cudaStream_t st) {
+#define GO(TIN, DD)                                                                                               \
+  return seqs.ragged ? launch_finish<TIN, DD, kSeqMax>(s, w, q, k, seqs, theta, shape, init, want_kt, key_stream, \
+                                                       reverse, programmatic, st)                                 \
+                     : launch_finish<TIN, DD, 1>(s, w, q, k, seqs, theta, shape, init, want_kt, key_stream, reverse, \
+                                                 programmatic, st)
+  if (dtype == DELTA_F32) {
+    if (s.d == 64) { GO(float, 64); } else { GO(float, 128); }
+  } else {
+    if (s.d == 64) { GO(__nv_bfloat16, 64); } else { GO(__nv_bfloat16, 128); }
+  }
+#undef GO
 }
 
 }  // namespace delta

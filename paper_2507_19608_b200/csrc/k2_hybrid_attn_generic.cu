@@ -118,11 +118,13 @@ __device__ __forceinline__ void mma_parts(float (&big)[4], float (&small)[4], co
 }
 }  // namespace
 
-template <typename TIn, int D, int KS>
+template <typename TIn, int D, int KS, int N>
 __global__ void __launch_bounds__(NT, D == 64 ? 2 : 1) hybrid_attn_f32_kernel(
     const TIn* __restrict__ q, const TIn* __restrict__ k, const TIn* __restrict__ v, TIn* __restrict__ out,
-    const float* __restrict__ ckpt, unsigned long long* __restrict__ counters, int T, int T_max, int n_ckpt, int H, int g,
-    int W, int shape, float theta, int basis_row, float scale_log2e) {
+    const float* __restrict__ ckpt, unsigned long long* __restrict__ counters, const __grid_constant__ SeqList<N> seqs,
+    int T_max, int n_ckpt, int H, int g, int shape, float theta, int basis_row, float scale_log2e) {
+  const Seq& sq = seqs.s[N == 1 ? 0 : blockIdx.z];
+  const int T = sq.T, W = sq.W;
   constexpr int NP = sizeof(TIn) == 4 ? 3 : 1;
   using SM = F32Smem<D, KS, NP>;
   constexpr int BM = SM::BM, NB = D / 64;          // NB: 64-channel blocks of a row
@@ -135,8 +137,10 @@ __global__ void __launch_bounds__(NT, D == 64 ? 2 : 1) hybrid_attn_f32_kernel(
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int g8 = lane >> 2, t4 = lane & 3;         // row of the fragments, thread of the row
   const int rg = warp / KS, kg = warp % KS;        // the warp's 16 rows, its share of a tile's keys
-  const int qt = (int)gridDim.x - 1 - (int)blockIdx.x;     // longest walks first
-  const int bh = blockIdx.y, b = bh / H, h = bh - b * H;
+  const int qt = (T + BM - 1) / BM - 1 - (int)blockIdx.x;  // longest walks first
+  if (N > 1 && qt < 0) return;                             // (a shorter sequence of a ragged group)
+  const int bh = sq.b * H + (int)blockIdx.y, b = bh / H, h = bh - b * H;
+  const size_t io = sq.q_off + (size_t)blockIdx.y * T * D;      // the head's rows in q and out
   const size_t bkv = (size_t)b * (H / g) + h / g;
   const int i0 = qt * BM, i1 = min(i0 + BM, T) - 1;
   const TIn* const kp = k + bkv * T_max * D;
@@ -166,7 +170,7 @@ __global__ void __launch_bounds__(NT, D == 64 ? 2 : 1) hybrid_attn_f32_kernel(
   for (int e = tid; e < BM * (D / 8); e += NT) {
     const int r = e / (D / 8), c = e % (D / 8);
     float x[8] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
-    if (i0 + r < T) load8f(q + ((size_t)bh * T + i0 + r) * D + 8 * c, x);
+    if (i0 + r < T) load8f(q + io + (size_t)(i0 + r) * D + 8 * c, x);
     store_parts<NP>(base + (c >> 3) * (BM * 128), SM::QPART, r, c & 7, x);
 #pragma unroll
     for (int i = 0; i < 8; i += 4)
@@ -393,7 +397,7 @@ __global__ void __launch_bounds__(NT, D == 64 ? 2 : 1) hybrid_attn_f32_kernel(
     const int i = e2 ? ib : ia;
     if (i < T && DELTA_IN(i, T, counters)) {
       const float inv = 1.0f / l[e2];
-      TIn* const op = out + ((size_t)bh * T + i) * D + 2 * t4;
+      TIn* const op = out + io + (size_t)i * D + 2 * t4;
 #pragma unroll
       for (int x = 0; x < NB; ++x)
 #pragma unroll
@@ -406,10 +410,10 @@ __global__ void __launch_bounds__(NT, D == 64 ? 2 : 1) hybrid_attn_f32_kernel(
   }
 }
 
-template <typename TIn, int D, int KS>
+template <typename TIn, int D, int KS, int N>
 static cudaError_t launch_f32(const Shape& s, const Workspace& w, const void* q, const void* k, const void* v, void* out,
-                              int T, float theta, int init, int window, int shape, cudaStream_t st) {
-  auto kern = hybrid_attn_f32_kernel<TIn, D, KS>;
+                              const SeqBatch& seqs, float theta, int init, int shape, cudaStream_t st) {
+  auto kern = hybrid_attn_f32_kernel<TIn, D, KS, N>;
   constexpr size_t smem = F32Smem<D, KS, sizeof(TIn) == 4 ? 3 : 1>::bytes;
   static std::atomic<uint64_t> ready{0};
   if (!device_done(ready)) {
@@ -417,8 +421,11 @@ static cudaError_t launch_f32(const Shape& s, const Workspace& w, const void* q,
     if (e != cudaSuccess) return e;
     device_mark(ready);
   }
+  SeqList<N> list;
+  for (int i = 0; i < N; ++i) list.s[i] = seqs.s[i < seqs.n ? i : 0];
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)((T + 64 / KS - 1) / (64 / KS)), (unsigned)(s.B * s.H));
+  cfg.gridDim = dim3((unsigned)((seqs.T_longest + 64 / KS - 1) / (64 / KS)), (unsigned)(seqs.ragged ? s.H : s.B * s.H),
+                     (unsigned)seqs.n);
   cfg.blockDim = dim3(NT);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
@@ -429,31 +436,42 @@ static cudaError_t launch_f32(const Shape& s, const Workspace& w, const void* q,
   cfg.numAttrs = 1;
   const cudaError_t e =
       cudaLaunchKernelEx(&cfg, kern, (const TIn*)q, (const TIn*)k, (const TIn*)v, (TIn*)out, (const float*)w.ckpt, w.counters,
-                         T, s.T_max, s.n_ckpt(), s.H, s.g(), window, shape, theta, init == DELTA_INIT_BASIS_EXACT ? 0 : -1,
+                         list, s.T_max, s.n_ckpt(), s.H, s.g(), shape, theta, init == DELTA_INIT_BASIS_EXACT ? 0 : -1,
                          1.4426950408889634f / sqrtf((float)s.d));
   count_launch();
-  return e;
+  return e != cudaSuccess ? e : cudaGetLastError();
 }
 
-cudaError_t launch_hybrid_attn_generic(const Shape& s, const Workspace& w, const void* q, const void* k, const void* v,
-                                       void* out, int T, float theta, int init, int window, int shape, int dtype,
-                                       cudaStream_t st) {
+template <typename TIn, int D, int N>
+static cudaError_t launch_f32_form(const Shape& s, const Workspace& w, const void* q, const void* k, const void* v, void* out,
+                                   const SeqBatch& seqs, float theta, int init, int shape, cudaStream_t st) {
   // Warps per row group.  A key tile of 64 costs 3.3 / 2.2 / 1.4 us where a CTA walks alone and takes
   // 4.0 / 2.2 / 1.6 us of an SM where the chip is full (KS = 1 / 2 / 4; d = 64, 1 to 256 heads of 128 to
   // 4000 tokens); every halving of the rows doubles the tiles.  The longest walk bounds a small
   // grid, the sum of all tiles, with half a walk for the uneven end, a large one.
   int ks = 1;
-  float best = 3.4e38f;
+  float best = 3.4e38f, pairs = 0.0f;
+  for (int i = 0; i < seqs.n; ++i) {
+    const float t = (float)((seqs.s[i].T + BN - 1) / BN);
+    pairs += 0.5f * t * (t + 1.0f) * (float)((seqs.ragged ? 1 : s.B) * s.H);
+  }
   for (int c = 0; c < 3; ++c) {
     constexpr float alone[3] = {3.3f, 2.2f, 1.4f}, full[3] = {4.0f, 2.2f, 1.6f};
-    const float walk = (float)((T + BN - 1) / BN), tiles = 0.5f * walk * (walk + 1.0f) * (float)(1 << c) * (float)(s.B * s.H);
-    const float us = fmaxf(walk * alone[c], tiles / (float)device_sm_count() * full[c] + 0.5f * walk * alone[c]);
+    const float walk = (float)((seqs.T_longest + BN - 1) / BN) * alone[c];
+    const float us = fmaxf(walk, pairs * (float)(1 << c) / (float)device_sm_count() * full[c] + 0.5f * walk);
     if (us < best) { best = us; ks = 1 << c; }
   }
-#define GO(TIN, DD)                                                                                            \
-  return ks == 4   ? launch_f32<TIN, DD, 4>(s, w, q, k, v, out, T, theta, init, window, shape, st)            \
-         : ks == 2 ? launch_f32<TIN, DD, 2>(s, w, q, k, v, out, T, theta, init, window, shape, st)            \
-                    : launch_f32<TIN, DD, 1>(s, w, q, k, v, out, T, theta, init, window, shape, st)
+  return ks == 4   ? launch_f32<TIn, D, 4, N>(s, w, q, k, v, out, seqs, theta, init, shape, st)
+         : ks == 2 ? launch_f32<TIn, D, 2, N>(s, w, q, k, v, out, seqs, theta, init, shape, st)
+                   : launch_f32<TIn, D, 1, N>(s, w, q, k, v, out, seqs, theta, init, shape, st);
+}
+
+cudaError_t launch_hybrid_attn_generic(const Shape& s, const Workspace& w, const void* q, const void* k, const void* v,
+                                       void* out, const SeqBatch& seqs, float theta, int init, int shape, int dtype,
+                                       cudaStream_t st) {
+#define GO(TIN, DD)                                                                                       \
+  return seqs.ragged ? launch_f32_form<TIN, DD, kSeqMax>(s, w, q, k, v, out, seqs, theta, init, shape, st) \
+                     : launch_f32_form<TIN, DD, 1>(s, w, q, k, v, out, seqs, theta, init, shape, st)
   if (dtype == DELTA_F32) {
     if (s.d == 64) { GO(float, 64); } else { GO(float, 128); }
   } else {

@@ -114,13 +114,18 @@ struct TqParams {
   __nv_bfloat16* out;
   unsigned long long* counters;
   const float* ckpt;           // [B,H,n_ckpt,D] reference in front of every 8-row block (query deltas only)
-  int T, T_max, n_ckpt, H, g, W, shape;
-  int BH;            // heads in all (batch x query heads)
+  int T_max, n_ckpt, H, g, shape;
+  int BH;            // heads of one entry of the sequence list (uniform batch: batch x query heads)
+  int nqt;           // query tiles of the longest sequence
   int n_one;         // two-head layout: the n_one heaviest query tiles of every head go one head per CTA
   int reverse;       // strategy (2): Eq. 2-3 runs from row T-1 down to row 0
-  int basis_row;     // the un-thresholded basis row (0, or T-1 in reverse), -1 if there is none
+  int basis;         // is the first row taken (0, or T-1 in reverse) the un-thresholded basis?
   float scale_log2e, theta;
 };
+
+// Tensor maps of one entry of the sequence list: queries, reference-key rows, keys, values (rows 0..T-1).
+struct TqMaps { CUtensorMap q, qh, k, v; };
+template <int N> struct TqMapList { TqMaps m[N]; };
 
 // Barrier of the eight softmax warps (id 1, 256 threads; immediate id: a register operand would
 // make the compiler reserve all sixteen hardware barriers).
@@ -211,11 +216,12 @@ __device__ __forceinline__ void build_ref_rows(const unsigned char* q_src, unsig
 // and with it every register spill of the kernel.
 // FORM: 0 = every CTA one head; 1 = every CTA two heads; 2 = two-head layout, the form of a CTA
 // follows its place in the grid (see below).
-template <int D, bool KEY, int FORM, bool MIXED>
+// N: entries of the sequence list: 1 (a uniform batch), or kSeqMax (a ragged group: the grid is
+// [heads of all sequences][query tiles of the longest]; CTAs past their sequence's tiles return).
+template <int D, bool KEY, int FORM, bool MIXED, int N>
 __global__ void __launch_bounds__(NTHR, 1)
-hybrid_attn_tcq_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_qh,
-                       const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ CUtensorMap tm_v,
-                       const TqParams p) {
+hybrid_attn_tcq_kernel(const __grid_constant__ TqMapList<N> maps, const __grid_constant__ SeqList<N> seqs,
+                       const __grid_constant__ TqParams p) {
   extern __shared__ unsigned char smem_raw[];
   const uint32_t raw = smem_u32(smem_raw);
   const uint32_t base = (raw + 1023u) & ~1023u;
@@ -237,10 +243,17 @@ hybrid_attn_tcq_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
   // others the same query tile of two neighbouring heads of one KV group, bh and bh + 1 (group
   // X of the softmax warps takes head bh + X and every key tile).  pr: this CTA is of the
   // second kind.
-  int qt, bh;
+  int qt, bh, si = 0;
   bool pr = false;
-  if (PAIR) {
-    const int nqt = (p.T + BM - 1) / BM, idx = (int)blockIdx.x, n1 = (FORM == 1) ? 0 : p.BH * p.n_one;
+  if (N > 1) {
+    const int per = PAIR ? p.BH / 2 : p.BH, x = (int)blockIdx.x;
+    si = x / per;
+    bh = (x - si * per) * (PAIR ? 2 : 1);
+    pr = PAIR;
+    qt = (seqs.s[si].T + BM - 1) / BM - 1 - (int)blockIdx.y;
+    if (qt < 0) return;
+  } else if (PAIR) {
+    const int nqt = p.nqt, idx = (int)blockIdx.x, n1 = (FORM == 1) ? 0 : p.BH * p.n_one;
     if (FORM == 2 && idx < n1) {
       qt = nqt - 1 - idx / p.BH;
       bh = idx % p.BH;
@@ -254,9 +267,14 @@ hybrid_attn_tcq_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
     qt = (int)gridDim.y - 1 - (int)blockIdx.y;
     bh = (int)blockIdx.x;
   }
+  // (bh, bkv: head and KV head within the entry of the sequence list; g_bh: of the workspace arrays)
   const int b = bh / p.H, h = bh - b * p.H;
   const int bkv = b * (p.H / p.g) + h / p.g;
-  const int T = p.T, W = p.W, shape = p.shape;
+  const Seq& sq = seqs.s[si];
+  const int g_bh = sq.b * p.H;
+  const CUtensorMap &tm_q = maps.m[si].q, &tm_qh = maps.m[si].qh, &tm_k = maps.m[si].k, &tm_v = maps.m[si].v;
+  const int T = sq.T, W = sq.W, shape = p.shape;
+  const int basis_row = !p.basis ? -1 : p.reverse ? T - 1 : 0;
   const int i0 = qt * BM;
   const int i1 = min(i0 + BM, T) - 1;
   const int n = qt + 1;                                 // key tiles up to the diagonal
@@ -531,17 +549,17 @@ hybrid_attn_tcq_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
       // every CTA has come by here (the last wave included) it may run on the SMs left idle
       if (tid == 0) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
       const int r00 = i0 + seg * SEG;              // the thread's first row
-      const float* const ck = p.ckpt + ((size_t)bh_x * p.n_ckpt + r00 / DELTA_CKPT_ROWS) * D + c;
+      const float* const ck = p.ckpt + ((size_t)(g_bh + bh_x) * p.n_ckpt + r00 / DELTA_CKPT_ROWS) * D + c;
       const float2 ref0 = (r00 < T && DELTA_IN(min(r00 + SEG - 1, T - 1) / DELTA_CKPT_ROWS, p.n_ckpt, p.counters))
                               ? *reinterpret_cast<const float2*>(ck) : make_float2(0.0f, 0.0f);
       mbar_wait(BAR(BAR_Q), 0, abort_flag);      // the query tile has landed
       const unsigned char* const q_src = sm + OFF_Q + qsel + thr_off;
       unsigned char* const qh_dst = sm + OFF_QH + qsel + thr_off;
       unsigned char* const qm_dst = sm + OFF_QM + 2 * qsel + thr_off;
-      const bool check = (i0 + BM > T) || (p.basis_row >= i0 && p.basis_row < i0 + BM);
+      const bool check = (i0 + BM > T) || (basis_row >= i0 && basis_row < i0 + BM);
 #define BUILD(REV, CHECK)                                                                              \
   build_ref_rows<REV, CHECK>(q_src, qh_dst, qm_dst, SZ_TILE, offs, ck, D, ref0, nbk, p.theta, quarters, seg * SEG, \
-                                  i0, T, p.basis_row)
+                                  i0, T, basis_row)
       if (p.reverse) { if (check) BUILD(true, true); else BUILD(true, false); }
       else { if (check) BUILD(false, true); else BUILD(false, false); }
 #undef BUILD
@@ -806,7 +824,7 @@ hybrid_attn_tcq_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
             const __nv_bfloat162 t2 = __floats2bfloat162_rn(__uint_as_float(u[c]) * inv, __uint_as_float(u[c + 1]) * inv);
             w[c >> 1] = *reinterpret_cast<const uint32_t*>(&t2);
           }
-          uint4* op = reinterpret_cast<uint4*>(p.out + ((size_t)bh_x * T + i) * D + 32 * ch);
+          uint4* op = reinterpret_cast<uint4*>(p.out + sq.q_off + ((size_t)bh_x * T + i) * D + 32 * ch);
 #pragma unroll
           for (int q4 = 0; q4 < 4; ++q4) op[q4] = make_uint4(w[4 * q4], w[4 * q4 + 1], w[4 * q4 + 2], w[4 * q4 + 3]);
         }
@@ -859,7 +877,7 @@ hybrid_attn_tcq_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
           const __nv_bfloat162 t2 = __floats2bfloat162_rn(o0, o1);
           w[c >> 1] = *reinterpret_cast<const uint32_t*>(&t2);
         }
-        uint4* op = reinterpret_cast<uint4*>(p.out + ((size_t)bh * T + i) * D + HC * X + 32 * ch);
+        uint4* op = reinterpret_cast<uint4*>(p.out + sq.q_off + ((size_t)bh * T + i) * D + HC * X + 32 * ch);
 #pragma unroll
         for (int q4 = 0; q4 < 4; ++q4) op[q4] = make_uint4(w[4 * q4], w[4 * q4 + 1], w[4 * q4 + 2], w[4 * q4 + 3]);
       }
@@ -878,45 +896,61 @@ hybrid_attn_tcq_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
 #undef BAR
 }
 
-template <int D, bool KEY, int FORM, bool MIXED>
+template <int D, bool KEY, int FORM, bool MIXED, int N>
 static cudaError_t launch_tcq_m(const Shape& s, const Workspace& w, const void* q, const void* k, const void* v,
-                                void* out, int T, float theta, int init, int window, int shape, bool reverse,
+                                void* out, const SeqBatch& seqs, float theta, int init, int shape, bool reverse,
                                 int n_one, cudaStream_t st) {
   constexpr bool PAIR = FORM != 0;
-  const uint64_t BH = (uint64_t)s.B * s.H, BKV = (uint64_t)s.B * s.H_kv;
+  auto kern = hybrid_attn_tcq_kernel<D, KEY, FORM, MIXED, N>;
+  using TC = __nv_bfloat16;
+  const int nb = seqs.ragged ? 1 : s.B;
+  const uint64_t BH = (uint64_t)nb * s.H, BKV = (uint64_t)nb * s.H_kv;     // heads of one entry
   const uint64_t ref_heads = KEY ? BKV : BH;   // the reference rows follow the delta stream
-  CUtensorMap tq, tqh, tk, tv;
-  const bool ok =
-      encode3(&tq, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, q, D, (uint64_t)T, BH, D * 2, (uint64_t)T * D * 2, 64, 128,
-              CU_TENSOR_MAP_SWIZZLE_128B) &&
-      encode3(&tqh, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, w.qhat_rows, D, (uint64_t)T, ref_heads, D * 2,
-              (uint64_t)s.T_max * D * 2, 64, 128, CU_TENSOR_MAP_SWIZZLE_128B) &&
-      encode3(&tk, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, k, D, (uint64_t)T, BKV, D * 2, (uint64_t)s.T_max * D * 2, 64,
-              128, CU_TENSOR_MAP_SWIZZLE_128B) &&
-      encode3(&tv, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, v, D, (uint64_t)T, BKV, D * 2, (uint64_t)s.T_max * D * 2, 64,
-              128, CU_TENSOR_MAP_SWIZZLE_128B);
-  if (!ok) return cudaErrorInvalidValue;
-  cudaError_t err = cudaFuncSetAttribute(hybrid_attn_tcq_kernel<D, KEY, FORM, MIXED>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)TqSmem<D, PAIR>::BYTES);
-  if (err != cudaSuccess) return err;
+  TqMapList<N> maps;
+  SeqList<N> list;
+  for (int i = 0; i < seqs.n; ++i) {
+    const Seq& e = seqs.s[i];
+    const uint64_t T = (uint64_t)e.T;
+    const size_t kv = (size_t)e.b * s.H_kv * s.T_max * D, rf = (size_t)e.b * (KEY ? s.H_kv : s.H) * s.T_max * D;
+    TqMaps& m = maps.m[i];
+    list.s[i] = e;
+    const uint64_t cache = (uint64_t)s.T_max * D * 2;
+    if (!encode3(&m.q, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, (const TC*)q + e.q_off, D, T, BH, D * 2, T * D * 2, 64, 128,
+                 CU_TENSOR_MAP_SWIZZLE_128B) ||
+        !encode3(&m.k, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, (const TC*)k + kv, D, T, BKV, D * 2, cache, 64, 128,
+                 CU_TENSOR_MAP_SWIZZLE_128B) ||
+        !encode3(&m.v, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, (const TC*)v + kv, D, T, BKV, D * 2, cache, 64, 128,
+                 CU_TENSOR_MAP_SWIZZLE_128B) ||
+        (KEY && !encode3(&m.qh, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, w.qhat_rows + rf, D, T, ref_heads, D * 2, cache, 64, 128,
+                         CU_TENSOR_MAP_SWIZZLE_128B)))
+      return cudaErrorInvalidValue;
+  }
+  static std::atomic<uint64_t> ready{0};
+  if (!device_done(ready)) {
+    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TqSmem<D, PAIR>::BYTES);
+    if (e != cudaSuccess) return e;
+    device_mark(ready);
+  }
   TqParams p;
   p.out = (__nv_bfloat16*)out;
   p.counters = w.counters;
   p.ckpt = w.ckpt;
   p.T_max = s.T_max; p.n_ckpt = s.n_ckpt();
   p.theta = theta; p.reverse = reverse ? 1 : 0;
-  p.basis_row = (init == DELTA_INIT_BASIS_EXACT) ? (reverse ? T - 1 : 0) : -1;
-  p.T = T; p.H = s.H; p.g = s.g(); p.W = window; p.shape = shape;
+  p.basis = (init == DELTA_INIT_BASIS_EXACT) ? 1 : 0;
+  p.H = s.H; p.g = s.g(); p.shape = shape;
   p.scale_log2e = 1.4426950408889634f / sqrtf((float)s.d);
   // Launched with programmatic stream serialisation: the CTAs become resident and run their
   // prologue (tensor-memory allocation, barrier setup, query, key and value loads) while the
   // delta chain kernel in front is still running; they wait for its results with
   // griddepcontrol.wait.
   cudaLaunchConfig_t cfg = {};
-  const int nqt = (T + BM - 1) / BM;
+  const int nqt = (seqs.T_longest + BM - 1) / BM;
   p.BH = (int)BH;
+  p.nqt = nqt;
   p.n_one = (FORM == 2) ? (n_one < nqt ? n_one : nqt) : 0;
-  cfg.gridDim = PAIR ? dim3((unsigned)(BH * p.n_one + BH / 2 * (nqt - p.n_one))) : dim3((unsigned)BH, (unsigned)nqt);
+  if (N > 1) cfg.gridDim = dim3((unsigned)(seqs.n * (PAIR ? BH / 2 : BH)), (unsigned)nqt);
+  else cfg.gridDim = PAIR ? dim3((unsigned)(BH * p.n_one + BH / 2 * (nqt - p.n_one))) : dim3((unsigned)BH, (unsigned)nqt);
   cfg.blockDim = dim3(NTHR);
   cfg.dynamicSmemBytes = TqSmem<D, PAIR>::BYTES;
   cfg.stream = st;
@@ -925,7 +959,7 @@ static cudaError_t launch_tcq_m(const Shape& s, const Workspace& w, const void* 
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  err = cudaLaunchKernelEx(&cfg, hybrid_attn_tcq_kernel<D, KEY, FORM, MIXED>, tq, tqh, tk, tv, p);
+  const cudaError_t err = cudaLaunchKernelEx(&cfg, kern, maps, list, p);
   count_launch();
   return err != cudaSuccess ? err : cudaGetLastError();
 }
@@ -943,17 +977,20 @@ static bool mixed_tiles_possible(int window, int shape) {
 
 template <int D, bool KEY, int FORM>
 static cudaError_t launch_tcq(const Shape& s, const Workspace& w, const void* q, const void* k, const void* v,
-                              void* out, int T, float theta, int init, int window, int shape, bool reverse,
+                              void* out, const SeqBatch& seqs, float theta, int init, int shape, bool reverse,
                               int n_one, cudaStream_t st) {
-  return mixed_tiles_possible<D, KEY>(window, shape)
-             ? launch_tcq_m<D, KEY, FORM, true>(s, w, q, k, v, out, T, theta, init, window, shape, reverse, n_one, st)
-             : launch_tcq_m<D, KEY, FORM, false>(s, w, q, k, v, out, T, theta, init, window, shape, reverse, n_one, st);
+  if (seqs.ragged)       // (windows differ: with the mixed tiles' code)
+    return launch_tcq_m<D, KEY, FORM == 2 ? 0 : FORM, true, kSeqMax>(s, w, q, k, v, out, seqs, theta, init, shape, reverse, 0,
+                                                                    st);
+  return mixed_tiles_possible<D, KEY>(seqs.s[0].W, shape)
+             ? launch_tcq_m<D, KEY, FORM, true, 1>(s, w, q, k, v, out, seqs, theta, init, shape, reverse, n_one, st)
+             : launch_tcq_m<D, KEY, FORM, false, 1>(s, w, q, k, v, out, seqs, theta, init, shape, reverse, n_one, st);
 }
 
 bool tcq_kernel_shape(int d) { return d == 64 || d == 128; }
 
 cudaError_t launch_hybrid_attn_tcq(const Shape& s, const Workspace& w, const void* q, const void* k,
-                                   const void* v, void* out, int T, float theta, int init, int window,
+                                   const void* v, void* out, const SeqBatch& seqs, float theta, int init,
                                    int shape, bool key_deltas, bool reverse, int form, cudaStream_t st) {
   if (key_deltas && reverse) return cudaErrorNotSupported;
   if (!w.qhat_rows) return cudaErrorNotSupported;
@@ -966,9 +1003,12 @@ cudaError_t launch_hybrid_attn_tcq(const Shape& s, const Workspace& w, const voi
     // On a smaller grid that the one-head form cannot place in one wave, the heaviest query
     // tiles of every head go one head per CTA and the rest two heads per CTA, as many of the
     // former as one wave of SMs allows.
-    const long BH = (long)s.B * s.H, nqt = (T + BM - 1) / BM, sms = device_sm_count();
+    const long BH = (long)(seqs.ragged ? 1 : s.B) * s.H, sms = device_sm_count();
+    long nqt = 0;                         // query tiles of a head (ragged group: of a head of every sequence)
+    for (int i = 0; i < seqs.n; ++i) nqt += (seqs.s[i].T + BM - 1) / BM;
     int n_one = -1;                       // -1: the one-head kernel
-    if (form == 2) n_one = 0;
+    if (seqs.ragged) n_one = (two_heads_ok && form != 1 && BH / 2 * nqt >= 2 * sms) ? 0 : -1;
+    else if (form == 2) n_one = 0;
     else if (form == 3) n_one = 1;
     else if (form == 0 && two_heads_ok) {
       if (BH / 2 * nqt >= 2 * sms) n_one = 0;
@@ -976,21 +1016,21 @@ cudaError_t launch_hybrid_attn_tcq(const Shape& s, const Workspace& w, const voi
     }
     if (key_deltas) {
       if (n_one == 0)
-        return launch_tcq<64, true, 1>(s, w, q, k, v, out, T, theta, init, window, shape, reverse, 0, st);
+        return launch_tcq<64, true, 1>(s, w, q, k, v, out, seqs, theta, init, shape, reverse, 0, st);
       if (n_one > 0)
-        return launch_tcq<64, true, 2>(s, w, q, k, v, out, T, theta, init, window, shape, reverse, n_one, st);
-      return launch_tcq<64, true, 0>(s, w, q, k, v, out, T, theta, init, window, shape, reverse, 0, st);
+        return launch_tcq<64, true, 2>(s, w, q, k, v, out, seqs, theta, init, shape, reverse, n_one, st);
+      return launch_tcq<64, true, 0>(s, w, q, k, v, out, seqs, theta, init, shape, reverse, 0, st);
     }
     if (n_one == 0)
-      return launch_tcq<64, false, 1>(s, w, q, k, v, out, T, theta, init, window, shape, reverse, 0, st);
+      return launch_tcq<64, false, 1>(s, w, q, k, v, out, seqs, theta, init, shape, reverse, 0, st);
     if (n_one > 0)
-      return launch_tcq<64, false, 2>(s, w, q, k, v, out, T, theta, init, window, shape, reverse, n_one, st);
-    return launch_tcq<64, false, 0>(s, w, q, k, v, out, T, theta, init, window, shape, reverse, 0, st);
+      return launch_tcq<64, false, 2>(s, w, q, k, v, out, seqs, theta, init, shape, reverse, n_one, st);
+    return launch_tcq<64, false, 0>(s, w, q, k, v, out, seqs, theta, init, shape, reverse, 0, st);
   }
   if (s.d == 128)
     return key_deltas
-               ? launch_tcq<128, true, 0>(s, w, q, k, v, out, T, theta, init, window, shape, reverse, 0, st)
-               : launch_tcq<128, false, 0>(s, w, q, k, v, out, T, theta, init, window, shape, reverse, 0, st);
+               ? launch_tcq<128, true, 0>(s, w, q, k, v, out, seqs, theta, init, shape, reverse, 0, st)
+               : launch_tcq<128, false, 0>(s, w, q, k, v, out, seqs, theta, init, shape, reverse, 0, st);
   return cudaErrorNotSupported;
 }
 

@@ -19,6 +19,6 @@ bool tcq_kernel_shape(int d);
 // an even number of query heads per KV head; cudaErrorNotSupported otherwise); 3 = form 2 with
 // the heaviest query tile of every head in form 1; 0 = chosen by the size of the grid.
 cudaError_t launch_hybrid_attn_tcq(const Shape& s, const Workspace& w, const void* q, const void* k,
-                                   const void* v, void* out, int T, float theta, int init, int window,
+                                   const void* v, void* out, const SeqBatch& seqs, float theta, int init,
                                    int shape, bool key_deltas, bool reverse, int form, cudaStream_t st);
 }  // namespace delta
