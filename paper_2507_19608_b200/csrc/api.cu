@@ -3,6 +3,7 @@
 #include <cmath>
 #include <cstdio>
 #include <cstring>
+#include <mutex>
 #include <new>
 #include <vector>
 
@@ -305,45 +306,57 @@ static delta_status_t check_theta_window(float theta, int32_t window) {
 
 }  // extern "C"
 
-// The state's workspace and shape as one batch element sees them (every array is laid out batch
-// element by batch element; the counters are shared).
-static void view_of(const delta_state* st, int b, Shape* sh, Workspace* w) {
+// The state's workspace and shape as n consecutive (batch element, KV head) units from u on see them, as
+// one batch element of n KV heads (every array is laid out unit by unit; the counters are shared).
+static void view_units(const delta_state* st, int u, int n, Shape* sh, Workspace* w) {
   const delta_config_t& c = st->cfg;
+  const size_t g = c.H / c.H_kv, uu = (size_t)u;
+  const size_t hs = uu * (c.source == DELTA_SRC_KEY ? 1 : g);        // heads of the delta stream in front
+  const size_t nt = st->shape.n_tiles, nck = st->shape.n_ckpt();
   *sh = st->shape;
   sh->B = 1;
+  sh->H = n * (int)g;
+  sh->H_kv = n;
   *w = st->ws;
-  const size_t Hs = (c.source == DELTA_SRC_KEY) ? c.H_kv : c.H;      // heads of the delta stream
-  const size_t nt = st->shape.n_tiles, nck = st->shape.n_ckpt(), g = c.H / c.H_kv;
-  const size_t ub = (size_t)b;
-  w->dq += ub * Hs * c.T_max * c.d;
-  w->mask += ub * Hs * c.T_max * (c.d / 32);
-  w->row_nnz += ub * Hs * c.T_max;
-  w->tile_nnz += ub * Hs * nt;
-  w->idx += ub * Hs * c.T_max * c.d;
-  w->qhat_tile += ub * Hs * nt * c.d;
-  w->ckpt += ub * Hs * nck * c.d;
-  w->qhat[0] += ub * Hs * c.d;
-  w->qhat[1] += ub * Hs * c.d;
-  w->R += ub * c.H * c.T_max;
-  w->dec_partial += ub * c.H_kv * kMaxDecodeSplits * g * (c.d + 2);
-  w->dec_ticket += ub * c.H_kv;
-  if (w->kt) w->kt += ub * c.H_kv * c.d * (((size_t)c.T_max + 3) / 4 * 4);
-  if (w->qhat_rows) w->qhat_rows += ub * Hs * c.T_max * c.d;
+  w->dq += hs * c.T_max * c.d;
+  w->mask += hs * c.T_max * (c.d / 32);
+  w->row_nnz += hs * c.T_max;
+  w->tile_nnz += hs * nt;
+  w->idx += hs * c.T_max * c.d;
+  w->qhat_tile += hs * nt * c.d;
+  w->ckpt += hs * nck * c.d;
+  w->qhat[0] += hs * c.d;
+  w->qhat[1] += hs * c.d;
+  w->R += uu * g * c.T_max;
+  w->dec_partial += uu * kMaxDecodeSplits * g * (c.d + 2);
+  w->dec_ticket += uu;
+  if (w->kt) w->kt += uu * c.d * (((size_t)c.T_max + 3) / 4 * 4);
+  if (w->qhat_rows) w->qhat_rows += hs * c.T_max * c.d;
   if (w->kp_vals) {
     const size_t nseg = (size_t)keypack_segments(c.T_max);
-    w->kp_vals += ub * c.H_kv * keypack_capacity(c.T_max, c.d);
-    w->kp_segoff += ub * c.H_kv * (nseg + 1);
-    w->kp_base += ub * c.H_kv * nseg * c.d;
-    w->kp_used += ub * c.H_kv;
-    w->kp_mask += ub * c.H_kv * nseg * 32 * (c.d / 32);
-    w->kp_nnz += ub * c.H_kv * nseg * 32;
+    w->kp_vals += uu * keypack_capacity(c.T_max, c.d);
+    w->kp_segoff += uu * (nseg + 1);
+    w->kp_base += uu * nseg * c.d;
+    w->kp_used += uu;
+    w->kp_mask += uu * nseg * 32 * (c.d / 32);
+    w->kp_nnz += uu * nseg * 32;
   }
 }
+// ... as one batch element sees them.
+static void view_of(const delta_state* st, int b, Shape* sh, Workspace* w) {
+  view_units(st, b * st->cfg.H_kv, st->cfg.H_kv, sh, w);
+}
 
-// The three kernels of a prefill over a uniform batch or a group of sequences of different lengths.
+// The kernels of a prefill over a uniform batch or a group of sequences of different lengths.  parts:
+// PREFILL_ALL, or in two calls where the finish kernel comes last: PREFILL_FRONT (chain, attention) and
+// PREFILL_FINISH.
+enum { PREFILL_FRONT = 1, PREFILL_FINISH = 2, PREFILL_ALL = 3 };
+static bool finish_comes_last(const delta_state* st) {
+  return st->cfg.source != DELTA_SRC_KEY && delta_state_prefill_kernel(st) != 1;
+}
 static delta_status_t prefill_launch(delta_state* st, const Shape& shape, const Workspace& ws, const void* q,
                                      const void* k, const void* v, void* out, const SeqBatch& seqs, float theta,
-                                     cudaStream_t cs, bool prof) {
+                                     cudaStream_t cs, bool prof, int parts = PREFILL_ALL) {
   const delta_config_t& c = st->cfg;
   cudaError_t e;
   // a pending reset: the chain kernel clears the span, less the front of qhat[0] that the chain
@@ -370,6 +383,9 @@ static delta_status_t prefill_launch(delta_state* st, const Shape& shape, const 
   // the finish kernel's launch overlaps the end of the attention kernel.  With per-kernel
   // timing on, the kernels run in their natural order with events between them.
   const bool chained = !use_tc && !prof;
+  if (parts == PREFILL_FINISH)
+    return (e = launch_delta_finish(shape, ws, q, k, seqs, theta, c.prefill_window, c.dtype, c.init, false, key, rev, 1,
+                                    cs)) == cudaSuccess ? DELTA_OK : cuda_fail(e);
   MARK(0);
   // the delta stream: the queries (strategy 1) or the keys, per KV head (strategy 3)
   if ((e = launch_delta_chain(shape, ws, key ? k : q, seqs, theta, c.dtype, c.init, key, rev, zero_ptr, zero_bytes, cs)) != cudaSuccess)
@@ -384,7 +400,7 @@ static delta_status_t prefill_launch(delta_state* st, const Shape& shape, const 
   if (chained && !key) {
     if ((e = attention()) != cudaSuccess) return cuda_fail(e);
     // (released by the attention CTAs once the chain is complete: it runs beside their last wave)
-    if ((e = launch_delta_finish(shape, ws, q, k, seqs, theta, c.prefill_window, c.dtype, c.init,
+    if (parts == PREFILL_ALL && (e = launch_delta_finish(shape, ws, q, k, seqs, theta, c.prefill_window, c.dtype, c.init,
                                  use_tc, key, rev, 2, cs)) != cudaSuccess)
       return cuda_fail(e);
   } else if (chained) {
@@ -422,6 +438,81 @@ static delta_status_t prefill_launch(delta_state* st, const Shape& shape, const 
   return DELTA_OK;
 }
 
+// Host-side bookkeeping behind a prefill of T tokens for every batch element.
+static void prefilled(delta_state* st, int T, int window) {
+  const double B = (double)st->cfg.B;
+  st->n = T;
+  st->n_b.assign((size_t)st->cfg.B, T);
+  st->ragged = false;
+  st->qhat_sel = 0;
+  st->win_sum[0] += B * (double)(window < T ? window : T);
+  st->len_sum[0] += B * (double)T;
+}
+
+// Streams and events of a host-buffer prefill.  A call takes a set for its duration (it synchronises
+// before it returns) and gives it back to a pool per device; more than kTransferKeep sets at once
+// (concurrent host threads) are made and destroyed by their calls.
+namespace {
+constexpr int kTransferChunks = 4;
+constexpr size_t kTransferKeep = 4;
+struct Transfer {
+  int dev = 0;
+  cudaStream_t up = nullptr, down = nullptr;
+  cudaEvent_t start = nullptr, arrived[kTransferChunks] = {}, computed[kTransferChunks] = {};
+  cudaError_t create() {
+    cudaError_t e = cudaGetDevice(&dev);
+    auto ok = [&](cudaError_t x) { if (e == cudaSuccess) e = x; };
+    if (e != cudaSuccess) return e;
+    ok(cudaStreamCreateWithFlags(&up, cudaStreamNonBlocking));
+    ok(cudaStreamCreateWithFlags(&down, cudaStreamNonBlocking));
+    ok(cudaEventCreateWithFlags(&start, cudaEventDisableTiming));
+    for (int i = 0; i < kTransferChunks; ++i) {
+      ok(cudaEventCreateWithFlags(&arrived[i], cudaEventDisableTiming));
+      ok(cudaEventCreateWithFlags(&computed[i], cudaEventDisableTiming));
+    }
+    return e;
+  }
+  void destroy() {
+    if (up) cudaStreamDestroy(up);
+    if (down) cudaStreamDestroy(down);
+    if (start) cudaEventDestroy(start);
+    for (int i = 0; i < kTransferChunks; ++i) {
+      if (arrived[i]) cudaEventDestroy(arrived[i]);
+      if (computed[i]) cudaEventDestroy(computed[i]);
+    }
+  }
+};
+std::mutex g_transfer_mu;
+std::vector<Transfer*> g_transfers;      // idle sets
+struct TransferGuard {
+  Transfer* t = nullptr;
+  cudaError_t open() {
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    {
+      std::lock_guard<std::mutex> lock(g_transfer_mu);
+      for (size_t i = 0; i < g_transfers.size() && !t; ++i)
+        if (g_transfers[i]->dev == dev) { t = g_transfers[i]; g_transfers.erase(g_transfers.begin() + (long)i); }
+    }
+    if (t) return cudaSuccess;
+    t = new (std::nothrow) Transfer();
+    if (!t) return cudaErrorMemoryAllocation;
+    if ((e = t->create()) != cudaSuccess) { t->destroy(); delete t; t = nullptr; }
+    return e;
+  }
+  ~TransferGuard() {
+    if (!t) return;
+    {
+      std::lock_guard<std::mutex> lock(g_transfer_mu);
+      if (g_transfers.size() < kTransferKeep) { g_transfers.push_back(t); return; }
+    }
+    t->destroy();
+    delete t;
+  }
+};
+}  // namespace
+
 extern "C" {
 
 delta_status_t delta_attn_prefill(delta_state_t* st, const void* q, const void* k, const void* v,
@@ -444,12 +535,7 @@ delta_status_t delta_attn_prefill(delta_state_t* st, const void* q, const void* 
   s = prefill_launch(st, st->shape, st->ws, q, k, v, out, seqs, theta, (cudaStream_t)stream, prof);
   if (s != DELTA_OK) return s;
   st->profiled = prof;
-  st->n = T;
-  st->n_b.assign((size_t)c.B, T);
-  st->ragged = false;
-  st->qhat_sel = 0;
-  st->win_sum[0] += (double)c.B * (double)(window < T ? window : T);
-  st->len_sum[0] += (double)c.B * (double)T;
+  prefilled(st, T, window);
   return DELTA_OK;
 }
 
@@ -548,24 +634,79 @@ delta_status_t delta_attn_prefill_host(delta_state_t* st, const void* q_host, co
   char* dk = dout + qb;
   char* dv = dk + kb;
   cudaStream_t cs = (cudaStream_t)stream;
-  cudaError_t e;
-  if ((e = cudaMemcpyAsync(dq_, q_host, q_bytes, cudaMemcpyHostToDevice, cs)) != cudaSuccess) return cuda_fail(e);
+  // The call is bound by PCIe (6.3 MB up and 4.2 MB down around 35 us of kernels at the Llama layer; 51 GB/s
+  // one way, 80 both ways together): keys and values come up first, then the queries in chunks of KV
+  // heads, and while a chunk is computed on the caller's stream the next one comes up on a stream of
+  // the pool and the last one's output goes down on another.  At most four chunks of at least a
+  // megabyte: a small copy beside one in the other direction waits for it (queries, keys and values in
+  // chunks: 275 us).  Llama layer, 1024 tokens: 252 us in one piece, 225 so; batch 4: 860, 723.
+  const int units = c.B * c.H_kv;
+  const size_t es2 = (size_t)c.d * es, g = c.H / c.H_kv;
+  int chunks = (int)(q_bytes >> 20);
+  if (chunks > kTransferChunks) chunks = kTransferChunks;
+  if (chunks > units) chunks = units;
+  if (chunks < 1 || st->profiling) chunks = 1;
+  // (one chunk: all on the caller's stream, nothing to overlap)
+  TransferGuard tg;
+  cudaError_t e = chunks > 1 ? tg.open() : cudaSuccess;
+  if (e != cudaSuccess) return cuda_fail(e);
+  Transfer* const x = tg.t;
+  const cudaStream_t s_up = x ? x->up : cs, s_down = x ? x->down : cs;
+  auto fail = [&](cudaError_t err) {      // nothing of this call may still touch the buffers
+    cudaStreamSynchronize(s_up);
+    cudaStreamSynchronize(s_down);
+    cudaStreamSynchronize(cs);
+    return cuda_fail(err);
+  };
+#define DO(call) do { if ((e = (call)) != cudaSuccess) return fail(e); } while (0)
   // host K/V hold T rows per head; the device copy uses the cache layout with T_max rows
-  const size_t row = (size_t)c.d * es;
-  const size_t units = (size_t)c.B * c.H_kv;
-  if (T == c.T_max) {      // the two layouts coincide: one contiguous copy each
-    if ((e = cudaMemcpyAsync(dk, k_host, units * T * row, cudaMemcpyHostToDevice, cs)) != cudaSuccess) return cuda_fail(e);
-    if ((e = cudaMemcpyAsync(dv, v_host, units * T * row, cudaMemcpyHostToDevice, cs)) != cudaSuccess) return cuda_fail(e);
-  } else {
-    if ((e = cudaMemcpy2DAsync(dk, (size_t)c.T_max * row, k_host, (size_t)T * row, (size_t)T * row, units,
-                               cudaMemcpyHostToDevice, cs)) != cudaSuccess) return cuda_fail(e);
-    if ((e = cudaMemcpy2DAsync(dv, (size_t)c.T_max * row, v_host, (size_t)T * row, (size_t)T * row, units,
-                               cudaMemcpyHostToDevice, cs)) != cudaSuccess) return cuda_fail(e);
+  auto up_rows = [&](char* dst, const char* src, int u0, int n) -> cudaError_t {
+    const size_t w = (size_t)T * es2, p = (size_t)c.T_max * es2;
+    if (T == c.T_max) return cudaMemcpyAsync(dst + u0 * w, src + u0 * w, n * w, cudaMemcpyHostToDevice, s_up);
+    return cudaMemcpy2DAsync(dst + u0 * p, p, src + u0 * w, w, w, n, cudaMemcpyHostToDevice, s_up);
+  };
+  if (x) {
+    DO(cudaEventRecord(x->start, cs));
+    DO(cudaStreamWaitEvent(s_up, x->start, 0));
   }
-  s = delta_attn_prefill(st, dq_, dk, dv, dout, T, c.H, c.H_kv, c.d, theta, window, stream);
-  if (s != DELTA_OK) return s;
-  if ((e = cudaMemcpyAsync(out_host, dout, q_bytes, cudaMemcpyDeviceToHost, cs)) != cudaSuccess) return cuda_fail(e);
-  if ((e = cudaStreamSynchronize(cs)) != cudaSuccess) return cuda_fail(e);
+  const size_t unit_q = g * T * es2;      // bytes of a unit's queries
+  DO(up_rows(dk, (const char*)k_host, 0, units));
+  DO(up_rows(dv, (const char*)v_host, 0, units));
+  for (int i = 0; i < chunks; ++i) {
+    const int u0 = (int)((long)units * i / chunks), n = (int)((long)units * (i + 1) / chunks) - u0;
+    DO(cudaMemcpyAsync(dq_ + u0 * unit_q, (const char*)q_host + u0 * unit_q, n * unit_q, cudaMemcpyHostToDevice, s_up));
+    if (x) DO(cudaEventRecord(x->arrived[i], s_up));
+  }
+  const bool late = x && finish_comes_last(st);
+  SeqBatch seqs;
+  seqs.n = 1; seqs.T_longest = T; seqs.ragged = false;
+  seqs.s[0] = Seq{T, window, 0, 0};
+  for (int i = 0; i < chunks; ++i) {
+    const int u0 = (int)((long)units * i / chunks), n = (int)((long)units * (i + 1) / chunks) - u0;
+    const size_t kv = (size_t)u0 * c.T_max * es2, qo = u0 * unit_q;
+    Shape sh = st->shape;
+    Workspace ws = st->ws;
+    if (chunks > 1) view_units(st, u0, n, &sh, &ws);
+    if (x) DO(cudaStreamWaitEvent(cs, x->arrived[i], 0));
+    s = prefill_launch(st, sh, ws, dq_ + qo, dk + kv, dv + kv, dout + qo, seqs, theta, cs, st->profiling,
+                       late ? PREFILL_FRONT : PREFILL_ALL);
+    if (s != DELTA_OK) { fail(cudaSuccess); return s; }
+    if (x) {
+      DO(cudaEventRecord(x->computed[i], cs));
+      DO(cudaStreamWaitEvent(s_down, x->computed[i], 0));
+    }
+    DO(cudaMemcpyAsync((char*)out_host + qo, dout + qo, n * unit_q, cudaMemcpyDeviceToHost, s_down));
+  }
+  // delta arrays, counters and the hand-off row of all chunks, while the last output goes down
+  if (late) {
+    s = prefill_launch(st, st->shape, st->ws, dq_, dk, dv, dout, seqs, theta, cs, false, PREFILL_FINISH);
+    if (s != DELTA_OK) { fail(cudaSuccess); return s; }
+  }
+  if (x) DO(cudaStreamSynchronize(s_down));
+  DO(cudaStreamSynchronize(cs));
+#undef DO
+  st->profiled = st->profiling;
+  prefilled(st, T, window);
   return DELTA_OK;
 }
 
