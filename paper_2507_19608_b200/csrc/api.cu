@@ -750,6 +750,10 @@ delta_status_t delta_attn_decode_step(delta_state_t* st, const void* q_new, cons
                                st->ragged ? st->n_b.data() : nullptr, theta, window, st->qhat_sel,
                                c.source == DELTA_SRC_KEY, key_packed, st->dec_maps, cs);
     if (e != cudaSuccess) return cuda_fail(e);
+  } else if (c.dtype == DELTA_F32 && st->forced_decode_kernel < 0) {
+    e = launch_decode_step_f32(st->shape, st->ws, q_new, k_new, v_new, k_cache, v_cache, out, st->n,
+                               st->ragged ? st->n_b.data() : nullptr, theta, window, st->qhat_sel, st->dec_maps, cs);
+    if (e != cudaSuccess) return cuda_fail(e);
   } else if (!st->ragged) {
     e = decode_launch(st, st->shape, st->ws, q_new, k_new, v_new, k_cache, v_cache, out, st->n, theta, window, cs);
     if (e != cudaSuccess) return cuda_fail(e);

@@ -1,0 +1,174 @@
+// Pieces shared by the decode-step kernels whose warps work on units of 32 keys each on their own: how
+// a step is sliced, and how the warps' partial results meet.
+//
+// Merge.  The result of a (batch, KV head), G heads x D channels, is cut into blocks of 16 channels of one
+// head.  The slices of the (batch, KV head) are one thread-block cluster of cs CTAs; block q is finished by
+// slice q mod cs (by the CTA itself without a cluster), to whose shared memory every warp of every
+// slice sends its part: a record of 16 channels at recs + ((q / cs) * nsrc + source) * REC * 4 and a
+// (maximum, row sum) pair at mls + (..) * 8.
+#pragma once
+#include "decode_common.cuh"
+#include "tc_common.cuh"
+
+namespace delta {
+namespace {
+
+constexpr int UK = 32;                    // keys a warp works on at a time
+constexpr int kMaxCluster = 16;           // slices merged through distributed shared memory
+constexpr int kRaggedMax = 64;            // batch elements of one ragged launch
+constexpr int REC = 16;                   // floats of a partial result's record: 16 channels of one head
+
+__device__ __forceinline__ void async16(uint32_t dst, const void* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
+}
+__device__ __forceinline__ void async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+__device__ __forceinline__ uint32_t cluster_map(uint32_t addr, uint32_t rank) {
+  uint32_t r;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
+  return r;
+}
+// Stores into the shared memory of a CTA of the cluster that count their bytes on its barrier: the
+// receiver waits for the bytes, and nothing of the sender's (its global stores least of all) has to
+// be flushed first, as a cluster barrier with release semantics would.
+__device__ __forceinline__ void cluster_send4(uint32_t addr, uint32_t bar, float a, float b, float c, float d) {
+  asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v4.f32 [%0], {%2, %3, %4, %5}, [%1];" ::"r"(addr),
+               "r"(bar), "f"(a), "f"(b), "f"(c), "f"(d) : "memory");
+}
+__device__ __forceinline__ void cluster_send2(uint32_t addr, uint32_t bar, float a, float b) {
+  asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v2.f32 [%0], {%2, %3}, [%1];" ::"r"(addr),
+               "r"(bar), "f"(a), "f"(b) : "memory");
+}
+__device__ __forceinline__ void sts_f4(uint32_t addr, float a, float b, float c, float d) {
+  asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "f"(a), "f"(b), "f"(c), "f"(d) : "memory");
+}
+__device__ __forceinline__ void sts_f2(uint32_t addr, float a, float b) {
+  asm volatile("st.shared.v2.f32 [%0], {%1, %2};" ::"r"(addr), "f"(a), "f"(b) : "memory");
+}
+__device__ __forceinline__ float2 lds_f2(uint32_t addr) {
+  float2 v;
+  asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(addr));
+  return v;
+}
+__device__ __forceinline__ float4 lds_f4(uint32_t addr) { return tc::lds128(addr); }
+__device__ __forceinline__ void store4(__nv_bfloat16* p, float a, float b, float c, float d) {
+  const __nv_bfloat162 x = __floats2bfloat162_rn(a, b), y = __floats2bfloat162_rn(c, d);
+  *reinterpret_cast<uint2*>(p) = make_uint2(*reinterpret_cast<const uint32_t*>(&x), *reinterpret_cast<const uint32_t*>(&y));
+}
+__device__ __forceinline__ void store4(float* p, float a, float b, float c, float d) {
+  *reinterpret_cast<float4*>(p) = make_float4(a, b, c, d);
+}
+__device__ __forceinline__ int warp_sum(int x) {
+#pragma unroll
+  for (int s = 16; s > 0; s >>= 1) x += __shfl_xor_sync(0xffffffffu, x, s);
+  return x;
+}
+
+// The finishing half, once all records are there: combine this CTA's blocks and store them, or, where
+// a (batch, KV head) has more slices (ns) than a cluster, leave this slice's part in global memory
+// for the last CTA to arrive.  out0: first output of the group.
+template <typename TO, int D, int G, int MNW, bool CLUSTER>
+__device__ __forceinline__ void decode_merge(uint32_t recs, uint32_t mls, int rank, int cs, int nsrc, int ns, int split,
+                                             int bkv, size_t out0, float* __restrict__ partial,
+                                             uint32_t* __restrict__ ticket, TO* __restrict__ out, int* s_last) {
+  // One warp per block: lane = (4 channels, one of 8 groups of parts).
+  constexpr int NB = G * D / 16;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int c4 = lane & 3, sg = lane >> 2;
+  for (int slot = warp; slot * cs + rank < NB; slot += MNW) {
+    const int q = slot * cs + rank;
+    const uint32_t rb = recs + (uint32_t)(slot * nsrc) * (REC * 4) + 16 * c4, mb = mls + (uint32_t)(slot * nsrc) * 8;
+    float M = -INFINITY;
+#pragma unroll
+    for (int x = 0; x < (CLUSTER ? kMaxCluster : 1) * MNW; x += 32)
+      if (x + lane < nsrc) M = fmaxf(M, lds_f2(mb + 8 * (x + lane)).x);
+#pragma unroll
+    for (int x = 1; x < 32; x <<= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, x));
+    float a[5] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
+#pragma unroll 4
+    for (int x = sg; x < nsrc; x += 8) {
+      const float2 ml = lds_f2(mb + 8 * x);
+      const float4 o = lds_f4(rb + x * (REC * 4));
+      const float f = tc::ex2(ml.x - M);                     // 0 for a warp without keys
+      a[0] = fmaf(f, o.x, a[0]); a[1] = fmaf(f, o.y, a[1]); a[2] = fmaf(f, o.z, a[2]); a[3] = fmaf(f, o.w, a[3]);
+      a[4] = fmaf(f, ml.y, a[4]);
+    }
+#pragma unroll
+    for (int x = 4; x < 32; x <<= 1)
+#pragma unroll
+      for (int e = 0; e < 5; ++e) a[e] += __shfl_xor_sync(0xffffffffu, a[e], x);
+    const int hh = q / (D / 16), ch = (q % (D / 16)) * 16 + 4 * c4;
+    if (sg == 0) {
+      if (CLUSTER || ns == 1) {
+        const float inv = 1.0f / a[4];
+        store4(out + out0 + (size_t)hh * D + ch, a[0] * inv, a[1] * inv, a[2] * inv, a[3] * inv);
+      } else {
+        // slices through global memory: this slice's part
+        float* const pg = partial + (((size_t)bkv * kMaxDecodeSplits + split) * G + hh) * (D + 2);
+        pg[ch] = a[0]; pg[ch + 1] = a[1]; pg[ch + 2] = a[2]; pg[ch + 3] = a[3];
+        if (ch == 0) { pg[D] = M; pg[D + 1] = a[4]; }
+      }
+    }
+  }
+  if (CLUSTER || ns == 1) return;
+
+  // ---- the last CTA of the (batch, KV head) to arrive merges the slices
+  __threadfence();
+  __syncthreads();
+  if (tid == 0) *s_last = atomicAdd(&ticket[bkv], 1u) == (uint32_t)ns - 1u;
+  __syncthreads();
+  if (!*s_last) return;
+  __threadfence();
+  const float* const pb = partial + (size_t)bkv * kMaxDecodeSplits * G * (D + 2);
+  for (int e = tid; e < G * D; e += 32 * MNW) {
+    const int hh = e / D, c = e - hh * D;
+    float M = -INFINITY, nu = 0.0f, de = 0.0f;
+#pragma unroll 8
+    for (int r = 0; r < ns; ++r) M = fmaxf(M, __ldcg(pb + ((size_t)r * G + hh) * (D + 2) + D));
+#pragma unroll 8
+    for (int r = 0; r < ns; ++r) {
+      const float* const pr = pb + ((size_t)r * G + hh) * (D + 2);
+      const float f = tc::ex2(__ldcg(pr + D) - M);
+      nu = fmaf(f, __ldcg(pr + c), nu);
+      de = fmaf(f, __ldcg(pr + D + 1), de);
+    }
+    out[out0 + (size_t)hh * D + c] = from_f32<TO>(nu / de);
+  }
+  if (tid == 0) ticket[bkv] = 0;                          // ready for the next step
+}
+
+// Slices of a step over sequences of up to L keys (the new one included).  A step takes 4 to 5 us plus,
+// for every unit a warp works through, 1.1 us (d = 64) or 1.3 us (d = 128) while a CTA has its SM for
+// itself and 1.75 us where two share one (measured from 1 to 192 KV heads, 300 to 16000 keys); the
+// slices are those that minimise that.  All slices of a KV head form one cluster, and clusters have to
+// find room in a GPC: from 1.75 CTAs per SM on (1.6 for clusters of 9 to 12, 1.35 for 13 to 16) some
+// wait for a second wave (batch 16, 2048 keys: 256 CTAs 12 us, 384 CTAs 17 us).  Very long caches of
+// few heads: up to 64 slices merged through global memory (4.5 us more than a cluster).  The compressed
+// key cache: 2.5 us more per unit, for the rebuilding.
+// nw: warps per CTA; us_alone, us_shared: a unit's time with the SM for itself, and shared (0: a CTA fills
+// its SM); us_more: a kernel's own extra time per unit.
+inline void decode_slices(const Shape& s, int L, int nw, float us_shared, float us_alone, float us_more, int* nsplit_out,
+                          int* chunk_out, bool* cluster_out) {
+  const int bkv = s.B * s.H_kv, sms = device_sm_count();
+  const int units = (L + UK - 1) / UK;
+  float best = 3.4e38f;
+  int best_ns = 1;
+  for (int ns = 1; ns <= kMaxDecodeSplits && (ns - 1) * nw < units; ++ns) {       // a unit per warp at least
+    const long ctas = (long)bkv * ns;
+    const bool alone = ctas * 100 <= (long)sms * 92;
+    if (ns > kMaxCluster && ctas > sms) break;
+    if (ns > 1 && us_shared == 0.0f && !alone) continue;
+    if (ns > 1 && ns <= kMaxCluster && ctas * 100 > (long)sms * (ns <= 8 ? 175 : ns <= 12 ? 160 : 135)) continue;
+    const int per = (units + ns - 1) / ns;                       // units per slice; per warp mostly the longest counts
+    const float rounds = 0.8f * (float)((per + nw - 1) / nw) + 0.2f * (float)per / (float)nw;
+    const float us = rounds * ((alone || us_shared == 0.0f ? us_alone : us_shared) + us_more) +
+                     (ns > kMaxCluster ? 4.5f + 0.15f * (float)(ns - 24) : (ns > 8 ? 0.075f : 0.06f) * (float)ns);
+    if (us < best - 0.02f) { best = us; best_ns = ns; }
+  }
+  const int chunk = (units + best_ns - 1) / best_ns * UK;
+  *nsplit_out = (L + chunk - 1) / chunk;
+  *chunk_out = chunk;
+  *cluster_out = *nsplit_out > 1 && *nsplit_out <= kMaxCluster;
+}
+
+}  // namespace
+}  // namespace delta

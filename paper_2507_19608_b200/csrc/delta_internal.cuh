@@ -139,6 +139,10 @@ cudaError_t launch_decode_step_mma(const Shape& s, const Workspace& w, const voi
                                    const void* v_new, void* k_cache, void* v_cache, void* out, int n, const int* n_b,
                                    float theta, int window, int qhat_sel, bool key, bool packed, DecodeTmapCache* maps,
                                    cudaStream_t st);
+// K3 for fp32 caches (query deltas), arguments as above.
+cudaError_t launch_decode_step_f32(const Shape& s, const Workspace& w, const void* q_new, const void* k_new,
+                                   const void* v_new, void* k_cache, void* v_cache, void* out, int n, const int* n_b,
+                                   float theta, int window, int qhat_sel, DecodeTmapCache* map, cudaStream_t st);
 // The compressed key-delta cache (packed = true above decodes from it): the kernel that builds it
 // behind a prefill, and its geometry (values per KV head at most, 32-row segments).
 size_t keypack_capacity(int T_max, int d);

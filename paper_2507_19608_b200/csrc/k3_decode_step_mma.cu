@@ -36,6 +36,7 @@
 #include <cuda.h>
 
 #include "decode_common.cuh"
+#include "decode_merge.cuh"
 #include "tc_common.cuh"
 
 namespace delta {
@@ -43,10 +44,6 @@ namespace delta {
 namespace {
 
 template <int D> constexpr int kWarps = D == 64 ? 8 : 4;    // warps per CTA
-constexpr int UK = 32;                    // keys a warp works on at a time
-constexpr int kMaxCluster = 16;           // slices merged through distributed shared memory
-constexpr int kRaggedMax = 64;            // batch elements of one ragged launch
-constexpr int REC = 16;                   // floats of a partial result's record: 16 channels of one head
 
 struct MmaDecodeParams {
   const __nv_bfloat16 *q_new, *k_new, *v_new;
@@ -67,10 +64,6 @@ struct MmaDecodeParams {
   int n_b[kRaggedMax];                    // ragged: tokens seen per batch element b0 ..
 };
 
-__device__ __forceinline__ void async16(uint32_t dst, const void* src) {
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
-}
-__device__ __forceinline__ void async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 __device__ __forceinline__ void sts128z(uint32_t dst) {
   asm volatile("st.shared.v4.u32 [%0], {%1, %1, %1, %1};" ::"r"(dst), "r"(0) : "memory");
 }
@@ -91,35 +84,6 @@ __device__ __forceinline__ void split3(float lo, float hi, uint32_t& p0, uint32_
   p1 = pack_bf16(r0, r1);
   p2 = pack_bf16(r0 - __uint_as_float(p1 << 16), r1 - __uint_as_float(p1 & 0xffff0000u));
 }
-__device__ __forceinline__ uint32_t cluster_map(uint32_t addr, uint32_t rank) {
-  uint32_t r;
-  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
-  return r;
-}
-// Stores into the shared memory of a CTA of the cluster that count their bytes on its barrier: the
-// receiver waits for the bytes, and nothing of the sender's (its global stores least of all) has to
-// be flushed first, as a cluster barrier with release semantics would.
-__device__ __forceinline__ void cluster_send4(uint32_t addr, uint32_t bar, float a, float b, float c, float d) {
-  asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v4.f32 [%0], {%2, %3, %4, %5}, [%1];" ::"r"(addr),
-               "r"(bar), "f"(a), "f"(b), "f"(c), "f"(d) : "memory");
-}
-__device__ __forceinline__ void cluster_send2(uint32_t addr, uint32_t bar, float a, float b) {
-  asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v2.f32 [%0], {%2, %3}, [%1];" ::"r"(addr),
-               "r"(bar), "f"(a), "f"(b) : "memory");
-}
-__device__ __forceinline__ void sts_f4(uint32_t addr, float a, float b, float c, float d) {
-  asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "f"(a), "f"(b), "f"(c), "f"(d) : "memory");
-}
-__device__ __forceinline__ void sts_f2(uint32_t addr, float a, float b) {
-  asm volatile("st.shared.v2.f32 [%0], {%1, %2};" ::"r"(addr), "f"(a), "f"(b) : "memory");
-}
-__device__ __forceinline__ float2 lds_f2(uint32_t addr) {
-  float2 v;
-  asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(addr));
-  return v;
-}
-__device__ __forceinline__ float4 lds_f4(uint32_t addr) { return tc::lds128(addr); }
-
 __device__ __forceinline__ uint32_t lds_u32(uint32_t a) {
   uint32_t v;
   asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(a));
@@ -131,12 +95,6 @@ __device__ __forceinline__ uint32_t lds_u16(uint32_t a) {
   return v;
 }
 __device__ __forceinline__ void sts_u32(uint32_t a, uint32_t v) { asm volatile("st.shared.u32 [%0], %1;" ::"r"(a), "r"(v) : "memory"); }
-__device__ __forceinline__ int warp_sum(int x) {
-#pragma unroll
-  for (int s = 16; s > 0; s >>= 1) x += __shfl_xor_sync(0xffffffffu, x, s);
-  return x;
-}
-
 // Shared memory: per warp one unit of keys and values (128-byte swizzle, blocks of [32 rows][64
 // channels]), then the merge's records [slot][slice x warp][REC] and (maximum, row sum) pairs.
 // PACKED: per warp also the encoding of one 32-row segment: values, mask words, the reference in front.
@@ -635,101 +593,8 @@ decode_step_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_co
   }
   if (tid == 0 && s_fail) atomicMax(&p.counters[CNT_STATUS], (unsigned long long)DELTA_ERR_TIMEOUT);
 
-  // One warp per block: lane = (4 channels, one of 8 groups of parts).
-  const int c4 = lane & 3, sg = lane >> 2;
-  const int ns = (L + p.chunk - 1) / p.chunk;               // slices of this sequence
-  for (int slot = warp; slot * cs + rank < SM::NB; slot += MNW) {
-    const int q = slot * cs + rank;
-    const uint32_t rb = recs + (uint32_t)(slot * nsrc) * (REC * 4) + 16 * c4, mb = mls + (uint32_t)(slot * nsrc) * 8;
-    float M = -INFINITY;
-#pragma unroll
-    for (int x = 0; x < (CLUSTER ? kMaxCluster : 1) * MNW; x += 32)
-      if (x + lane < nsrc) M = fmaxf(M, lds_f2(mb + 8 * (x + lane)).x);
-#pragma unroll
-    for (int x = 1; x < 32; x <<= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, x));
-    float a[5] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
-#pragma unroll 4
-    for (int x = sg; x < nsrc; x += 8) {
-      const float2 ml = lds_f2(mb + 8 * x);
-      const float4 o = lds_f4(rb + x * (REC * 4));
-      const float f = tc::ex2(ml.x - M);                     // 0 for a warp without keys
-      a[0] = fmaf(f, o.x, a[0]); a[1] = fmaf(f, o.y, a[1]); a[2] = fmaf(f, o.z, a[2]); a[3] = fmaf(f, o.w, a[3]);
-      a[4] = fmaf(f, ml.y, a[4]);
-    }
-#pragma unroll
-    for (int x = 4; x < 32; x <<= 1)
-#pragma unroll
-      for (int e = 0; e < 5; ++e) a[e] += __shfl_xor_sync(0xffffffffu, a[e], x);
-    const int hh = q / (D / 16), ch = (q % (D / 16)) * 16 + 4 * c4;
-    if (sg == 0) {
-      if (CLUSTER || ns == 1) {
-        const float inv = 1.0f / a[4];
-        *reinterpret_cast<uint2*>(p.out + ((size_t)b * p.H + kvh * G + hh) * D + ch) =
-            make_uint2(pack_bf16(a[0] * inv, a[1] * inv), pack_bf16(a[2] * inv, a[3] * inv));
-      } else {
-        // slices through global memory: this slice's part
-        float* const pg = p.partial + (((size_t)bkv * kMaxDecodeSplits + split) * G + hh) * (D + 2);
-        pg[ch] = a[0]; pg[ch + 1] = a[1]; pg[ch + 2] = a[2]; pg[ch + 3] = a[3];
-        if (ch == 0) { pg[D] = M; pg[D + 1] = a[4]; }
-      }
-    }
-  }
-  if (CLUSTER || ns == 1) return;
-
-  // ---- the last CTA of the (batch, KV head) to arrive merges the slices
-  __threadfence();
-  __syncthreads();
-  if (tid == 0) s_last = atomicAdd(&p.ticket[bkv], 1u) == (uint32_t)ns - 1u;
-  __syncthreads();
-  if (!s_last) return;
-  __threadfence();
-  const float* const pb = p.partial + (size_t)bkv * kMaxDecodeSplits * G * (D + 2);
-  for (int e = tid; e < G * D; e += 32 * MNW) {
-    const int hh = e / D, c = e - hh * D;
-    float M = -INFINITY, nu = 0.0f, de = 0.0f;
-#pragma unroll 8
-    for (int r = 0; r < ns; ++r) M = fmaxf(M, __ldcg(pb + ((size_t)r * G + hh) * (D + 2) + D));
-#pragma unroll 8
-    for (int r = 0; r < ns; ++r) {
-      const float* const pr = pb + ((size_t)r * G + hh) * (D + 2);
-      const float f = tc::ex2(__ldcg(pr + D) - M);
-      nu = fmaf(f, __ldcg(pr + c), nu);
-      de = fmaf(f, __ldcg(pr + D + 1), de);
-    }
-    p.out[((size_t)b * p.H + kvh * G + hh) * D + c] = __float2bfloat16_rn(nu / de);
-  }
-  if (tid == 0) p.ticket[bkv] = 0;                          // ready for the next step
-}
-
-// Slices of a step over sequences of up to L keys (the new one included).  A step takes 4 to 5 us plus,
-// for every unit a warp works through, 1.1 us (d = 64) or 1.3 us (d = 128) while a CTA has its SM for
-// itself and 1.75 us where two share one (measured from 1 to 192 KV heads, 300 to 16000 keys); the
-// slices are those that minimise that.  All slices of a KV head form one cluster, and clusters have to
-// find room in a GPC: from 1.75 CTAs per SM on (1.6 for clusters of 9 to 12, 1.35 for 13 to 16) some
-// wait for a second wave (batch 16, 2048 keys: 256 CTAs 12 us, 384 CTAs 17 us).  Very long caches of
-// few heads: up to 64 slices merged through global memory (4.5 us more than a cluster).  The compressed
-// key cache: 2.5 us more per unit, for the rebuilding.
-static void decode_mma_slices(const Shape& s, int L, bool packed, int* nsplit_out, int* chunk_out, bool* cluster_out) {
-  const int bkv = s.B * s.H_kv, sms = device_sm_count();
-  const int nw = s.d == 64 ? kWarps<64> : kWarps<128>;
-  const int units = (L + UK - 1) / UK;
-  float best = 3.4e38f;
-  int best_ns = 1;
-  for (int ns = 1; ns <= kMaxDecodeSplits && (ns - 1) * nw < units; ++ns) {       // a unit per warp at least
-    const long ctas = (long)bkv * ns;
-    const bool alone = ctas * 100 <= (long)sms * 92;
-    if (ns > kMaxCluster && ctas > sms) break;
-    if (ns > 1 && ns <= kMaxCluster && ctas * 100 > (long)sms * (ns <= 8 ? 175 : ns <= 12 ? 160 : 135)) continue;
-    const int per = (units + ns - 1) / ns;                       // units per slice; per warp mostly the longest counts
-    const float rounds = 0.8f * (float)((per + nw - 1) / nw) + 0.2f * (float)per / (float)nw;
-    const float us = rounds * ((!alone ? 1.75f : s.d == 64 ? 1.1f : 1.3f) + (packed ? 2.5f : 0.0f)) +
-                     (ns > kMaxCluster ? 4.5f + 0.15f * (float)(ns - 24) : (ns > 8 ? 0.075f : 0.06f) * (float)ns);
-    if (us < best - 0.02f) { best = us; best_ns = ns; }
-  }
-  const int chunk = (units + best_ns - 1) / best_ns * UK;
-  *nsplit_out = (L + chunk - 1) / chunk;
-  *chunk_out = chunk;
-  *cluster_out = *nsplit_out > 1 && *nsplit_out <= kMaxCluster;
+  decode_merge<TC, D, G, MNW, CLUSTER>(recs, mls, rank, cs, nsrc, (L + p.chunk - 1) / p.chunk, split, bkv,
+                                       ((size_t)b * p.H + kvh * G) * D, p.partial, p.ticket, p.out, &s_last);
 }
 
 template <int D, int G, int MODE, bool CLUSTER>
@@ -740,7 +605,8 @@ static cudaError_t launch_mma(const CUtensorMap& tk, const CUtensorMap& tv, cons
   const size_t smem = SM::bytes(CLUSTER ? p.nsplit : 1);
   static std::atomic<uint64_t> ready{0};
   if (!device_done(ready)) {
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SM::bytes(kMaxCluster - 1));
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(SM::bytes(kMaxCluster) > SM::bytes(kMaxCluster - 1) ? SM::bytes(kMaxCluster)
+                                                                                               : SM::bytes(kMaxCluster - 1)));
     // (two CTAs per SM need the largest shared-memory carve-out)
     if (e == cudaSuccess) e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout,
                                                    (int)cudaSharedmemCarveoutMaxShared);
@@ -806,7 +672,7 @@ cudaError_t launch_decode_step_mma(const Shape& s, const Workspace& w, const voi
   p.b0 = 0;
   const int G = s.g();
   bool cluster;
-  decode_mma_slices(s, n + 1, packed, &p.nsplit, &p.chunk, &cluster);
+  decode_slices(s, n + 1, s.d == 64 ? kWarps<64> : kWarps<128>, 1.75f, s.d == 64 ? 1.1f : 1.3f, packed ? 2.5f : 0.0f, &p.nsplit, &p.chunk, &cluster);
   if (p.nsplit > kMaxDecodeSplits) return cudaErrorInvalidValue;
   cudaError_t err = cudaSuccess;
   for (; p.b0 < s.B && err == cudaSuccess; p.b0 += kRaggedMax) {
