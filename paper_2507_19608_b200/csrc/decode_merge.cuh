@@ -57,6 +57,12 @@ __device__ __forceinline__ void store4(__nv_bfloat16* p, float a, float b, float
 __device__ __forceinline__ void store4(float* p, float a, float b, float c, float d) {
   *reinterpret_cast<float4*>(p) = make_float4(a, b, c, d);
 }
+// maximum over the warp in one instruction
+__device__ __forceinline__ float warp_max(float x) {
+  float r;
+  asm volatile("redux.sync.max.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(x));
+  return r;
+}
 __device__ __forceinline__ int warp_sum(int x) {
 #pragma unroll
   for (int s = 16; s > 0; s >>= 1) x += __shfl_xor_sync(0xffffffffu, x, s);
@@ -81,8 +87,7 @@ __device__ __forceinline__ void decode_merge(uint32_t recs, uint32_t mls, int ra
 #pragma unroll
     for (int x = 0; x < (CLUSTER ? kMaxCluster : 1) * MNW; x += 32)
       if (x + lane < nsrc) M = fmaxf(M, lds_f2(mb + 8 * (x + lane)).x);
-#pragma unroll
-    for (int x = 1; x < 32; x <<= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, x));
+    M = warp_max(M);
     float a[5] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
 #pragma unroll 4
     for (int x = sg; x < nsrc; x += 8) {

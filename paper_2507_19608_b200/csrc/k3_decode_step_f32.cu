@@ -38,11 +38,6 @@ template <int D, int G> struct F32DecSmem {
   __host__ __device__ static constexpr uint32_t nrec(int cs) { return (uint32_t)((NB + cs - 1) / cs * cs) * NW; }
   static constexpr size_t bytes(int cs) { return 1024 + RING + nrec(cs) * (REC + 2) * 4 + PROBS + ROWS; }
 };
-__device__ __forceinline__ float warp_max(float x) {
-  float r;
-  asm volatile("redux.sync.max.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(x));
-  return r;
-}
 }  // namespace
 
 template <int D, int G, bool CLUSTER>
@@ -164,6 +159,7 @@ decode_step_f32_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_co
     for (int c = 0; c < CPL; ++c) o[h][c] = 0.0f;
   }
   uint32_t ph = 0;
+  bool owns_new = false;                     // the warp owns the row that arrives with the step
   float* const pw = s_p + (size_t)warp * UK * G;
   // the lane's key against G rows of operands
   auto dots = [&](const float* rows, float (&s)[G]) {
@@ -250,11 +246,7 @@ decode_step_f32_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_co
     __syncwarp();                            // the warp is done with the unit
     ph ^= 1u;
     if (jn < j1) fetch(jn);
-    if (owner && lane < D / 4 && DELTA_IN(n, T_max, p.counters)) {
-      // the row that arrives with the step joins the caches
-      reinterpret_cast<float4*>(p.k_cache + (row0 + n) * D)[lane] = __ldcg(reinterpret_cast<const float4*>(kn) + lane);
-      reinterpret_cast<float4*>(p.v_cache + (row0 + n) * D)[lane] = __ldcg(reinterpret_cast<const float4*>(vn) + lane);
-    }
+    owns_new = owner;
   }
 
   // ---- merge: every warp sends its part to where it is finished
@@ -278,6 +270,11 @@ decode_step_f32_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_co
     if (lane % LPB == 0) {
       if (CLUSTER) cluster_send2(dml, rbar, m[h], l[h]); else sts_f2(dml, m[h], l[h]);
     }
+  }
+  if (owns_new && lane < D / 4 && DELTA_IN(n, T_max, p.counters)) {
+    // the row that arrives with the step joins the caches while the parts travel
+    reinterpret_cast<float4*>(p.k_cache + (row0 + n) * D)[lane] = __ldcg(reinterpret_cast<const float4*>(kn) + lane);
+    reinterpret_cast<float4*>(p.v_cache + (row0 + n) * D)[lane] = __ldcg(reinterpret_cast<const float4*>(vn) + lane);
   }
   if (CLUSTER) {
     if (!mbar_wait(bar_m, 0)) s_fail = 1;

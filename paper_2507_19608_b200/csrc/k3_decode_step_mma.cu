@@ -237,6 +237,14 @@ decode_step_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_co
         }
     }
   };
+  // where this thread's part of the result goes: slice and record (a division; ahead of the wait)
+  uint32_t to_rank[NV], to_rec[NV];
+#pragma unroll
+  for (int c = 0; c < NV; ++c) {
+    const int q = hd * (D / 16) + 4 * c + t;
+    to_rank[c] = (uint32_t)(q % cs);
+    to_rec[c] = (uint32_t)(q / cs * nsrc + rank * MNW + warp);
+  }
   // Reference-key rows and their encoding are the library's own: all but the row (segment) the step in
   // front may be writing is final before this kernel can start, since that step releases it only
   // behind its own wait, and is requested ahead of the wait.  (Key and value rows are the caller's.)
@@ -248,10 +256,6 @@ decode_step_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_co
   // The next step's CTAs may become resident from here on.  (Released at the kernel's start they
   // take the places of this step's own late CTAs: 30 us per step for 18 at batch 16.)
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  if (jg < j1) {
-    if (!early_k) fetch_k(jg);
-    fetch_v(jg);
-  }
 
   // ---- threshold step (Eq. 2-3): the operand rows, straight into registers
   uint32_t ar[NC][4], aq[NC][4];             // rows g and g + 8 of A, channels 32 c + 8 t ..
@@ -271,6 +275,11 @@ decode_step_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_co
       r4[c][0] = __ldcg(reinterpret_cast<const float4*>(rp + ch));
       r4[c][1] = __ldcg(reinterpret_cast<const float4*>(rp + ch) + 1);
       if (KEY) x4[c] = __ldcg(reinterpret_cast<const uint4*>(kn + ch));
+    }
+    // (behind those loads: they are what the warp waits for next)
+    if (jg < j1) {
+      if (!early_k) fetch_k(jg);
+      fetch_v(jg);
     }
 #pragma unroll
     for (int c = 0; c < NC; ++c) {
@@ -310,6 +319,7 @@ decode_step_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_co
 #pragma unroll
     for (int e = 0; e < 4; ++e) o_acc[i][e] = 0.0f;
   float m = -INFINITY, l = 0.0f;
+  bool first = true;
   unsigned done = 0;
   uint32_t ph_k = 0, ph_v = 0;
   // Column x of a score block stands for key x ^ (4 (x & 1)) of its 8 keys: with the swizzle, the
@@ -407,8 +417,25 @@ decode_step_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_co
       p.kp_nnz[(size_t)bkv * p.nseg_max * UK + n] = (uint16_t)nz;
     }
   };
+  // What a unit leaves behind its products is stored when the next unit, or the merge, is under way.
+  float s[4][4];
+  int j_done = -1;                           // the unit whose scores s holds
+  unsigned nz = 0;                           // KEY: its multiply-adds per query, of key j_done + lane
+  bool owns_new = false;                     // the warp owns the row that arrives with the step
+  auto store_r = [&]() {
+    if (!KEY && part == 0 && j_done >= 0) {  // R[j] = q_hat . k_j
+#pragma unroll
+      for (int h = 0; h < 4; ++h) {
+        const int ja = j_done + 8 * h + kx0, jb = j_done + 8 * h + kx1;
+        if ((!owns_new || ja <= n) && DELTA_IN(ja, T_max, p.counters)) Rg[ja] = s[h][0];
+        if ((!owns_new || jb <= n) && DELTA_IN(jb, T_max, p.counters)) Rg[jb] = s[h][1];
+      }
+    }
+  };
   for (; jg < j1; jg += UK * MNW) {
     const int jn = jg + UK * MNW;            // the warp's next unit
+    store_r();
+    done += nz;
     const bool owner = n < jg + UK;          // of the row that arrives with the step
     const bool packed = from_pack(jg), tma_k = !packed && k_plain(jg), tma_v = jg + UK <= n;
     if (packed) {
@@ -422,7 +449,6 @@ decode_step_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_co
       async_wait_all();
       __syncwarp();
     }
-    float s[4][4];
 #pragma unroll
     for (int h = 0; h < 4; ++h) {
 #pragma unroll
@@ -437,26 +463,23 @@ decode_step_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_co
         mma16816(s[h], ar[c][2], aq[c][2], ar[c][3], aq[c][3], k4.z, k4.w);
       }
     }
-    int nz_new = 0;
+    j_done = jg;
+    owns_new = owner;
     if (KEY) {
-      // multiply-adds: d inside the window, nnz(Delta k_j) outside
+      // multiply-adds: d inside the window, nnz(Delta k_j) outside (added when the load is back)
       const int j = jg + lane;
-      if (owner) {
-        nz_new = warp_sum(fired);
-        if (lane == 0 && DELTA_IN(n, T_max, p.counters)) p.row_nnz[row0 + n] = (uint16_t)nz_new;
-      }
-      if (j < j1) done += (n - j < W) ? (unsigned)D : (j == n) ? (unsigned)nz_new : (unsigned)p.row_nnz[row0 + j];
+      nz = (j > n || j >= j1) ? 0u : (n - j < W) ? (unsigned)D : j == n ? 0u : (unsigned)p.row_nnz[row0 + j];
       if (!tma_k) tc::fence_proxy_async();                 // rows written by the warp, TMA overwrites them
     }
     __syncwarp();                            // every key of the unit has been used
     if (jn < j1) fetch_k(jn);
 
-    // hybrid select, scale, running maximum of the row (4 threads hold it)
+    // hybrid select, running maximum of the row (4 threads hold it); the scale joins the exponential
     float v[8];
 #pragma unroll
     for (int h = 0; h < 4; ++h) {
-      v[2 * h] = ((KEY || jg + 8 * h + kx0 < wl) ? s[h][0] : s[h][2]) * p.scale_log2e;
-      v[2 * h + 1] = ((KEY || jg + 8 * h + kx1 < wl) ? s[h][1] : s[h][3]) * p.scale_log2e;
+      v[2 * h] = (KEY || jg + 8 * h + kx0 < wl) ? s[h][0] : s[h][2];
+      v[2 * h + 1] = (KEY || jg + 8 * h + kx1 < wl) ? s[h][1] : s[h][3];
     }
     if (owner) {
 #pragma unroll
@@ -467,8 +490,11 @@ decode_step_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_co
     }
     float mx = tc::fmax3(fmaxf(v[0], v[1]), tc::fmax3(v[2], v[3], v[4]), tc::fmax3(v[5], v[6], v[7]));
     mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
-    mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
-    if (__any_sync(0xffffffffu, mx > m)) {
+    mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 2)) * p.scale_log2e;
+    if (first) {
+      m = mx;
+      first = false;
+    } else if (__any_sync(0xffffffffu, mx > m)) {
       const float mn = fmaxf(m, mx), al = tc::ex2(m - mn);
       m = mn;
       l *= al;
@@ -479,7 +505,7 @@ decode_step_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_co
     }
     float pr[8];
 #pragma unroll
-    for (int e = 0; e < 8; ++e) pr[e] = tc::ex2(v[e] - m);
+    for (int e = 0; e < 8; ++e) pr[e] = tc::ex2(fmaf(v[e], p.scale_log2e, -m));
     l += ((pr[0] + pr[1]) + (pr[2] + pr[3])) + ((pr[4] + pr[5]) + (pr[6] + pr[7]));
     if (tma_v) {
       if (!mbar_wait(bar_v, ph_v)) s_fail = 1;
@@ -516,27 +542,6 @@ decode_step_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_co
     }
     __syncwarp();
     if (jn < j1) fetch_v(jn);
-    if (!KEY && part == 0) {                 // R[j] = q_hat . k_j
-#pragma unroll
-      for (int h = 0; h < 4; ++h) {
-        const int ja = jg + 8 * h + kx0, jb = jg + 8 * h + kx1;
-        if ((!owner || ja <= n) && DELTA_IN(ja, T_max, p.counters)) Rg[ja] = s[h][0];
-        if ((!owner || jb <= n) && DELTA_IN(jb, T_max, p.counters)) Rg[jb] = s[h][1];
-      }
-    }
-    if (owner && DELTA_IN(n, T_max, p.counters)) {
-      // the row that arrives with the step joins the caches
-      if (lane < D / 8) {
-        reinterpret_cast<uint4*>(p.k_cache + (row0 + n) * D)[lane] = __ldcg(reinterpret_cast<const uint4*>(kn) + lane);
-        reinterpret_cast<uint4*>(p.v_cache + (row0 + n) * D)[lane] = __ldcg(reinterpret_cast<const uint4*>(vn) + lane);
-      }
-      if constexpr (PACKED) append(nz_new);
-      if (MODE == 1 && g == 0)
-#pragma unroll
-        for (int c = 0; c < NC; ++c)
-          *reinterpret_cast<uint4*>(p.khat_cache + (row0 + n) * D + 32 * c + 8 * t) =
-              make_uint4(khat_new[c][0], khat_new[c][1], khat_new[c][2], khat_new[c][3]);
-    }
   }
 
   // ---- the warp's result: the parts of P meet again, the row sum over the row's four threads
@@ -552,14 +557,13 @@ decode_step_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_co
     }
   }
   // ---- merge: every warp sends its part to where it is finished
-  const int src = rank * MNW + warp;
   if (CLUSTER) asm volatile("barrier.cluster.wait.aligned;" ::: "memory");          // every slice runs
   if (part == 0) {
 #pragma unroll
     for (int c = 0; c < NV; ++c) {
       // tile 8c + i, accumulator column x holds channel 64 c + 8 x + i; this thread has columns 2t, 2t + 1
-      const int q = hd * (D / 16) + 4 * c + t, r = q % cs, rec = (q / cs) * nsrc + src;
-      uint32_t dst = recs + (uint32_t)rec * (REC * 4), dml = mls + (uint32_t)rec * 8, rbar = bar_m;
+      const uint32_t r = to_rank[c];
+      uint32_t dst = recs + to_rec[c] * (REC * 4), dml = mls + to_rec[c] * 8, rbar = bar_m;
       if (CLUSTER) { dst = cluster_map(dst, r); dml = cluster_map(dml, r); rbar = cluster_map(bar_m, r); }
 #pragma unroll
       for (int e = 0; e < 4; ++e) {
@@ -570,20 +574,35 @@ decode_step_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_co
       if (CLUSTER) cluster_send2(dml, rbar, m, l); else sts_f2(dml, m, l);
     }
   }
-  if (keep) {
-    const int f = warp_sum(fired);
-    if (lane == 0) {
-      const int n_in = min(L, max(W, 0));
-      atomicAdd(&p.counters[CNT_DECODE_NNZ], (unsigned long long)f);
-      atomicAdd(&p.counters[CNT_DECODE_ELEMS], (unsigned long long)(KEY ? D : G * D));
-      atomicAdd(&p.counters[CNT_DECODE_MACS_DENSE], (unsigned long long)L * D * G);
-      if (!KEY)
-        atomicAdd(&p.counters[CNT_DECODE_MACS_DONE],
-                  (unsigned long long)n_in * D * G + (unsigned long long)(L - n_in) * f);
+  // ---- while the parts travel: the last unit's score row, the caches' new row, the counters
+  store_r();
+  const int f_all = (keep || (KEY && owns_new)) ? warp_sum(fired) : 0;
+  if (owns_new && DELTA_IN(n, T_max, p.counters)) {
+    // the row that arrives with the step joins the caches
+    if (lane < D / 8) {
+      reinterpret_cast<uint4*>(p.k_cache + (row0 + n) * D)[lane] = __ldcg(reinterpret_cast<const uint4*>(kn) + lane);
+      reinterpret_cast<uint4*>(p.v_cache + (row0 + n) * D)[lane] = __ldcg(reinterpret_cast<const uint4*>(vn) + lane);
     }
+    if (KEY && lane == 0) p.row_nnz[row0 + n] = (uint16_t)f_all;
+    if constexpr (PACKED) append(f_all);
+    if (MODE == 1 && g == 0)
+#pragma unroll
+      for (int c = 0; c < NC; ++c)
+        *reinterpret_cast<uint4*>(p.khat_cache + (row0 + n) * D + 32 * c + 8 * t) =
+            make_uint4(khat_new[c][0], khat_new[c][1], khat_new[c][2], khat_new[c][3]);
+  }
+  if (keep && lane == 0) {
+    const int n_in = min(L, max(W, 0));
+    atomicAdd(&p.counters[CNT_DECODE_NNZ], (unsigned long long)f_all);
+    atomicAdd(&p.counters[CNT_DECODE_ELEMS], (unsigned long long)(KEY ? D : G * D));
+    atomicAdd(&p.counters[CNT_DECODE_MACS_DENSE], (unsigned long long)L * D * G);
+    if (!KEY)
+      atomicAdd(&p.counters[CNT_DECODE_MACS_DONE],
+                (unsigned long long)n_in * D * G + (unsigned long long)(L - n_in) * f_all);
   }
   if (KEY) {
-    const int d = warp_sum((int)done);
+    // (the new key: inside any window of at least one key, else its own count)
+    const unsigned d = __reduce_add_sync(0xffffffffu, done + nz) + (owns_new && W <= 0 ? (unsigned)f_all : 0u);
     if (lane == 0 && d) atomicAdd(&p.counters[CNT_DECODE_MACS_DONE], (unsigned long long)d * G);
   }
   if (CLUSTER) {
