@@ -30,9 +30,15 @@
 //
 // Key tiles and the window (Section III-B).  A tile none of whose pairs is inside the window is
 // scored by the telescoped product alone; a tile all of whose causal pairs are inside it by
-// Q.K^T alone; a mixed tile takes the telescoped product first and then, one half of 64 keys
-// at a time, hands the half the threads have read into registers back for Q.K^T, from which
-// they take the in-window elements.
+// Q.K^T alone.  A mixed tile takes both, one half of 64 keys at a time.  d = 64: the half's two
+// products stand side by side in the score buffer (64 columns each), and the second half's are
+// issued as soon as the threads have read the first's, so they run under its exponentials: two
+// hand-overs per tile, and the register allocator finds room without a spill.  (Against handing a
+// half that is held in registers back for its exact product, three hand-overs and spills in every
+// tile of the launch: 4 x 32 heads, 1777 keys, key deltas, sliding window of 100 174 -> 133 us, no
+// window 109; 32 heads, 1900 keys, block window of 95 65 -> 56 us, of 64 51; six ragged sequences
+// of 99 to 1900 keys with windows of 4 to 95 167 -> 134 us.)  d = 128 has the probabilities over the
+// scores and no such room: it hands the half back.
 //
 // Head dimensions 64 and 128 (template parameter).
 //
@@ -75,6 +81,9 @@ template <int D, bool PAIR> struct TqSmem {
   static constexpr uint32_t NQ = PAIR ? 2 : 1;            // query tiles (heads) per CTA
   static constexpr uint32_t NKS = PAIR ? 3 : (D == 64) ? 4 : 3;      // key ring stages
   static constexpr uint32_t NVS = PAIR ? 3 : (D == 64) ? 4 : 2;      // value ring stages
+  // original keys of mixed tiles (key deltas), from OFF_QH on: d = 64 has the scores of two mixed
+  // tiles in flight at a time
+  static constexpr uint32_t NKX = (D == 64) ? 2 : 1;
   static constexpr uint32_t OFF_Q = 0;                    // [NQ] query tiles
   static constexpr uint32_t OFF_QH = OFF_Q + NQ * SZ_TILE;   // [NQ] reference-query tiles
   // d = 64, query deltas: two operand tiles mixed by row halves, [Q rows 0-63; Q_hat rows
@@ -99,8 +108,9 @@ enum Bar {
   BAR_KFREE0 = BAR_KFULL0 + 4,
   BAR_VFULL0 = BAR_KFREE0 + 4,
   BAR_VFREE0 = BAR_VFULL0 + 4,
-  BAR_KXFULL = BAR_VFREE0 + 4, BAR_KXFREE,    // original keys of a window tile (key deltas)
-  BAR_SFULL0, BAR_SFULL1,    // a score product of the group is complete (tcgen05.commit)
+  BAR_KXFULL0 = BAR_VFREE0 + 4,               // original keys of a mixed tile (key deltas; + slot, up to 2)
+  BAR_KXFREE0 = BAR_KXFULL0 + 2,
+  BAR_SFULL0 = BAR_KXFREE0 + 2, BAR_SFULL1,    // a score product of the group is complete (tcgen05.commit)
   BAR_PRDY0, BAR_PRDY1,      // probabilities written (4 warps)
   BAR_SXREQ0, BAR_SXREQ1,    // telescoped scores read, the exact pass may overwrite them (4 warps)
   BAR_ODONE0, BAR_ODONE1,    // the group's last P.V is complete
@@ -212,8 +222,8 @@ __device__ __forceinline__ void build_ref_rows(const unsigned char* q_src, unsig
 // and the original keys are fetched only for tiles that touch the window.
 // MIXED = false: no key tile of the launch is mixed (no window; a block window of whole
 // 128-key tiles; or, query deltas at d = 64, a block window whose edges fall on multiples of
-// 64): the code of the mixed tiles is left out,
-// and with it every register spill of the kernel.
+// 64): the code of the mixed tiles is left out (at d = 128 every register spill of the kernel is
+// there; at d = 64 it costs the other tiles registers, 144 -> 168, and some percent).
 // FORM: 0 = every CTA one head; 1 = every CTA two heads; 2 = two-head layout, the form of a CTA
 // follows its place in the grid (see below).
 // N: entries of the sequence list: 1 (a uniform batch), or kSeqMax (a ragged group: the grid is
@@ -228,7 +238,7 @@ hybrid_attn_tcq_kernel(const __grid_constant__ TqMapList<N> maps, const __grid_c
   unsigned char* sm = smem_raw + (base - raw);
   constexpr bool PAIR = FORM != 0;       // the layout holds two query tiles
   using SM = TqSmem<D, PAIR>;
-  constexpr uint32_t NKB = SM::NKB, SZ_TILE = SM::SZ_TILE, NKS = SM::NKS, NVS = SM::NVS;
+  constexpr uint32_t NKB = SM::NKB, SZ_TILE = SM::SZ_TILE, NKS = SM::NKS, NVS = SM::NVS, NKX = SM::NKX;
   constexpr uint32_t OFF_Q = SM::OFF_Q, OFF_QH = SM::OFF_QH, OFF_K = SM::OFF_K, OFF_V = SM::OFF_V,
                      OFF_BAR = SM::OFF_BAR, OFF_MISC = SM::OFF_MISC, OFF_QM = SM::OFF_QM;
   volatile uint32_t* sMisc = reinterpret_cast<volatile uint32_t*>(sm + OFF_MISC);
@@ -378,9 +388,10 @@ hybrid_attn_tcq_kernel(const __grid_constant__ TqMapList<N> maps, const __grid_c
         const int cls = tile_class(t);
         load_tile(base + OFF_K + ks * SZ_TILE, (KEY && cls == 2) ? &tm_k : tm_ring, BAR(BAR_KFULL0 + ks), t * BN, bkv);
         if (MIXED && KEY && cls == 1) {
-          if (n_kx > 0) mbar_wait(BAR(BAR_KXFREE), (n_kx - 1) & 1, abort_flag);
-          mbar_expect_tx(BAR(BAR_KXFULL), SZ_TILE);
-          load_tile(base + OFF_QH, &tm_k, BAR(BAR_KXFULL), t * BN, bkv);
+          const uint32_t xs = (uint32_t)n_kx % NKX;
+          if (n_kx >= (int)NKX) mbar_wait(BAR(BAR_KXFREE0 + xs), ((n_kx / (int)NKX) - 1) & 1, abort_flag);
+          mbar_expect_tx(BAR(BAR_KXFULL0 + xs), SZ_TILE);
+          load_tile(base + OFF_QH + xs * SZ_TILE, &tm_k, BAR(BAR_KXFULL0 + xs), t * BN, bkv);
           ++n_kx;
         }
         if (t >= (int)NVS) mbar_wait(BAR(BAR_VFREE0 + vs), ((t / NVS) - 1) & 1, abort_flag);
@@ -403,7 +414,26 @@ hybrid_attn_tcq_kernel(const __grid_constant__ TqMapList<N> maps, const __grid_c
         tc_commit(BAR(BAR_SFULL0 + X));
       };
       const uint32_t IDESC_QK64 = make_idesc(64, 0);
-      int n_kx = 0, n_sx0 = 0, n_sx1 = 0;
+      int n_kx0 = 0, n_kx = 0, n_sx0 = 0, n_sx1 = 0;   // mixed tiles whose first / last products are issued
+      // d = 64, mixed tile: both products of one half of 64 keys side by side in the score buffer,
+      // telescoped in columns 0-63, exact in columns 64-127
+      auto mixed_half_scores = [&](int u, int hf, int ord) {
+        const int t = tile_of(u);
+        const uint32_t X = (uint32_t)u & 1u, qsel = pr ? X * SZ_TILE : 0u;
+        tc_fence_after();
+        const uint32_t ring = base + OFF_K + ((uint32_t)t % NKS) * SZ_TILE;
+        const uint32_t kx = KEY ? base + OFF_QH + ((uint32_t)ord % NKX) * SZ_TILE : ring;
+        const uint32_t qt_ = base + (KEY ? OFF_Q : OFF_QH) + qsel, qx = base + OFF_Q + qsel;
+#pragma unroll
+        for (int w = 0; w < 2; ++w)
+#pragma unroll
+          for (int ks = 0; ks < D / 16; ++ks)
+            tc_mma(tmem + TMEM_S + 128u * X + 64u * w,
+                   make_desc((w ? qx : qt_) + (ks >> 2) * SZ_BLK + (ks & 3) * 32, 16, 1024),
+                   make_desc((w ? kx : ring) + 8192u * hf + (ks >> 2) * SZ_BLK + (ks & 3) * 32, 16, 1024), IDESC_QK64,
+                   ks > 0 ? 1u : 0u);
+        tc_commit(BAR(BAR_SFULL0 + X));
+      };
       // first scores of unit u, for group u & 1: telescoped, or exact where the whole tile
       // lies inside the window
       auto first_scores = [&](int u) {
@@ -435,6 +465,13 @@ hybrid_attn_tcq_kernel(const __grid_constant__ TqMapList<N> maps, const __grid_c
           tc_commit(BAR(BAR_SFULL0 + X));
           return;
         }
+        if (MIXED && !ALIAS && cls == 1) {
+          // (head pairs: the same tile of keys for both heads)
+          if (KEY) mbar_poll(BAR(BAR_KXFULL0 + (uint32_t)n_kx0 % NKX), (n_kx0 / (int)NKX) & 1, abort_flag);
+          mixed_half_scores(u, 0, n_kx0);
+          if (!pr || X == 1u) ++n_kx0;
+          return;
+        }
         const bool q_exact = KEY || cls == 2;
         scores(X, base + (q_exact ? OFF_Q : OFF_QH) + qsel, ring);
       };
@@ -447,26 +484,35 @@ hybrid_attn_tcq_kernel(const __grid_constant__ TqMapList<N> maps, const __grid_c
         const int t = tile_of(u);
         const uint32_t X = (uint32_t)u & 1u;
         if (MIXED && tile_class(t) == 1) {
-          // mixed tile: Q.K^T over each half of 64 keys once the group has that half's
-          // telescoped scores in registers
-          if (KEY) mbar_poll(BAR(BAR_KXFULL), n_kx & 1, abort_flag);   // (head pairs: the same tile for both heads)
           int& n_sx = X ? n_sx1 : n_sx0;
-          const uint32_t kx = KEY ? base + OFF_QH : base + OFF_K + ((uint32_t)t % NKS) * SZ_TILE;
-          const uint32_t qx = base + OFF_Q + (pr ? X * SZ_TILE : 0u);
-#pragma unroll
-          for (int hf = 0; hf < 2; ++hf) {
+          if (!ALIAS) {
+            // the second half's products once the group has read the first half's
             mbar_poll(BAR(BAR_SXREQ0 + X), n_sx & 1, abort_flag);
             ++n_sx;
-            tc_fence_after();
+            mixed_half_scores(u, 1, n_kx);
+          } else {
+            // d = 128 (the probabilities lie over the scores): Q.K^T over each half of 64 keys once the
+            // group has that half's telescoped scores in registers
+            if (KEY) mbar_poll(BAR(BAR_KXFULL0), n_kx & 1, abort_flag);
+            const uint32_t kx = KEY ? base + OFF_QH : base + OFF_K + ((uint32_t)t % NKS) * SZ_TILE;
 #pragma unroll
-            for (int ks = 0; ks < D / 16; ++ks)
-              tc_mma(tmem + TMEM_S + 128u * X + 64u * hf,
-                     make_desc(qx + (ks >> 2) * SZ_BLK + (ks & 3) * 32, 16, 1024),
-                     make_desc(kx + 8192u * hf + (ks >> 2) * SZ_BLK + (ks & 3) * 32, 16, 1024), IDESC_QK64,
-                     ks > 0 ? 1u : 0u);
-            tc_commit(BAR(BAR_SFULL0 + X));
+            for (int hf = 0; hf < 2; ++hf) {
+              mbar_poll(BAR(BAR_SXREQ0 + X), n_sx & 1, abort_flag);
+              ++n_sx;
+              tc_fence_after();
+#pragma unroll
+              for (int ks = 0; ks < D / 16; ++ks)
+                tc_mma(tmem + TMEM_S + 128u * X + 64u * hf,
+                       make_desc(base + OFF_Q + (ks >> 2) * SZ_BLK + (ks & 3) * 32, 16, 1024),
+                       make_desc(kx + 8192u * hf + (ks >> 2) * SZ_BLK + (ks & 3) * 32, 16, 1024), IDESC_QK64,
+                       ks > 0 ? 1u : 0u);
+              tc_commit(BAR(BAR_SFULL0 + X));
+            }
           }
-          if (KEY && (!pr || X == 1u)) { tc_commit(BAR(BAR_KXFREE)); ++n_kx; }
+          if (!pr || X == 1u) {
+            if (KEY) tc_commit(BAR(BAR_KXFREE0 + (uint32_t)n_kx % NKX));
+            ++n_kx;
+          }
         }
         // every product that reads this key stage is issued (head pairs: after the second head's)
         if (!pr || X == 1u) tc_commit(BAR(BAR_KFREE0 + (uint32_t)t % NKS));
@@ -568,11 +614,8 @@ hybrid_attn_tcq_kernel(const __grid_constant__ TqMapList<N> maps, const __grid_c
       if (lane == 0) mbar_arrive(BAR(BAR_QH));
     };
 
-    int wlo = 0, whi = 0;       // exact keys of row i: wlo <= j < whi
-    if (W > 0) {
-      if (shape == 0) { wlo = (i / W) * W; whi = wlo + W; }
-      else { wlo = i - W + 1; whi = i + 1; }
-    }
+    // exact keys of row i: from wlo on (every window reaches past i, and past i the causal mask rules)
+    const int wlo = W == 0 ? i + 1 : shape == 0 ? (i / W) * W : i - W + 1;
     float m_used = -INFINITY;   // the scale (log2 domain) the row's P and O are stored at
     float l_sum = 0.0f;
     uint32_t s_phase = 0;
@@ -757,32 +800,43 @@ hybrid_attn_tcq_kernel(const __grid_constant__ TqMapList<N> maps, const __grid_c
           for (int hf = 0; hf < 2; ++hf) exp_half(hf);
         }
       } else {
-        // ---- a mixed tile (Section III-B hybrid select), one half of 64 keys at a time: the
-        // half's telescoped scores go to registers, its columns go back for the exact product,
-        // the in-window elements are taken from that
+        // ---- a mixed tile (Section III-B hybrid select), one half of 64 keys at a time.  d = 64: the
+        // half's telescoped and exact scores stand side by side in the score buffer, and the second
+        // half's products run under the first half's exponentials.  d = 128: the half's telescoped
+        // scores go to registers, its columns go back for the exact product.
         auto mixed_half = [&](int hf) {
+          if (!ALIAS && hf == 1) {
+            mbar_wait(BAR(BAR_SFULL0 + X), s_phase & 1u, abort_flag);
+            ++s_phase;
+            tc_fence_after();
+          }
           float v[64];
           {
             uint32_t u[64];
-            tc_ld64(t_s + 64u * hf, u);
+            tc_ld64(t_s + (ALIAS ? 64u * hf : 0u), u);
 #pragma unroll
             for (int c = 0; c < 64; ++c) v[c] = __uint_as_float(u[c]);
           }
-          tc_fence_before();
-          __syncwarp();
-          if (lane == 0) mbar_arrive(BAR(BAR_SXREQ0 + X));
-          mbar_wait(BAR(BAR_SFULL0 + X), s_phase & 1u, abort_flag);
-          ++s_phase;
-          tc_fence_after();
+          if (ALIAS) {
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(BAR(BAR_SXREQ0 + X));
+            mbar_wait(BAR(BAR_SFULL0 + X), s_phase & 1u, abort_flag);
+            ++s_phase;
+            tc_fence_after();
+          }
 #pragma unroll
           for (int ch = 0; ch < 2; ++ch) {
             uint32_t u[32];
-            tc_ld32(t_s + 64u * hf + 32u * ch, u);
+            tc_ld32(t_s + (ALIAS ? 64u * hf : 64u) + 32u * ch, u);
 #pragma unroll
-            for (int c = 0; c < 32; ++c) {
-              const int j = j0 + 64 * hf + 32 * ch + c;
-              if (j >= wlo && j < whi) v[32 * ch + c] = __uint_as_float(u[c]);
-            }
+            for (int c = 0; c < 32; ++c)
+              if (c >= wlo - j0 - 64 * hf - 32 * ch) v[32 * ch + c] = __uint_as_float(u[c]);
+          }
+          if (!ALIAS && hf == 0) {                 // the second half's products may have the buffer
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(BAR(BAR_SXREQ0 + X));
           }
           if (hf == 1) s_consumed();
           if (diag) {
@@ -791,7 +845,8 @@ hybrid_attn_tcq_kernel(const __grid_constant__ TqMapList<N> maps, const __grid_c
               if (j0 + 64 * hf + c > i) v[c] = -INFINITY;
           }
           settle_scale(u, max64(v), u >= 2, hf == 1);
-          exp_store(v, hf, u, 2);
+          // (diagonal tile: no exponentials for the 32-column chunks behind the warp's rows)
+          exp_store(v, hf, u, diag ? min(max(w4 + 1 - 2 * hf, 0), 2) : 2);
         };
         if (D == 64) {
           mixed_half(0);
