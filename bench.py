@@ -219,7 +219,7 @@ def to_dev(x, dtype, torch):
     return torch.from_numpy(np.ascontiguousarray(x)).cuda()
 
 
-KERNEL_NAMES = {0: "generic (FP32 pipes)", 1: "tcgen05 + FP32 delta path", 2: "tcgen05 telescoped"}
+KERNEL_NAMES = {0: "fp32 arithmetic (tensor cores, split operands)", 1: "tcgen05 + FP32 delta path", 2: "tcgen05 telescoped"}
 
 
 def flop_model(w, stats, kernel):
@@ -229,9 +229,9 @@ def flop_model(w, stats, kernel):
       score stage (d per in-window pair, nnz(dq_i) per out-of-window pair: the library's macs_done)
       plus 2 d per causal pair for P.V.  This is the figure the roofline fraction is taken from.
     executed: what the selected kernel really runs.  Kernel 2 (telescoped) multiplies q_hat.k
-      densely, d multiply-adds for every pair, on the tensor cores and skips nothing; kernel 1
-      runs the sparse products (plus one dense seed row per 128-row query tile) on the FP32 pipes;
-      kernel 0 runs everything on the FP32 pipes.
+      densely, d multiply-adds for every pair, on the tensor cores and skips nothing, and so does
+      kernel 0, at fp32 precision (several products per multiply-add); kernel 1
+      runs the sparse products (plus one dense seed row per 128-row query tile) on the FP32 pipes.
     dense_equiv: 4 d per causal pair, what dense attention would be credited with."""
     BH = w.B * w.H
     N_c = w.T * (w.T + 1) // 2
@@ -243,12 +243,10 @@ def flop_model(w, stats, kernel):
     seeds = 2.0 * w.d * (N_c - n_in) * BH / 128.0               # one dense row per 128-row query tile
     dense_equiv = 4.0 * w.d * N_c * BH
     method = qk + pv
-    if kernel == 2:
+    if kernel != 1:
         return dict(method=method, executed=dense_equiv, alu=0.0, tensor=dense_equiv, dense_equiv=dense_equiv)
-    if kernel == 1:
-        return dict(method=method, executed=qk + seeds + pv, alu=(qk - qk_in) + seeds, tensor=qk_in + pv,
-                    dense_equiv=dense_equiv)
-    return dict(method=method, executed=qk + seeds + pv, alu=qk + seeds + pv, tensor=0.0, dense_equiv=dense_equiv)
+    return dict(method=method, executed=qk + seeds + pv, alu=(qk - qk_in) + seeds, tensor=qk_in + pv,
+                dense_equiv=dense_equiv)
 
 
 def k2_roofline(w, stats, kernel, k2_ms, peaks, n_sm, sustained=False):
@@ -263,7 +261,7 @@ def k2_roofline(w, stats, kernel, k2_ms, peaks, n_sm, sustained=False):
               "method_gflop_per_launch": fm["method"] / 1e9, "executed_gflop_per_launch": fm["executed"] / 1e9,
               "method_tflops": fm["method"] / t / 1e12, "executed_tflops": fm["executed"] / t / 1e12,
               "dense_equiv_tflops": fm["dense_equiv"] / t / 1e12, "traffic": measured_traffic(kernel, w.name)}
-    if kernel == 2:
+    if kernel != 1:
         key = "bf16_tflops_sustained" if sustained and "bf16_tflops_sustained" in peaks else "bf16_tflops"
         peak = float(peaks[key])
         a = fm["method"] / t / 1e12
@@ -646,7 +644,7 @@ def run_decode(args, B, torch, peaks, source="query", names=("llama32_1b_decode_
             "us_per_step_eager": statistics.median(eager), "us_per_step_graph": graph_us,
             "us_per_step_l2_flushed": flushed_us, "us_per_step_l2_flushed_by_read": flushed_read_us,
             "graph_matches_eager": graph_ok, "steps": w.n_decode,
-            "decode_kernel": ("FP32 pipes, compressed key-delta cache" if packed else
+            "decode_kernel": ("tensor cores, compressed key-delta cache" if packed else
                               "tensor-core scores" if B.delta_state_decode_kernel(st) == 1 else "FP32 pipes"),
             "key_cache_bytes": cache_bytes, "cache_tokens": w.T, "theta": theta,
             "window": w.window, "algorithmic_bytes_per_step": bytes_step,
@@ -980,7 +978,7 @@ def main():
     ap.add_argument("--impl", default="ours", choices=["ours", "reference"])
     ap.add_argument("--workload", default="llama32_1b_prefill")
     ap.add_argument("--theta", type=float, default=HEADLINE_THETA)
-    ap.add_argument("--kernel", type=int, default=-1, help="-1 auto, 0 generic, 1 tcgen05 + FP32 delta path, 2 tcgen05 telescoped")
+    ap.add_argument("--kernel", type=int, default=-1, help="-1 auto, 0 fp32 arithmetic, 1 tcgen05 + FP32 delta path, 2 tcgen05 telescoped")
     ap.add_argument("--quick", action="store_true", help="prefill timing only (used for ncu launch lists)")
     ap.add_argument("--only", default="", choices=["", "decode_b1", "decode_b16", "stack_layer", "stack", "bitnet"],
                     help="run one secondary leg alone on one GPU (small ncu captures of its kernels)")

@@ -19,7 +19,7 @@
 //
 // Bound: a few MB of reads and writes.  One CTA per eight segments of a KV head (a warp each); every
 // CTA derives the segment offsets from the row counts itself, a scan over T / 32 sums, which costs
-// less than a launch of its own.  (One CTA per KV head took 46 us for 32 heads of 1024 keys, this 6.)
+// less than a launch of its own.  (One CTA per KV head took 46 us for 32 heads of 1024 keys, this 10.)
 #include "delta_internal.cuh"
 
 namespace delta {

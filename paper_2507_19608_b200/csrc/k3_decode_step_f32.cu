@@ -11,7 +11,7 @@
 //           packed fma.rn.f32x2; queries only where the unit touches the window;
 //   P.V     lane = D / 32 channels, probabilities broadcast.
 // Bound: dependent latencies at the sizes fp32 is used at (16 heads over 1000 keys move 2 MB): 10.3 us per
-// step with block barriers around every tile and a merge through global memory, 5.5 so.
+// step with block barriers around every tile and a merge through global memory, 5.0 so.
 #include "decode_common.cuh"
 #include "decode_merge.cuh"
 

@@ -30,9 +30,9 @@
 // bytes on the receiver's barrier (a merge through global memory takes 2 us more; a cluster barrier
 // with release semantics waits 0.7 us for the step's global stores).
 // Measured, us per step, against the kernel before it (tcgen05 scores for d = 64, FP32 pipes for
-// d = 128): Llama layer at 2048 keys, batch 1 8.9 -> 4.8, batch 4 10.3 -> 7.0, batch 16 18.4 -> 12.3
-// (5.9 TB/s); batch 8 at 4096 keys 18.0 -> 11.8; BitNet layer (d = 128) at 1531 keys, batch 2
-// 16.7 -> 6.5, at 2000 keys, batch 16 45.5 -> 14.9; key deltas, batch 4 at 1777 keys 12.1 -> 6.8.
+// d = 128): Llama layer at 2048 keys, batch 1 8.9 -> 4.4, batch 4 10.3 -> 7.0, batch 16 18.4 -> 12.2
+// (5.9 TB/s); batch 8 at 4096 keys 18.0 -> 11.6; BitNet layer (d = 128) at 1531 keys, batch 2
+// 16.7 -> 6.1, at 2000 keys, batch 16 45.5 -> 14.2; key deltas, batch 4 at 1777 keys 12.1 -> 6.4.
 #include <cuda.h>
 
 #include "decode_common.cuh"
