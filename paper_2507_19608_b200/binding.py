@@ -162,12 +162,13 @@ def _stream(stream):
 
 
 def _load_calls():
-    """The CPython entry points of the two calls on a serving loop's path (csrc/py_calls.cpp)."""
+    """The CPython entry points of the calls on a serving loop's path (csrc/py_calls.cpp)."""
     loader = importlib.machinery.ExtensionFileLoader("_calls", _build.build_calls())
     mod = importlib.util.module_from_spec(importlib.util.spec_from_loader("_calls", loader))
     loader.exec_module(mod)
     address = lambda f: C.cast(f, C.c_void_p).value      # noqa: E731
-    mod.setup(address(lib.delta_attn_decode_step), address(lib.delta_attn_prefill), _ptr, _stream, _check, _torch_streams)
+    mod.setup(address(lib.delta_attn_decode_step), address(lib.delta_attn_prefill), address(lib.delta_state_reset),
+              address(lib.delta_state_view), _ptr, _stream, _check, _torch_streams, _make_view)
     return mod
 
 
@@ -209,12 +210,29 @@ def delta_state_init(cfg: delta_config_t, device="cuda", stream=None, workspace=
     return DeltaState(cfg, h, workspace)
 
 
-def delta_state_reset(st: DeltaState, stream=None):
-    # (host-side only: the library does not use the stream)
-    _check(lib.delta_state_reset(st.handle, None if stream is None else _stream(stream)), "delta_state_reset")
+def _make_view(st: DeltaState, what: int, address: int, nbytes: int):
+    """The tensor of delta_state_view for an array and address, kept in st.views."""
+    import torch
+    off = address - st.workspace.data_ptr()
+    raw = st.workspace[off:off + nbytes]
+    c = st.cfg
+    nt = (c.T_max + DELTA_TILE_ROWS - 1) // DELTA_TILE_ROWS
+    shapes = {DELTA_VIEW_DQ: (c.B, c.H, c.T_max, c.d), DELTA_VIEW_MASK: (c.B, c.H, c.T_max, c.d // 32),
+              DELTA_VIEW_ROW_NNZ: (c.B, c.H, c.T_max), DELTA_VIEW_TILE_NNZ: (c.B, c.H, nt),
+              DELTA_VIEW_IDX: (c.B, c.H, c.T_max, c.d), DELTA_VIEW_QHAT_TILE: (c.B, c.H, nt, c.d),
+              DELTA_VIEW_QHAT: (c.B, c.H, c.d), DELTA_VIEW_R: (c.B, c.H, c.T_max),
+              DELTA_VIEW_COUNTERS: (nbytes // 8,)}
+    t = st.views[(what, address)] = raw.view(getattr(torch, _VIEW_DTYPES[what])).view(shapes[what])
+    return t
 
 
 _calls = _load_calls()
+
+# delta_state_reset(st, stream=None): host-side only, the library does not use the stream
+delta_state_reset = _calls.delta_state_reset
+
+# delta_state_view(st, what): a torch tensor aliasing one of the state's arrays (shape per include/delta_attn.h)
+delta_state_view = _calls.delta_state_view
 
 # delta_attn_prefill(st, q, k, v, out, T, H, H_kv, d, theta, window, stream=None)
 delta_attn_prefill = _calls.delta_attn_prefill
@@ -327,24 +345,3 @@ def delta_launch_count() -> int:
 _VIEW_DTYPES = {DELTA_VIEW_DQ: "float32", DELTA_VIEW_MASK: "int32", DELTA_VIEW_ROW_NNZ: "int16",
                 DELTA_VIEW_TILE_NNZ: "int32", DELTA_VIEW_IDX: "uint8", DELTA_VIEW_QHAT_TILE: "float32",
                 DELTA_VIEW_QHAT: "float32", DELTA_VIEW_R: "float32", DELTA_VIEW_COUNTERS: "int64"}
-
-
-def delta_state_view(st: DeltaState, what: int):
-    """A torch tensor aliasing one of the state's arrays (shape per include/delta_attn.h)."""
-    import torch
-    p, n = C.c_void_p(), C.c_size_t(0)
-    _check(lib.delta_state_view(st.handle, what, C.byref(p), C.byref(n)), "delta_state_view")
-    t = st.views.get((what, p.value))
-    if t is not None:
-        return t.detach()               # another tensor over the same memory
-    off = p.value - st.workspace.data_ptr()
-    raw = st.workspace[off:off + n.value]
-    c = st.cfg
-    nt = (c.T_max + DELTA_TILE_ROWS - 1) // DELTA_TILE_ROWS
-    shapes = {DELTA_VIEW_DQ: (c.B, c.H, c.T_max, c.d), DELTA_VIEW_MASK: (c.B, c.H, c.T_max, c.d // 32),
-              DELTA_VIEW_ROW_NNZ: (c.B, c.H, c.T_max), DELTA_VIEW_TILE_NNZ: (c.B, c.H, nt),
-              DELTA_VIEW_IDX: (c.B, c.H, c.T_max, c.d), DELTA_VIEW_QHAT_TILE: (c.B, c.H, nt, c.d),
-              DELTA_VIEW_QHAT: (c.B, c.H, c.d), DELTA_VIEW_R: (c.B, c.H, c.T_max),
-              DELTA_VIEW_COUNTERS: (n.value // 8,)}
-    t = st.views[(what, p.value)] = raw.view(getattr(torch, _VIEW_DTYPES[what])).view(shapes[what])
-    return t.detach()

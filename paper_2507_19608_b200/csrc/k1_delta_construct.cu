@@ -278,8 +278,11 @@ static cudaError_t launch_delta_chain_tables(const Shape& s, const Workspace& w,
   do {                                                                                           \
     auto kern = delta_chain_kernel<TIN, DD>;                                                     \
     const size_t smem = (size_t)NS * RC * CH * sizeof(TIN) + (size_t)NZ * Z_STAGE * sizeof(float4); \
-    err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);    \
-    if (err != cudaSuccess) return err;                                                          \
+    static std::atomic<uint64_t> ready{0};                                                       \
+    if (!device_done(ready)) {                                                                   \
+      if ((err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess) return err; \
+      device_mark(ready);                                                                        \
+    }                                                                                            \
     kern<<<heads * (DD / CH), CHAIN_THREADS, smem, st>>>(tm, w.qhat_tile, w.qhat[0], w.ckpt, w.counters, T, \
                                                          s.n_tiles, s.n_ckpt(), theta, basis, reverse ? 1 : 0, \
                                                          (uint4*)zero_ptr, (unsigned)(zero_bytes / 16)); \

@@ -1,5 +1,5 @@
 // CPython entry points for the calls a serving loop makes once per layer and token
-// (delta_attn_decode_step) or once per prompt (delta_attn_prefill): argument marshalling for the C ABI
+// (delta_attn_decode_step) or once per prompt (delta_state_reset, delta_attn_prefill, delta_state_view): argument marshalling for the C ABI
 // of libdelta_attn.so without an interpreted line.  A decode step of one sequence takes 4 to 5 us on
 // the device; in Python (six _ptr calls, torch.cuda.current_stream, a ctypes call of eleven
 // converted arguments) its marshalling took 5 us on top of the launch itself, here 0.6 us.
@@ -13,13 +13,17 @@ namespace {
 typedef int (*decode_fn)(void*, const void*, const void*, const void*, void*, void*, void*, float, int32_t, void*);
 typedef int (*prefill_fn)(void*, const void*, const void*, const void*, void*, int32_t, int32_t, int32_t, int32_t, float,
                           int32_t, void*);
+typedef int (*reset_fn)(void*, void*);
+typedef int (*view_fn)(const void*, int32_t, const void**, size_t*);
 
 decode_fn g_decode;
 prefill_fn g_prefill;
-PyObject *g_ptr, *g_stream, *g_check;                 // the binding's _ptr, _stream, _check
+reset_fn g_reset;
+view_fn g_view;
+PyObject *g_ptr, *g_stream, *g_check, *g_make_view;   // the binding's _ptr, _stream, _check, _make_view
 PyObject* g_streams;                                  // gives (current device, raw stream of a device), once torch is up
 PyObject *g_get_device, *g_get_stream;                // those two
-PyObject *s_data_ptr, *s_raw, *s_decode, *s_prefill;  // interned names
+PyObject *s_data_ptr, *s_raw, *s_views, *s_detach, *s_decode, *s_prefill, *s_reset, *s_view;  // interned names
 
 // Device (or host) address of a tensor, array, integer or None.
 bool address(PyObject* o, void** out) {
@@ -84,9 +88,10 @@ bool int_of(PyObject* o, int32_t* out) {
   return true;
 }
 
-// Positional and keyword arguments into slots[0..n); the last one (stream) may be missing.
+// Positional and keyword arguments into slots[0..n); the last one (stream) may be missing, or as many
+// are needed as `needed` says.
 bool collect(const char* fn, const char* const* names, int n, PyObject* const* args, Py_ssize_t nargs, PyObject* kwnames,
-             PyObject** slots) {
+             PyObject** slots, int needed = -1) {
   for (int i = 0; i < n; ++i) slots[i] = nullptr;
   if (nargs > n) {
     PyErr_Format(PyExc_TypeError, "%s() takes at most %d arguments (%zd given)", fn, n, nargs);
@@ -106,7 +111,7 @@ bool collect(const char* fn, const char* const* names, int n, PyObject* const* a
     }
     slots[at] = args[nargs + k];
   }
-  for (int i = 0; i < n - 1; ++i)
+  for (int i = 0; i < (needed < 0 ? n - 1 : needed); ++i)
     if (!slots[i]) {
       PyErr_Format(PyExc_TypeError, "%s() missing required argument: '%s'", fn, names[i]);
       return false;
@@ -164,15 +169,59 @@ PyObject* prefill(PyObject*, PyObject* const* args, Py_ssize_t nargs, PyObject* 
   return finish(status, s_prefill);
 }
 
-// setup(decode address, prefill address, _ptr, _stream, _check, _torch_streams)
+PyObject* reset(PyObject*, PyObject* const* args, Py_ssize_t nargs, PyObject* kwnames) {
+  static const char* const names[] = {"st", "stream"};
+  PyObject* a[2];
+  if (!collect("delta_state_reset", names, 2, args, nargs, kwnames, a)) return nullptr;
+  void *h, *stream = nullptr;                         // (host-side only: the library does not use the stream)
+  if (!handle_of(a[0], &h)) return nullptr;
+  if (a[1] && a[1] != Py_None && !stream_of(a[1], &stream)) return nullptr;
+  return finish(g_reset(h, stream), s_reset);
+}
+
+// A tensor over one of the state's arrays: another one over the memory of the tensor kept in st.views, or a
+// first one (the binding's _make_view).
+PyObject* view(PyObject*, PyObject* const* args, Py_ssize_t nargs, PyObject* kwnames) {
+  static const char* const names[] = {"st", "what"};
+  PyObject* a[2];
+  if (!collect("delta_state_view", names, 2, args, nargs, kwnames, a, 2)) return nullptr;
+  void* h;
+  int32_t what;
+  if (!handle_of(a[0], &h) || !int_of(a[1], &what)) return nullptr;
+  const void* p = nullptr;
+  size_t n = 0;
+  const int status = g_view(h, what, &p, &n);
+  if (status != 0) return finish(status, s_view);
+  PyObject* at = PyLong_FromVoidPtr((void*)p);
+  PyObject* key = at ? PyTuple_Pack(2, a[1], at) : nullptr;
+  PyObject* views = key ? PyObject_GetAttr(a[0], s_views) : nullptr;
+  PyObject* t = nullptr;
+  if (views && PyDict_Check(views)) t = Py_XNewRef(PyDict_GetItemWithError(views, key));
+  if (views && !t && !PyErr_Occurred()) {
+    PyObject* size = PyLong_FromSize_t(n);
+    PyObject* argv[4] = {a[0], a[1], at, size};
+    if (size) t = PyObject_Vectorcall(g_make_view, argv, 4, nullptr);
+    Py_XDECREF(size);
+  }
+  PyObject* r = t ? PyObject_CallMethodNoArgs(t, s_detach) : nullptr;
+  Py_XDECREF(t);
+  Py_XDECREF(views);
+  Py_XDECREF(key);
+  Py_XDECREF(at);
+  return r;
+}
+
+// setup(addresses of decode, prefill, reset, view, _ptr, _stream, _check, _torch_streams, _make_view)
 PyObject* setup(PyObject*, PyObject* args) {
-  unsigned long long d, f;
-  PyObject* o[4];
-  if (!PyArg_ParseTuple(args, "KKOOOO", &d, &f, &o[0], &o[1], &o[2], &o[3])) return nullptr;
-  g_decode = (decode_fn)(uintptr_t)d;
-  g_prefill = (prefill_fn)(uintptr_t)f;
-  PyObject** to[4] = {&g_ptr, &g_stream, &g_check, &g_streams};
-  for (int i = 0; i < 4; ++i) { Py_XDECREF(*to[i]); *to[i] = Py_NewRef(o[i]); }
+  unsigned long long f[4];
+  PyObject* o[5];
+  if (!PyArg_ParseTuple(args, "KKKKOOOOO", &f[0], &f[1], &f[2], &f[3], &o[0], &o[1], &o[2], &o[3], &o[4])) return nullptr;
+  g_decode = (decode_fn)(uintptr_t)f[0];
+  g_prefill = (prefill_fn)(uintptr_t)f[1];
+  g_reset = (reset_fn)(uintptr_t)f[2];
+  g_view = (view_fn)(uintptr_t)f[3];
+  PyObject** to[5] = {&g_ptr, &g_stream, &g_check, &g_streams, &g_make_view};
+  for (int i = 0; i < 5; ++i) { Py_XDECREF(*to[i]); *to[i] = Py_NewRef(o[i]); }
   Py_RETURN_NONE;
 }
 
@@ -180,6 +229,8 @@ PyMethodDef methods[] = {
     {"setup", setup, METH_VARARGS, nullptr},
     {"delta_attn_decode_step", (PyCFunction)(void (*)(void))decode_step, METH_FASTCALL | METH_KEYWORDS, nullptr},
     {"delta_attn_prefill", (PyCFunction)(void (*)(void))prefill, METH_FASTCALL | METH_KEYWORDS, nullptr},
+    {"delta_state_reset", (PyCFunction)(void (*)(void))reset, METH_FASTCALL | METH_KEYWORDS, nullptr},
+    {"delta_state_view", (PyCFunction)(void (*)(void))view, METH_FASTCALL | METH_KEYWORDS, nullptr},
     {nullptr, nullptr, 0, nullptr}};
 PyModuleDef module = {PyModuleDef_HEAD_INIT, "_calls", nullptr, -1, methods, nullptr, nullptr, nullptr, nullptr};
 
@@ -190,5 +241,9 @@ PyMODINIT_FUNC PyInit__calls(void) {
   s_raw = PyUnicode_InternFromString("raw");
   s_decode = PyUnicode_InternFromString("delta_attn_decode_step");
   s_prefill = PyUnicode_InternFromString("delta_attn_prefill");
+  s_reset = PyUnicode_InternFromString("delta_state_reset");
+  s_view = PyUnicode_InternFromString("delta_state_view");
+  s_views = PyUnicode_InternFromString("views");
+  s_detach = PyUnicode_InternFromString("detach");
   return PyModule_Create(&module);
 }
