@@ -246,7 +246,8 @@ hybrid_attn_tcq_kernel(const __grid_constant__ TqMapList<N> maps, const __grid_c
   const uint32_t bar0 = base + OFF_BAR;
 #define BAR(i) (bar0 + 8u * (uint32_t)(i))
 
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  // (the warp index by shuffle: known to be the same in every lane)
+  const int tid = threadIdx.x, lane = tid & 31, warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
   // Heaviest query tiles of every head first.  PAIR (the layout holds two query tiles): a
   // one-dimensional grid; its first BH * n_one CTAs take the n_one heaviest query tiles of every
   // head in the one-head form (key tiles dealt to the two softmax groups, merge at the end), the
@@ -337,7 +338,7 @@ hybrid_attn_tcq_kernel(const __grid_constant__ TqMapList<N> maps, const __grid_c
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  const uint32_t tmem = sMisc[0];
+  const uint32_t tmem = __shfl_sync(0xffffffffu, sMisc[0], 0);
 
   // Keys that some row of this query tile scores exactly: ex_lo <= j <= ex_hi (empty if W = 0).
   // Block window: the window blocks that rows i0..i1 fall into; sliding: i0-W+1 .. i1.
@@ -402,16 +403,18 @@ hybrid_attn_tcq_kernel(const __grid_constant__ TqMapList<N> maps, const __grid_c
     __syncwarp();
   } else if (warp == WARP_QK) {
     // =========================== tensor-core issue: scores (d = 128: and P.V) ================
-    if (lane == 0) {
+    {
+      const uint32_t lead = lane == 0;
+      auto poll = [&](uint32_t bar, uint32_t parity, volatile uint32_t* flag) { mbar_poll(bar, parity, flag); __syncwarp(); };
       const uint32_t IDESC_QK = make_idesc(BN, 0);
       const uint32_t IDESC_PV = make_idesc(D, 1);
       // S = A . B^T into the score buffer of group X
       auto scores = [&](uint32_t X, uint32_t a, uint32_t bq) {
 #pragma unroll
         for (int ks = 0; ks < D / 16; ++ks)
-          tc_mma(tmem + TMEM_S + 128u * X, make_desc(a + (ks >> 2) * SZ_BLK + (ks & 3) * 32, 16, 1024),
+          tc_mma_if(lead, tmem + TMEM_S + 128u * X, make_desc(a + (ks >> 2) * SZ_BLK + (ks & 3) * 32, 16, 1024),
                  make_desc(bq + (ks >> 2) * SZ_BLK + (ks & 3) * 32, 16, 1024), IDESC_QK, ks > 0 ? 1u : 0u);
-        tc_commit(BAR(BAR_SFULL0 + X));
+        tc_commit_if(lead, BAR(BAR_SFULL0 + X));
       };
       const uint32_t IDESC_QK64 = make_idesc(64, 0);
       int n_kx0 = 0, n_kx = 0, n_sx0 = 0, n_sx1 = 0;   // mixed tiles whose first / last products are issued
@@ -428,11 +431,11 @@ hybrid_attn_tcq_kernel(const __grid_constant__ TqMapList<N> maps, const __grid_c
         for (int w = 0; w < 2; ++w)
 #pragma unroll
           for (int ks = 0; ks < D / 16; ++ks)
-            tc_mma(tmem + TMEM_S + 128u * X + 64u * w,
+            tc_mma_if(lead, tmem + TMEM_S + 128u * X + 64u * w,
                    make_desc((w ? qx : qt_) + (ks >> 2) * SZ_BLK + (ks & 3) * 32, 16, 1024),
                    make_desc((w ? kx : ring) + 8192u * hf + (ks >> 2) * SZ_BLK + (ks & 3) * 32, 16, 1024), IDESC_QK64,
                    ks > 0 ? 1u : 0u);
-        tc_commit(BAR(BAR_SFULL0 + X));
+        tc_commit_if(lead, BAR(BAR_SFULL0 + X));
       };
       // first scores of unit u, for group u & 1: telescoped, or exact where the whole tile
       // lies inside the window
@@ -440,7 +443,7 @@ hybrid_attn_tcq_kernel(const __grid_constant__ TqMapList<N> maps, const __grid_c
         const int t = tile_of(u);
         const uint32_t X = (uint32_t)u & 1u;
         const uint32_t qsel = pr ? X * SZ_TILE : 0u;         // the group's own query tiles
-        mbar_poll(BAR(BAR_KFULL0 + (uint32_t)t % NKS), (t / NKS) & 1, abort_flag);
+        poll(BAR(BAR_KFULL0 + (uint32_t)t % NKS), (t / NKS) & 1, abort_flag);
         tc_fence_after();
         // query deltas: Q for an exact tile, Q_hat otherwise, against the keys; key deltas: Q
         // against what the loader put into the stage (original keys for an exact tile)
@@ -458,16 +461,16 @@ hybrid_attn_tcq_kernel(const __grid_constant__ TqMapList<N> maps, const __grid_c
                                            : (in1 ? OFF_QM + 2 * qsel + SZ_TILE : OFF_QH + qsel));
 #pragma unroll
             for (int ks = 0; ks < D / 16; ++ks)
-              tc_mma(tmem + TMEM_S + 128u * X + 64u * hf, make_desc(a + (ks >> 2) * SZ_BLK + (ks & 3) * 32, 16, 1024),
+              tc_mma_if(lead, tmem + TMEM_S + 128u * X + 64u * hf, make_desc(a + (ks >> 2) * SZ_BLK + (ks & 3) * 32, 16, 1024),
                      make_desc(ring + 8192u * hf + (ks >> 2) * SZ_BLK + (ks & 3) * 32, 16, 1024), IDESC_QK64,
                      ks > 0 ? 1u : 0u);
           }
-          tc_commit(BAR(BAR_SFULL0 + X));
+          tc_commit_if(lead, BAR(BAR_SFULL0 + X));
           return;
         }
         if (MIXED && !ALIAS && cls == 1) {
           // (head pairs: the same tile of keys for both heads)
-          if (KEY) mbar_poll(BAR(BAR_KXFULL0 + (uint32_t)n_kx0 % NKX), (n_kx0 / (int)NKX) & 1, abort_flag);
+          if (KEY) poll(BAR(BAR_KXFULL0 + (uint32_t)n_kx0 % NKX), (n_kx0 / (int)NKX) & 1, abort_flag);
           mixed_half_scores(u, 0, n_kx0);
           if (!pr || X == 1u) ++n_kx0;
           return;
@@ -475,8 +478,8 @@ hybrid_attn_tcq_kernel(const __grid_constant__ TqMapList<N> maps, const __grid_c
         const bool q_exact = KEY || cls == 2;
         scores(X, base + (q_exact ? OFF_Q : OFF_QH) + qsel, ring);
       };
-      mbar_poll(BAR(BAR_Q), 0, abort_flag);
-      if (!KEY) mbar_poll(BAR(BAR_QH), 0, abort_flag);   // the softmax warps have built Q_hat
+      poll(BAR(BAR_Q), 0, abort_flag);
+      if (!KEY) poll(BAR(BAR_QH), 0, abort_flag);   // the softmax warps have built Q_hat
       tc_fence_after();
       first_scores(0);
       if (U > 1) first_scores(1);
@@ -487,51 +490,51 @@ hybrid_attn_tcq_kernel(const __grid_constant__ TqMapList<N> maps, const __grid_c
           int& n_sx = X ? n_sx1 : n_sx0;
           if (!ALIAS) {
             // the second half's products once the group has read the first half's
-            mbar_poll(BAR(BAR_SXREQ0 + X), n_sx & 1, abort_flag);
+            poll(BAR(BAR_SXREQ0 + X), n_sx & 1, abort_flag);
             ++n_sx;
             mixed_half_scores(u, 1, n_kx);
           } else {
             // d = 128 (the probabilities lie over the scores): Q.K^T over each half of 64 keys once the
             // group has that half's telescoped scores in registers
-            if (KEY) mbar_poll(BAR(BAR_KXFULL0), n_kx & 1, abort_flag);
+            if (KEY) poll(BAR(BAR_KXFULL0), n_kx & 1, abort_flag);
             const uint32_t kx = KEY ? base + OFF_QH : base + OFF_K + ((uint32_t)t % NKS) * SZ_TILE;
 #pragma unroll
             for (int hf = 0; hf < 2; ++hf) {
-              mbar_poll(BAR(BAR_SXREQ0 + X), n_sx & 1, abort_flag);
+              poll(BAR(BAR_SXREQ0 + X), n_sx & 1, abort_flag);
               ++n_sx;
               tc_fence_after();
 #pragma unroll
               for (int ks = 0; ks < D / 16; ++ks)
-                tc_mma(tmem + TMEM_S + 128u * X + 64u * hf,
+                tc_mma_if(lead, tmem + TMEM_S + 128u * X + 64u * hf,
                        make_desc(base + OFF_Q + (ks >> 2) * SZ_BLK + (ks & 3) * 32, 16, 1024),
                        make_desc(kx + 8192u * hf + (ks >> 2) * SZ_BLK + (ks & 3) * 32, 16, 1024), IDESC_QK64,
                        ks > 0 ? 1u : 0u);
-              tc_commit(BAR(BAR_SFULL0 + X));
+              tc_commit_if(lead, BAR(BAR_SFULL0 + X));
             }
           }
           if (!pr || X == 1u) {
-            if (KEY) tc_commit(BAR(BAR_KXFREE0 + (uint32_t)n_kx % NKX));
+            if (KEY) tc_commit_if(lead, BAR(BAR_KXFREE0 + (uint32_t)n_kx % NKX));
             ++n_kx;
           }
         }
         // every product that reads this key stage is issued (head pairs: after the second head's)
-        if (!pr || X == 1u) tc_commit(BAR(BAR_KFREE0 + (uint32_t)t % NKS));
+        if (!pr || X == 1u) tc_commit_if(lead, BAR(BAR_KFREE0 + (uint32_t)t % NKS));
         if (ALIAS) {
           // P.V of this tile into the group's output tile, then the group's next scores at once
-          mbar_poll(BAR(BAR_VFULL0 + (uint32_t)t % NVS), (t / NVS) & 1, abort_flag);
-          mbar_poll(BAR(BAR_PRDY0 + X), (u >> 1) & 1, abort_flag);
+          poll(BAR(BAR_VFULL0 + (uint32_t)t % NVS), (t / NVS) & 1, abort_flag);
+          poll(BAR(BAR_PRDY0 + X), (u >> 1) & 1, abort_flag);
           tc_fence_after();
           const uint32_t vb = base + OFF_V + ((uint32_t)t % NVS) * SZ_TILE;
 #pragma unroll
           for (int ks = 0; ks < BN / 16; ++ks)
-            tc_mma_ts(tmem + TMEM_O + (uint32_t)D * X, tmem + TMEM_S + 128u * X + 8u * ks,
+            tc_mma_ts_if(lead, tmem + TMEM_O + (uint32_t)D * X, tmem + TMEM_S + 128u * X + 8u * ks,
                       make_desc(vb + ks * 2048, SZ_BLK, 1024), IDESC_PV, (u >= 2 || ks > 0) ? 1u : 0u);
-          tc_commit(BAR(BAR_VFREE0 + (uint32_t)t % NVS));
-          if (u + 2 >= U) tc_commit(BAR(BAR_ODONE0 + X));   // the group's last product
+          tc_commit_if(lead, BAR(BAR_VFREE0 + (uint32_t)t % NVS));
+          if (u + 2 >= U) tc_commit_if(lead, BAR(BAR_ODONE0 + X));   // the group's last product
           else first_scores(u + 2);
         } else if (u + 2 < U) {
           // the group's next scores as soon as it has read this unit's
-          mbar_poll(BAR(BAR_SCONS0 + X), (u >> 1) & 1, abort_flag);
+          poll(BAR(BAR_SCONS0 + X), (u >> 1) & 1, abort_flag);
           first_scores(u + 2);
         }
       }
@@ -539,22 +542,24 @@ hybrid_attn_tcq_kernel(const __grid_constant__ TqMapList<N> maps, const __grid_c
     __syncwarp();
   } else if (warp == WARP_PV) {
     // =========================== tensor-core issue: P.V (d = 64) ============================
-    if (!ALIAS && lane == 0) {
+    if (!ALIAS) {
+      const uint32_t lead = lane == 0;
+      auto poll = [&](uint32_t bar, uint32_t parity, volatile uint32_t* flag) { mbar_poll(bar, parity, flag); __syncwarp(); };
       const uint32_t IDESC_PV = make_idesc(D, 1);
       for (int u = 0; u < U; ++u) {
         const int t = tile_of(u);
         const uint32_t X = (uint32_t)u & 1u;
-        mbar_poll(BAR(BAR_VFULL0 + (uint32_t)t % NVS), (t / NVS) & 1, abort_flag);
-        mbar_poll(BAR(BAR_PRDY0 + X), (u >> 1) & 1, abort_flag);
+        poll(BAR(BAR_VFULL0 + (uint32_t)t % NVS), (t / NVS) & 1, abort_flag);
+        poll(BAR(BAR_PRDY0 + X), (u >> 1) & 1, abort_flag);
         tc_fence_after();
         const uint32_t vb = base + OFF_V + ((uint32_t)t % NVS) * SZ_TILE;
 #pragma unroll
         for (int ks = 0; ks < BN / 16; ++ks)
-          tc_mma_ts(tmem + TMEM_O + (uint32_t)D * X, tmem + TMEM_P64 + 64u * X + 8u * ks,
+          tc_mma_ts_if(lead, tmem + TMEM_O + (uint32_t)D * X, tmem + TMEM_P64 + 64u * X + 8u * ks,
                     make_desc(vb + ks * 2048, SZ_BLK, 1024), IDESC_PV, (u >= 2 || ks > 0) ? 1u : 0u);
-        if (!pr || X == 1u) tc_commit(BAR(BAR_VFREE0 + (uint32_t)t % NVS));
-        if (u + 2 >= U) tc_commit(BAR(BAR_ODONE0 + X));   // the group's last product
-        else tc_commit(BAR(BAR_PFREE0 + X));              // the group may write its next probabilities
+        if (!pr || X == 1u) tc_commit_if(lead, BAR(BAR_VFREE0 + (uint32_t)t % NVS));
+        if (u + 2 >= U) tc_commit_if(lead, BAR(BAR_ODONE0 + X));   // the group's last product
+        else tc_commit_if(lead, BAR(BAR_PFREE0 + X));              // the group may write its next probabilities
       }
     }
     __syncwarp();
