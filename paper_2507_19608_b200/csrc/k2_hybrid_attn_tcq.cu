@@ -410,10 +410,11 @@ hybrid_attn_tcq_kernel(const __grid_constant__ TqMapList<N> maps, const __grid_c
       const uint32_t IDESC_PV = make_idesc(D, 1);
       // S = A . B^T into the score buffer of group X
       auto scores = [&](uint32_t X, uint32_t a, uint32_t bq) {
+        const uint64_t da = make_desc(a, 16, 1024), db = make_desc(bq, 16, 1024);
 #pragma unroll
         for (int ks = 0; ks < D / 16; ++ks)
-          tc_mma_if(lead, tmem + TMEM_S + 128u * X, make_desc(a + (ks >> 2) * SZ_BLK + (ks & 3) * 32, 16, 1024),
-                 make_desc(bq + (ks >> 2) * SZ_BLK + (ks & 3) * 32, 16, 1024), IDESC_QK, ks > 0 ? 1u : 0u);
+          tc_mma_if(lead, tmem + TMEM_S + 128u * X, desc_at(da, (ks >> 2) * SZ_BLK + (ks & 3) * 32),
+                    desc_at(db, (ks >> 2) * SZ_BLK + (ks & 3) * 32), IDESC_QK, ks > 0 ? 1u : 0u);
         tc_commit_if(lead, BAR(BAR_SFULL0 + X));
       };
       const uint32_t IDESC_QK64 = make_idesc(64, 0);
@@ -524,11 +525,11 @@ hybrid_attn_tcq_kernel(const __grid_constant__ TqMapList<N> maps, const __grid_c
           poll(BAR(BAR_VFULL0 + (uint32_t)t % NVS), (t / NVS) & 1, abort_flag);
           poll(BAR(BAR_PRDY0 + X), (u >> 1) & 1, abort_flag);
           tc_fence_after();
-          const uint32_t vb = base + OFF_V + ((uint32_t)t % NVS) * SZ_TILE;
+          const uint64_t dv = make_desc(base + OFF_V + ((uint32_t)t % NVS) * SZ_TILE, SZ_BLK, 1024);
 #pragma unroll
           for (int ks = 0; ks < BN / 16; ++ks)
             tc_mma_ts_if(lead, tmem + TMEM_O + (uint32_t)D * X, tmem + TMEM_S + 128u * X + 8u * ks,
-                      make_desc(vb + ks * 2048, SZ_BLK, 1024), IDESC_PV, (u >= 2 || ks > 0) ? 1u : 0u);
+                         desc_at(dv, ks * 2048), IDESC_PV, (u >= 2 || ks > 0) ? 1u : 0u);
           tc_commit_if(lead, BAR(BAR_VFREE0 + (uint32_t)t % NVS));
           if (u + 2 >= U) tc_commit_if(lead, BAR(BAR_ODONE0 + X));   // the group's last product
           else first_scores(u + 2);
@@ -552,11 +553,11 @@ hybrid_attn_tcq_kernel(const __grid_constant__ TqMapList<N> maps, const __grid_c
         poll(BAR(BAR_VFULL0 + (uint32_t)t % NVS), (t / NVS) & 1, abort_flag);
         poll(BAR(BAR_PRDY0 + X), (u >> 1) & 1, abort_flag);
         tc_fence_after();
-        const uint32_t vb = base + OFF_V + ((uint32_t)t % NVS) * SZ_TILE;
+        const uint64_t dv = make_desc(base + OFF_V + ((uint32_t)t % NVS) * SZ_TILE, SZ_BLK, 1024);
 #pragma unroll
         for (int ks = 0; ks < BN / 16; ++ks)
           tc_mma_ts_if(lead, tmem + TMEM_O + (uint32_t)D * X, tmem + TMEM_P64 + 64u * X + 8u * ks,
-                    make_desc(vb + ks * 2048, SZ_BLK, 1024), IDESC_PV, (u >= 2 || ks > 0) ? 1u : 0u);
+                       desc_at(dv, ks * 2048), IDESC_PV, (u >= 2 || ks > 0) ? 1u : 0u);
         if (!pr || X == 1u) tc_commit_if(lead, BAR(BAR_VFREE0 + (uint32_t)t % NVS));
         if (u + 2 >= U) tc_commit_if(lead, BAR(BAR_ODONE0 + X));   // the group's last product
         else tc_commit_if(lead, BAR(BAR_PFREE0 + X));              // the group may write its next probabilities
