@@ -652,12 +652,12 @@ delta_status_t delta_attn_prefill_host(delta_state_t* st, const void* q_host, co
   if (e != cudaSuccess) return cuda_fail(e);
   Transfer* const x = tg.t;
   const cudaStream_t s_up = x ? x->up : cs, s_down = x ? x->down : cs;
-  auto fail = [&](cudaError_t err) {      // nothing of this call may still touch the buffers
+  auto settle = [&] {                     // nothing of a failed call may still touch the buffers
     cudaStreamSynchronize(s_up);
     cudaStreamSynchronize(s_down);
     cudaStreamSynchronize(cs);
-    return cuda_fail(err);
   };
+  auto fail = [&](cudaError_t err) { settle(); return cuda_fail(err); };
 #define DO(call) do { if ((e = (call)) != cudaSuccess) return fail(e); } while (0)
   // host K/V hold T rows per head; the device copy uses the cache layout with T_max rows
   auto up_rows = [&](char* dst, const char* src, int u0, int n) -> cudaError_t {
@@ -690,7 +690,7 @@ delta_status_t delta_attn_prefill_host(delta_state_t* st, const void* q_host, co
     if (x) DO(cudaStreamWaitEvent(cs, x->arrived[i], 0));
     s = prefill_launch(st, sh, ws, dq_ + qo, dk + kv, dv + kv, dout + qo, seqs, theta, cs, st->profiling,
                        late ? PREFILL_FRONT : PREFILL_ALL);
-    if (s != DELTA_OK) { fail(cudaSuccess); return s; }
+    if (s != DELTA_OK) { settle(); return s; }      // (prefill_launch has recorded the error's text)
     if (x) {
       DO(cudaEventRecord(x->computed[i], cs));
       DO(cudaStreamWaitEvent(s_down, x->computed[i], 0));
@@ -700,7 +700,7 @@ delta_status_t delta_attn_prefill_host(delta_state_t* st, const void* q_host, co
   // delta arrays, counters and the hand-off row of all chunks, while the last output goes down
   if (late) {
     s = prefill_launch(st, st->shape, st->ws, dq_, dk, dv, dout, seqs, theta, cs, false, PREFILL_FINISH);
-    if (s != DELTA_OK) { fail(cudaSuccess); return s; }
+    if (s != DELTA_OK) { settle(); return s; }      // (prefill_launch has recorded the error's text)
   }
   if (x) DO(cudaStreamSynchronize(s_down));
   DO(cudaStreamSynchronize(cs));

@@ -1,0 +1,65 @@
+"""The host side of the library (csrc/api.cu) against fakes of the CUDA runtime and of the kernel launchers
+(host_runtime_fake.cpp): what a call launches, keeps and reports, without a GPU."""
+import ctypes as C
+import os
+import subprocess
+
+import pytest
+
+from paper_2507_19608_b200 import _build
+from paper_2507_19608_b200 import binding as B
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+CUDA_INCLUDE = os.path.join(os.path.dirname(os.path.dirname(os.path.realpath(_build._nvcc()))), "include")
+LAUNCH_FAILURE = 719
+
+
+@pytest.fixture(scope="module")
+def fake(tmp_path_factory):
+    so = str(tmp_path_factory.mktemp("fake") / "fake.so")
+    subprocess.run(["g++", "-std=c++17", "-O1", "-shared", "-fPIC", "-fvisibility=hidden", "-Wl,-Bsymbolic", "-DNVTX_NO_IMPL",
+                    "-DDELTA_BUILDING_LIB", "-I", CUDA_INCLUDE, "-o", so, "-x", "c++", os.path.join(_build.CSRC, "api.cu"),
+                    os.path.join(HERE, "host_runtime_fake.cpp")], check=True)
+    lib = C.CDLL(so)
+    for name in ("delta_last_cuda_error", "fake_log"):
+        getattr(lib, name).restype = C.c_char_p
+    return lib
+
+
+class Host:
+    """A state over the fake runtime, and host buffers nothing reads."""
+
+    def __init__(self, lib, H=32, H_kv=8, T=1024, source=B.DELTA_SRC_QUERY, dtype="bf16", Bn=1):
+        self.lib, self.T, self.cfg = lib, T, B.make_config(Bn, H, H_kv, 64, T + 64, dtype, source=source)
+        lib.fake_clear()
+        lib.fake_device(0)
+        n = C.c_size_t()
+        assert lib.delta_state_workspace_bytes(C.byref(self.cfg), C.byref(n)) == 0
+        self.st = C.c_void_p()
+        assert lib.delta_state_init(C.byref(self.cfg), C.c_void_p(1 << 40), n, None, C.byref(self.st)) == 0
+        self.buf = C.c_void_p(1 << 44)
+        self.call_log()
+
+    def prefill_host(self):
+        n = C.c_size_t()
+        assert self.lib.delta_prefill_staging_bytes(C.byref(self.cfg), self.T, C.byref(n)) == 0
+        return self.lib.delta_attn_prefill_host(self.st, self.buf, self.buf, self.buf, self.buf, self.buf, n, self.T,
+                                                C.c_float(0.3), 64, None)
+
+    def reset(self):
+        assert self.lib.delta_state_reset(self.st, None) == 0
+
+    def call_log(self):
+        log = self.lib.fake_log().decode().splitlines()
+        self.lib.fake_clear()
+        return log
+
+
+@pytest.mark.parametrize("name", ["chain", "attn", "finish", "memcpy", "synchronize"])
+def test_host_prefill_reports_the_error_of_the_failed_call(fake, name):
+    h = Host(fake)
+    fake.fake_fail(name.encode(), LAUNCH_FAILURE)
+    assert h.prefill_host() == B.DELTA_ERR_CUDA
+    assert fake.delta_last_cuda_error() == b"fakeError: code 719"
+    assert h.call_log()[-1] == "synchronize"        # nothing of the call is left in flight
+    assert fake.delta_state_position(h.st) == 0
