@@ -6,6 +6,8 @@ import os
 import shutil
 import subprocess
 import sysconfig
+import tempfile
+from concurrent.futures import ThreadPoolExecutor
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
@@ -16,8 +18,8 @@ CALLS_SOURCE = "py_calls.cpp"
 SOURCES = ["api.cu", "k1_delta_construct.cu", "k2_hybrid_attn_generic.cu", "k2_hybrid_attn_tc.cu", "k2_hybrid_attn_tcq.cu",
            "k3_decode_step.cu", "k3_decode_step_mma.cu", "k3_decode_step_f32.cu", "k3_decode_step_key.cu", "k1_pack_keys.cu", "decode_noalloc.cu"]
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
-              "--shared", "-Xcompiler", "-fPIC", "-Xcompiler", "-fvisibility=hidden",
-              "-DDELTA_BUILDING_LIB", "-lcuda"]
+              "-Xcompiler", "-fPIC", "-Xcompiler", "-fvisibility=hidden", "-DDELTA_BUILDING_LIB"]
+LINK_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "--shared", "-lcuda"]
 
 
 def _nvcc() -> str:
@@ -57,17 +59,23 @@ def build(force: bool = False, verbose: bool = False, debug_bounds: bool = False
     lib = LIB_DEBUG if debug_bounds else LIB
     if not force and not _stale(lib):
         return lib
-    flags = NVCC_FLAGS + (["-DDELTA_DEBUG_BOUNDS"] if debug_bounds else [])
-    cmd = [_nvcc(), *flags, "-o", lib + ".tmp", *[os.path.join(CSRC, s) for s in SOURCES]]
-    if verbose:
-        cmd.insert(1, "-Xptxas")
-        cmd.insert(2, "-v")
-    r = subprocess.run(cmd, capture_output=True, text=True)
-    if r.returncode != 0:
-        raise RuntimeError("nvcc failed:\n" + r.stdout + r.stderr)
+    flags = NVCC_FLAGS + (["-DDELTA_DEBUG_BOUNDS"] if debug_bounds else []) + (["-Xptxas", "-v"] if verbose else [])
+    nvcc = _nvcc()
+
+    def run(cmd: list) -> str:
+        r = subprocess.run(cmd, capture_output=True, text=True)
+        if r.returncode != 0:
+            raise RuntimeError("nvcc failed:\n" + r.stdout + r.stderr)
+        return r.stderr
+
+    # the files side by side: they share no device symbols, and one nvcc call would compile them in turn
+    with tempfile.TemporaryDirectory() as tmp, ThreadPoolExecutor(os.cpu_count()) as pool:
+        objs = [os.path.join(tmp, s + ".o") for s in SOURCES]
+        logs = list(pool.map(run, [[nvcc, *flags, "-c", os.path.join(CSRC, s), "-o", o] for s, o in zip(SOURCES, objs)]))
+        run([nvcc, *LINK_FLAGS, "-o", lib + ".tmp", *objs])
     os.replace(lib + ".tmp", lib)
     if verbose:
-        print(r.stderr)
+        print("".join(logs))
     return lib
 
 
