@@ -13,7 +13,9 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libdelta_attn.so")
 LIB_DEBUG = os.path.join(HERE, "libdelta_attn_dbg.so")      # the same sources with -DDELTA_DEBUG_BOUNDS
-CALLS = os.path.join(HERE, "_calls.so")                      # CPython entry points over the library
+# CPython entry points over the library: compiled against this interpreter's headers, so its file carries the
+# interpreter's ABI tag and another version of Python builds its own
+CALLS = os.path.join(HERE, "_calls" + sysconfig.get_config_var("EXT_SUFFIX"))
 CALLS_SOURCE = "py_calls.cpp"
 SOURCES = ["api.cu", "k1_delta_construct.cu", "k2_hybrid_attn_generic.cu", "k2_hybrid_attn_tc.cu", "k2_hybrid_attn_tcq.cu",
            "k3_decode_step.cu", "k3_decode_step_mma.cu", "k3_decode_step_f32.cu", "k3_decode_step_key.cu", "k1_pack_keys.cu", "decode_noalloc.cu"]

@@ -3,6 +3,7 @@ header declares, rejects bad arguments before touching the device, and Eq. 5 mat
 import ctypes as C
 import os
 import re
+import sysconfig
 
 import pytest
 
@@ -29,6 +30,14 @@ def test_library_exports_every_declared_symbol():
     for n in names:
         assert hasattr(raw, n), f"{n} declared in include/ but not exported"
     assert set(names) == set(B.EXPORTED)
+
+
+def test_native_calls_are_built_for_this_interpreter():
+    """The CPython entry points do not use the limited API: a module that another version of Python built in the
+    same tree must not be loaded here."""
+    from paper_2507_19608_b200 import _build
+    tag = sysconfig.get_config_var("EXT_SUFFIX")
+    assert tag != ".so" and B._calls.__file__ == _build.CALLS and _build.CALLS.endswith(tag)
 
 
 def test_status_strings():
