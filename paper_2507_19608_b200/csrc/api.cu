@@ -616,6 +616,7 @@ delta_status_t delta_attn_prefill_host(delta_state_t* st, const void* q_host, co
                                        const void* v_host, void* out_host, void* staging,
                                        size_t staging_bytes, int32_t T, float theta,
                                        int32_t window, void* stream) {
+  NvtxRange range("delta_attn_prefill_host");
   if (!st || !q_host || !k_host || !v_host || !out_host || !staging) return DELTA_ERR_INVALID_ARG;
   const delta_config_t& c = st->cfg;
   size_t need = 0;

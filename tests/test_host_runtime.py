@@ -49,10 +49,10 @@ class Host:
     def reset(self):
         assert self.lib.delta_state_reset(self.st, None) == 0
 
-    def call_log(self):
+    def call_log(self, nvtx=False):
         log = self.lib.fake_log().decode().splitlines()
         self.lib.fake_clear()
-        return log
+        return [x for x in log if nvtx or not x.startswith(("push", "pop"))]
 
 
 @pytest.mark.parametrize("name", ["chain", "attn", "finish", "memcpy", "synchronize"])
@@ -63,3 +63,11 @@ def test_host_prefill_reports_the_error_of_the_failed_call(fake, name):
     assert fake.delta_last_cuda_error() == b"fakeError: code 719"
     assert h.call_log()[-1] == "synchronize"        # nothing of the call is left in flight
     assert fake.delta_state_position(h.st) == 0
+
+
+def test_host_prefill_opens_an_nvtx_range(fake):
+    h = Host(fake)
+    assert h.prefill_host() == 0
+    log = h.call_log(nvtx=True)
+    assert log[0] == "push delta_attn_prefill_host" and log[-1] == "pop"
+    assert sum(x.startswith("push") for x in log) == sum(x == "pop" for x in log)
