@@ -449,14 +449,15 @@ static void prefilled(delta_state* st, int T, int window) {
   st->len_sum[0] += B * (double)T;
 }
 
-// Streams and events of a host-buffer prefill.  A call takes a set for its duration (it synchronises
-// before it returns) and gives it back to a pool per device; more than kTransferKeep sets at once
-// (concurrent host threads) are made and destroyed by their calls.
+// Streams and events of a host-buffer prefill.  A call takes a set of its device for its duration (it
+// synchronises before it returns) and gives it back to the list of idle sets, which keeps up to
+// kTransferKeep of every device; what more host threads use at once is made and destroyed by their calls.
 namespace {
 constexpr int kTransferChunks = 4;
-constexpr size_t kTransferKeep = 4;
+constexpr int kTransferKeep = 4;
 struct Transfer {
   int dev = 0;
+  Transfer* next = nullptr;               // in the list of idle sets
   cudaStream_t up = nullptr, down = nullptr;
   cudaEvent_t start = nullptr, arrived[kTransferChunks] = {}, computed[kTransferChunks] = {};
   cudaError_t create() {
@@ -483,7 +484,7 @@ struct Transfer {
   }
 };
 std::mutex g_transfer_mu;
-std::vector<Transfer*> g_transfers;      // idle sets
+Transfer* g_transfers = nullptr;         // idle sets (linked through the sets: giving one back allocates nothing)
 struct TransferGuard {
   Transfer* t = nullptr;
   cudaError_t open() {
@@ -492,8 +493,8 @@ struct TransferGuard {
     if (e != cudaSuccess) return e;
     {
       std::lock_guard<std::mutex> lock(g_transfer_mu);
-      for (size_t i = 0; i < g_transfers.size() && !t; ++i)
-        if (g_transfers[i]->dev == dev) { t = g_transfers[i]; g_transfers.erase(g_transfers.begin() + (long)i); }
+      for (Transfer** at = &g_transfers; *at; at = &(*at)->next)
+        if ((*at)->dev == dev) { t = *at; *at = t->next; break; }
     }
     if (t) return cudaSuccess;
     t = new (std::nothrow) Transfer();
@@ -505,7 +506,9 @@ struct TransferGuard {
     if (!t) return;
     {
       std::lock_guard<std::mutex> lock(g_transfer_mu);
-      if (g_transfers.size() < kTransferKeep) { g_transfers.push_back(t); return; }
+      int idle = 0;                       // of this device
+      for (const Transfer* x = g_transfers; x; x = x->next) idle += x->dev == t->dev;
+      if (idle < kTransferKeep) { t->next = g_transfers; g_transfers = t; return; }
     }
     t->destroy();
     delete t;

@@ -71,3 +71,16 @@ def test_host_prefill_opens_an_nvtx_range(fake):
     log = h.call_log(nvtx=True)
     assert log[0] == "push delta_attn_prefill_host" and log[-1] == "pop"
     assert sum(x.startswith("push") for x in log) == sum(x == "pop" for x in log)
+
+
+def test_streams_of_the_host_prefill_are_kept_per_device(fake):
+    """Six devices in turn, twice: the second round makes and destroys nothing."""
+    h = Host(fake)
+    for turn in range(2):
+        for dev in range(10, 16):
+            fake.fake_device(dev)
+            h.reset()
+            assert h.prefill_host() == 0
+            log = h.call_log()
+            assert log.count(f"stream_create dev={dev}") == (2 if turn == 0 else 0)
+            assert not any("destroy" in x for x in log)
