@@ -164,7 +164,8 @@ DELTA_API delta_status_t delta_attn_prefill_varlen(delta_state_t* st, const void
 /* delta_attn_prefill_host -- the same call for HOST buffers (q, k, v, out are host pointers
  * with the shapes above; k and v hold T rows per head, i.e. [B, H_kv, T, d]).  `staging` is
  * a DEVICE buffer of at least delta_prefill_staging_bytes(cfg, T) bytes that receives the
- * copies.  Copies in, runs the prefill, copies `out` back and synchronises the stream. */
+ * copies.  Copies in, runs the prefill, copies `out` back and synchronises the stream (so a
+ * stream under capture is refused: DELTA_ERR_CUDA, nothing enqueued). */
 DELTA_API delta_status_t delta_prefill_staging_bytes(const delta_config_t* cfg, int32_t T, size_t* bytes);
 DELTA_API delta_status_t delta_attn_prefill_host(delta_state_t* st, const void* q_host, const void* k_host,
                                        const void* v_host, void* out_host, void* staging,

@@ -638,6 +638,12 @@ delta_status_t delta_attn_prefill_host(delta_state_t* st, const void* q_host, co
   char* dk = dout + qb;
   char* dv = dk + kb;
   cudaStream_t cs = (cudaStream_t)stream;
+  // A call that synchronises cannot be captured; refused before a stream of the pool joins the capture (it
+  // would go back to the pool in it, and the next call that takes it would fail until the capture ends).
+  cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+  cudaError_t e = cudaStreamIsCapturing(cs, &capture);
+  if (e == cudaSuccess && capture != cudaStreamCaptureStatusNone) e = cudaErrorStreamCaptureUnsupported;
+  if (e != cudaSuccess) return cuda_fail(e);
   // The call is bound by PCIe (6.3 MB up and 4.2 MB down around 35 us of kernels at the Llama layer; 51 GB/s
   // one way, 80 both ways together): keys and values come up first, then the queries in chunks of KV
   // heads, and while a chunk is computed on the caller's stream the next one comes up on a stream of
@@ -652,7 +658,7 @@ delta_status_t delta_attn_prefill_host(delta_state_t* st, const void* q_host, co
   if (chunks < 1 || st->profiling) chunks = 1;
   // (one chunk: all on the caller's stream, nothing to overlap)
   TransferGuard tg;
-  cudaError_t e = chunks > 1 ? tg.open() : cudaSuccess;
+  e = chunks > 1 ? tg.open() : cudaSuccess;
   if (e != cudaSuccess) return cuda_fail(e);
   Transfer* const x = tg.t;
   const cudaStream_t s_up = x ? x->up : cs, s_down = x ? x->down : cs;

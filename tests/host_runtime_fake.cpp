@@ -13,7 +13,7 @@ namespace {
 std::mutex g_mu;
 std::string g_log;
 std::map<std::string, int> g_fail;      // call -> error of its next run
-int g_device = 0;
+int g_device = 0, g_capturing = 0;
 size_t g_handle = 0x1000;
 
 cudaError_t call(const char* name, const std::string& args = "") {
@@ -38,6 +38,7 @@ extern "C" {
 EXPORT const char* fake_log() { return g_log.c_str(); }
 EXPORT void fake_clear() { g_log.clear(); g_fail.clear(); }
 EXPORT void fake_fail(const char* name, int error) { g_fail[name] = error; }
+EXPORT void fake_capturing(int on) { g_capturing = on; }
 EXPORT void fake_device(int dev) { g_device = dev; }
 
 const char* cudaGetErrorName(cudaError_t e) { return e == cudaSuccess ? "cudaSuccess" : "fakeError"; }
@@ -54,6 +55,10 @@ cudaError_t cudaMemcpy2DAsync(void*, size_t, const void*, size_t, size_t, size_t
 }
 cudaError_t cudaStreamCreateWithFlags(cudaStream_t* s, unsigned) { return make("stream_create", s); }
 cudaError_t cudaStreamDestroy(cudaStream_t) { return call("stream_destroy"); }
+cudaError_t cudaStreamIsCapturing(cudaStream_t, cudaStreamCaptureStatus* s) {
+  *s = g_capturing ? cudaStreamCaptureStatusActive : cudaStreamCaptureStatusNone;
+  return cudaSuccess;
+}
 cudaError_t cudaStreamSynchronize(cudaStream_t) { return call("synchronize"); }
 cudaError_t cudaStreamWaitEvent(cudaStream_t, cudaEvent_t, unsigned) { return call("wait_event"); }
 cudaError_t cudaEventCreate(cudaEvent_t* e) { return make("event_create", e); }

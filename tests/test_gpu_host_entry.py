@@ -75,3 +75,22 @@ def test_host_calls_from_several_threads():
     for t in threads:
         t.join()
     assert not errors, errors
+
+
+def test_host_call_on_a_capturing_stream_is_refused_and_leaves_the_capture_valid():
+    from paper_2507_19608_b200 import binding as B
+    T, x = 1024, torch.ones(1024, device="cuda")
+    cfg = B.make_config(1, 32, 8, 64, T, "bf16")
+    host = [torch.zeros(1, h, T, 64, dtype=torch.bfloat16).pin_memory() for h in (32, 8, 8, 32)]
+    st = B.delta_state_init(cfg)
+    staging = torch.empty(B.delta_prefill_staging_bytes(cfg, T), dtype=torch.uint8, device="cuda")
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        with pytest.raises(B.DeltaError):
+            B.delta_attn_prefill_host(st, *host, staging, T, 0.4, 64)
+        x += 1
+    g.replay()
+    B.delta_attn_prefill_host(st, *host, staging, T, 0.4, 64)
+    torch.cuda.synchronize()
+    assert bool((x == 2).all()) and B.delta_state_position(st) == T

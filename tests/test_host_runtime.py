@@ -84,3 +84,14 @@ def test_streams_of_the_host_prefill_are_kept_per_device(fake):
             log = h.call_log()
             assert log.count(f"stream_create dev={dev}") == (2 if turn == 0 else 0)
             assert not any("destroy" in x for x in log)
+
+
+def test_host_prefill_on_a_capturing_stream_touches_nothing(fake):
+    """The call synchronises, so it cannot be captured: refused before a pooled stream joins the capture."""
+    h = Host(fake)
+    fake.fake_capturing(1)
+    status = h.prefill_host()
+    fake.fake_capturing(0)
+    assert status == B.DELTA_ERR_CUDA and h.call_log() == []
+    assert fake.delta_last_cuda_error() == b"fakeError: code 900"       # cudaErrorStreamCaptureUnsupported
+    assert h.prefill_host() == 0
