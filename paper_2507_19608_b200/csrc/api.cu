@@ -47,6 +47,7 @@ struct delta_state {
   double win_sum[2], len_sum[2];
   DecodeTmapCache dec_maps[3];     // tensor maps of the key, value and reference-key caches the decode steps read
   int forced_decode_kernel = -1;   // -1: chosen per step
+  bool stepped = false;            // a decode step has been enqueued behind the prefill
   bool key_cache_packed = false;   // key deltas: decode from the compressed key-delta cache
   // optional per-kernel timing of prefill (host-side event objects)
   bool profiling = false, profiled = false;
@@ -151,6 +152,7 @@ static delta_status_t zero_state(delta_state* st, cudaStream_t stream, bool defe
   st->n = 0;
   st->n_b.assign((size_t)st->cfg.B, 0);
   st->ragged = false;
+  st->stepped = false;
   st->qhat_sel = 0;
   st->win_sum[0] = st->win_sum[1] = st->len_sum[0] = st->len_sum[1] = 0.0;
   return DELTA_OK;
@@ -758,7 +760,7 @@ delta_status_t delta_attn_decode_step(delta_state_t* st, const void* q_new, cons
     // one launch, whether the batch elements stand at one position or at different ones
     e = launch_decode_step_mma(st->shape, st->ws, q_new, k_new, v_new, k_cache, v_cache, out, st->n,
                                st->ragged ? st->n_b.data() : nullptr, theta, window, st->qhat_sel,
-                               c.source == DELTA_SRC_KEY, key_packed, st->dec_maps, cs);
+                               c.source == DELTA_SRC_KEY, key_packed, st->stepped, st->dec_maps, cs);
     if (e != cudaSuccess) return cuda_fail(e);
   } else if (c.dtype == DELTA_F32 && st->forced_decode_kernel < 0) {
     e = launch_decode_step_f32(st->shape, st->ws, q_new, k_new, v_new, k_cache, v_cache, out, st->n,
@@ -788,6 +790,7 @@ delta_status_t delta_attn_decode_step(delta_state_t* st, const void* q_new, cons
   }
   for (auto& nb : st->n_b) nb += 1;
   st->qhat_sel ^= 1;
+  st->stepped = true;
   st->n += 1;
   return DELTA_OK;
 }

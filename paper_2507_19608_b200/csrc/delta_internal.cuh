@@ -133,12 +133,13 @@ struct DecodeTmapCache {
 };
 // K3 for bf16 caches (query and key deltas; key: w.qhat_rows is the reference-key cache).  n: tokens
 // seen (the longest sequence's); n_b: null, or the tokens seen by every batch element of a ragged
-// batch; maps: the state's tensor maps of the key, value and reference-key caches.
+// batch; behind_step: the state's last kernel was a decode step, not a prefill's; maps: the state's tensor
+// maps of the key, value and reference-key caches.
 bool decode_mma_applies(const Shape& s, int dtype);
 cudaError_t launch_decode_step_mma(const Shape& s, const Workspace& w, const void* q_new, const void* k_new,
                                    const void* v_new, void* k_cache, void* v_cache, void* out, int n, const int* n_b,
-                                   float theta, int window, int qhat_sel, bool key, bool packed, DecodeTmapCache* maps,
-                                   cudaStream_t st);
+                                   float theta, int window, int qhat_sel, bool key, bool packed, bool behind_step,
+                                   DecodeTmapCache* maps, cudaStream_t st);
 // K3 for fp32 caches (query deltas), arguments as above.
 cudaError_t launch_decode_step_f32(const Shape& s, const Workspace& w, const void* q_new, const void* k_new,
                                    const void* v_new, void* k_cache, void* v_cache, void* out, int n, const int* n_b,

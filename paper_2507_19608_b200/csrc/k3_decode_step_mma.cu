@@ -59,6 +59,7 @@ struct MmaDecodeParams {
   uint32_t* ticket;
   unsigned long long* counters;
   int n, T_max, H, chunk, nsplit, W, b0;
+  int early;                              // reference keys may be fetched ahead of the wait (see there)
   float theta, scale_log2e;
   int ragged;
   int n_b[kRaggedMax];                    // ragged: tokens seen per batch element b0 ..
@@ -245,11 +246,13 @@ decode_step_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_co
     to_rank[c] = (uint32_t)(q % cs);
     to_rec[c] = (uint32_t)(q / cs * nsrc + rank * MNW + warp);
   }
-  // Reference-key rows and their encoding are the library's own: all but the row (segment) the step in
-  // front may be writing is final before this kernel can start, since that step releases it only
-  // behind its own wait, and is requested ahead of the wait.  (Key and value rows are the caller's.)
+  // Reference-key rows and their encoding are the library's own: behind another step (p.early) all but the
+  // row (segment) that step may be writing is final before this kernel can start, since a step releases
+  // the next one only behind its own wait, and is requested ahead of the wait.  Not so behind a prefill:
+  // its last kernel (the packing kernel least of all) releases nothing itself, and what it writes is
+  // certain to be seen only behind the wait.  (Key and value rows are the caller's.)
   int jg = j0 + UK * warp;
-  const bool early_k = KEY && jg < j1 && jg + UK <= min(n - 1, wl);
+  const bool early_k = KEY && p.early && jg < j1 && jg + UK <= min(n - 1, wl);
   if (early_k) fetch_k(jg);
   // the step in front (or the prefill) has written the reference, row n - 1 of the caches, the tickets
   asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -670,7 +673,8 @@ bool decode_mma_applies(const Shape& s, int dtype) { return dtype == DELTA_BF16 
 
 cudaError_t launch_decode_step_mma(const Shape& s, const Workspace& w, const void* q_new, const void* k_new,
                                    const void* v_new, void* k_cache, void* v_cache, void* out, int n, const int* n_b,
-                                   float theta, int window, int qhat_sel, bool key, bool packed, DecodeTmapCache* maps, cudaStream_t st) {
+                                   float theta, int window, int qhat_sel, bool key, bool packed, bool behind_step,
+                                   DecodeTmapCache* maps, cudaStream_t st) {
   if ((key && !w.qhat_rows) || (packed && (!key || !w.kp_vals))) return cudaErrorNotSupported;
   using TC = __nv_bfloat16;
   const CUtensorMap* const tk = row_map(&maps[0], k_cache, s);
@@ -688,6 +692,7 @@ cudaError_t launch_decode_step_mma(const Shape& s, const Workspace& w, const voi
   p.kp_nnz = w.kp_nnz; p.vals = w.kp_vals; p.base = w.kp_base;
   p.cap = keypack_capacity(s.T_max, s.d); p.nseg_max = keypack_segments(s.T_max);
   p.ragged = n_b != nullptr;
+  p.early = behind_step ? 1 : 0;
   p.b0 = 0;
   const int G = s.g();
   bool cluster;

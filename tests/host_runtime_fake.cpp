@@ -92,7 +92,9 @@ cudaError_t launch_pack_keys(const Shape&, const Workspace&, const void*, int, c
 cudaError_t launch_decode_step(const Shape&, const Workspace&, const void*, const void*, const void*, void*, void*, void*, int, float,
                                int, int, int, cudaStream_t) { return call("decode"); }
 cudaError_t launch_decode_step_mma(const Shape&, const Workspace&, const void*, const void*, const void*, void*, void*, void*, int,
-                                   const int*, float, int, int, bool, bool, DecodeTmapCache*, cudaStream_t) { return call("decode_mma"); }
+                                   const int*, float, int, int, bool, bool, bool behind_step, DecodeTmapCache*, cudaStream_t) {
+  return call("decode_mma", num("behind_step", behind_step));
+}
 cudaError_t launch_decode_step_f32(const Shape&, const Workspace&, const void*, const void*, const void*, void*, void*, void*, int,
                                    const int*, float, int, int, DecodeTmapCache*, cudaStream_t) { return call("decode_f32"); }
 cudaError_t launch_decode_step_key(const Shape&, const Workspace&, const void*, const void*, const void*, void*, void*, void*, int,

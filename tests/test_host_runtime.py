@@ -46,6 +46,13 @@ class Host:
         return self.lib.delta_attn_prefill_host(self.st, self.buf, self.buf, self.buf, self.buf, self.buf, n, self.T,
                                                 C.c_float(0.3), 64, None)
 
+    def prefill(self):
+        c = self.cfg
+        return self.lib.delta_attn_prefill(self.st, *[self.buf] * 4, self.T, c.H, c.H_kv, c.d, C.c_float(0.3), 64, None)
+
+    def decode(self):
+        return self.lib.delta_attn_decode_step(self.st, *[self.buf] * 6, C.c_float(0.3), 64, None)
+
     def reset(self):
         assert self.lib.delta_state_reset(self.st, None) == 0
 
@@ -95,3 +102,15 @@ def test_host_prefill_on_a_capturing_stream_touches_nothing(fake):
     assert status == B.DELTA_ERR_CUDA and h.call_log() == []
     assert fake.delta_last_cuda_error() == b"fakeError: code 900"       # cudaErrorStreamCaptureUnsupported
     assert h.prefill_host() == 0
+
+
+@pytest.mark.parametrize("packed", [0, 1])
+def test_only_a_step_behind_a_step_may_fetch_ahead_of_its_wait(fake, packed):
+    """The first step behind a prefill must take what the prefill's last kernel wrote behind its wait for it."""
+    h = Host(fake, source=B.DELTA_SRC_KEY)
+    assert fake.delta_state_set_key_cache(h.st, packed) == 0
+    for _ in range(2):
+        assert h.prefill() == 0
+        assert [h.decode() for _ in range(3)] == [0, 0, 0]
+        assert [x[-1] for x in h.call_log() if x.startswith("decode_mma")] == ["0", "1", "1"]
+        h.reset()
