@@ -111,8 +111,9 @@ cudaError_t launch_delta_chain(const Shape& s, const Workspace& w, const void* x
 int device_sm_count();
 // programmatic: 1 = launched with programmatic stream serialisation (its launch overlaps the end
 // of the kernel in front; the kernel waits for that kernel's completion itself); 2 = the same, but
-// the kernel does not wait: the kernel in front releases it once the chain kernel's results are
-// complete (query deltas behind the telescoped attention kernel); 0 = an ordinary launch.
+// the kernel does not wait before its work, only before its end: the kernel in front releases it once the
+// chain kernel's results are complete (query deltas behind the telescoped or the fp32 attention
+// kernel); 0 = an ordinary launch.
 cudaError_t launch_delta_finish(const Shape& s, const Workspace& w, const void* q, const void* k, const SeqBatch& seqs,
                                 float theta, int shape, int dtype, int init, bool want_kt,
                                 bool key_stream, bool reverse, int programmatic, cudaStream_t st);

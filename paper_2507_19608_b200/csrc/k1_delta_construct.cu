@@ -654,7 +654,10 @@ __global__ void __launch_bounds__(256, D == 64 ? 5 : 4) delta_finish_kernel(
   // deltas behind the telescoped attention kernel, of which this kernel needs nothing): every
   // CTA of the attention kernel has released this kernel after its own wait for the chain
   // kernel, so the chain's results are complete; they are read past the L1 cache (ld.global.cg),
-  // and the blocks run on the SMs the attention kernel's last wave leaves idle.
+  // and the blocks run on the SMs the attention kernel's last wave leaves idle.  One thread of the
+  // grid waits at its end: a kernel serialised programmatically behind this one (a decode step) waits for
+  // this kernel only, and with it has to have waited for the attention kernel's stores too.  (Every
+  // CTA of the attention kernel is resident by then, so nothing can be kept from starting.)
   if (wait_front) asm volatile("griddepcontrol.wait;" ::: "memory");
   // key deltas: the attention kernel is serialised programmatically behind this one and may set
   // itself up meanwhile (it waits for this kernel's results itself)
@@ -741,6 +744,7 @@ __global__ void __launch_bounds__(256, D == 64 ? 5 : 4) delta_finish_kernel(
       atomicAdd(&cs[1], (unsigned long long)rows * D);
       atomicAdd(&cs[2], b2);
       atomicAdd(&cs[3], c2);
+      if (!wait_front && blockIdx.x == 0 && blockIdx.y == 0) asm volatile("griddepcontrol.wait;" ::: "memory");
     }
     return;
   }
