@@ -312,14 +312,16 @@ DELTA_API int32_t delta_state_sequence_position(const delta_state_t* st, int32_t
 DELTA_API int32_t delta_state_prefill_kernel(const delta_state_t* st);
 
 /* Which kernel the next delta_attn_decode_step of this state would use: 1 = score and value
- * products on the tensor cores (bf16, top-down query deltas or key deltas: the telescoped form of
- * Eq. 4, see delta_attn_decode_step), 0 = the FP32-pipe kernel, -1 for a null state.  Both compute
- * the same step and keep the same state. */
+ * products on the tensor cores (bf16, top-down query deltas or key deltas; with the compressed key
+ * cache always, only this kernel reads it), 0 = an FP32-pipe kernel (fp32 inputs: a kernel of its own
+ * by default, the stepwise one when 0 is forced; both report 0), -1 for a null state.  All compute the
+ * same step and keep the same state; all but the forced stepwise kernels take Eq. 4 in its telescoped
+ * form (see delta_attn_decode_step). */
 DELTA_API int32_t delta_state_decode_kernel(const delta_state_t* st);
 
 /* Force the decode kernel of a state: 1 = tensor cores (DELTA_ERR_UNSUPPORTED unless bf16, top-down
- * query deltas or key deltas), 0 = FP32 pipes, -1 = the library's choice (the default).  Host-side
- * only. */
+ * query deltas or key deltas), 0 = the stepwise FP32-pipe kernels (no effect while the compressed key
+ * cache is on), -1 = the library's choice (the default).  Host-side only. */
 DELTA_API delta_status_t delta_state_set_decode_kernel(delta_state_t* st, int32_t which);
 DELTA_API delta_status_t delta_state_set_prefill_kernel(delta_state_t* st, int32_t which);
 

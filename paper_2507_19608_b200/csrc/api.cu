@@ -249,6 +249,7 @@ static bool decode_tc_possible(const delta_state* st) {
 int32_t delta_state_decode_kernel(const delta_state_t* st) {
   if (!st) return -1;
   if (!decode_tc_possible(st)) return 0;
+  if (st->key_cache_packed) return 1;          // only that kernel reads the encoding
   return st->forced_decode_kernel >= 0 ? st->forced_decode_kernel : 1;
 }
 
@@ -756,7 +757,7 @@ delta_status_t delta_attn_decode_step(delta_state_t* st, const void* q_new, cons
   cudaStream_t cs = (cudaStream_t)stream;
   cudaError_t e = cudaSuccess;
   const bool key_packed = c.source == DELTA_SRC_KEY && st->key_cache_packed;
-  if (key_packed || delta_state_decode_kernel(st) == 1) {
+  if (delta_state_decode_kernel(st) == 1) {
     // one launch, whether the batch elements stand at one position or at different ones
     e = launch_decode_step_mma(st->shape, st->ws, q_new, k_new, v_new, k_cache, v_cache, out, st->n,
                                st->ragged ? st->n_b.data() : nullptr, theta, window, st->qhat_sel,

@@ -114,3 +114,20 @@ def test_only_a_step_behind_a_step_may_fetch_ahead_of_its_wait(fake, packed):
         assert [h.decode() for _ in range(3)] == [0, 0, 0]
         assert [x[-1] for x in h.call_log() if x.startswith("decode_mma")] == ["0", "1", "1"]
         h.reset()
+
+
+@pytest.mark.parametrize("source,dtype,packed,forced,reported,launched", [
+    (B.DELTA_SRC_QUERY, "bf16", 0, -1, 1, "decode_mma"), (B.DELTA_SRC_QUERY, "bf16", 0, 0, 0, "decode"),
+    (B.DELTA_SRC_KEY, "bf16", 0, -1, 1, "decode_mma"), (B.DELTA_SRC_KEY, "bf16", 0, 0, 0, "decode_key"),
+    (B.DELTA_SRC_KEY, "bf16", 1, -1, 1, "decode_mma"), (B.DELTA_SRC_KEY, "bf16", 1, 0, 1, "decode_mma"),
+    (B.DELTA_SRC_QUERY, "f32", 0, -1, 0, "decode_f32"), (B.DELTA_SRC_QUERY, "f32", 0, 0, 0, "decode")])
+def test_the_reported_decode_kernel_is_the_one_that_runs(fake, source, dtype, packed, forced, reported, launched):
+    h = Host(fake, source=source, dtype=dtype)
+    if packed:
+        assert fake.delta_state_set_key_cache(h.st, 1) == 0
+    assert fake.delta_state_set_decode_kernel(h.st, forced) == 0
+    assert h.prefill() == 0
+    h.call_log()
+    assert fake.delta_state_decode_kernel(h.st) == reported
+    assert h.decode() == 0
+    assert [x.split()[0] for x in h.call_log()] == [launched]
