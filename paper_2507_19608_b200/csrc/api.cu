@@ -692,7 +692,7 @@ delta_status_t delta_attn_prefill_host(delta_state_t* st, const void* q_host, co
   }
   const bool late = x && finish_comes_last(st);
   SeqBatch seqs;
-  seqs.n = 1; seqs.T_longest = T; seqs.ragged = false;
+  seqs.n = 1; seqs.T_longest = T; seqs.ragged = false; seqs.grid_heads = c.B * c.H;
   seqs.s[0] = Seq{T, window, 0, 0};
   for (int i = 0; i < chunks; ++i) {
     const int u0 = (int)((long)units * i / chunks), n = (int)((long)units * (i + 1) / chunks) - u0;

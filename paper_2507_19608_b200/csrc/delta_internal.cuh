@@ -69,10 +69,17 @@ struct Seq {
 };
 template <int N> struct SeqList { Seq s[N]; };
 // The sequences of a launch: n = 1 (uniform, covering the whole batch) or a ragged group.
+// grid_heads: the query heads of the whole call where a launch covers a part of a uniform batch, else 0.  The
+// forms of the attention kernels follow the size of the grid and round differently (which keys share a
+// running maximum, whose probabilities meet): the call's grid decides, not the part's, so that a
+// head's result does not depend on how its call was cut.
 struct SeqBatch {
   int n, T_longest;
   bool ragged;
+  int grid_heads = 0;
   Seq s[kSeqMax];
+  // query heads of the grid that chooses the form (ragged: of every sequence's grid)
+  long form_heads(const Shape& sh) const { return grid_heads ? grid_heads : (long)(ragged ? 1 : sh.B) * sh.H; }
 };
 
 // What a launcher does once per device (function attributes, which the runtime keeps): has it been

@@ -453,7 +453,7 @@ static cudaError_t launch_f32_form(const Shape& s, const Workspace& w, const voi
   float best = 3.4e38f, pairs = 0.0f;
   for (int i = 0; i < seqs.n; ++i) {
     const float t = (float)((seqs.s[i].T + BN - 1) / BN);
-    pairs += 0.5f * t * (t + 1.0f) * (float)((seqs.ragged ? 1 : s.B) * s.H);
+    pairs += 0.5f * t * (t + 1.0f) * (float)seqs.form_heads(s);
   }
   for (int c = 0; c < 3; ++c) {
     constexpr float alone[3] = {3.3f, 2.2f, 1.4f}, full[3] = {4.0f, 2.2f, 1.6f};

@@ -1064,7 +1064,7 @@ cudaError_t launch_hybrid_attn_tcq(const Shape& s, const Workspace& w, const voi
     // On a smaller grid that the one-head form cannot place in one wave, the heaviest query
     // tiles of every head go one head per CTA and the rest two heads per CTA, as many of the
     // former as one wave of SMs allows.
-    const long BH = (long)(seqs.ragged ? 1 : s.B) * s.H, sms = device_sm_count();
+    const long BH = seqs.form_heads(s), sms = device_sm_count();
     long nqt = 0;                         // query tiles of a head (ragged group: of a head of every sequence)
     for (int i = 0; i < seqs.n; ++i) nqt += (seqs.s[i].T + BM - 1) / BM;
     int n_one = -1;                       // -1: the one-head kernel

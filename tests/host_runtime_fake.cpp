@@ -84,10 +84,14 @@ cudaError_t launch_delta_finish(const Shape& s, const Workspace&, const void*, c
                                 bool, bool, int, cudaStream_t) { return call("finish", num("heads", s.B * s.H)); }
 cudaError_t launch_hybrid_attn_tc(const Shape& s, const Workspace&, const void*, const void*, const void*, void*, int, int, int,
                                   cudaStream_t) { return call("attn_tc", num("heads", s.B * s.H)); }
-cudaError_t launch_hybrid_attn_tcq(const Shape& s, const Workspace&, const void*, const void*, const void*, void*, const SeqBatch&,
-                                   float, int, int, bool, bool, int, cudaStream_t) { return call("attn", num("heads", s.B * s.H)); }
-cudaError_t launch_hybrid_attn_generic(const Shape& s, const Workspace&, const void*, const void*, const void*, void*, const SeqBatch&,
-                                       float, int, int, int, cudaStream_t) { return call("attn", num("heads", s.B * s.H)); }
+cudaError_t launch_hybrid_attn_tcq(const Shape& s, const Workspace&, const void*, const void*, const void*, void*, const SeqBatch& q,
+                                   float, int, int, bool, bool, int, cudaStream_t) {
+  return call("attn", num("heads", s.B * s.H) + num("form_heads", q.form_heads(s)));
+}
+cudaError_t launch_hybrid_attn_generic(const Shape& s, const Workspace&, const void*, const void*, const void*, void*,
+                                       const SeqBatch& q, float, int, int, int, cudaStream_t) {
+  return call("attn", num("heads", s.B * s.H) + num("form_heads", q.form_heads(s)));
+}
 cudaError_t launch_pack_keys(const Shape&, const Workspace&, const void*, int, cudaStream_t) { return call("pack"); }
 cudaError_t launch_decode_step(const Shape&, const Workspace&, const void*, const void*, const void*, void*, void*, void*, int, float,
                                int, int, int, cudaStream_t) { return call("decode"); }

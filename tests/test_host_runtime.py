@@ -131,3 +131,12 @@ def test_the_reported_decode_kernel_is_the_one_that_runs(fake, source, dtype, pa
     assert fake.delta_state_decode_kernel(h.st) == reported
     assert h.decode() == 0
     assert [x.split()[0] for x in h.call_log()] == [launched]
+
+
+@pytest.mark.parametrize("Bn,H,H_kv,dtype,parts", [(1, 32, 8, "bf16", [8] * 4), (3, 20, 5, "bf16", [12, 16, 16, 16]),
+                                                   (1, 8, 8, "f32", [4, 4])])
+def test_a_call_in_parts_takes_the_form_of_the_whole_call(fake, Bn, H, H_kv, dtype, parts):
+    """The attention kernels round by their form; the host-buffer call cuts a batch and must not change it."""
+    h = Host(fake, H=H, H_kv=H_kv, Bn=Bn, dtype=dtype)
+    assert h.prefill_host() == 0
+    assert [x for x in h.call_log() if x.startswith("attn")] == [f"attn heads={n} form_heads={Bn * H}" for n in parts]
