@@ -137,7 +137,10 @@ DELTA_API delta_status_t delta_state_destroy(delta_state_t* st);
  * scale 1/sqrt(d), causal online softmax, P.V (Eq. 1)), the hand-off of q_hat(T-1) and
  * R(T-1)[0..T-1] for decode, and the sparsity counters (Eq. 6).
  * H, H_kv, d must equal the configuration.  Needs a fresh or reset state (else
- * DELTA_ERR_STATE); 1 <= T <= T_max (else DELTA_ERR_CAPACITY). */
+ * DELTA_ERR_STATE); 1 <= T <= T_max (else DELTA_ERR_CAPACITY).
+ * Rounding: the form of the attention kernel (which keys share a running maximum and a sum) follows
+ * the sizes of the call, B, H and T, alone; the same sequence in batches of different sizes agrees to the
+ * rounding of the probabilities (a bf16 step for bf16), the delta arrays and counters exactly. */
 DELTA_API delta_status_t delta_attn_prefill(delta_state_t* st, const void* q, const void* k, const void* v,
                                   void* out, int32_t T, int32_t H, int32_t H_kv, int32_t d,
                                   float theta, int32_t window, void* stream);
@@ -151,7 +154,8 @@ DELTA_API delta_status_t delta_attn_prefill(delta_state_t* st, const void* q, co
  *              the other in batch order (sequence b starts H * d * (seq_lens[0] + .. + seq_lens[b-1])
  *              elements into the array)
  *   k, v     : [B, H_kv, T_max, d] (KV-cache layout; rows 0 .. seq_lens[b]-1 of element b are read)
- * Every sequence is what delta_attn_prefill computes for a batch of one: its own delta chains,
+ * Every sequence is what delta_attn_prefill computes for a batch of one, bit for bit (the attention
+ * kernel takes each in the form of its own length, whatever stands beside it): its own delta chains,
  * window, counters (Eq. 6 sums over the sequences: S_c_eq6 uses sum min(W_b, n_b) / sum n_b) and
  * decode hand-off.  Afterwards the batch elements stand at different positions:
  * delta_state_sequence_position reports each, delta_state_position the longest, and
@@ -161,7 +165,7 @@ DELTA_API delta_status_t delta_attn_prefill_varlen(delta_state_t* st, const void
                                          void* out, const int32_t* seq_lens, const int32_t* windows,
                                          float theta, void* stream);
 
-/* delta_attn_prefill_host -- the same call for HOST buffers (q, k, v, out are host pointers
+/* delta_attn_prefill_host -- delta_attn_prefill, bit for bit, for HOST buffers (q, k, v, out are host pointers
  * with the shapes above; k and v hold T rows per head, i.e. [B, H_kv, T, d]).  `staging` is
  * a DEVICE buffer of at least delta_prefill_staging_bytes(cfg, T) bytes that receives the
  * copies.  Copies in, runs the prefill, copies `out` back and synchronises the stream (so a

@@ -26,6 +26,8 @@
 // A tile takes Q_hat.K^T where none of its pairs is inside the window, Q.K^T where all causal ones are,
 // both where it is mixed.  The reference rows are rebuilt from the 8-row checkpoints of the chain
 // kernel (Eq. 2-3 re-run per block), so nothing of the finish kernel is read.
+#include <algorithm>
+
 #include "delta_internal.cuh"
 #include "tc_common.cuh"
 
@@ -116,14 +118,30 @@ __device__ __forceinline__ void mma_parts(float (&big)[4], float (&small)[4], co
     if constexpr (NB == 1) mma(small, a[2], b[0][2 * half], b[0][2 * half + 1]);
   }
 }
-}  // namespace
+// Forms (KS) of the sequences of a ragged group.
+struct F32Forms { int ks[kSeqMax]; };
+template <typename TIn> struct F32Args {
+  const TIn *q, *k, *v;
+  TIn* out;
+  const float* ckpt;
+  unsigned long long* counters;
+  int T_max, n_ckpt, H, g, shape;
+  float theta;
+  int basis_row;
+  float scale_log2e;
+};
 
-template <typename TIn, int D, int KS, int N>
-__global__ void __launch_bounds__(NT, D == 64 ? 2 : 1) hybrid_attn_f32_kernel(
-    const TIn* __restrict__ q, const TIn* __restrict__ k, const TIn* __restrict__ v, TIn* __restrict__ out,
-    const float* __restrict__ ckpt, unsigned long long* __restrict__ counters, const __grid_constant__ SeqList<N> seqs,
-    int T_max, int n_ckpt, int H, int g, int shape, float theta, int basis_row, float scale_log2e) {
-  const Seq& sq = seqs.s[N == 1 ? 0 : blockIdx.z];
+// One query tile (of 64 / KS rows) of one head; tile 0 is the last one of the sequence.
+template <typename TIn, int D, int KS>
+__device__ __forceinline__ void attn_f32_tile(const F32Args<TIn>& p, const Seq& sq, int tile, int head) {
+  const TIn* __restrict__ const q = p.q;
+  const TIn* __restrict__ const k = p.k;
+  const TIn* __restrict__ const v = p.v;
+  TIn* __restrict__ const out = p.out;
+  const float* __restrict__ const ckpt = p.ckpt;
+  unsigned long long* __restrict__ const counters = p.counters;
+  const int T_max = p.T_max, n_ckpt = p.n_ckpt, H = p.H, g = p.g, shape = p.shape, basis_row = p.basis_row;
+  const float theta = p.theta, scale_log2e = p.scale_log2e;
   const int T = sq.T, W = sq.W;
   constexpr int NP = sizeof(TIn) == 4 ? 3 : 1;
   using SM = F32Smem<D, KS, NP>;
@@ -137,10 +155,10 @@ __global__ void __launch_bounds__(NT, D == 64 ? 2 : 1) hybrid_attn_f32_kernel(
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int g8 = lane >> 2, t4 = lane & 3;         // row of the fragments, thread of the row
   const int rg = warp / KS, kg = warp % KS;        // the warp's 16 rows, its share of a tile's keys
-  const int qt = (T + BM - 1) / BM - 1 - (int)blockIdx.x;  // longest walks first
-  if (N > 1 && qt < 0) return;                             // (a shorter sequence of a ragged group)
-  const int bh = sq.b * H + (int)blockIdx.y, b = bh / H, h = bh - b * H;
-  const size_t io = sq.q_off + (size_t)blockIdx.y * T * D;      // the head's rows in q and out
+  const int qt = (T + BM - 1) / BM - 1 - tile;     // longest walks first
+  if (qt < 0) return;                              // (a shorter sequence of a ragged group)
+  const int bh = sq.b * H + head, b = bh / H, h = bh - b * H;
+  const size_t io = sq.q_off + (size_t)head * T * D;            // the head's rows in q and out
   const size_t bkv = (size_t)b * (H / g) + h / g;
   const int i0 = qt * BM, i1 = min(i0 + BM, T) - 1;
   const TIn* const kp = k + bkv * T_max * D;
@@ -410,22 +428,34 @@ __global__ void __launch_bounds__(NT, D == 64 ? 2 : 1) hybrid_attn_f32_kernel(
   }
 }
 
-template <typename TIn, int D, int KS, int N>
-static cudaError_t launch_f32(const Shape& s, const Workspace& w, const void* q, const void* k, const void* v, void* out,
-                              const SeqBatch& seqs, float theta, int init, int shape, cudaStream_t st) {
-  auto kern = hybrid_attn_f32_kernel<TIn, D, KS, N>;
-  constexpr size_t smem = F32Smem<D, KS, sizeof(TIn) == 4 ? 3 : 1>::bytes;
-  static std::atomic<uint64_t> ready{0};
+}  // namespace
+
+// A uniform batch.
+template <typename TIn, int D, int KS>
+__global__ void __launch_bounds__(NT, D == 64 ? 2 : 1)
+hybrid_attn_f32_kernel(const __grid_constant__ F32Args<TIn> p, const __grid_constant__ SeqList<1> seqs) {
+  attn_f32_tile<TIn, D, KS>(p, seqs.s[0], (int)blockIdx.x, (int)blockIdx.y);
+}
+// A ragged group: every sequence in the form of a batch of its own.
+template <typename TIn, int D>
+__global__ void __launch_bounds__(NT, D == 64 ? 2 : 1)
+hybrid_attn_f32_ragged_kernel(const __grid_constant__ F32Args<TIn> p, const __grid_constant__ SeqList<kSeqMax> seqs,
+                              const __grid_constant__ F32Forms forms) {
+  const int i = (int)blockIdx.z, ks = forms.ks[i];
+  if (ks == 1) attn_f32_tile<TIn, D, 1>(p, seqs.s[i], (int)blockIdx.x, (int)blockIdx.y);
+  else if (ks == 2) attn_f32_tile<TIn, D, 2>(p, seqs.s[i], (int)blockIdx.x, (int)blockIdx.y);
+  else attn_f32_tile<TIn, D, 4>(p, seqs.s[i], (int)blockIdx.x, (int)blockIdx.y);
+}
+
+template <typename K, typename... A>
+static cudaError_t launch_f32(K kern, std::atomic<uint64_t>& ready, size_t smem, dim3 grid, cudaStream_t st, const A&... args) {
   if (!device_done(ready)) {
     const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     device_mark(ready);
   }
-  SeqList<N> list;
-  for (int i = 0; i < N; ++i) list.s[i] = seqs.s[i < seqs.n ? i : 0];
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)((seqs.T_longest + 64 / KS - 1) / (64 / KS)), (unsigned)(seqs.ragged ? s.H : s.B * s.H),
-                     (unsigned)seqs.n);
+  cfg.gridDim = grid;
   cfg.blockDim = dim3(NT);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
@@ -434,44 +464,69 @@ static cudaError_t launch_f32(const Shape& s, const Workspace& w, const void* q,
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  const cudaError_t e =
-      cudaLaunchKernelEx(&cfg, kern, (const TIn*)q, (const TIn*)k, (const TIn*)v, (TIn*)out, (const float*)w.ckpt, w.counters,
-                         list, s.T_max, s.n_ckpt(), s.H, s.g(), shape, theta, init == DELTA_INIT_BASIS_EXACT ? 0 : -1,
-                         1.4426950408889634f / sqrtf((float)s.d));
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, args...);
   count_launch();
   return e != cudaSuccess ? e : cudaGetLastError();
 }
 
-template <typename TIn, int D, int N>
-static cudaError_t launch_f32_form(const Shape& s, const Workspace& w, const void* q, const void* k, const void* v, void* out,
-                                   const SeqBatch& seqs, float theta, int init, int shape, cudaStream_t st) {
-  // Warps per row group.  A key tile of 64 costs 3.3 / 2.2 / 1.4 us where a CTA walks alone and takes
-  // 4.0 / 2.2 / 1.6 us of an SM where the chip is full (KS = 1 / 2 / 4; d = 64, 1 to 256 heads of 128 to
-  // 4000 tokens); every halving of the rows doubles the tiles.  The longest walk bounds a small
-  // grid, the sum of all tiles, with half a walk for the uneven end, a large one.
+// Warps per row group for `heads` heads of T tokens.  A key tile of 64 costs 3.3 / 2.2 / 1.4 us where a CTA
+// walks alone and takes 4.0 / 2.2 / 1.6 us of an SM where the chip is full (KS = 1 / 2 / 4; d = 64, 1 to
+// 256 heads of 128 to 4000 tokens); every halving of the rows doubles the tiles.  The longest walk bounds a
+// small grid, the sum of all tiles, with half a walk for the uneven end, a large one.  A sequence of a
+// ragged group takes the form of a batch of its own (the forms round differently: its result does not
+// depend on the sequences beside it).
+static int f32_form(long heads, int T) {
   int ks = 1;
-  float best = 3.4e38f, pairs = 0.0f;
-  for (int i = 0; i < seqs.n; ++i) {
-    const float t = (float)((seqs.s[i].T + BN - 1) / BN);
-    pairs += 0.5f * t * (t + 1.0f) * (float)seqs.form_heads(s);
-  }
+  float best = 3.4e38f;
+  const float t = (float)((T + BN - 1) / BN), pairs = 0.5f * t * (t + 1.0f) * (float)heads;
   for (int c = 0; c < 3; ++c) {
     constexpr float alone[3] = {3.3f, 2.2f, 1.4f}, full[3] = {4.0f, 2.2f, 1.6f};
-    const float walk = (float)((seqs.T_longest + BN - 1) / BN) * alone[c];
+    const float walk = t * alone[c];
     const float us = fmaxf(walk, pairs * (float)(1 << c) / (float)device_sm_count() * full[c] + 0.5f * walk);
     if (us < best) { best = us; ks = 1 << c; }
   }
-  return ks == 4   ? launch_f32<TIn, D, 4, N>(s, w, q, k, v, out, seqs, theta, init, shape, st)
-         : ks == 2 ? launch_f32<TIn, D, 2, N>(s, w, q, k, v, out, seqs, theta, init, shape, st)
-                   : launch_f32<TIn, D, 1, N>(s, w, q, k, v, out, seqs, theta, init, shape, st);
+  return ks;
+}
+
+template <typename TIn, int D>
+static cudaError_t launch_f32_form(const Shape& s, const Workspace& w, const void* q, const void* k, const void* v, void* out,
+                                   const SeqBatch& seqs, float theta, int init, int shape, cudaStream_t st) {
+  constexpr int NP = sizeof(TIn) == 4 ? 3 : 1;
+  const F32Args<TIn> p{(const TIn*)q, (const TIn*)k, (const TIn*)v, (TIn*)out, w.ckpt, w.counters, s.T_max, s.n_ckpt(), s.H,
+                       s.g(), shape, theta, init == DELTA_INIT_BASIS_EXACT ? 0 : -1, 1.4426950408889634f / sqrtf((float)s.d)};
+  const long heads = seqs.form_heads(s);
+  static std::atomic<uint64_t> ready[4] = {};
+  if (seqs.ragged) {
+    SeqList<kSeqMax> list;
+    F32Forms forms;
+    unsigned tiles = 0;
+    for (int i = 0; i < kSeqMax; ++i) {
+      list.s[i] = seqs.s[i < seqs.n ? i : 0];
+      forms.ks[i] = f32_form(heads, list.s[i].T);
+      const unsigned bm = 64u / (unsigned)forms.ks[i], n = ((unsigned)list.s[i].T + bm - 1) / bm;
+      tiles = n > tiles ? n : tiles;
+    }
+    return launch_f32(hybrid_attn_f32_ragged_kernel<TIn, D>, ready[3],
+                      std::max({F32Smem<D, 1, NP>::bytes, F32Smem<D, 2, NP>::bytes, F32Smem<D, 4, NP>::bytes}),
+                      dim3(tiles, (unsigned)s.H, (unsigned)seqs.n), st, p, list, forms);
+  }
+  SeqList<1> list;
+  list.s[0] = seqs.s[0];
+  const unsigned T = (unsigned)list.s[0].T, bh = (unsigned)(s.B * s.H);
+  const int ks = f32_form(heads, (int)T);
+#define GO(KS)                                                                                               \
+  return launch_f32(hybrid_attn_f32_kernel<TIn, D, KS>, ready[KS / 2], F32Smem<D, KS, NP>::bytes,            \
+                    dim3((T + 64 / KS - 1) / (64 / KS), bh), st, p, list)
+  if (ks == 4) GO(4);
+  if (ks == 2) GO(2);
+  GO(1);
+#undef GO
 }
 
 cudaError_t launch_hybrid_attn_generic(const Shape& s, const Workspace& w, const void* q, const void* k, const void* v,
                                        void* out, const SeqBatch& seqs, float theta, int init, int shape, int dtype,
                                        cudaStream_t st) {
-#define GO(TIN, DD)                                                                                       \
-  return seqs.ragged ? launch_f32_form<TIN, DD, kSeqMax>(s, w, q, k, v, out, seqs, theta, init, shape, st) \
-                     : launch_f32_form<TIN, DD, 1>(s, w, q, k, v, out, seqs, theta, init, shape, st)
+#define GO(TIN, DD) return launch_f32_form<TIN, DD>(s, w, q, k, v, out, seqs, theta, init, shape, st)
   if (dtype == DELTA_F32) {
     if (s.d == 64) { GO(float, 64); } else { GO(float, 128); }
   } else {

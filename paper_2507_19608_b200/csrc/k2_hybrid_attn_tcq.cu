@@ -46,6 +46,8 @@
 // nothing is stored and the status word records DELTA_ERR_TIMEOUT.
 #include <cuda.h>
 
+#include <climits>
+
 #include "k2_tc.cuh"
 #include "tc_common.cuh"
 
@@ -126,15 +128,15 @@ struct TqParams {
   const float* ckpt;           // [B,H,n_ckpt,D] reference in front of every 8-row block (query deltas only)
   int T_max, n_ckpt, H, g, shape;
   int BH;            // heads of one entry of the sequence list (uniform batch: batch x query heads)
-  int nqt;           // query tiles of the longest sequence
-  int n_one;         // two-head layout: the n_one heaviest query tiles of every head go one head per CTA
   int reverse;       // strategy (2): Eq. 2-3 runs from row T-1 down to row 0
   int basis;         // is the first row taken (0, or T-1 in reverse) the un-thresholded basis?
   float scale_log2e, theta;
 };
 
-// Tensor maps of one entry of the sequence list: queries, reference-key rows, keys, values (rows 0..T-1).
-struct TqMaps { CUtensorMap q, qh, k, v; };
+// One entry of the sequence list: tensor maps of queries, reference-key rows, keys, values (rows
+// 0..T-1), its first CTA in the grid (INT_MAX: no entry), its query tiles and, two-head layout, how many
+// of the heaviest ones of every head go one head per CTA.
+struct TqMaps { CUtensorMap q, qh, k, v; int first, nqt, n_one; };
 template <int N> struct TqMapList { TqMaps m[N]; };
 
 // Barrier of the eight softmax warps (id 1, 256 threads; immediate id: a register operand would
@@ -226,8 +228,8 @@ __device__ __forceinline__ void build_ref_rows(const unsigned char* q_src, unsig
 // there; at d = 64 it costs the other tiles registers, 144 -> 168, and some percent).
 // FORM: 0 = every CTA one head; 1 = every CTA two heads; 2 = two-head layout, the form of a CTA
 // follows its place in the grid (see below).
-// N: entries of the sequence list: 1 (a uniform batch), or kSeqMax (a ragged group: the grid is
-// [heads of all sequences][query tiles of the longest]; CTAs past their sequence's tiles return).
+// N: entries of the sequence list: 1 (a uniform batch), or kSeqMax (a ragged group: the CTAs of the
+// sequences one behind the other, the longest sequence first, each as in a batch of its own).
 template <int D, bool KEY, int FORM, bool MIXED, int N>
 __global__ void __launch_bounds__(NTHR, 1)
 hybrid_attn_tcq_kernel(const __grid_constant__ TqMapList<N> maps, const __grid_constant__ SeqList<N> seqs,
@@ -248,8 +250,8 @@ hybrid_attn_tcq_kernel(const __grid_constant__ TqMapList<N> maps, const __grid_c
 
   // (the warp index by shuffle: known to be the same in every lane)
   const int tid = threadIdx.x, lane = tid & 31, warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
-  // Heaviest query tiles of every head first.  PAIR (the layout holds two query tiles): a
-  // one-dimensional grid; its first BH * n_one CTAs take the n_one heaviest query tiles of every
+  // Heaviest query tiles of every head first.  PAIR (the layout holds two query tiles): an entry's
+  // first BH * n_one CTAs take the n_one heaviest query tiles of every
   // head in the one-head form (key tiles dealt to the two softmax groups, merge at the end), the
   // others the same query tile of two neighbouring heads of one KV group, bh and bh + 1 (group
   // X of the softmax warps takes head bh + X and every key tile).  pr: this CTA is of the
@@ -257,26 +259,21 @@ hybrid_attn_tcq_kernel(const __grid_constant__ TqMapList<N> maps, const __grid_c
   int qt, bh, si = 0;
   bool pr = false;
   if (N > 1) {
-    const int per = PAIR ? p.BH / 2 : p.BH, x = (int)blockIdx.x;
-    si = x / per;
-    bh = (x - si * per) * (PAIR ? 2 : 1);
-    pr = PAIR;
-    qt = (seqs.s[si].T + BM - 1) / BM - 1 - (int)blockIdx.y;
-    if (qt < 0) return;
-  } else if (PAIR) {
-    const int nqt = p.nqt, idx = (int)blockIdx.x, n1 = (FORM == 1) ? 0 : p.BH * p.n_one;
-    if (FORM == 2 && idx < n1) {
+#pragma unroll
+    for (int i = 1; i < N; ++i) si = (int)blockIdx.x >= maps.m[i].first ? i : si;
+  }
+  {
+    const int nqt = maps.m[si].nqt, idx = (int)blockIdx.x - (N > 1 ? maps.m[si].first : 0);
+    const int n_one = FORM == 0 ? nqt : FORM == 1 ? 0 : maps.m[si].n_one, n1 = p.BH * n_one;
+    if (FORM != 1 && (FORM == 0 || idx < n1)) {
       qt = nqt - 1 - idx / p.BH;
       bh = idx % p.BH;
     } else {
       const int j = idx - n1, hp = p.BH / 2;
       pr = true;
-      qt = nqt - ((FORM == 1) ? 0 : p.n_one) - 1 - j / hp;
+      qt = nqt - n_one - 1 - j / hp;
       bh = 2 * (j % hp);
     }
-  } else {
-    qt = (int)gridDim.y - 1 - (int)blockIdx.y;
-    bh = (int)blockIdx.x;
   }
   // (bh, bkv: head and KV head within the entry of the sequence list; g_bh: of the workspace arrays)
   const int b = bh / p.H, h = bh - b * p.H;
@@ -340,10 +337,11 @@ hybrid_attn_tcq_kernel(const __grid_constant__ TqMapList<N> maps, const __grid_c
   tc_fence_after();
   const uint32_t tmem = __shfl_sync(0xffffffffu, sMisc[0], 0);
 
-  // Keys that some row of this query tile scores exactly: ex_lo <= j <= ex_hi (empty if W = 0).
+  // Keys that some row of this query tile scores exactly: ex_lo <= j <= ex_hi (W = 0: no key tile's
+  // last key reaches ex_lo).
   // Block window: the window blocks that rows i0..i1 fall into; sliding: i0-W+1 .. i1.
   // Computed once: the per-tile test below must not divide.
-  int ex_lo = 1, ex_hi = 0;
+  int ex_lo = INT_MAX, ex_hi = -1;
   if (W > 0) {
     if (shape == 0) { ex_lo = (i0 / W) * W; ex_hi = (i1 / W) * W + W - 1; }
     else { ex_lo = i0 - W + 1; ex_hi = i1; }
@@ -959,8 +957,8 @@ hybrid_attn_tcq_kernel(const __grid_constant__ TqMapList<N> maps, const __grid_c
 
 template <int D, bool KEY, int FORM, bool MIXED, int N>
 static cudaError_t launch_tcq_m(const Shape& s, const Workspace& w, const void* q, const void* k, const void* v,
-                                void* out, const SeqBatch& seqs, float theta, int init, int shape, bool reverse,
-                                int n_one, cudaStream_t st) {
+                                void* out, const SeqBatch& seqs, const int (&n_one)[kSeqMax], float theta, int init, int shape,
+                                bool reverse, cudaStream_t st) {
   constexpr bool PAIR = FORM != 0;
   auto kern = hybrid_attn_tcq_kernel<D, KEY, FORM, MIXED, N>;
   using TC = __nv_bfloat16;
@@ -969,12 +967,23 @@ static cudaError_t launch_tcq_m(const Shape& s, const Workspace& w, const void* 
   const uint64_t ref_heads = KEY ? BKV : BH;   // the reference rows follow the delta stream
   TqMapList<N> maps;
   SeqList<N> list;
+  int order[N];                            // the entries, longest first
   for (int i = 0; i < seqs.n; ++i) {
-    const Seq& e = seqs.s[i];
+    int at = i;
+    for (; at > 0 && seqs.s[order[at - 1]].T < seqs.s[i].T; --at) order[at] = order[at - 1];
+    order[at] = i;
+  }
+  int ctas = 0;
+  for (int i = 0; i < seqs.n; ++i) {
+    const Seq& e = seqs.s[order[i]];
     const uint64_t T = (uint64_t)e.T;
     const size_t kv = (size_t)e.b * s.H_kv * s.T_max * D, rf = (size_t)e.b * (KEY ? s.H_kv : s.H) * s.T_max * D;
     TqMaps& m = maps.m[i];
     list.s[i] = e;
+    m.first = ctas;
+    m.nqt = (e.T + BM - 1) / BM;
+    m.n_one = FORM == 0 ? m.nqt : FORM == 1 ? 0 : n_one[order[i]] < m.nqt ? n_one[order[i]] : m.nqt;
+    ctas += (int)BH * m.n_one + (int)(BH / 2) * (m.nqt - m.n_one);
     const uint64_t cache = (uint64_t)s.T_max * D * 2;
     if (!encode3(&m.q, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, (const TC*)q + e.q_off, D, T, BH, D * 2, T * D * 2, 64, 128,
                  CU_TENSOR_MAP_SWIZZLE_128B) ||
@@ -986,6 +995,7 @@ static cudaError_t launch_tcq_m(const Shape& s, const Workspace& w, const void* 
                          CU_TENSOR_MAP_SWIZZLE_128B)))
       return cudaErrorInvalidValue;
   }
+  for (int i = seqs.n; i < N; ++i) { list.s[i] = list.s[0]; maps.m[i].first = INT_MAX; }
   static std::atomic<uint64_t> ready{0};
   if (!device_done(ready)) {
     const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TqSmem<D, PAIR>::BYTES);
@@ -1006,12 +1016,8 @@ static cudaError_t launch_tcq_m(const Shape& s, const Workspace& w, const void* 
   // delta chain kernel in front is still running; they wait for its results with
   // griddepcontrol.wait.
   cudaLaunchConfig_t cfg = {};
-  const int nqt = (seqs.T_longest + BM - 1) / BM;
   p.BH = (int)BH;
-  p.nqt = nqt;
-  p.n_one = (FORM == 2) ? (n_one < nqt ? n_one : nqt) : 0;
-  if (N > 1) cfg.gridDim = dim3((unsigned)(seqs.n * (PAIR ? BH / 2 : BH)), (unsigned)nqt);
-  else cfg.gridDim = PAIR ? dim3((unsigned)(BH * p.n_one + BH / 2 * (nqt - p.n_one))) : dim3((unsigned)BH, (unsigned)nqt);
+  cfg.gridDim = dim3((unsigned)ctas);
   cfg.blockDim = dim3(NTHR);
   cfg.dynamicSmemBytes = TqSmem<D, PAIR>::BYTES;
   cfg.stream = st;
@@ -1038,14 +1044,14 @@ static bool mixed_tiles_possible(int window, int shape) {
 
 template <int D, bool KEY, int FORM>
 static cudaError_t launch_tcq(const Shape& s, const Workspace& w, const void* q, const void* k, const void* v,
-                              void* out, const SeqBatch& seqs, float theta, int init, int shape, bool reverse,
-                              int n_one, cudaStream_t st) {
-  if (seqs.ragged)       // (windows differ: with the mixed tiles' code)
-    return launch_tcq_m<D, KEY, FORM == 2 ? 0 : FORM, true, kSeqMax>(s, w, q, k, v, out, seqs, theta, init, shape, reverse, 0,
-                                                                    st);
+                              void* out, const SeqBatch& seqs, const int (&n_one)[kSeqMax], float theta, int init, int shape,
+                              bool reverse, cudaStream_t st) {
+  if (seqs.ragged)       // (windows differ: with the mixed tiles' code; the form is each sequence's)
+    return launch_tcq_m<D, KEY, FORM == 0 ? 0 : 2, true, kSeqMax>(s, w, q, k, v, out, seqs, n_one, theta, init, shape, reverse,
+                                                                 st);
   return mixed_tiles_possible<D, KEY>(seqs.s[0].W, shape)
-             ? launch_tcq_m<D, KEY, FORM, true, 1>(s, w, q, k, v, out, seqs, theta, init, shape, reverse, n_one, st)
-             : launch_tcq_m<D, KEY, FORM, false, 1>(s, w, q, k, v, out, seqs, theta, init, shape, reverse, n_one, st);
+             ? launch_tcq_m<D, KEY, FORM, true, 1>(s, w, q, k, v, out, seqs, n_one, theta, init, shape, reverse, st)
+             : launch_tcq_m<D, KEY, FORM, false, 1>(s, w, q, k, v, out, seqs, n_one, theta, init, shape, reverse, st);
 }
 
 bool tcq_kernel_shape(int d) { return d == 64 || d == 128; }
@@ -1057,41 +1063,45 @@ cudaError_t launch_hybrid_attn_tcq(const Shape& s, const Workspace& w, const voi
   if (!w.qhat_rows) return cudaErrorNotSupported;
   const bool two_heads_ok = s.d == 64 && (s.g() % 2) == 0;
   if ((form == 2 || form == 3) && !two_heads_ok) return cudaErrorNotSupported;
-  if (s.d == 64) {
-    // Two heads of a KV group per CTA share every key and value tile and need no merge, but a
-    // head's key tiles are then walked by one softmax group instead of two.  That pays once
-    // there are at least two such CTAs per SM (stack layer: 0.925 of the one-head form's time).
-    // On a smaller grid that the one-head form cannot place in one wave, the heaviest query
-    // tiles of every head go one head per CTA and the rest two heads per CTA, as many of the
-    // former as one wave of SMs allows.
-    const long BH = seqs.form_heads(s), sms = device_sm_count();
-    long nqt = 0;                         // query tiles of a head (ragged group: of a head of every sequence)
-    for (int i = 0; i < seqs.n; ++i) nqt += (seqs.s[i].T + BM - 1) / BM;
-    int n_one = -1;                       // -1: the one-head kernel
-    if (seqs.ragged) n_one = (two_heads_ok && form != 1 && BH / 2 * nqt >= 2 * sms) ? 0 : -1;
-    else if (form == 2) n_one = 0;
-    else if (form == 3) n_one = 1;
+  // Two heads of a KV group per CTA share every key and value tile and need no merge, but a
+  // head's key tiles are then walked by one softmax group instead of two.  That pays once
+  // there are at least two such CTAs per SM (stack layer: 0.925 of the one-head form's time).
+  // On a smaller grid that the one-head form cannot place in one wave, the heaviest query
+  // tiles of every head go one head per CTA and the rest two heads per CTA, as many of the
+  // former as one wave of SMs allows.  The forms round differently: a sequence of a ragged group takes the
+  // form of a batch of its own, so that its result does not depend on the sequences beside it.
+  const long BH = seqs.form_heads(s), sms = device_sm_count();
+  int n_one[kSeqMax];                     // query tiles of every head in the one-head form
+  bool all_one = true, all_two = true;
+  for (int i = 0; i < seqs.n; ++i) {
+    const long nqt = (seqs.s[i].T + BM - 1) / BM;
+    long n1 = nqt;
+    if (form == 2) n1 = 0;
+    else if (form == 3) n1 = 1;
     else if (form == 0 && two_heads_ok) {
-      if (BH / 2 * nqt >= 2 * sms) n_one = 0;
-      else if (BH * nqt > sms && BH / 2 * nqt <= sms) n_one = (int)((sms - BH / 2 * nqt) / (BH / 2));
+      if (BH / 2 * nqt >= 2 * sms) n1 = 0;
+      else if (BH * nqt > sms && BH / 2 * nqt <= sms) n1 = (sms - BH / 2 * nqt) / (BH / 2);
     }
-    if (key_deltas) {
-      if (n_one == 0)
-        return launch_tcq<64, true, 1>(s, w, q, k, v, out, seqs, theta, init, shape, reverse, 0, st);
-      if (n_one > 0)
-        return launch_tcq<64, true, 2>(s, w, q, k, v, out, seqs, theta, init, shape, reverse, n_one, st);
-      return launch_tcq<64, true, 0>(s, w, q, k, v, out, seqs, theta, init, shape, reverse, 0, st);
-    }
-    if (n_one == 0)
-      return launch_tcq<64, false, 1>(s, w, q, k, v, out, seqs, theta, init, shape, reverse, 0, st);
-    if (n_one > 0)
-      return launch_tcq<64, false, 2>(s, w, q, k, v, out, seqs, theta, init, shape, reverse, n_one, st);
-    return launch_tcq<64, false, 0>(s, w, q, k, v, out, seqs, theta, init, shape, reverse, 0, st);
+    n_one[i] = (int)n1;
+    all_one = all_one && n1 >= nqt;
+    all_two = all_two && n1 == 0;
   }
-  if (s.d == 128)
-    return key_deltas
-               ? launch_tcq<128, true, 0>(s, w, q, k, v, out, seqs, theta, init, shape, reverse, 0, st)
-               : launch_tcq<128, false, 0>(s, w, q, k, v, out, seqs, theta, init, shape, reverse, 0, st);
+#define GO(DD, K, F) return launch_tcq<DD, K, F>(s, w, q, k, v, out, seqs, n_one, theta, init, shape, reverse, st)
+  if (s.d == 64) {
+    if (key_deltas) {
+      if (all_one) GO(64, true, 0);
+      if (all_two) GO(64, true, 1);
+      GO(64, true, 2);
+    }
+    if (all_one) GO(64, false, 0);
+    if (all_two) GO(64, false, 1);
+    GO(64, false, 2);
+  }
+  if (s.d == 128) {
+    if (key_deltas) GO(128, true, 0);
+    GO(128, false, 0);
+  }
+#undef GO
   return cudaErrorNotSupported;
 }
 
