@@ -10,7 +10,9 @@ threshold that gives about 60 % delta sparsity on the synthetic AR(1) streams.  
 step (cache prefilled to 2048 tokens, 256 steps, batch 1 and 16) is a different workload and
 is timed in its own region of the same run; it is reported under "decode".
 
-Rank 0 prints one JSON line.  With N > 1 every rank runs an independent replica of the
+Rank 0 prints one JSON line on stdout: the contract's keys, the rooflines, the end-to-end and CPU figures and
+the decode times.  The secondary legs in full (kernel variants, threshold sweep, decode, key deltas, window
+grid, larger configurations) go to stderr, one JSON line each, and with --report FILE into a file.  With N > 1 every rank runs an independent replica of the
 workload (different seed): the path shards over (batch, KV-head group, layer) with no
 exchange step, so there is no collective on the data path ("scaling": "weak").
 """
@@ -277,6 +279,30 @@ def k2_roofline(w, stats, kernel, k2_ms, peaks, n_sm, sustained=False):
 
 
 
+SECONDARY_LEGS = ("kernel_variants", "theta_sweep", "decode", "key_deltas", "strategies", "window_grid",
+                  "delta_pass_large", "configs")
+
+
+def headline(report: dict) -> dict:
+    """The stdout line of a full report: the secondary legs left out (whoever keeps a run's tail has to find the
+    whole line in it), of the decode leg the times per step."""
+    line = {k: v for k, v in report.items() if k not in SECONDARY_LEGS}
+    times = ("us_per_step_eager", "us_per_step_graph", "us_per_step_l2_flushed", "us_per_step_l2_flushed_by_read")
+    if "decode" in report:
+        line["decode"] = {batch: {t: leg.get(t) for t in times} for batch, leg in report["decode"].items()}
+    return line
+
+
+def print_report(report: dict, path: str = "") -> None:
+    for leg in SECONDARY_LEGS:
+        if leg in report:
+            print(json.dumps({"leg": leg, "result": report[leg]}), file=sys.stderr, flush=True)
+    if path:
+        with open(path, "w") as f:
+            json.dump(report, f, indent=1)
+    print(json.dumps(headline(report)), flush=True)
+
+
 def replica_layer(rank: int) -> int:
     """Input stream of a rank: every rank is an independent replica with its own seeds
     (workloads.make_qkv's `layer` argument), so N ranks do N times the work."""
@@ -431,7 +457,7 @@ def run_ours(args):
                                        "algorithmic_bytes_per_step": d16["algorithmic_bytes_per_step"],
                                        "note": "L2 flushed (256 MiB write) before every step, each step timed alone by events"}
         line["cpu_baseline"] = run_cpu_baseline(args, w, tens, theta)
-    print(json.dumps(line))
+    print_report(line, args.report)
     if dist is not None:
         dist.barrier()
         dist.destroy_process_group()
@@ -980,6 +1006,7 @@ def main():
     ap.add_argument("--theta", type=float, default=HEADLINE_THETA)
     ap.add_argument("--kernel", type=int, default=-1, help="-1 auto, 0 fp32 arithmetic, 1 tcgen05 + FP32 delta path, 2 tcgen05 telescoped")
     ap.add_argument("--quick", action="store_true", help="prefill timing only (used for ncu launch lists)")
+    ap.add_argument("--report", default="", help="file for the full report, secondary legs included")
     ap.add_argument("--only", default="", choices=["", "decode_b1", "decode_b16", "stack_layer", "stack", "bitnet"],
                     help="run one secondary leg alone on one GPU (small ncu captures of its kernels)")
     ap.add_argument("--ref-heads", type=int, default=4, help="heads per reference step")
