@@ -39,7 +39,7 @@ FLUSH_BYTES = 256 << 20       # > 126 MB of L2, written between timed iterations
 FALLBACK_PEAKS = {"hbm_gbs": 6650.0, "bf16_tflops": 1590.0, "bf16_tflops_sustained": 1400.0,
                   "sm_max_mhz": 1965.0}
 TRAFFIC_FILE = os.path.join(ROOT, "profiles", "hybrid_attn_dram_traffic.txt")
-KERNEL_SOURCES = {2: "k2_hybrid_attn_tcq.cu", 1: "k2_hybrid_attn_tc.cu", 0: "k2_hybrid_attn_generic.cu"}
+KERNEL_SOURCES = {2: "k2_hybrid_attn_tcq.cu", 1: "k2_hybrid_attn_tc.cu", 0: "k2_hybrid_attn_f32.cu"}
 
 
 def kernel_source_digest(kernel: int) -> str:

@@ -17,7 +17,7 @@ LIB_DEBUG = os.path.join(HERE, "libdelta_attn_dbg.so")      # the same sources w
 # interpreter's ABI tag and another version of Python builds its own
 CALLS = os.path.join(HERE, "_calls" + sysconfig.get_config_var("EXT_SUFFIX"))
 CALLS_SOURCE = "py_calls.cpp"
-SOURCES = ["api.cu", "k1_delta_construct.cu", "k2_hybrid_attn_generic.cu", "k2_hybrid_attn_tc.cu", "k2_hybrid_attn_tcq.cu",
+SOURCES = ["api.cu", "k1_delta_construct.cu", "k2_hybrid_attn_f32.cu", "k2_hybrid_attn_tc.cu", "k2_hybrid_attn_tcq.cu",
            "k3_decode_step.cu", "k3_decode_step_mma.cu", "k3_decode_step_f32.cu", "k3_decode_step_key.cu", "k1_pack_keys.cu", "decode_noalloc.cu"]
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
               "-Xcompiler", "-fPIC", "-Xcompiler", "-fvisibility=hidden", "-DDELTA_BUILDING_LIB"]

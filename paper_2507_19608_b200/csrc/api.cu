@@ -42,7 +42,7 @@ struct delta_state {
   std::vector<int> n_b;   // tokens seen per batch element
   bool ragged = false;    // the batch elements stand at different positions
   int qhat_sel;  // which q_hat buffer is current
-  int forced_kernel;  // -1 auto, 0 generic, 1 tensor-core
+  int forced_kernel;  // -1 auto, else a kernel of delta_state_set_prefill_kernel
   // Eq. 6 bookkeeping that needs no device work: sum of window lengths and sequence lengths
   double win_sum[2], len_sum[2];
   DecodeTmapCache dec_maps[3];     // tensor maps of the key, value and reference-key caches the decode steps read
@@ -398,7 +398,7 @@ static delta_status_t prefill_launch(delta_state* st, const Shape& shape, const 
     if (tcq)
       return launch_hybrid_attn_tcq(shape, ws, q, k, v, out, seqs, theta, c.init, c.prefill_window, key,
                                     rev, /*form=*/which == 3 ? 1 : which == 4 ? 2 : which == 5 ? 3 : 0, cs);
-    return launch_hybrid_attn_generic(shape, ws, q, k, v, out, seqs, theta, c.init, c.prefill_window, c.dtype, cs);
+    return launch_hybrid_attn_f32(shape, ws, q, k, v, out, seqs, theta, c.init, c.prefill_window, c.dtype, cs);
   };
   if (chained && !key) {
     if ((e = attention()) != cudaSuccess) return cuda_fail(e);

@@ -124,8 +124,9 @@ int device_sm_count();
 cudaError_t launch_delta_finish(const Shape& s, const Workspace& w, const void* q, const void* k, const SeqBatch& seqs,
                                 float theta, int shape, int dtype, int init, bool want_kt,
                                 bool key_stream, bool reverse, int programmatic, cudaStream_t st);
-// K2 on the FP32 pipes, either dtype; reads the chain kernel's checkpoints and nothing of the finish kernel's.
-cudaError_t launch_hybrid_attn_generic(const Shape& s, const Workspace& w, const void* q, const void* k, const void* v,
+// K2 at fp32 precision (three-part bf16 products on the tensor cores), either dtype; reads the chain kernel's
+// checkpoints and nothing of the finish kernel's.
+cudaError_t launch_hybrid_attn_f32(const Shape& s, const Workspace& w, const void* q, const void* k, const void* v,
                                        void* out, const SeqBatch& seqs, float theta, int init, int shape, int dtype,
                                        cudaStream_t st);
 // K3: one decode step.
@@ -188,12 +189,8 @@ template <> __device__ __forceinline__ __nv_bfloat16 from_f32<__nv_bfloat16>(flo
   return __float2bfloat16_rn(x);
 }
 
-// Is the causal pair (i, j <= i) inside the exact window?  shape: 0 block, 1 sliding.
-__host__ __device__ __forceinline__ bool in_window(int i, int j, int W, int shape) {
-  if (W <= 0) return false;
-  return shape == 0 ? (i / W) == (j / W) : (i - j) < W;
-}
-// Number of in-window keys of query row i.
+// Number of in-window keys of query row i.  The causal pair (i, j <= i) is inside the exact window iff
+// i / W == j / W (shape 0, block) or i - j < W (shape 1, sliding).
 __host__ __device__ __forceinline__ int in_window_count(int i, int W, int shape) {
   if (W <= 0) return 0;
   return shape == 0 ? (i % W) + 1 : (i + 1 < W ? i + 1 : W);

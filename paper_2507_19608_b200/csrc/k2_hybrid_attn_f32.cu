@@ -523,7 +523,7 @@ static cudaError_t launch_f32_form(const Shape& s, const Workspace& w, const voi
 #undef GO
 }
 
-cudaError_t launch_hybrid_attn_generic(const Shape& s, const Workspace& w, const void* q, const void* k, const void* v,
+cudaError_t launch_hybrid_attn_f32(const Shape& s, const Workspace& w, const void* q, const void* k, const void* v,
                                        void* out, const SeqBatch& seqs, float theta, int init, int shape, int dtype,
                                        cudaStream_t st) {
 #define GO(TIN, DD) return launch_f32_form<TIN, DD>(s, w, q, k, v, out, seqs, theta, init, shape, st)

@@ -12,16 +12,18 @@
 // Organisation.  One CTA owns one 128-row query tile of one head and walks its key tiles up to
 // the diagonal; the key tiles are dealt alternately to two groups of softmax warps, each with
 // its own score buffer, running maximum, row sum and output tile in tensor memory (the two
-// partial results are merged once, at the end).  Ten warps:
+// partial results are merged once, at the end).  Where heads of a KV group share a CTA (d = 64), each
+// group takes every key tile for a head of its own and there is no merge.  Eleven warps:
 //   warps 0-3  softmax of the even key tiles, warps 4-7 of the odd ones: ONE THREAD PER SCORE
 //              ROW.  A thread reads its 128 scores of a key tile out of tensor memory, takes the
 //              row maximum and the exponentials without talking to any other thread, and writes
 //              the probabilities back into tensor memory as bf16, over the scores it has read;
-//   warp 8     one thread issues the score products S = Q_hat.K^T (A and B operands in shared
-//              memory); warp 9: one thread issues O += P.V with P read from tensor memory (for
-//              d = 128, where P lies over S, warp 8 issues both in turn);
+//   warp 8     issues the score products S = Q_hat.K^T (A and B operands in shared memory); warp 9
+//              issues O += P.V with P read from tensor memory (for d = 128, where P lies over S,
+//              warp 8 issues both in turn).  The whole warp runs the issuing loop, one lane's products
+//              and commits count (tc_common.cuh has the reason);
 //   warp 10    one thread streams key and value tiles by TMA through a ring of stages.
-
+//
 // The output tiles stay in tensor memory for the whole key loop (the products accumulate);
 // a row is rescaled only when its running maximum has grown by more than 2^8 since the scale
 // it is stored at, by the softmax thread that owns the row.  While one group exponentiates,
@@ -293,9 +295,9 @@ hybrid_attn_tcq_kernel(const __grid_constant__ TqMapList<N> maps, const __grid_c
   auto tile_of = [&](int u) -> int { return pr ? (u >> 1) : u; };
   // d = 128 fills tensor memory with two score buffers and two output tiles: the probabilities
   // overwrite the scores they come from and a group's next score product has to follow its
-  // P.V (one issuing thread does both).  d = 64 leaves room for the probabilities beside the
+  // P.V (one issuing warp does both).  d = 64 leaves room for the probabilities beside the
   // scores: the next score product is issued as soon as the group has read the buffer, by a
-  // thread of its own, while another thread issues the P.V products.
+  // warp of its own, while another one issues the P.V products.
   constexpr bool ALIAS = (D == 128);
 
   if (warp == 0) {

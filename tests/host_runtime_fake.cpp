@@ -88,7 +88,7 @@ cudaError_t launch_hybrid_attn_tcq(const Shape& s, const Workspace&, const void*
                                    float, int, int, bool, bool, int, cudaStream_t) {
   return call("attn", num("heads", s.B * s.H) + num("form_heads", q.form_heads(s)));
 }
-cudaError_t launch_hybrid_attn_generic(const Shape& s, const Workspace&, const void*, const void*, const void*, void*,
+cudaError_t launch_hybrid_attn_f32(const Shape& s, const Workspace&, const void*, const void*, const void*, void*,
                                        const SeqBatch& q, float, int, int, int, cudaStream_t) {
   return call("attn", num("heads", s.B * s.H) + num("form_heads", q.form_heads(s)));
 }
