@@ -159,8 +159,8 @@ DELTA_API delta_status_t delta_attn_prefill(delta_state_t* st, const void* q, co
  * window, counters (Eq. 6 sums over the sequences: S_c_eq6 uses sum min(W_b, n_b) / sum n_b) and
  * decode hand-off.  Afterwards the batch elements stand at different positions:
  * delta_state_sequence_position reports each, delta_state_position the longest, and
- * delta_attn_decode_step advances every sequence by one token from where it stands (in one launch
- * where delta_state_decode_kernel reports 1 and the compressed key cache is off).  Needs a fresh or reset state. */
+ * delta_attn_decode_step advances every sequence by one token from where it stands (one launch for up to 64
+ * sequences; one per sequence where a stepwise kernel is forced).  Needs a fresh or reset state. */
 DELTA_API delta_status_t delta_attn_prefill_varlen(delta_state_t* st, const void* q, const void* k, const void* v,
                                          void* out, const int32_t* seq_lens, const int32_t* windows,
                                          float theta, void* stream);
@@ -185,10 +185,12 @@ DELTA_API delta_status_t delta_attn_prefill_host(delta_state_t* st, const void* 
  * that arrives now; score j is q_new.k_j if n - j < window else R[j]; softmax over the n + 1
  * keys; out = P.V; position becomes n + 1.  Needs n >= 1 (else DELTA_ERR_STATE) and
  * n < T_max (else DELTA_ERR_CAPACITY).
- * Eq. 4's sum telescopes to R[j] = q_hat . k_j (exactly, up to the order of the fp32
- * additions, for bf16 inputs, whose references are copies of input elements); where
- * delta_state_decode_kernel reports 1 the step computes R[j] in that form on the tensor cores
- * and writes it back without reading it.
+ * Eq. 4's sum telescopes to R[j] = q_hat . k_j (up to fp32 rounding, of which this form has less: the
+ * references are copies of input elements, no rounded differences are added up); the step computes R[j] in that form, on the
+ * tensor cores for bf16 and on the FP32 pipes for fp32 inputs, and writes it without reading it.  (The
+ * stepwise kernels that delta_state_set_decode_kernel(st, 0) forces update it in place.)
+ * Rounding: how the keys are dealt to CTAs and warps follows B, H_kv, d and the longest sequence, so the same
+ * sequence in different batches agrees to the order of the fp32 additions.
  * All six tensor pointers must be 16-byte aligned (the kernels stage cache tiles with bulk
  * copies and read rows as 16-byte vectors): DELTA_ERR_INVALID_ARG otherwise, nothing launched.
  * With DELTA_SRC_KEY the step thresholds k_new against the carried reference key instead
@@ -306,7 +308,8 @@ DELTA_API int32_t delta_state_sequence_position(const delta_state_t* st, int32_t
  *       A CTA takes one head's query tile and splits its key tiles between two softmax
  *       groups, or (d = 64 with an even number of query heads per KV head)
  *       the same query tile of two heads of a KV group, so that every key and value tile
- *       is fetched once for both; which CTAs take which form follows the size of the grid;
+ *       is fetched once for both; which CTAs take which form follows the size of the call's grid (of
+ *       each sequence's own in delta_attn_prefill_varlen);
  *   3 = kernel 2 with every CTA in the one-head form, 4 = every CTA in the two-heads form,
  *   5 = the two-heads form with the heaviest query tile of every head in the one-head form
  *       (3 to 5 are never chosen as such; for comparison and tests).
@@ -338,7 +341,7 @@ DELTA_API delta_status_t delta_state_set_prefill_kernel(delta_state_t* st, int32
  *     and the offsets of those 32-row segments; a decode step rebuilds the reference-key rows of
  *     a tile in shared memory from that.  The keys inside the decode window are read from
  *     k_cache.  Same results bit for bit; the bytes a step reads for the keys shrink with the
- *     delta sparsity (delta_key_cache_bytes), the step itself runs on the FP32 pipes.
+ *     delta sparsity (delta_key_cache_bytes); the products run on the tensor cores as from dense rows.
  * Set it on a fresh or reset state (DELTA_ERR_STATE otherwise): the prefill builds the encoding.
  * The workspace reserves the packed pool for the worst case (every element fires) beside the
  * dense rows the prefill kernel streams, so the choice changes what decoding reads, not what

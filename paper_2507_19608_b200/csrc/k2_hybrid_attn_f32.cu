@@ -14,7 +14,9 @@
 // pipes, whose 74 TFLOP/s a fused kernel reaches to a quarter (each 16-byte shared-memory operand feeds
 // few multiply-adds): the same kernel on packed fma.rn.f32x2 ran at 20 TFLOP/s, the kernel before it,
 // sparse delta sums on the FP32 pipes, at 6.  Relative error against fp64 dense attention at 1000
-// tokens: 1.8e-7 (FP32-pipe kernel 3.7e-7).  Measured, whole prefill: 24 heads x 1425 tokens, d = 64:
+// tokens: 1.8e-7 (FP32-pipe kernel 3.7e-7).  mma.sync and not tcgen05: accumulators in registers make the
+// separate small-product sums and the per-tile fresh output sums free to join in fp32, and no key tile waits
+// for a hand-over through tensor memory; whether tcgen05 at the same precision would pay has not been measured.  Measured, whole prefill: 24 heads x 1425 tokens, d = 64:
 // 212 us = 29 TFLOP/s; 16 heads x 1000: 350 -> 95 us; one head x 128: 54 -> 13 us (the kernel 42 -> 6).
 //
 // Bound: mma.sync issue (m16n8k16 every 8 clocks per scheduler) once the chip is full, the walk of the
@@ -472,7 +474,12 @@ static cudaError_t launch_f32(K kern, std::atomic<uint64_t>& ready, size_t smem,
 // Warps per row group for `heads` heads of T tokens.  A key tile of 64 costs 3.3 / 2.2 / 1.4 us where a CTA
 // walks alone and takes 4.0 / 2.2 / 1.6 us of an SM where the chip is full (KS = 1 / 2 / 4; d = 64, 1 to
 // 256 heads of 128 to 4000 tokens); every halving of the rows doubles the tiles.  The longest walk bounds a
-// small grid, the sum of all tiles, with half a walk for the uneven end, a large one.  A sequence of a
+// small grid, the sum of all tiles, with half a walk for the uneven end, a large one.  Only the ratios count,
+// and they carry over to d = 128 (one CTA per SM, two to three times the time) and to bf16 inputs: with each
+// form timed at 1 to 128 heads of 128 to 4000 tokens (30 shapes per type and d) the chosen one is the
+// fastest or, fp32, within 6 % of it (64 or 128 heads of 128 tokens: 10 to 15 %); bf16, which runs here only
+// when kernel 0 is forced, within 16 % (there: 23 %).  16 heads x 1000, d = 64 / 128, KS = 1, 2, 4: 82, 81, 92 us
+// / 185, 170, 207; 32 x 2000: 375, 408, 521 / 930, 988, 1306.  A sequence of a
 // ragged group takes the form of a batch of its own (the forms round differently: its result does not
 // depend on the sequences beside it).
 static int f32_form(long heads, int T) {
