@@ -281,6 +281,7 @@ delta_status_t delta_key_cache_bytes(const delta_state_t* st, uint64_t* packed_b
   uint64_t packed = 0, dense = 0;
   for (int b = 0; b < c.B; ++b) {
     const uint64_t rows = (uint64_t)st->n_b[(size_t)b], segs = (rows + 31) / 32;
+    if (rows == 0) continue;         // nothing encoded yet; the device word is an earlier prompt's, or unset
     for (int h = 0; h < c.H_kv; ++h)
       packed += 2ull * used[(size_t)b * c.H_kv + h]            // values (with the segments' padding)
                 + rows * (uint64_t)(c.d / 8)                    // mask words

@@ -2,6 +2,7 @@
 // tests of its host side without a GPU: every call is written to a log, a named call can be made to
 // fail, and the current device is what the test says.
 #include <cstdio>
+#include <cstring>
 #include <map>
 #include <mutex>
 #include <string>
@@ -13,7 +14,7 @@ namespace {
 std::mutex g_mu;
 std::string g_log;
 std::map<std::string, int> g_fail;      // call -> error of its next run
-int g_device = 0, g_capturing = 0;
+int g_device = 0, g_capturing = 0, g_fill = -1;
 size_t g_handle = 0x1000;
 
 cudaError_t call(const char* name, const std::string& args = "") {
@@ -38,6 +39,7 @@ extern "C" {
 EXPORT const char* fake_log() { return g_log.c_str(); }
 EXPORT void fake_clear() { g_log.clear(); g_fail.clear(); }
 EXPORT void fake_fail(const char* name, int error) { g_fail[name] = error; }
+EXPORT void fake_fill(int byte) { g_fill = byte; }      // what copies leave at their destination (-1: nothing)
 EXPORT void fake_capturing(int on) { g_capturing = on; }
 EXPORT void fake_device(int dev) { g_device = dev; }
 
@@ -49,7 +51,10 @@ const char* cudaGetErrorString(cudaError_t e) {
 }
 cudaError_t cudaGetDevice(int* dev) { *dev = g_device; return cudaSuccess; }
 cudaError_t cudaMemsetAsync(void*, int, size_t, cudaStream_t) { return call("memset"); }
-cudaError_t cudaMemcpyAsync(void*, const void*, size_t, cudaMemcpyKind kind, cudaStream_t) { return call("memcpy", num("kind", kind)); }
+cudaError_t cudaMemcpyAsync(void* dst, const void*, size_t n, cudaMemcpyKind kind, cudaStream_t) {
+  if (g_fill >= 0) memset(dst, g_fill, n);
+  return call("memcpy", num("kind", kind));
+}
 cudaError_t cudaMemcpy2DAsync(void*, size_t, const void*, size_t, size_t, size_t, cudaMemcpyKind kind, cudaStream_t) {
   return call("memcpy", num("kind", kind));
 }

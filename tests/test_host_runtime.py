@@ -140,3 +140,14 @@ def test_a_call_in_parts_takes_the_form_of_the_whole_call(fake, Bn, H, H_kv, dty
     h = Host(fake, H=H, H_kv=H_kv, Bn=Bn, dtype=dtype)
     assert h.prefill_host() == 0
     assert [x for x in h.call_log() if x.startswith("attn")] == [f"attn heads={n} form_heads={Bn * H}" for n in parts]
+
+
+def test_compressed_cache_bytes_are_zero_before_a_prefill(fake):
+    """The fill words on the device are an earlier prompt's, or unset, until a prefill has written them."""
+    h = Host(fake, source=B.DELTA_SRC_KEY)
+    assert fake.delta_state_set_key_cache(h.st, 1) == 0
+    packed, dense = C.c_uint64(7), C.c_uint64(7)
+    fake.fake_fill(0x5a)
+    status = fake.delta_key_cache_bytes(h.st, C.byref(packed), C.byref(dense), None)
+    fake.fake_fill(-1)
+    assert (status, packed.value, dense.value) == (0, 0, 0)
