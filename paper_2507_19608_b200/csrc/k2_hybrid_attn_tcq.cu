@@ -38,8 +38,7 @@
 // hand-overs per tile, and the register allocator finds room without a spill.  (Against handing a
 // half that is held in registers back for its exact product, three hand-overs and spills in every
 // tile of the launch: 4 x 32 heads, 1777 keys, key deltas, sliding window of 100 174 -> 133 us, no
-// window 109; 32 heads, 1900 keys, block window of 95 65 -> 56 us, of 64 51; six ragged sequences
-// of 99 to 1900 keys with windows of 4 to 95 167 -> 134 us.)  d = 128 has the probabilities over the
+// window 109; 32 heads, 1900 keys, block window of 95 65 -> 56 us, of 64 51.)  d = 128 has the probabilities over the
 // scores and no such room: it hands the half back.
 //
 // Head dimensions 64 and 128 (template parameter).
@@ -130,16 +129,18 @@ struct TqParams {
   const float* ckpt;           // [B,H,n_ckpt,D] reference in front of every 8-row block (query deltas only)
   int T_max, n_ckpt, H, g, shape;
   int BH;            // heads of one entry of the sequence list (uniform batch: batch x query heads)
+  int nqt;           // uniform batch: its query tiles
+  int n_one;         // ... and, two-head layout, how many of the heaviest ones of every head go one head per CTA
   int reverse;       // strategy (2): Eq. 2-3 runs from row T-1 down to row 0
   int basis;         // is the first row taken (0, or T-1 in reverse) the un-thresholded basis?
   float scale_log2e, theta;
 };
 
-// One entry of the sequence list: tensor maps of queries, reference-key rows, keys, values (rows
-// 0..T-1), its first CTA in the grid (INT_MAX: no entry), its query tiles and, two-head layout, how many
-// of the heaviest ones of every head go one head per CTA.
-struct TqMaps { CUtensorMap q, qh, k, v; int first, nqt, n_one; };
-template <int N> struct TqMapList { TqMaps m[N]; };
+// Tensor maps of one entry of the sequence list: queries, reference-key rows, keys, values (rows 0..T-1).
+struct TqMaps { CUtensorMap q, qh, k, v; };
+// The entries; of a ragged group also each one's first CTA in the grid (INT_MAX: no entry) and its n_one.
+template <int N> struct TqMapList { TqMaps m[N]; int first[N], n_one[N]; };
+template <> struct TqMapList<1> { TqMaps m[1]; };
 
 // Barrier of the eight softmax warps (id 1, 256 threads; immediate id: a register operand would
 // make the compiler reserve all sixteen hardware barriers).
@@ -260,14 +261,17 @@ hybrid_attn_tcq_kernel(const __grid_constant__ TqMapList<N> maps, const __grid_c
   // second kind.
   int qt, bh, si = 0;
   bool pr = false;
-  if (N > 1) {
+  int nqt = p.nqt, n_one = (FORM == 1) ? 0 : p.n_one, idx = (int)blockIdx.x;
+  if constexpr (N > 1) {
 #pragma unroll
-    for (int i = 1; i < N; ++i) si = (int)blockIdx.x >= maps.m[i].first ? i : si;
+    for (int i = 1; i < N; ++i) si = idx >= maps.first[i] ? i : si;
+    nqt = (seqs.s[si].T + BM - 1) / BM;
+    n_one = maps.n_one[si];
+    idx -= maps.first[si];
   }
-  {
-    const int nqt = maps.m[si].nqt, idx = (int)blockIdx.x - (N > 1 ? maps.m[si].first : 0);
-    const int n_one = FORM == 0 ? nqt : FORM == 1 ? 0 : maps.m[si].n_one, n1 = p.BH * n_one;
-    if (FORM != 1 && (FORM == 0 || idx < n1)) {
+  if (PAIR) {
+    const int n1 = (FORM == 1) ? 0 : p.BH * n_one;
+    if (FORM == 2 && idx < n1) {
       qt = nqt - 1 - idx / p.BH;
       bh = idx % p.BH;
     } else {
@@ -276,6 +280,12 @@ hybrid_attn_tcq_kernel(const __grid_constant__ TqMapList<N> maps, const __grid_c
       qt = nqt - n_one - 1 - j / hp;
       bh = 2 * (j % hp);
     }
+  } else if (N > 1) {
+    qt = nqt - 1 - idx / p.BH;
+    bh = idx % p.BH;
+  } else {
+    qt = (int)gridDim.y - 1 - (int)blockIdx.y;
+    bh = (int)blockIdx.x;
   }
   // (bh, bkv: head and KV head within the entry of the sequence list; g_bh: of the workspace arrays)
   const int b = bh / p.H, h = bh - b * p.H;
@@ -976,16 +986,18 @@ static cudaError_t launch_tcq_m(const Shape& s, const Workspace& w, const void* 
     order[at] = i;
   }
   int ctas = 0;
+  TqParams p;
   for (int i = 0; i < seqs.n; ++i) {
     const Seq& e = seqs.s[order[i]];
     const uint64_t T = (uint64_t)e.T;
     const size_t kv = (size_t)e.b * s.H_kv * s.T_max * D, rf = (size_t)e.b * (KEY ? s.H_kv : s.H) * s.T_max * D;
     TqMaps& m = maps.m[i];
     list.s[i] = e;
-    m.first = ctas;
-    m.nqt = (e.T + BM - 1) / BM;
-    m.n_one = FORM == 0 ? m.nqt : FORM == 1 ? 0 : n_one[order[i]] < m.nqt ? n_one[order[i]] : m.nqt;
-    ctas += (int)BH * m.n_one + (int)(BH / 2) * (m.nqt - m.n_one);
+    const int nqt = (e.T + BM - 1) / BM;
+    const int n1 = FORM == 0 ? nqt : FORM == 1 ? 0 : n_one[order[i]] < nqt ? n_one[order[i]] : nqt;
+    if constexpr (N > 1) { maps.first[i] = ctas; maps.n_one[i] = n1; }
+    p.nqt = nqt; p.n_one = n1;               // (uniform batch)
+    ctas += (int)BH * n1 + (int)(BH / 2) * (nqt - n1);
     const uint64_t cache = (uint64_t)s.T_max * D * 2;
     if (!encode3(&m.q, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, (const TC*)q + e.q_off, D, T, BH, D * 2, T * D * 2, 64, 128,
                  CU_TENSOR_MAP_SWIZZLE_128B) ||
@@ -997,14 +1009,14 @@ static cudaError_t launch_tcq_m(const Shape& s, const Workspace& w, const void* 
                          CU_TENSOR_MAP_SWIZZLE_128B)))
       return cudaErrorInvalidValue;
   }
-  for (int i = seqs.n; i < N; ++i) { list.s[i] = list.s[0]; maps.m[i].first = INT_MAX; }
+  if constexpr (N > 1)
+    for (int i = seqs.n; i < N; ++i) { list.s[i] = list.s[0]; maps.first[i] = INT_MAX; maps.n_one[i] = 0; }
   static std::atomic<uint64_t> ready{0};
   if (!device_done(ready)) {
     const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TqSmem<D, PAIR>::BYTES);
     if (e != cudaSuccess) return e;
     device_mark(ready);
   }
-  TqParams p;
   p.out = (__nv_bfloat16*)out;
   p.counters = w.counters;
   p.ckpt = w.ckpt;
@@ -1019,7 +1031,7 @@ static cudaError_t launch_tcq_m(const Shape& s, const Workspace& w, const void* 
   // griddepcontrol.wait.
   cudaLaunchConfig_t cfg = {};
   p.BH = (int)BH;
-  cfg.gridDim = dim3((unsigned)ctas);
+  cfg.gridDim = (PAIR || N > 1) ? dim3((unsigned)ctas) : dim3((unsigned)BH, (unsigned)p.nqt);
   cfg.blockDim = dim3(NTHR);
   cfg.dynamicSmemBytes = TqSmem<D, PAIR>::BYTES;
   cfg.stream = st;
@@ -1071,7 +1083,9 @@ cudaError_t launch_hybrid_attn_tcq(const Shape& s, const Workspace& w, const voi
   // On a smaller grid that the one-head form cannot place in one wave, the heaviest query
   // tiles of every head go one head per CTA and the rest two heads per CTA, as many of the
   // former as one wave of SMs allows.  The forms round differently: a sequence of a ragged group takes the
-  // form of a batch of its own, so that its result does not depend on the sequences beside it.
+  // form of a batch of its own, so that its result does not depend on the sequences beside it.  (Two heads per
+  // CTA throughout, by the size of the group, is faster: six sequences of 99 to 1900 tokens, 32 heads, with 24
+  // steps behind them 292 us, so 305.)
   const long BH = seqs.form_heads(s), sms = device_sm_count();
   int n_one[kSeqMax];                     // query tiles of every head in the one-head form
   bool all_one = true, all_two = true;
