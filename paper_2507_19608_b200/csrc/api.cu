@@ -651,15 +651,18 @@ delta_status_t delta_attn_prefill_host(delta_state_t* st, const void* q_host, co
   // The call is bound by PCIe (6.3 MB up and 4.2 MB down around 35 us of kernels at the Llama layer; 51 GB/s
   // one way, 80 both ways together): keys and values come up first, then the queries in chunks of KV
   // heads, and while a chunk is computed on the caller's stream the next one comes up on a stream of
-  // the pool and the last one's output goes down on another.  At most four chunks of at least a
-  // megabyte: a small copy beside one in the other direction waits for it (queries, keys and values in
-  // chunks: 275 us).  Llama layer, 1024 tokens: 252 us in one piece, 225 so; batch 4: 860, 723.
+  // the pool and the last one's output goes down on another.  Two chunks from 1.25 MB of queries on, four
+  // above 4.5 MB: the kernels of a chunk are one latency (the chain, then the heaviest query tile), so more chunks
+  // than the copies need lengthen the call, and a small copy beside one in the other direction waits for it
+  // (queries, keys and values in chunks: 275 us).  us with 1, 2, 3, 4 chunks, 32 heads over 8 KV heads: 1.0 MB
+  // 91, 91, 94, 101; 1.4 110, 106, 109, 117; 2.5 183, 152, 158, 162; 4.0 (Llama layer, 1024 tokens) 252, 220,
+  // 225, 233; 4.7 331, 272, 263, 244; 6.6 404, 349, 353, 323; 16 861, 719, 704, 720; 20 heads, d = 128, 2.5 MB 195,
+  // 162, 164, 170; 7.3 428, 388, 387, 371.
   const int units = c.B * c.H_kv;
   const size_t es2 = (size_t)c.d * es, g = c.H / c.H_kv;
-  int chunks = (int)(q_bytes >> 20);
-  if (chunks > kTransferChunks) chunks = kTransferChunks;
+  int chunks = q_bytes > (9u << 19) ? kTransferChunks : q_bytes >= (5u << 18) ? 2 : 1;
   if (chunks > units) chunks = units;
-  if (chunks < 1 || st->profiling) chunks = 1;
+  if (st->profiling) chunks = 1;
   // (one chunk: all on the caller's stream, nothing to overlap)
   TransferGuard tg;
   e = chunks > 1 ? tg.open() : cudaSuccess;

@@ -1,5 +1,5 @@
 """The host-buffer prefill in chunks of KV heads: same output bit for bit, delta arrays and counters as the device call,
-for one to four chunks (uneven ones included), every source, both cache layouts, pinned and pageable
+for one, two and four chunks (uneven ones included), every source, both cache layouts, pinned and pageable
 buffers, and from several host threads at once."""
 import threading
 
@@ -50,7 +50,8 @@ def _both(B, Bn, H, Hk, d, T, T_max, source, dtype, seed, pinned=True, stream=No
     (1, 4, 1, 64, 100, 100, "query", "bf16"), (1, 32, 8, 64, 1024, 1024, "query", "bf16"),
     (1, 20, 5, 128, 900, 950, "query", "bf16"), (3, 6, 3, 64, 1500, 1503, "key", "bf16"),
     (2, 12, 3, 64, 1300, 1310, "key_packed", "bf16"), (1, 14, 7, 64, 1111, 1111, "bottom_up", "bf16"),
-    (1, 8, 8, 64, 700, 701, "query", "f32"), (4, 32, 8, 64, 1024, 1030, "query", "bf16")])
+    (1, 8, 8, 64, 700, 701, "query", "f32"), (4, 32, 8, 64, 1024, 1030, "query", "bf16"),
+    (3, 20, 5, 64, 1024, 1030, "query", "bf16"), (3, 12, 3, 128, 1100, 1100, "key_packed", "bf16")])
 def test_host_call_equals_device_call(Bn, H, Hk, d, T, T_max, source, dtype):
     from paper_2507_19608_b200 import binding as B
     _both(B, Bn, H, Hk, d, T, T_max, source, dtype, seed=T)

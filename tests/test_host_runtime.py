@@ -133,7 +133,7 @@ def test_the_reported_decode_kernel_is_the_one_that_runs(fake, source, dtype, pa
     assert [x.split()[0] for x in h.call_log()] == [launched]
 
 
-@pytest.mark.parametrize("Bn,H,H_kv,dtype,parts", [(1, 32, 8, "bf16", [8] * 4), (3, 20, 5, "bf16", [12, 16, 16, 16]),
+@pytest.mark.parametrize("Bn,H,H_kv,dtype,parts", [(1, 32, 8, "bf16", [16] * 2), (3, 20, 5, "bf16", [12, 16, 16, 16]),
                                                    (1, 8, 8, "f32", [4, 4])])
 def test_a_call_in_parts_takes_the_form_of_the_whole_call(fake, Bn, H, H_kv, dtype, parts):
     """The attention kernels round by their form; the host-buffer call cuts a batch and must not change it."""
