@@ -377,7 +377,7 @@ def run_ours(args):
         flush.zero_()
         e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
         e0.record()
-        B.delta_state_reset(st)                 # the memset a fresh sequence needs is part of the step
+        B.delta_state_reset(st)                 # (its clearing is done by the step's first kernel)
         B.delta_attn_prefill(st, q, k, v, out, w.T, w.H, w.H_kv, w.d, theta, w.window)
         e1.record()
         evs.append((e0, e1))

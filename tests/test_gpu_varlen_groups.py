@@ -74,11 +74,15 @@ def test_ragged_call_equals_single_calls(source, dtype, d, g, shape):
     assert [s["prefill"][k] for k in ("nnz", "elements", "macs_done", "macs_dense")] == total and s["device_status"] == 0
 
 
-@pytest.mark.parametrize("source,dtype,H,Hk,lens", [
-    ("query", "bf16", 32, 8, (1024, 2500, 300, 1900, 640)),      # query tiles: 8 (both forms), 20 (two heads), 3, 15, 5 (one)
-    ("key", "bf16", 32, 8, (640, 2433, 1100, 90)), ("bottom_up", "bf16", 32, 16, (1152, 2500, 513)),
-    ("query", "f32", 16, 4, (100, 1500, 500, 1000))])            # 4, 1 and 2 warps per row group
-def test_sequences_of_a_ragged_call_keep_the_form_of_their_own_call(source, dtype, H, Hk, lens):
+@pytest.mark.parametrize("source,dtype,H,Hk,lens,kernel", [
+    # query tiles: 8 (both forms), 20 (two heads), 3, 15, 5 (one)
+    ("query", "bf16", 32, 8, (1024, 2500, 300, 1900, 640), -1),
+    ("key", "bf16", 32, 8, (640, 2433, 1100, 90), -1), ("bottom_up", "bf16", 32, 16, (1152, 2500, 513), -1),
+    ("query", "f32", 16, 4, (100, 1500, 500, 1000), -1),         # 4, 1 and 2 warps per row group
+    # one form forced: one head per CTA, two, both
+    ("query", "bf16", 8, 4, (300, 128, 700), 3), ("query", "bf16", 8, 4, (300, 128, 700), 4),
+    ("query", "bf16", 8, 4, (300, 128, 700), 5), ("key", "bf16", 8, 4, (300, 128, 700), 5)])
+def test_sequences_of_a_ragged_call_keep_the_form_of_their_own_call(source, dtype, H, Hk, lens, kernel):
     """The attention kernels' forms round differently; which one a sequence takes follows its own length and
     heads, so a neighbour never changes its bits (here: each with and without the others)."""
     from paper_2507_19608_b200 import binding as B
@@ -91,10 +95,12 @@ def test_sequences_of_a_ragged_call_keep_the_form_of_their_own_call(source, dtyp
     packed = torch.cat([x.reshape(-1) for x in qs])
     out = torch.full_like(packed, float("nan"))
     st = B.delta_state_init(B.make_config(n, H, Hk, d, T_max, dtype, source=src))
+    B.delta_state_set_prefill_kernel(st, kernel)
     B.delta_attn_prefill_varlen(st, packed, kc, vc, out, lens, wins, 0.6)
     at = 0
     for b, T in enumerate(lens):
         one = B.delta_state_init(B.make_config(1, H, Hk, d, T_max, dtype, source=src))
+        B.delta_state_set_prefill_kernel(one, kernel)
         o = torch.empty_like(qs[b])
         B.delta_attn_prefill(one, qs[b], kc[b], vc[b], o, T, H, Hk, d, 0.6, wins[b])
         assert torch.equal(out[at:at + o.numel()].view_as(o), o), (b, T)
