@@ -657,7 +657,9 @@ __global__ void __launch_bounds__(256, D == 64 ? 5 : 4) delta_finish_kernel(
   // and the blocks run on the SMs the attention kernel's last wave leaves idle.  One thread of the
   // grid waits at its end: a kernel serialised programmatically behind this one (a decode step) waits for
   // this kernel only, and with it has to have waited for the attention kernel's stores too.  (Every
-  // CTA of the attention kernel is resident by then, so nothing can be kept from starting.)
+  // CTA of the attention kernel is resident by then, so nothing can be kept from starting.  It costs up to
+  // 1.1 us where the attention kernel ends last -- three ragged sequences of up to 392 tokens, d = 128:
+  // 22.9 -> 24.1 us; BitNet layer 63.8 -> 64.2 -- and nothing at the Llama layer.)
   if (wait_front) asm volatile("griddepcontrol.wait;" ::: "memory");
   // key deltas: the attention kernel is serialised programmatically behind this one and may set
   // itself up meanwhile (it waits for this kernel's results itself)
