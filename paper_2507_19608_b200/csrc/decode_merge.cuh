@@ -69,6 +69,35 @@ __device__ __forceinline__ int warp_sum(int x) {
   return x;
 }
 
+// The last CTA of a (batch, KV head) to arrive merges the slices' parts in global memory.
+template <typename TO, int D, int G, int MNW>
+__device__ __forceinline__ void merge_global(int ns, int bkv, size_t out0, float* __restrict__ partial, uint32_t* __restrict__ ticket,
+                                             TO* __restrict__ out, int* s_last) {
+  const int tid = threadIdx.x;
+  __threadfence();
+  __syncthreads();
+  if (tid == 0) *s_last = atomicAdd(&ticket[bkv], 1u) == (uint32_t)ns - 1u;
+  __syncthreads();
+  if (!*s_last) return;
+  __threadfence();
+  const float* const pb = partial + (size_t)bkv * kMaxDecodeSplits * G * (D + 2);
+  for (int e = tid; e < G * D; e += 32 * MNW) {
+    const int hh = e / D, c = e - hh * D;
+    float M = -INFINITY, nu = 0.0f, de = 0.0f;
+#pragma unroll 8
+    for (int r = 0; r < ns; ++r) M = fmaxf(M, __ldcg(pb + ((size_t)r * G + hh) * (D + 2) + D));
+#pragma unroll 8
+    for (int r = 0; r < ns; ++r) {
+      const float* const pr = pb + ((size_t)r * G + hh) * (D + 2);
+      const float f = tc::ex2(__ldcg(pr + D) - M);
+      nu = fmaf(f, __ldcg(pr + c), nu);
+      de = fmaf(f, __ldcg(pr + D + 1), de);
+    }
+    out[out0 + (size_t)hh * D + c] = from_f32<TO>(nu / de);
+  }
+  if (tid == 0) ticket[bkv] = 0;                          // ready for the next step
+}
+
 // The finishing half, once all records are there: combine this CTA's blocks and store them, or, where
 // a (batch, KV head) has more slices (ns) than a cluster, leave this slice's part in global memory
 // for the last CTA to arrive.  out0: first output of the group.
@@ -116,31 +145,87 @@ __device__ __forceinline__ void decode_merge(uint32_t recs, uint32_t mls, int ra
   }
   if (CLUSTER || ns == 1) return;
 
-  // ---- the last CTA of the (batch, KV head) to arrive merges the slices
-  __threadfence();
-  __syncthreads();
-  if (tid == 0) *s_last = atomicAdd(&ticket[bkv], 1u) == (uint32_t)ns - 1u;
-  __syncthreads();
-  if (!*s_last) return;
-  __threadfence();
-  const float* const pb = partial + (size_t)bkv * kMaxDecodeSplits * G * (D + 2);
-  for (int e = tid; e < G * D; e += 32 * MNW) {
-    const int hh = e / D, c = e - hh * D;
-    float M = -INFINITY, nu = 0.0f, de = 0.0f;
-#pragma unroll 8
-    for (int r = 0; r < ns; ++r) M = fmaxf(M, __ldcg(pb + ((size_t)r * G + hh) * (D + 2) + D));
-#pragma unroll 8
-    for (int r = 0; r < ns; ++r) {
-      const float* const pr = pb + ((size_t)r * G + hh) * (D + 2);
-      const float f = tc::ex2(__ldcg(pr + D) - M);
-      nu = fmaf(f, __ldcg(pr + c), nu);
-      de = fmaf(f, __ldcg(pr + D + 1), de);
-    }
-    out[out0 + (size_t)hh * D + c] = from_f32<TO>(nu / de);
-  }
-  if (tid == 0) ticket[bkv] = 0;                          // ready for the next step
+  merge_global<TO, D, G, MNW>(ns, bkv, out0, partial, ticket, out, s_last);
 }
 
+// The merge in two steps, for kernels whose warps leave their results as fp32 rows in the CTA's shared memory:
+// every `stride` bytes from part on a warp's [head][D + 8] (8 floats apart: the heads' rows fall on
+// different banks) and behind them its [head] (maximum, row sum).  The CTA combines its warps' parts first and sends one record of 20 floats (16
+// channels of one head, maximum, row sum) per block to the slice that finishes the block.  Sent by every warp
+// instead, a record's five packets per lane queue at the receivers: eight times as many of them.
+// recs: this CTA's records, [slot][slice][REC2]; bar: their barrier.
+constexpr int REC2 = 20;
+template <int D, int G> __host__ __device__ constexpr uint32_t merge_slots(int cs) { return (uint32_t)((G * D / 16 + cs - 1) / cs); }
+template <int D, int G> struct MergePart {
+  static constexpr uint32_t LD = D + 8, ML = G * LD * 4, BYTES = ML + G * 8;
+};
+// The CTA's own parts (all threads, behind a CTA-wide barrier).
+template <typename TO, int D, int G, int MNW, bool CLUSTER>
+__device__ __forceinline__ void merge_warps(uint32_t part, uint32_t stride, uint32_t recs, uint32_t bar, int rank, int cs, int ns, int split,
+                                            int bkv, size_t out0, float* __restrict__ partial, TO* __restrict__ out) {
+  using MP = MergePart<D, G>;
+  constexpr int NTH = 32 * MNW;
+#pragma unroll
+  for (int e0 = 0; e0 < G * D / 4; e0 += NTH) {
+    const int e = e0 + (int)threadIdx.x;
+    if (G * D / 4 % NTH != 0 && e >= G * D / 4) break;
+    const int hh = e / (D / 4), c = 4 * (e % (D / 4));
+    float2 ml[MNW];
+    float4 o[MNW];
+#pragma unroll
+    for (int w = 0; w < MNW; ++w) ml[w] = lds_f2(part + w * stride + MP::ML + hh * 8);
+#pragma unroll
+    for (int w = 0; w < MNW; ++w) o[w] = lds_f4(part + w * stride + (hh * MP::LD + c) * 4);
+    float M = ml[0].x, l = 0.0f;
+#pragma unroll
+    for (int w = 1; w < MNW; ++w) M = fmaxf(M, ml[w].x);
+    float4 a = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    // (a warp without keys: maximum -inf, zeros; a slice without keys: all of them)
+    const float Mf = M == -INFINITY ? 0.0f : M;
+#pragma unroll
+    for (int w = 0; w < MNW; ++w) {
+      const float f = tc::ex2(ml[w].x - Mf);
+      a.x = fmaf(f, o[w].x, a.x); a.y = fmaf(f, o[w].y, a.y); a.z = fmaf(f, o[w].z, a.z); a.w = fmaf(f, o[w].w, a.w);
+      l = fmaf(f, ml[w].y, l);
+    }
+    if (CLUSTER) {
+      const int q = hh * (D / 16) + c / 16, r = q % cs;
+      const uint32_t dst = cluster_map(recs + (uint32_t)((q / cs) * cs + rank) * (REC2 * 4), r), rbar = cluster_map(bar, r);
+      cluster_send4(dst + 4 * (c & 15), rbar, a.x, a.y, a.z, a.w);
+      if ((c & 15) == 0) cluster_send2(dst + 64, rbar, M, l);
+    } else if (ns == 1) {
+      const float inv = 1.0f / l;
+      store4(out + out0 + (size_t)hh * D + c, a.x * inv, a.y * inv, a.z * inv, a.w * inv);
+    } else {
+      // slices through global memory: this slice's part
+      float* const pg = partial + (((size_t)bkv * kMaxDecodeSplits + split) * G + hh) * (D + 2);
+      pg[c] = a.x; pg[c + 1] = a.y; pg[c + 2] = a.z; pg[c + 3] = a.w;
+      if (c == 0) { pg[D] = M; pg[D + 1] = l; }
+    }
+  }
+}
+// The blocks this slice finishes, once the records of every slice are there.
+template <typename TO, int D, int G>
+__device__ __forceinline__ void merge_slices(uint32_t recs, int rank, int cs, size_t out0, TO* __restrict__ out) {
+  constexpr int NB = G * D / 16;
+  const int slot = threadIdx.x >> 2, c4 = threadIdx.x & 3, q = slot * cs + rank;
+  if (q >= NB) return;
+  const uint32_t rb = recs + (uint32_t)(slot * cs) * (REC2 * 4);
+  float M = -INFINITY, l = 0.0f;
+#pragma unroll 8
+  for (int x = 0; x < cs; ++x) M = fmaxf(M, lds_f2(rb + x * (REC2 * 4) + 64).x);
+  float4 a = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+#pragma unroll 8
+  for (int x = 0; x < cs; ++x) {
+    const float2 ml = lds_f2(rb + x * (REC2 * 4) + 64);
+    const float4 o = lds_f4(rb + x * (REC2 * 4) + 16 * c4);
+    const float f = tc::ex2(ml.x - M);                       // 0 for a slice without keys
+    a.x = fmaf(f, o.x, a.x); a.y = fmaf(f, o.y, a.y); a.z = fmaf(f, o.z, a.z); a.w = fmaf(f, o.w, a.w);
+    l = fmaf(f, ml.y, l);
+  }
+  const float inv = 1.0f / l;
+  store4(out + out0 + (size_t)(q / (D / 16)) * D + (q % (D / 16)) * 16 + 4 * c4, a.x * inv, a.y * inv, a.z * inv, a.w * inv);
+}
 // Slices of a step over sequences of up to L keys (the new one included).  A step takes 4 to 5 us plus,
 // for every unit a warp works through, 1.1 us (d = 64) or 1.3 us (d = 128) while a CTA has its SM for
 // itself and 1.75 us where two share one (measured from 1 to 192 KV heads, 300 to 16000 keys); the

@@ -10,9 +10,13 @@
 // Bound: one pass over the key and value cache (HBM, or L2 for a layer stepped in a loop); for a few
 // sequences the chain of dependent latencies in front of and behind that pass.  So a warp works alone:
 // it owns units of 32 keys, brings their key and value rows in by TMA (one box each, 128-byte swizzle,
-// its own two barriers), multiplies on mma.sync (m16n8k16) straight from the swizzled rows and keeps
+// a ring of three halves), multiplies on mma.sync (m16n8k16) straight from the swizzled rows and keeps
 // its own running softmax; warps meet once, at the end.  Staging by per-thread cp.async instead of TMA
 // was bound by the SM's load path at half the rate (batch 16, 2048 keys: 18.9 us per step, TMA 12.2).
+// With the copies ahead of their use, a unit's time is its instructions (two CTAs per SM: 3060 clocks a
+// round, now 2030; 64 MB from L2 in 5 us are 1560): copies are issued under a predicate, not in one lane's branch;
+// values come by ldmatrix.trans instead of 32 byte permutations; the row scale moves only past 2^8; the unit of the
+// new row comes by TMA like any other (row by row it made its warp the last of every step by 0.8 us).
 // G <= 8 query rows against the cache are no shape for a 128-row tcgen05 tile, whose operands,
 // commits and tensor-memory reads put four hand-overs between a key tile and its softmax; the score
 // product here fills 16 rows with the G references and the G queries, so that one thread receives both
@@ -24,15 +28,18 @@
 //           P keeps fp32 precision as a sum of three bf16 parts: rows 0-7 of A carry the first part,
 //           rows 8-15 the second (the same thread holds both), the third goes to rows G .. 2G-1,
 //           whose lanes duplicate the scores of rows 0 .. G-1 (G <= 4), or to a second product (G = 8).
-// The row that arrives with the step is scored from k_new and v_new and written to the caches by the
-// warp that owns its unit.  The slices of a (batch, KV head) are one thread-block cluster: every warp
-// sends its partial result to the CTA that finishes those channels with st.async, which counts its
-// bytes on the receiver's barrier (a merge through global memory takes 2 us more; a cluster barrier
-// with release semantics waits 0.7 us for the step's global stores).
-// Measured, us per step, against the kernel before it (tcgen05 scores for d = 64, FP32 pipes for
-// d = 128): Llama layer at 2048 keys, batch 1 8.9 -> 4.4, batch 4 10.3 -> 7.0, batch 16 18.4 -> 12.2
-// (5.9 TB/s); batch 8 at 4096 keys 18.0 -> 11.6; BitNet layer (d = 128) at 1531 keys, batch 2
-// 16.7 -> 6.1, at 2000 keys, batch 16 45.5 -> 14.2; key deltas, batch 4 at 1777 keys 12.1 -> 6.4.
+// The row that arrives with the step is scored from k_new and v_new, written over its row of the unit (zeros
+// behind it: what the caches hold there is anything), and joins the caches through the warp that owns its unit.
+// The slices of a (batch, KV head) are one thread-block cluster: a CTA's warps meet in its shared memory, and one
+// record per block of 16 channels goes to the CTA that finishes the block with st.async, which counts its
+// bytes on the receiver's barrier (every warp sending for itself: 0.4 us more, the packets queue at the
+// receivers; a merge through global memory 2 us more; a cluster barrier with release semantics waits 0.7 us for
+// the step's global stores).
+// Measured, us per step of a loop of steps, before -> after the changes above: Llama layer at 2048 keys, batch 1
+// 4.4 -> 4.1 (the caller's host time; 3.3 on the device), batch 16 12.2 -> 9.3 (7.6 TB/s from L2); batch 8 at 4096 keys
+// 11.6 -> 9.5; BitNet layer (d = 128) at 1531 keys, batch 2 6.1 -> 5.0; key deltas, batch 4 at 1777 keys 6.4 -> 5.0.
+// Tried and dropped: the next unit's scores issued under a unit's softmax and P.V (twice the code, spills: batch 16
+// 10.3); three slots without the rest (nothing: no warp was waiting for its copies).
 #include <cuda.h>
 
 #include "decode_common.cuh"
@@ -44,6 +51,7 @@ namespace delta {
 namespace {
 
 template <int D> constexpr int kWarps = D == 64 ? 8 : 4;    // warps per CTA
+constexpr float RESCALE_LOG2 = 8.0f;
 
 struct MmaDecodeParams {
   const __nv_bfloat16 *q_new, *k_new, *v_new;
@@ -74,6 +82,19 @@ __device__ __forceinline__ void mma16816(float (&c)[4], uint32_t a0, uint32_t a1
                "{%0, %1, %2, %3};"
                : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3]) : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
 }
+// (the accumulators start at zero)
+__device__ __forceinline__ void mma16816_first(float (&c)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0,
+                                               uint32_t b1) {
+  asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, "
+               "{%10, %10, %10, %10};"
+               : "=f"(c[0]), "=f"(c[1]), "=f"(c[2]), "=f"(c[3])
+               : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1), "f"(0.0f));
+}
+// four 8 x 8 tiles, transposed: lane l gives the address of row l % 8 of tile l / 8
+__device__ __forceinline__ void ldsm4t(uint32_t addr, uint32_t (&r)[4]) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0, %1, %2, %3}, [%4];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr));
+}
 __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
   const __nv_bfloat162 t = __floats2bfloat162_rn(lo, hi);
   return *reinterpret_cast<const uint32_t*>(&t);
@@ -95,19 +116,47 @@ __device__ __forceinline__ uint32_t lds_u16(uint32_t a) {
   asm volatile("ld.shared.u16 %0, [%1];" : "=r"(v) : "r"(a));
   return v;
 }
+__device__ __forceinline__ void sts_u4(uint32_t a, uint4 v) {
+  asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(a), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w) : "memory");
+}
 __device__ __forceinline__ void sts_u32(uint32_t a, uint32_t v) { asm volatile("st.shared.u32 [%0], %1;" ::"r"(a), "r"(v) : "memory"); }
-// Shared memory: per warp one unit of keys and values (128-byte swizzle, blocks of [32 rows][64
-// channels]), then the merge's records [slot][slice x warp][REC] and (maximum, row sum) pairs.
+// N consecutive elements, as fp32, past the L1 cache
+template <int N> __device__ __forceinline__ void load_bf16(const __nv_bfloat16* p, float (&x)[N]) {
+  static_assert(N == 1 || N == 2 || N == 4 || N == 8, "");
+  uint32_t w[N == 1 ? 1 : N / 2];
+  if constexpr (N == 1) w[0] = __ldcg(reinterpret_cast<const unsigned short*>(p));
+  else if constexpr (N == 2) w[0] = __ldcg(reinterpret_cast<const uint32_t*>(p));
+  else if constexpr (N == 4) { const uint2 u = __ldcg(reinterpret_cast<const uint2*>(p)); w[0] = u.x; w[1] = u.y; }
+  else { const uint4 u = __ldcg(reinterpret_cast<const uint4*>(p)); w[0] = u.x; w[1] = u.y; w[2] = u.z; w[3] = u.w; }
+#pragma unroll
+  for (int i = 0; i < N; ++i) x[i] = __uint_as_float((i & 1) ? w[i >> 1] & 0xffff0000u : w[i >> 1] << 16);
+}
+template <int N> __device__ __forceinline__ void load_f32(const float* p, float (&x)[N]) {
+  if constexpr (N == 1) x[0] = __ldcg(p);
+  else if constexpr (N == 2) { const float2 u = __ldcg(reinterpret_cast<const float2*>(p)); x[0] = u.x; x[1] = u.y; }
+  else
+#pragma unroll
+    for (int i = 0; i < N; i += 4) {
+      const float4 u = __ldcg(reinterpret_cast<const float4*>(p + i));
+      x[i] = u.x; x[i + 1] = u.y; x[i + 2] = u.z; x[i + 3] = u.w;
+    }
+}
+// Shared memory: per warp a ring of NS halves of units (the keys, or the values, of one unit: 128-byte
+// swizzle, blocks of [32 rows][64 channels]), whose first slot takes the warp's result in the end, then the merge's records.
 // PACKED: per warp also the encoding of one 32-row segment: values, mask words, the reference in front.
 template <int D, int G, bool PACKED> struct MmaSmem {
   static constexpr int NW = kWarps<D>;
   static constexpr uint32_t VALS = UK * D * 2 + 16, MASKS = UK * (D / 32) * 4, PACK = PACKED ? VALS + MASKS + D * 2 : 0;
   static constexpr uint32_t HALF = UK * D * 2;             // keys, or values, of a unit
-  static constexpr uint32_t RING = NW * 2 * HALF;
+  static constexpr int NS = PACKED ? 2 : 3;                // (two CTAs per SM: 2 x 113 KB)
+  static constexpr uint32_t RING = NW * NS * HALF;
   static constexpr int NB = G * D / 16;                    // 16-channel blocks of the result
+  static_assert(MergePart<D, G>::BYTES <= HALF, "a warp's result fits its first slot");
   // records of a CTA of a cluster of cs
-  __host__ __device__ static constexpr uint32_t nrec(int cs) { return (uint32_t)((NB + cs - 1) / cs * cs) * NW; }
-  static constexpr size_t bytes(int cs) { return 1024 + RING + nrec(cs) * (REC + 2) * 4 + NW * PACK; }
+  __host__ __device__ static constexpr uint32_t rec_bytes(int cs) { return merge_slots<D, G>(cs) * cs * REC2 * 4; }
+  static constexpr uint32_t NEW = 2 * D * 2;               // the key and value row that arrive with the step
+  static constexpr size_t bytes(int cs) { return 1024 + RING + rec_bytes(cs) + NW * PACK + NEW; }
+  static constexpr size_t bytes_max = 1024 + RING + (NB + kMaxCluster - 1) * REC2 * 4 + NW * PACK + NEW;
 };
 
 }  // namespace
@@ -127,12 +176,14 @@ decode_step_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_co
   constexpr int NV = D / 64;                 // 64-channel blocks of a row
   constexpr int NT8 = D / 8;                 // n-tiles of P.V
   extern __shared__ unsigned char dsm_raw[];
-  __shared__ __align__(8) unsigned long long bars[2 * MNW + 1];
+  __shared__ __align__(8) unsigned long long bars[SM::NS * MNW + 1];
   __shared__ int s_last, s_fail;
   const uint32_t ring = (smem_u32(dsm_raw) + 1023u) & ~1023u;
-  const uint32_t recs = ring + SM::RING, mls = recs + SM::nrec(CLUSTER ? p.nsplit : 1) * REC * 4;
+  const uint32_t recs = ring + SM::RING, packs = recs + SM::rec_bytes(CLUSTER ? p.nsplit : 1);
 
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  // (the warp index by shuffle: known to be the same in every lane, so that addresses of copies stay in uniform registers)
+  const int tid = threadIdx.x, lane = tid & 31, warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
+  const uint32_t lead = lane == 0;
   const int g = lane >> 2, t = lane & 3;     // row of the accumulators, thread of the row
   const int hd = g % G, part = g / G;        // the head this thread's row stands for; which part of P it feeds
   const int split = blockIdx.x, bkv = p.b0 * (p.H / G) + blockIdx.y;
@@ -144,15 +195,14 @@ decode_step_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_co
   const float theta = p.theta;
 
   // the merge: blocks of 16 channels of one head; slice r of the cluster finishes blocks r, r + cs, ..
-  // (a CTA without a cluster all of them), each from the records of every warp of every slice
-  const int cs = CLUSTER ? p.nsplit : 1, rank = CLUSTER ? split : 0, nsrc = cs * MNW;
-  const uint32_t bar_m = smem_u32(&bars[2 * MNW]);
+  // (a CTA without a cluster all of them), each from the records of every slice
+  const int cs = CLUSTER ? p.nsplit : 1, rank = CLUSTER ? split : 0;
+  const uint32_t bar_m = smem_u32(&bars[SM::NS * MNW]);
   if (CLUSTER) {
     if (tid == 0) {
       tc::mbar_init(bar_m, 1);
       asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-      const int slots = (SM::NB - rank + cs - 1) / cs;
-      tc::mbar_expect_tx(bar_m, (uint32_t)(slots * nsrc) * (REC + 2) * 4);
+      tc::mbar_expect_tx(bar_m, (uint32_t)((SM::NB - rank + cs - 1) / cs * cs) * (16 + 2) * 4);
     }
     __syncwarp();
     asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
@@ -167,25 +217,35 @@ decode_step_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_co
   const TC* const vn = p.v_new + (size_t)bkv * D;
   const int wl = n - W + 1;                  // first key inside the decode window
 
-  // ---- the warp's ring: one unit of keys, one of values.  Row r, 16-byte chunk c of a 64-channel
-  // block lies at r * 128 + ((c ^ (r & 7)) << 4): what TMA's 128-byte swizzle writes.
-  const uint32_t slot_k = ring + (uint32_t)warp * 2 * SM::HALF, slot_v = slot_k + SM::HALF;
-  const uint32_t bar_k = smem_u32(&bars[2 * warp]), bar_v = bar_k + 8;
+  // ---- the warp's ring: halves K, V, K, V, .. of its units in turn, half h in slot h mod NS.  Row r,
+  // 16-byte chunk c of a 64-channel block lies at r * 128 + ((c ^ (r & 7)) << 4): what TMA's 128-byte
+  // swizzle writes.
+  constexpr int NS = SM::NS;
+  const uint32_t slots = ring + (uint32_t)warp * NS * SM::HALF;
+  const uint32_t bars0 = smem_u32(&bars[NS * warp]);
   if (lane == 0) {
-    tc::mbar_init(bar_k, 1);
-    tc::mbar_init(bar_v, 1);
+    if (warp == 0) {
+      // (a copy that has to fetch its tensor map first takes 0.25 us longer)
+      asm volatile("prefetch.tensormap [%0];" ::"l"(&tm_k) : "memory");
+      asm volatile("prefetch.tensormap [%0];" ::"l"(&tm_v) : "memory");
+      if (MODE == 1) asm volatile("prefetch.tensormap [%0];" ::"l"(&tm_h) : "memory");
+    }
+#pragma unroll
+    for (int i = 0; i < NS; ++i) tc::mbar_init(bars0 + 8 * i, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     tc::fence_proxy_async();
   }
   if (tid == 0) s_fail = 0;
   __syncwarp();
-  // A unit whose rows come from one cache goes by TMA; the unit of the row that arrives with the
-  // step (rows behind it: zeros) and, key deltas, the unit of the window's edge row by row.
-  auto k_plain = [&](int jg) { return jg + UK <= n && (!KEY || jg + UK <= wl || jg >= wl); };
-  const uint32_t pack_s = mls + SM::nrec(CLUSTER ? p.nsplit : 1) * 8 + (uint32_t)warp * SM::PACK;       // values, mask words, base
+  // A unit whose rows come from one cache goes by TMA, the unit of the row that arrives with the step
+  // too (rows behind the cached ones hold anything: that row and zeros are written over them); key
+  // deltas: the unit of the window's edge row by row.
+  auto k_plain = [&](int jg) { return !KEY || jg + UK <= wl || jg >= wl; };
+  const uint32_t pack_s = packs + (uint32_t)warp * SM::PACK;       // values, mask words, base
   const uint32_t* const so = PACKED ? p.seg_off + (size_t)bkv * (p.nseg_max + 1) : nullptr;
   auto from_pack = [&](int jg) { return PACKED && jg < wl && jg < n; };          // some row is a cached reference row
-  auto fetch_k = [&](int jg) {
+  auto fetch_k = [&](int jg, int slot) {
+    const uint32_t bar_k = bars0 + 8 * slot, slot_k = slots + slot * SM::HALF;
     if (from_pack(jg)) {
       // (the entry behind the last cached segment is being rewritten by this step's owner where the new
       // row extends or follows that segment: old and new value both bound the cached values)
@@ -200,12 +260,10 @@ decode_step_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_co
       }
       // (the original keys of a mixed unit's window rows follow when the rows are rebuilt)
     } else if (k_plain(jg)) {
-      if (lane == 0) {
-        tc::mbar_expect_tx(bar_k, SM::HALF);
-        const CUtensorMap* tm = (MODE == 1 && jg < wl) ? &tm_h : &tm_k;
+      tc::mbar_expect_tx_if(lead, bar_k, SM::HALF);
+      const CUtensorMap* tm = (MODE == 1 && jg < wl) ? &tm_h : &tm_k;
 #pragma unroll
-        for (int c = 0; c < NV; ++c) tc::tma_load_3d(slot_k + c * UK * 128, tm, bar_k, 64 * c, jg, bkv);
-      }
+      for (int c = 0; c < NV; ++c) tc::tma_load_3d_if(lead, slot_k + c * UK * 128, tm, bar_k, 64 * c, jg, bkv);
     } else {
 #pragma unroll
       for (int c = 0; c < NV; ++c)
@@ -219,33 +277,18 @@ decode_step_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_co
         }
     }
   };
-  auto fetch_v = [&](int jg) {
-    if (jg + UK <= n) {
-      if (lane == 0) {
-        tc::mbar_expect_tx(bar_v, SM::HALF);
+  auto fetch_v = [&](int jg, int slot) {
+    const uint32_t bar_v = bars0 + 8 * slot, slot_v = slots + slot * SM::HALF;
+    tc::mbar_expect_tx_if(lead, bar_v, SM::HALF);
 #pragma unroll
-        for (int c = 0; c < NV; ++c) tc::tma_load_3d(slot_v + c * UK * 128, &tm_v, bar_v, 64 * c, jg, bkv);
-      }
-    } else {
-#pragma unroll
-      for (int c = 0; c < NV; ++c)
-#pragma unroll
-        for (int i = 0; i < UK / 4; ++i) {
-          const int r = 4 * i + (lane >> 3), ch = lane & 7, j = jg + r;
-          const uint32_t dst = slot_v + c * UK * 128 + r * 128 + ((ch ^ (r & 7)) << 4);
-          if (j <= n) async16(dst, (j < n ? vc + (size_t)j * D : vn) + 64 * c + 8 * ch);
-          else sts128z(dst);
-        }
-    }
+    for (int c = 0; c < NV; ++c) tc::tma_load_3d_if(lead, slot_v + c * UK * 128, &tm_v, bar_v, 64 * c, jg, bkv);
   };
-  // where this thread's part of the result goes: slice and record (a division; ahead of the wait)
-  uint32_t to_rank[NV], to_rec[NV];
-#pragma unroll
-  for (int c = 0; c < NV; ++c) {
-    const int q = hd * (D / 16) + 4 * c + t;
-    to_rank[c] = (uint32_t)(q % cs);
-    to_rec[c] = (uint32_t)(q / cs * nsrc + rank * MNW + warp);
-  }
+  // the warp that owns the row arriving with the step, and that row in shared memory (keys, values)
+  const bool has_new = j1 == L && j0 < L && ((n - j0) / UK) % MNW == warp;
+  const uint32_t new_s = packs + MNW * SM::PACK;
+  auto row_at = [&](uint32_t slot, int r, int ch) {          // 16-byte piece ch of row r
+    return slot + (ch >> 3) * UK * 128 + r * 128 + (((ch & 7) ^ (r & 7)) << 4);
+  };
   // Reference-key rows and their encoding are the library's own: behind another step (p.early) all but the
   // row (segment) that step may be writing is final before this kernel can start, since a step releases
   // the next one only behind its own wait, and is requested ahead of the wait.  Not so behind a prefill:
@@ -253,66 +296,85 @@ decode_step_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_co
   // certain to be seen only behind the wait.  (Key and value rows are the caller's.)
   int jg = j0 + UK * warp;
   const bool early_k = KEY && p.early && jg < j1 && jg + UK <= min(n - 1, wl);
-  if (early_k) fetch_k(jg);
+  if (early_k) fetch_k(jg, 0);
   // the step in front (or the prefill) has written the reference, row n - 1 of the caches, the tickets
   asm volatile("griddepcontrol.wait;" ::: "memory");
   // The next step's CTAs may become resident from here on.  (Released at the kernel's start they
   // take the places of this step's own late CTAs: 30 us per step for 18 at batch 16.)
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 
-  // ---- threshold step (Eq. 2-3): the operand rows, straight into registers
-  uint32_t ar[NC][4], aq[NC][4];             // rows g and g + 8 of A, channels 32 c + 8 t ..
-  uint32_t khat_new[KEY ? NC : 1][4];        // KEY: the reference key after this step
-  int fired = 0;
-  uint32_t fbits = 0;                        // PACKED: which of this thread's channels fired, 8 per piece
+  // ---- threshold step (Eq. 2-3), a few elements per thread; the references meet in shared memory, from
+  // where every warp takes its operand rows (each warp on its own: 150 instructions more per warp, 0.2 us
+  // alone and 0.4 us where two CTAs share an SM)
   const bool keep = split == 0 && warp == 0;
+  constexpr int NTH = 32 * MNW, NE = KEY ? D : G * D, EPT = NE <= NTH ? 1 : NE / NTH;
+  constexpr uint32_t REF_LD = 2 * D + (KEY ? 0 : 64);       // bytes (the 64: rows on different banks)
+  __shared__ __align__(16) unsigned char s_ref[(KEY ? 1 : G) * REF_LD];
+  __shared__ int s_fired[MNW];               // fired elements of every warp
+  __shared__ uint32_t s_word[NC];            // KEY: mask words of the new key
+  const uint32_t refs = smem_u32(s_ref);
+  uint32_t ar[NC][4], aq[NC][4];             // rows g and g + 8 of A, channels 32 c + 8 t ..
   {
-    const size_t o = ((size_t)b * p.H + kvh * G + hd) * D;
-    const float* const rp = p.ref_in + (KEY ? (size_t)bkv * D : o);
-    uint4 q4[NC], x4[NC];
-    float4 r4[NC][2];
-#pragma unroll
-    for (int c = 0; c < NC; ++c) {
-      const int ch = 32 * c + 8 * t;
-      q4[c] = __ldcg(reinterpret_cast<const uint4*>(p.q_new + o + ch));
-      r4[c][0] = __ldcg(reinterpret_cast<const float4*>(rp + ch));
-      r4[c][1] = __ldcg(reinterpret_cast<const float4*>(rp + ch) + 1);
-      if (KEY) x4[c] = __ldcg(reinterpret_cast<const uint4*>(kn + ch));
+    const size_t o0 = ((size_t)b * p.H + kvh * G) * D;
+    const int e0 = tid * EPT;
+    const bool mine = NE >= NTH || e0 < NE;
+    float x[EPT], ref[EPT];
+    if (mine) {
+      load_bf16(KEY ? kn + e0 : p.q_new + o0 + e0, x);
+      load_f32(p.ref_in + (KEY ? (size_t)bkv * D : o0) + e0, ref);
     }
+    uint4 q4[NC];
+#pragma unroll
+    for (int c = 0; c < NC; ++c) q4[c] = __ldcg(reinterpret_cast<const uint4*>(p.q_new + o0 + hd * D + 32 * c + 8 * t));
     // (behind those loads: they are what the warp waits for next)
     if (jg < j1) {
-      if (!early_k) fetch_k(jg);
-      fetch_v(jg);
+      if (!early_k) fetch_k(jg, 0);
+      fetch_v(jg, 1);
+      if (NS == 3 && jg + UK * MNW < j1) fetch_k(jg + UK * MNW, 2);
     }
+    if (has_new) {
+#pragma unroll
+      for (int e = 0; e < 2 * (D / 8); e += 32)
+        if (e + lane < 2 * (D / 8)) {
+          const int ch = (e + lane) % (D / 8);
+          async16(new_s + 16 * (e + lane), (e + lane < D / 8 ? kn : vn) + 8 * ch);
+        }
+    }
+    int fired = 0;
+    if (mine) {
+#pragma unroll
+      for (int i = 0; i < EPT; ++i) {
+        const bool fire = fabsf(__fsub_rn(x[i], ref[i])) > theta;
+        ref[i] = fire ? x[i] : ref[i];
+        fired += fire ? 1 : 0;
+      }
+      // exactly bf16: copies of input elements (or the zero the reference starts from)
+      unsigned char* const at = s_ref + (KEY ? 0 : e0 / D) * REF_LD + 2 * (KEY ? e0 : e0 % D);
+      if constexpr (EPT == 1) *reinterpret_cast<uint16_t*>(at) = (uint16_t)(__float_as_uint(ref[0]) >> 16);
+      else
+#pragma unroll
+        for (int i = 0; i < EPT; i += 2)
+          *reinterpret_cast<uint32_t*>(at + 2 * i) = __byte_perm(__float_as_uint(ref[i]), __float_as_uint(ref[i + 1]), 0x7632);
+      if (split == 0) {
+        float* const rq = p.ref_out + (KEY ? (size_t)bkv * D : o0) + e0;
+#pragma unroll
+        for (int i = 0; i < EPT; ++i) rq[i] = ref[i];
+      }
+    }
+    if constexpr (KEY) {                     // (a thread, an element: a warp's vote is a mask word)
+      const uint32_t word = __ballot_sync(0xffffffffu, fired != 0);
+      if (lane == 0) { s_fired[warp] = __popc(word); if (warp < NC) s_word[warp] = word; }
+    } else {
+      fired = __reduce_add_sync(0xffffffffu, fired);
+      if (lane == 0) s_fired[warp] = fired;
+    }
+    __syncthreads();
 #pragma unroll
     for (int c = 0; c < NC; ++c) {
-      const uint32_t qw[4] = {q4[c].x, q4[c].y, q4[c].z, q4[c].w};
-      const uint4 xx = KEY ? x4[c] : q4[c];
-      const uint32_t xw[4] = {xx.x, xx.y, xx.z, xx.w};
-      float ref[8] = {r4[c][0].x, r4[c][0].y, r4[c][0].z, r4[c][0].w, r4[c][1].x, r4[c][1].y, r4[c][1].z, r4[c][1].w};
-#pragma unroll
-      for (int i = 0; i < 8; ++i) {
-        const float x = (i & 1) ? __uint_as_float(xw[i >> 1] & 0xffff0000u) : __uint_as_float(xw[i >> 1] << 16);
-        const bool fire = fabsf(__fsub_rn(x, ref[i])) > theta;
-        ref[i] = fire ? x : ref[i];
-        fired += fire ? 1 : 0;
-        if (PACKED) fbits |= (fire ? 1u : 0u) << (8 * c + i);
-      }
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        // exactly bf16: copies of input elements (or the zero the reference starts from)
-        const uint32_t rw = __byte_perm(__float_as_uint(ref[2 * i]), __float_as_uint(ref[2 * i + 1]), 0x7632);
-        ar[c][i] = KEY ? qw[i] : rw;
-        aq[c][i] = KEY ? 0u : qw[i];
-        if (KEY) khat_new[c][i] = rw;
-      }
-      if (keep && (KEY ? g == 0 : part == 0)) {
-        float4* rq = reinterpret_cast<float4*>(p.ref_out + (KEY ? (size_t)bkv * D : o) + 32 * c + 8 * t);
-        rq[0] = make_float4(ref[0], ref[1], ref[2], ref[3]);
-        rq[1] = make_float4(ref[4], ref[5], ref[6], ref[7]);
-      }
+      const uint4 r4 = KEY ? q4[c] : tc::lds128u(refs + hd * REF_LD + 64 * c + 16 * t);
+      ar[c][0] = r4.x; ar[c][1] = r4.y; ar[c][2] = r4.z; ar[c][3] = r4.w;
+      aq[c][0] = KEY ? 0u : q4[c].x; aq[c][1] = KEY ? 0u : q4[c].y; aq[c][2] = KEY ? 0u : q4[c].z; aq[c][3] = KEY ? 0u : q4[c].w;
     }
-    if (!(KEY ? g == 0 : part == 0)) fired = 0;
   }
 
   // ---- the warp's units
@@ -322,19 +384,22 @@ decode_step_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_co
 #pragma unroll
     for (int e = 0; e < 4; ++e) o_acc[i][e] = 0.0f;
   float m = -INFINITY, l = 0.0f;
-  bool first = true;
   unsigned done = 0;
-  uint32_t ph_k = 0, ph_v = 0;
+  uint32_t phases = 0;                       // of the slots' barriers, a bit each
+  int sk = 0, sv = 1;                        // the slots of the unit's keys and values
   // Column x of a score block stands for key x ^ (4 (x & 1)) of its 8 keys: with the swizzle, the
   // eight lanes of a shared-memory phase then touch eight different chunks, for keys and values alike.
   const int kx0 = 2 * t, kx1 = (2 * t + 1) ^ 4;            // this thread's two keys of a block
   const int kr = g ^ (4 * (g & 1));                        // the key row it reads
-  const uint32_t k_off = slot_k + kr * 128, k_sw = kr & 7;
-  const uint32_t v_off0 = slot_v + kx0 * 128 + ((g ^ kx0) << 4), v_off1 = slot_v + kx1 * 128 + ((g ^ kx1) << 4);
+  const uint32_t k_off = kr * 128, k_sw = kr & 7;
+  // lane l gives row l % 8 of 8-key block l / 8, read as the column it stands for; chunk c of it lies at
+  // v_off ^ (c << 4)
+  const int vr_ = (lane & 7) ^ (4 * (lane & 1));
+  const uint32_t v_off = (lane >> 3) * 1024 + vr_ * 128 + (vr_ << 4);
   float* const Rg = KEY ? nullptr : p.R + ((size_t)b * p.H + kvh * G + hd) * T_max;
   // Rows jg .. jg + 31 of the reference-key stream from their encoding, into the key slot: lane = two
   // channels (of a 64-channel block), walking the rows; the window's rows and the new one are keys.
-  auto rebuild = [&](int jg) {
+  auto rebuild = [&](int jg, uint32_t slot_k) {
     constexpr int NWD = D / 32;
     const int last = min(UK, min(n, wl) - jg);             // rows that are cached references
     const int hi = lane >> 4, sh = 2 * (lane & 15);        // this lane's channels: bits sh, sh + 1 of word 2 c + hi
@@ -383,18 +448,16 @@ decode_step_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_co
     uint32_t at = pos;
 #pragma unroll
     for (int c = 0; c < NC; ++c) {
-      // word c: thread t of row 0 holds its bits 8 t .. 8 t + 7
-      uint32_t byte = (fbits >> (8 * c)) & 0xffu;
-      uint32_t word = byte << (8 * t);
-      word |= __shfl_xor_sync(0xffffffffu, word, 1);
-      word |= __shfl_xor_sync(0xffffffffu, word, 2);
+      const uint32_t word = s_word[c], byte = (word >> (8 * t)) & 0xffu;
+      const uint4 kh4 = tc::lds128u(refs + 64 * c + 16 * t);
+      const uint32_t kh[4] = {kh4.x, kh4.y, kh4.z, kh4.w};
       if (g == 0) {
         uint32_t rank = at + __popc(word & ((1u << (8 * t)) - 1u));
 #pragma unroll
         for (int e = 0; e < 8; ++e)
           if ((byte >> e) & 1u) {
             // (a fired channel's new reference is the key value itself)
-            if (DELTA_IN(rank, p.cap, p.counters)) vg[rank] = (uint16_t)(khat_new[c][e >> 1] >> (16 * (e & 1)));
+            if (DELTA_IN(rank, p.cap, p.counters)) vg[rank] = (uint16_t)(kh[e >> 1] >> (16 * (e & 1)));
             ++rank;
           }
         if (t == 0) {
@@ -410,7 +473,7 @@ decode_step_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_co
             p.base[((size_t)bkv * p.nseg_max + sg) * D + 32 * c + 8 * t + e] = (uint16_t)(__float_as_uint(rr[e]) >> 16);
         }
       }
-      at += __popc(__shfl_sync(0xffffffffu, word, 0));
+      at += __popc(word);
     }
     if (lane == 0 && DELTA_IN(sg + 1, p.nseg_max + 1, p.counters)) {
       uint32_t* const sw = p.seg_off + (size_t)bkv * (p.nseg_max + 1);
@@ -427,27 +490,43 @@ decode_step_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_co
   bool owns_new = false;                     // the warp owns the row that arrives with the step
   auto store_r = [&]() {
     if (!KEY && part == 0 && j_done >= 0) {  // R[j] = q_hat . k_j
+      float *const ra = Rg + j_done + kx0, *const rb = Rg + j_done + kx1;
+      if (!owns_new) {
 #pragma unroll
-      for (int h = 0; h < 4; ++h) {
-        const int ja = j_done + 8 * h + kx0, jb = j_done + 8 * h + kx1;
-        if ((!owns_new || ja <= n) && DELTA_IN(ja, T_max, p.counters)) Rg[ja] = s[h][0];
-        if ((!owns_new || jb <= n) && DELTA_IN(jb, T_max, p.counters)) Rg[jb] = s[h][1];
+        for (int h = 0; h < 4; ++h)
+          if (DELTA_IN(j_done + 8 * h + 7, T_max, p.counters)) { ra[8 * h] = s[h][0]; rb[8 * h] = s[h][1]; }
+      } else {
+#pragma unroll
+        for (int h = 0; h < 4; ++h) {
+          if (j_done + 8 * h + kx0 <= n) ra[8 * h] = s[h][0];
+          if (j_done + 8 * h + kx1 <= n) rb[8 * h] = s[h][1];
+        }
       }
     }
   };
   for (; jg < j1; jg += UK * MNW) {
     const int jn = jg + UK * MNW;            // the warp's next unit
+    const uint32_t bar_k = bars0 + 8 * sk, bar_v = bars0 + 8 * sv, slot_k = slots + sk * SM::HALF, slot_v = slots + sv * SM::HALF;
     store_r();
     done += nz;
     const bool owner = n < jg + UK;          // of the row that arrives with the step
-    const bool packed = from_pack(jg), tma_k = !packed && k_plain(jg), tma_v = jg + UK <= n;
+    const bool packed = from_pack(jg), tma_k = !packed && k_plain(jg);
     if (packed) {
-      if (!mbar_wait(bar_k, ph_k)) s_fail = 1;
-      ph_k ^= 1u;
-      rebuild(jg);
+      if (!mbar_wait(bar_k, (phases >> sk) & 1u)) s_fail = 1;
+      phases ^= 1u << sk;
+      rebuild(jg, slot_k);
     } else if (tma_k) {
-      if (!mbar_wait(bar_k, ph_k)) s_fail = 1;
-      ph_k ^= 1u;
+      if (!mbar_wait(bar_k, (phases >> sk) & 1u)) s_fail = 1;
+      phases ^= 1u << sk;
+      if (owner) {                           // the new key's row (what the rows behind it hold is masked)
+        async_wait_all();
+        __syncwarp();
+        if (lane < D / 8) {
+          const uint4 x = tc::lds128u(new_s + 16 * lane);
+          sts_u4(row_at(slot_k, n - jg, lane), x);
+        }
+        __syncwarp();
+      }
     } else {
       async_wait_all();
       __syncwarp();
@@ -455,14 +534,13 @@ decode_step_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_co
 #pragma unroll
     for (int h = 0; h < 4; ++h) {
 #pragma unroll
-      for (int e = 0; e < 4; ++e) s[h][e] = 0.0f;
-#pragma unroll
       for (int c = 0; c < NC; ++c) {
         // channels 32 c + 8 t .. of the row: chunk 4 (c & 1) + t of block c >> 1
-        uint4 k4 = tc::lds128u(k_off + (c >> 1) * UK * 128 + h * 1024 + (((4 * (c & 1) + t) ^ k_sw) << 4));
+        uint4 k4 = tc::lds128u(slot_k + k_off + (c >> 1) * UK * 128 + h * 1024 + (((4 * (c & 1) + t) ^ k_sw) << 4));
         if (KEY && W <= 0 && jg + 8 * h + kr == n)         // no window: even the new key goes by its reference
-          k4 = make_uint4(khat_new[c][0], khat_new[c][1], khat_new[c][2], khat_new[c][3]);
-        mma16816(s[h], ar[c][0], aq[c][0], ar[c][1], aq[c][1], k4.x, k4.y);
+          k4 = tc::lds128u(refs + 64 * c + 16 * t);
+        if (c == 0) mma16816_first(s[h], ar[c][0], aq[c][0], ar[c][1], aq[c][1], k4.x, k4.y);
+        else mma16816(s[h], ar[c][0], aq[c][0], ar[c][1], aq[c][1], k4.x, k4.y);
         mma16816(s[h], ar[c][2], aq[c][2], ar[c][3], aq[c][3], k4.z, k4.w);
       }
     }
@@ -475,14 +553,20 @@ decode_step_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_co
       if (!tma_k) tc::fence_proxy_async();                 // rows written by the warp, TMA overwrites them
     }
     __syncwarp();                            // every key of the unit has been used
-    if (jn < j1) fetch_k(jn);
+    if (jn < j1) {
+      if (NS == 3) fetch_v(jn, sk); else fetch_k(jn, sk);
+    }
 
     // hybrid select, running maximum of the row (4 threads hold it); the scale joins the exponential
     float v[8];
 #pragma unroll
-    for (int h = 0; h < 4; ++h) {
-      v[2 * h] = (KEY || jg + 8 * h + kx0 < wl) ? s[h][0] : s[h][2];
-      v[2 * h + 1] = (KEY || jg + 8 * h + kx1 < wl) ? s[h][1] : s[h][3];
+    for (int h = 0; h < 4; ++h) { v[2 * h] = s[h][0]; v[2 * h + 1] = s[h][1]; }
+    if (!KEY && jg + UK > wl) {
+#pragma unroll
+      for (int h = 0; h < 4; ++h) {
+        if (jg + 8 * h + kx0 >= wl) v[2 * h] = s[h][2];
+        if (jg + 8 * h + kx1 >= wl) v[2 * h + 1] = s[h][3];
+      }
     }
     if (owner) {
 #pragma unroll
@@ -491,13 +575,12 @@ decode_step_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_co
         if (jg + 8 * h + kx1 > n) v[2 * h + 1] = -INFINITY;
       }
     }
-    float mx = tc::fmax3(fmaxf(v[0], v[1]), tc::fmax3(v[2], v[3], v[4]), tc::fmax3(v[5], v[6], v[7]));
-    mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
-    mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 2)) * p.scale_log2e;
-    if (first) {
-      m = mx;
-      first = false;
-    } else if (__any_sync(0xffffffffu, mx > m)) {
+    // The row's scale moves only when a score is more than 2^RESCALE_LOG2 above it (a warp's first unit: any
+    // is), so the four threads of a row compare notes in few units; P and its parts are as exact at any scale.
+    float mx = tc::fmax3(fmaxf(v[0], v[1]), tc::fmax3(v[2], v[3], v[4]), tc::fmax3(v[5], v[6], v[7])) * p.scale_log2e;
+    if (__any_sync(0xffffffffu, mx > m + RESCALE_LOG2)) {
+      mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
+      mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
       const float mn = fmaxf(m, mx), al = tc::ex2(m - mn);
       m = mn;
       l *= al;
@@ -507,14 +590,22 @@ decode_step_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_co
         for (int e = 0; e < 4; ++e) o_acc[i][e] *= al;
     }
     float pr[8];
+    uint32_t pa[2][4], p2[2][2];
 #pragma unroll
     for (int e = 0; e < 8; ++e) pr[e] = tc::ex2(fmaf(v[e], p.scale_log2e, -m));
     l += ((pr[0] + pr[1]) + (pr[2] + pr[3])) + ((pr[4] + pr[5]) + (pr[6] + pr[7]));
-    if (tma_v) {
-      if (!mbar_wait(bar_v, ph_v)) s_fail = 1;
-      ph_v ^= 1u;
-    } else {
+    if (!mbar_wait(bar_v, (phases >> sv) & 1u)) s_fail = 1;
+    phases ^= 1u << sv;
+    if (owner) {                             // the new value's row, zeros behind it
+      const int rn = n - jg;
       async_wait_all();
+      __syncwarp();
+      if (lane < D / 8) {
+        const uint4 x = tc::lds128u(new_s + D * 2 + 16 * lane);
+        sts_u4(row_at(slot_v, rn, lane), x);
+      }
+#pragma unroll 1
+      for (int e = (rn + 1) * (D / 8) + lane; e < UK * (D / 8); e += 32) sts128z(row_at(slot_v, e / (D / 8), e % (D / 8)));
       __syncwarp();
     }
 #pragma unroll
@@ -527,24 +618,29 @@ decode_step_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_co
         a0 = part == 0 ? f0 : part == 1 ? f2 : 0u; a1 = part == 0 ? f1 : 0u;
         a2 = part == 0 ? g0 : part == 1 ? g2 : 0u; a3 = part == 0 ? g1 : 0u;
       }
+      pa[q][0] = a0; pa[q][1] = a1; pa[q][2] = a2; pa[q][3] = a3;
+      if (G == 8) { p2[q][0] = f2; p2[q][1] = g2; }
+    }
 #pragma unroll
-      for (int c = 0; c < NV; ++c) {
-        uint4 vr[4];
+    for (int c = 0; c < NT8; ++c) {          // 8 channels: B tiles of the unit's four 8-key blocks
+      uint32_t vb[4];
+      ldsm4t(slot_v + (v_off ^ ((c & 7) << 4)) + (c >> 3) * UK * 128, vb);
 #pragma unroll
-        for (int r = 0; r < 4; ++r)
-          vr[r] = tc::lds128u(((r & 1) ? v_off1 : v_off0) + c * UK * 128 + (2 * q + (r >> 1)) * 1024);
-#pragma unroll
-        for (int i = 0; i < 8; ++i) {
-          auto word = [&](int r) { return i < 2 ? vr[r].x : i < 4 ? vr[r].y : i < 6 ? vr[r].z : vr[r].w; };
-          const uint32_t sel = (i & 1) ? 0x7632u : 0x5410u;
-          const uint32_t b0 = __byte_perm(word(0), word(1), sel), b1 = __byte_perm(word(2), word(3), sel);
-          mma16816(o_acc[8 * c + i], a0, a1, a2, a3, b0, b1);
-          if (G == 8) mma16816(o_acc[8 * c + i], f2, 0u, g2, 0u, b0, b1);
-        }
+      for (int q = 0; q < 2; ++q) {
+        mma16816(o_acc[c], pa[q][0], pa[q][1], pa[q][2], pa[q][3], vb[2 * q], vb[2 * q + 1]);
+        if (G == 8) mma16816(o_acc[c], p2[q][0], 0u, p2[q][1], 0u, vb[2 * q], vb[2 * q + 1]);
       }
     }
     __syncwarp();
-    if (jn < j1) fetch_v(jn);
+    if (NS == 2) {
+      if (jn < j1) fetch_v(jn, sv);
+    } else {
+      // two halves on, modulo three
+      if (jn + UK * MNW < j1) fetch_k(jn + UK * MNW, sv);
+      const int s0 = sk;
+      sk = sv == 2 ? 0 : sv + 1;
+      sv = s0;
+    }
   }
 
   // ---- the warp's result: the parts of P meet again, the row sum over the row's four threads
@@ -559,40 +655,37 @@ decode_step_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_co
       o_acc[i][1] += __shfl_down_sync(0xffffffffu, o_acc[i][1], 4 * G);
     }
   }
-  // ---- merge: every warp sends its part to where it is finished
-  if (CLUSTER) asm volatile("barrier.cluster.wait.aligned;" ::: "memory");          // every slice runs
+  // ---- merge: the warp's part into its first slot (every copy into it is complete and read)
   if (part == 0) {
+    using MP = MergePart<D, G>;
 #pragma unroll
-    for (int c = 0; c < NV; ++c) {
-      // tile 8c + i, accumulator column x holds channel 64 c + 8 x + i; this thread has columns 2t, 2t + 1
-      const uint32_t r = to_rank[c];
-      uint32_t dst = recs + to_rec[c] * (REC * 4), dml = mls + to_rec[c] * 8, rbar = bar_m;
-      if (CLUSTER) { dst = cluster_map(dst, r); dml = cluster_map(dml, r); rbar = cluster_map(bar_m, r); }
-#pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        const float* const oe = &o_acc[8 * c + 4 * (e & 1)][0] + (e >> 1);
-        if (CLUSTER) cluster_send4(dst + 16 * e, rbar, oe[0], oe[4], oe[8], oe[12]);
-        else sts_f4(dst + 16 * e, oe[0], oe[4], oe[8], oe[12]);
-      }
-      if (CLUSTER) cluster_send2(dml, rbar, m, l); else sts_f2(dml, m, l);
-    }
+    for (int i = 0; i < NT8; ++i) sts_f2(slots + (hd * MP::LD + 8 * i + 2 * t) * 4, o_acc[i][0], o_acc[i][1]);
+    if (t == 0) sts_f2(slots + MP::ML + hd * 8, m, l);
   }
+  __syncthreads();
+  if (CLUSTER) asm volatile("barrier.cluster.wait.aligned;" ::: "memory");          // every slice runs
+  const size_t out0 = ((size_t)b * p.H + kvh * G) * D;
+  const int n_slices = (L + p.chunk - 1) / p.chunk;
+  merge_warps<TC, D, G, MNW, CLUSTER>(ring, NS * SM::HALF, recs, bar_m, rank, cs, n_slices, split, bkv, out0, p.partial, p.out);
   // ---- while the parts travel: the last unit's score row, the caches' new row, the counters
   store_r();
-  const int f_all = (keep || (KEY && owns_new)) ? warp_sum(fired) : 0;
+  int f_all = 0;
+  if (keep || (KEY && owns_new)) {
+#pragma unroll
+    for (int w = 0; w < MNW; ++w) f_all += s_fired[w];
+  }
   if (owns_new && DELTA_IN(n, T_max, p.counters)) {
     // the row that arrives with the step joins the caches
     if (lane < D / 8) {
-      reinterpret_cast<uint4*>(p.k_cache + (row0 + n) * D)[lane] = __ldcg(reinterpret_cast<const uint4*>(kn) + lane);
-      reinterpret_cast<uint4*>(p.v_cache + (row0 + n) * D)[lane] = __ldcg(reinterpret_cast<const uint4*>(vn) + lane);
+      reinterpret_cast<uint4*>(p.k_cache + (row0 + n) * D)[lane] = tc::lds128u(new_s + 16 * lane);
+      reinterpret_cast<uint4*>(p.v_cache + (row0 + n) * D)[lane] = tc::lds128u(new_s + D * 2 + 16 * lane);
     }
     if (KEY && lane == 0) p.row_nnz[row0 + n] = (uint16_t)f_all;
     if constexpr (PACKED) append(f_all);
     if (MODE == 1 && g == 0)
 #pragma unroll
       for (int c = 0; c < NC; ++c)
-        *reinterpret_cast<uint4*>(p.khat_cache + (row0 + n) * D + 32 * c + 8 * t) =
-            make_uint4(khat_new[c][0], khat_new[c][1], khat_new[c][2], khat_new[c][3]);
+        *reinterpret_cast<uint4*>(p.khat_cache + (row0 + n) * D + 32 * c + 8 * t) = tc::lds128u(refs + 64 * c + 16 * t);
   }
   if (keep && lane == 0) {
     const int n_in = min(L, max(W, 0));
@@ -609,14 +702,13 @@ decode_step_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_co
     if (lane == 0 && d) atomicAdd(&p.counters[CNT_DECODE_MACS_DONE], (unsigned long long)d * G);
   }
   if (CLUSTER) {
+    // (every slice's block records: also what keeps this CTA until the last of them has been sent to it)
     if (!mbar_wait(bar_m, 0)) s_fail = 1;
-  } else {
-    __syncthreads();
+    merge_slices<TC, D, G>(recs, rank, cs, out0, p.out);
+  } else if (n_slices > 1) {
+    merge_global<TC, D, G, MNW>(n_slices, bkv, out0, p.partial, p.ticket, p.out, &s_last);
   }
-  if (tid == 0 && s_fail) atomicMax(&p.counters[CNT_STATUS], (unsigned long long)DELTA_ERR_TIMEOUT);
-
-  decode_merge<TC, D, G, MNW, CLUSTER>(recs, mls, rank, cs, nsrc, (L + p.chunk - 1) / p.chunk, split, bkv,
-                                       ((size_t)b * p.H + kvh * G) * D, p.partial, p.ticket, p.out, &s_last);
+  if (s_fail && lane == 0) atomicMax(&p.counters[CNT_STATUS], (unsigned long long)DELTA_ERR_TIMEOUT);
 }
 
 template <int D, int G, int MODE, bool CLUSTER>
@@ -627,8 +719,7 @@ static cudaError_t launch_mma(const CUtensorMap& tk, const CUtensorMap& tv, cons
   const size_t smem = SM::bytes(CLUSTER ? p.nsplit : 1);
   static std::atomic<uint64_t> ready{0};
   if (!device_done(ready)) {
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(SM::bytes(kMaxCluster) > SM::bytes(kMaxCluster - 1) ? SM::bytes(kMaxCluster)
-                                                                                               : SM::bytes(kMaxCluster - 1)));
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SM::bytes_max);
     // (two CTAs per SM need the largest shared-memory carve-out)
     if (e == cudaSuccess) e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout,
                                                    (int)cudaSharedmemCarveoutMaxShared);

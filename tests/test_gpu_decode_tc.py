@@ -17,8 +17,9 @@ def B():
     return binding
 
 
-def _run(B, kernel, source, Bn, H, Hk, d, lens, W_d, steps, seed):
-    """Prefill (ragged where the lengths differ), then decode steps with the given decode kernel."""
+def _run(B, kernel, source, Bn, H, Hk, d, lens, W_d, steps, seed, ramp=0.0):
+    """Prefill (ragged where the lengths differ), then decode steps with the given decode kernel.
+    ramp: every key is 2^ramp times as large as the one in front of it."""
     gen = torch.Generator("cuda").manual_seed(seed)
     dt = torch.float32 if source == "f32" else torch.bfloat16
     rnd = lambda *s: torch.randn(*s, generator=gen, device="cuda").to(dt)      # noqa: E731
@@ -31,6 +32,8 @@ def _run(B, kernel, source, Bn, H, Hk, d, lens, W_d, steps, seed):
     vc = kc.clone()
     for b, n in enumerate(lens):
         kc[b, :, :n], vc[b, :, :n] = rnd(Hk, n, d), rnd(Hk, n, d)
+        if ramp:
+            kc[b, :, :n] *= torch.exp2(ramp * torch.arange(n, device="cuda"))[:, None].to(dt)
     q = torch.cat([rnd(H, n, d).reshape(-1) for n in lens])
     out = torch.empty_like(q)
     B.delta_attn_prefill_varlen(st, q, kc, vc, out, lens, [16] * Bn, 0.7)
@@ -45,9 +48,9 @@ def _run(B, kernel, source, Bn, H, Hk, d, lens, W_d, steps, seed):
             B.delta_sparsity_stats(st))
 
 
-def _compare(B, source, Bn, H, Hk, d, lens, W_d, steps, seed=7):
-    a = _run(B, 1, source, Bn, H, Hk, d, lens, W_d, steps, seed)
-    r = _run(B, 0, source, Bn, H, Hk, d, lens, W_d, steps, seed)
+def _compare(B, source, Bn, H, Hk, d, lens, W_d, steps, seed=7, ramp=0.0):
+    a = _run(B, 1, source, Bn, H, Hk, d, lens, W_d, steps, seed, ramp)
+    r = _run(B, 0, source, Bn, H, Hk, d, lens, W_d, steps, seed, ramp)
     assert torch.isfinite(a[0]).all()
     rms = r[0].pow(2).mean(dim=-1, keepdim=True).sqrt()
     most, rel = (2e-5, 2e-6) if source == "f32" else (2e-2, 3e-3)
@@ -89,3 +92,12 @@ def test_slices(B, source, Bn, Hk, T, d):
 def test_ragged_batches(B, source, Bn, d):
     lens = [1 + (i * 7919) % 900 for i in range(Bn)]
     _compare(B, source, Bn, 2, 1, d, lens, 40, 3)
+
+
+@pytest.mark.parametrize("source", ["query", "key"])
+@pytest.mark.parametrize("d", [64, 128])
+@pytest.mark.parametrize("ramp", [0.004, -0.004])
+def test_scores_that_run_away(B, source, d, ramp):
+    # one CTA, several units per warp: a row's maximum moves by more than the 2^8 up to which the scale is kept
+    # (ramp 0.004 over the 256 keys between a warp's units: scores double from unit to unit, up to hundreds), or only falls
+    _compare(B, source, 40, 4, 1, d, [1100] * 40, 64, 2, ramp=ramp)
