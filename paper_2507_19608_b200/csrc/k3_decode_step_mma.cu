@@ -37,7 +37,8 @@
 // the step's global stores).
 // Measured, us per step of a loop of steps, before -> after the changes above: Llama layer at 2048 keys, batch 1
 // 4.4 -> 4.1 (the caller's host time; 3.3 on the device), batch 16 12.2 -> 9.3 (7.6 TB/s from L2); batch 8 at 4096 keys
-// 11.6 -> 9.5; BitNet layer (d = 128) at 1531 keys, batch 2 6.1 -> 5.0; key deltas, batch 4 at 1777 keys 6.4 -> 5.0.
+// 11.6 -> 9.5; BitNet layer (d = 128) at 1531 keys, batch 2 6.1 -> 5.0; key deltas, batch 4 at 1777 keys 6.4 -> 5.0;
+// compressed key cache, batch 4 at 1024 keys 8.0 -> 7.2.
 // Tried and dropped: the next unit's scores issued under a unit's softmax and P.V (twice the code, spills: batch 16
 // 10.3); three slots without the rest (nothing: no warp was waiting for its copies).
 #include <cuda.h>
@@ -119,6 +120,12 @@ __device__ __forceinline__ uint32_t lds_u16(uint32_t a) {
 __device__ __forceinline__ void sts_u4(uint32_t a, uint4 v) {
   asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(a), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w) : "memory");
 }
+__device__ __forceinline__ void lds_words(uint32_t a, uint32_t (&w)[2]) {
+  asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(w[0]), "=r"(w[1]) : "r"(a));
+}
+__device__ __forceinline__ void lds_words(uint32_t a, uint32_t (&w)[4]) {
+  asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(w[0]), "=r"(w[1]), "=r"(w[2]), "=r"(w[3]) : "r"(a));
+}
 __device__ __forceinline__ void sts_u32(uint32_t a, uint32_t v) { asm volatile("st.shared.u32 [%0], %1;" ::"r"(a), "r"(v) : "memory"); }
 // N consecutive elements, as fp32, past the L1 cache
 template <int N> __device__ __forceinline__ void load_bf16(const __nv_bfloat16* p, float (&x)[N]) {
@@ -143,10 +150,11 @@ template <int N> __device__ __forceinline__ void load_f32(const float* p, float 
 }
 // Shared memory: per warp a ring of NS halves of units (the keys, or the values, of one unit: 128-byte
 // swizzle, blocks of [32 rows][64 channels]), whose first slot takes the warp's result in the end, then the merge's records.
-// PACKED: per warp also the encoding of one 32-row segment: values, mask words, the reference in front.
+// PACKED: per warp also the encoding of one 32-row segment: values, mask words, the reference in front;
+// and a table of its rows (rebuild below).
 template <int D, int G, bool PACKED> struct MmaSmem {
   static constexpr int NW = kWarps<D>;
-  static constexpr uint32_t VALS = UK * D * 2 + 16, MASKS = UK * (D / 32) * 4, PACK = PACKED ? VALS + MASKS + D * 2 : 0;
+  static constexpr uint32_t VALS = UK * D * 2 + 16, MASKS = UK * (D / 32) * 4, ROWS = UK * 16, PACK = PACKED ? VALS + MASKS + D * 2 + ROWS : 0;
   static constexpr uint32_t HALF = UK * D * 2;             // keys, or values, of a unit
   static constexpr int NS = PACKED ? 2 : 3;                // (two CTAs per SM: 2 x 113 KB)
   static constexpr uint32_t RING = NW * NS * HALF;
@@ -244,6 +252,9 @@ decode_step_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_co
   const uint32_t pack_s = packs + (uint32_t)warp * SM::PACK;       // values, mask words, base
   const uint32_t* const so = PACKED ? p.seg_off + (size_t)bkv * (p.nseg_max + 1) : nullptr;
   auto from_pack = [&](int jg) { return PACKED && jg < wl && jg < n; };          // some row is a cached reference row
+  auto row_at = [&](uint32_t slot, int r, int ch) {          // 16-byte piece ch of row r
+    return slot + (ch >> 3) * UK * 128 + r * 128 + (((ch & 7) ^ (r & 7)) << 4);
+  };
   auto fetch_k = [&](int jg, int slot) {
     const uint32_t bar_k = bars0 + 8 * slot, slot_k = slots + slot * SM::HALF;
     if (from_pack(jg)) {
@@ -251,14 +262,23 @@ decode_step_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_co
       // row extends or follows that segment: old and new value both bound the cached values)
       if (lane == 0) {
         const int sg = jg / UK;
-        const uint32_t v0 = __ldcg(so + sg), v1 = __ldcg(so + sg + 1);
-        const uint32_t vb = min((v1 - v0 + 7u) & ~7u, (uint32_t)UK * D) * 2u;
+        // (the bounds hold for any encoding a prefill and at most T_max - T steps behind it have built; a
+        // captured step that is replayed appends its row again and again)
+        const uint32_t v0 = min(__ldcg(so + sg), (uint32_t)p.cap - D) & ~7u, v1 = __ldcg(so + sg + 1);
+        const uint32_t vb = min(min((v1 - v0 + 7u) & ~7u, (uint32_t)UK * D), (uint32_t)p.cap - v0) * 2u;
         tc::mbar_expect_tx(bar_k, vb + SM::MASKS + D * 2);
         if (vb) bulk_load(pack_s, p.vals + (size_t)bkv * p.cap + v0, vb, bar_k);
         bulk_load(pack_s + SM::VALS, p.kp_mask + ((size_t)bkv * p.nseg_max * UK + jg) * (D / 32), SM::MASKS, bar_k);
         bulk_load(pack_s + SM::VALS + SM::MASKS, p.base + ((size_t)bkv * p.nseg_max + sg) * D, D * 2, bar_k);
       }
-      // (the original keys of a mixed unit's window rows follow when the rows are rebuilt)
+      // rows of a mixed unit that are not cached references: original keys, the new one, zeros
+#pragma unroll 1
+      for (int e = min(UK, min(n, wl) - jg) * (D / 8) + lane; e < UK * (D / 8); e += 32) {
+        const int r = e / (D / 8), ch = e % (D / 8), j = jg + r;
+        const uint32_t dst = row_at(slot_k, r, ch);
+        if (j <= n) async16(dst, (j < n ? kc + (size_t)j * D : kn) + 8 * ch);
+        else sts128z(dst);
+      }
     } else if (k_plain(jg)) {
       tc::mbar_expect_tx_if(lead, bar_k, SM::HALF);
       const CUtensorMap* tm = (MODE == 1 && jg < wl) ? &tm_h : &tm_k;
@@ -286,9 +306,6 @@ decode_step_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_co
   // the warp that owns the row arriving with the step, and that row in shared memory (keys, values)
   const bool has_new = j1 == L && j0 < L && ((n - j0) / UK) % MNW == warp;
   const uint32_t new_s = packs + MNW * SM::PACK;
-  auto row_at = [&](uint32_t slot, int r, int ch) {          // 16-byte piece ch of row r
-    return slot + (ch >> 3) * UK * 128 + r * 128 + (((ch & 7) ^ (r & 7)) << 4);
-  };
   // Reference-key rows and their encoding are the library's own: behind another step (p.early) all but the
   // row (segment) that step may be writing is final before this kernel can start, since a step releases
   // the next one only behind its own wait, and is requested ahead of the wait.  Not so behind a prefill:
@@ -399,43 +416,58 @@ decode_step_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_co
   float* const Rg = KEY ? nullptr : p.R + ((size_t)b * p.H + kvh * G + hd) * T_max;
   // Rows jg .. jg + 31 of the reference-key stream from their encoding, into the key slot: lane = two
   // channels (of a 64-channel block), walking the rows; the window's rows and the new one are keys.
+  // Issue-bound, so what a row needs is laid out first, lane = row: for either half of the block's channels where the
+  // row's values of that half start and its mask word.  (Every lane counting for itself, and a row's loads behind the
+  // store of the one before: 147 clocks per row, a unit 2.5 us.)
   auto rebuild = [&](int jg, uint32_t slot_k) {
     constexpr int NWD = D / 32;
     const int last = min(UK, min(n, wl) - jg);             // rows that are cached references
     const int hi = lane >> 4, sh = 2 * (lane & 15);        // this lane's channels: bits sh, sh + 1 of word 2 c + hi
     const uint32_t lt = (1u << sh) - 1u;
+    const uint32_t table = pack_s + SM::VALS + SM::MASKS + D * 2;
+    uint32_t w[NWD], total = 0;
+    lds_words(pack_s + SM::VALS + 4 * NWD * lane, w);
+#pragma unroll
+    for (int k = 0; k < NWD; ++k) total += __popc(w[k]);
+    uint32_t at = total;                                   // values up to this row, then in front of it
+#pragma unroll
+    for (int x = 1; x < 32; x <<= 1) {
+      const uint32_t up = __shfl_up_sync(0xffffffffu, at, x);
+      at += lane >= x ? up : 0u;
+    }
+    at = pack_s + 2 * (at - total);
 #pragma unroll
     for (int c = 0; c < NV; ++c) {
-      uint32_t cur = lds_u32(pack_s + SM::VALS + SM::MASKS + 128 * c + 4 * lane), at = pack_s;
+      const uint32_t at1 = at + 2 * __popc(w[2 * c]);
+      sts_u4(table + 16 * lane, make_uint4(at, w[2 * c], at1, w[2 * c + 1]));
+      at = at1 + 2 * __popc(w[2 * c + 1]);
+      __syncwarp();
+      uint32_t cur = lds_u32(pack_s + SM::VALS + SM::MASKS + 128 * c + 4 * lane);
       const uint32_t dst = slot_k + c * UK * 128 + 4 * (lane & 3);
-#pragma unroll 8
-      for (int r = 0; r < last; ++r) {
-        uint32_t w[NWD], below = 0, total = 0;
-#pragma unroll
-        for (int i = 0; i < NWD; ++i) {
-          w[i] = lds_u32(pack_s + SM::VALS + 4 * (r * NWD + i));
-          if (i == 2 * c) below = total + (hi ? (uint32_t)__popc(w[i]) : 0u);
-          total += __popc(w[i]);
-        }
-        const uint32_t mine = hi ? w[2 * c + 1] : w[2 * c];
-        const uint32_t a = at + 2 * (below + __popc(mine & lt)), f = mine >> sh;
-        // (a channel that has not fired reads some value of the pool and drops it: no branch, and the
-        // loads of eight rows are in flight together)
-        const uint32_t x0 = lds_u16(a), x1 = lds_u16(a + 2 * (f & 1u));
-        cur = (f & 1u) ? __byte_perm(cur, x0, 0x3254) : cur;
-        cur = (f & 2u) ? __byte_perm(cur, x1, 0x5410) : cur;
-        sts_u32(dst + r * 128 + (((lane >> 2) ^ (r & 7)) << 4), cur);
-        at += 2 * total;
-      }
 #pragma unroll 1
-      for (int e = last * 8 + lane; e < UK * 8; e += 32) {
-        const int r = e >> 3, ch = e & 7, j = jg + r;
-        const uint32_t dst = slot_k + c * UK * 128 + r * 128 + ((ch ^ (r & 7)) << 4);
-        if (j <= n) async16(dst, (j < n ? kc + (size_t)j * D : kn) + 64 * c + 8 * ch);
-        else sts128z(dst);
+      for (int r0 = 0; r0 < last; r0 += 8) {
+        uint32_t f[8], a[8], x0[8], x1[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+          uint32_t e[2];
+          lds_words(table + 16 * (r0 + i) + 8 * hi, e);
+          a[i] = e[0] + 2 * __popc(e[1] & lt);
+          f[i] = e[1] >> sh;
+        }
+        // (a channel that has not fired reads some value of the pool and drops it: no branch)
+#pragma unroll
+        for (int i = 0; i < 8; ++i) { x0[i] = lds_u16(a[i]); x1[i] = lds_u16(a[i] + 2 * (f[i] & 1u)); }
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+          const int r = r0 + i;
+          cur = (f[i] & 1u) ? __byte_perm(cur, x0[i], 0x3254) : cur;
+          cur = (f[i] & 2u) ? __byte_perm(cur, x1[i], 0x5410) : cur;
+          if (r < last) sts_u32(dst + r * 128 + (((lane >> 2) ^ (r & 7)) << 4), cur);
+        }
       }
+      __syncwarp();
     }
-    async_wait_all();
+    async_wait_all();                                      // the rows that are not cached references (fetch_k)
     __syncwarp();
   };
   // The new row joins the encoding (the warp that owns its unit): values behind the pool's end (on a
@@ -443,7 +475,7 @@ decode_step_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_co
   auto append = [&](int nz) {
     const int sg = n / UK;
     const bool opens = (n % UK) == 0;
-    const uint32_t pool = __ldcg(p.used + bkv), pos = opens ? (pool + 7u) & ~7u : pool;
+    const uint32_t pool = __ldcg(p.used + bkv), pos = min(opens ? (pool + 7u) & ~7u : pool, (uint32_t)p.cap - D);
     uint16_t* const vg = p.vals + (size_t)bkv * p.cap;
     uint32_t at = pos;
 #pragma unroll
