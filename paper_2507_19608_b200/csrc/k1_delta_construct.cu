@@ -7,7 +7,7 @@
 // heads, or KV heads for key deltas).  The chain itself is three dependent FP32 operations per
 // token and a lone warp issues slowly, so everything else is kept off it: a producer warp
 // streams the rows into a ring of shared-memory stages with TMA (the rows do not depend on the
-// carried state), helper warps precompute everything about a four-row sub-block that does not
+// carried state), helper warps precompute everything about an eight-row sub-block that does not
 // involve the carried state (see the kernel), and the chain warp stores nothing but the
 // reference in front of every 8-row block (and every 64-row tile, and the final one).  Given
 // those checkpoints every 8-row block of Eq. 2-3 is independent of the others: fire bits,
@@ -28,14 +28,16 @@ namespace delta {
 namespace {
 
 constexpr int RC = 64;       // rows per ring stage (= one 64-row tile)
-constexpr int NS = 6;        // stages of staged rows
-constexpr int NZ = 2;        // stages of sub-block tables
+constexpr int NS = 8;        // stages of staged rows
+constexpr int NZ = 4;        // stages of sub-block tables
 constexpr int CH = 32;       // channels per CTA: one chain warp, thread = channel
-constexpr int SBR = 4;       // rows per sub-block
+constexpr int SBR = DELTA_CKPT_ROWS;     // rows per sub-block: one checkpoint each
 constexpr int NSB = RC / SBR;
-constexpr int NHELP = 3;     // warps that build the sub-block tables
-constexpr int Z_STAGE = NSB * 2 * CH;    // float4 per table stage: per (sub-block, channel) x0..x3 and z0..z2
-constexpr int CHAIN_THREADS = 32 * (1 + NHELP + 1);
+constexpr int NHELP = 12;    // warps that build the sub-block tables
+constexpr int ZV = 4;        // float4 per (sub-block, channel): x0..x7, z0..z6
+constexpr int Z_STAGE = NSB * ZV * CH;   // float4 per table stage
+constexpr int CHAIN_THREADS = 32 * (NHELP / 3 * 4);
+static_assert(SBR == 8 && NHELP % 3 == 0 && NHELP >= 6, "the kernel's tables and its warp roles");
 
 template <typename TIn> __device__ __forceinline__ float lds_elem(const TIn* p);
 template <> __device__ __forceinline__ float lds_elem<float>(const float* p) { return *p; }
@@ -48,13 +50,6 @@ __device__ __forceinline__ bool fires(float x, float x_ref, float theta) {
   return fabsf(__fsub_rn(x, x_ref)) > theta;
 }
 
-// Tight bounded poll of an mbarrier phase for the chain warp (a suspended wait wakes up late,
-// and the hand-over is on the chain's path); false once the CTA has given up.
-__device__ __forceinline__ bool poll_ok(uint32_t bar, uint32_t parity, volatile uint32_t* abort_flag) {
-  if (mbar_test_wait(bar, parity)) return true;
-  mbar_poll(bar, parity, abort_flag);
-  return *abort_flag == 0;
-}
 // The helpers' waits: suspended (they run ahead of the chain warp, and where several CTAs share
 // an SM a spinning helper would take issue slots from another CTA's chain warp).
 __device__ __forceinline__ bool wait_ok(uint32_t bar, uint32_t parity, volatile uint32_t* abort_flag) {
@@ -63,24 +58,67 @@ __device__ __forceinline__ bool wait_ok(uint32_t bar, uint32_t parity, volatile 
   return *abort_flag == 0;
 }
 
+// One arrival for the warp, predicated: a branch that one lane takes costs the chain warp its reconvergence.
+__device__ __forceinline__ void arrive_lane0(uint32_t bar, int lane) {
+  asm volatile("{\n\t.reg .pred p;\n\tsetp.eq.s32 p, %1, 0;\n\t@p mbarrier.arrive.shared::cta.b64 _, [%0];\n\t}"
+               ::"r"(bar), "r"(lane) : "memory");
+}
+
+// A sub-block's table for one channel: its rows and the end states z (z7 = x7), as the chain warp loads them.
+struct SubBlock {
+  float4 x[2], z[2];      // x0..x7, z0..z6
+};
+__device__ __forceinline__ SubBlock load_sub_block(const float4* p) {
+  SubBlock t;
+  t.x[0] = p[0];
+  t.x[1] = p[CH];
+  t.z[0] = p[2 * CH];
+  t.z[1] = p[3 * CH];
+  return t;
+}
+
+// The state behind a sub-block that is entered with state r: of the rows that fire against r (one IEEE subtraction,
+// strict compare, NaN false: see fires) the first one's end state, r where none does.  basis: row 0 is taken
+// un-thresholded.
+__device__ __forceinline__ float chain_sub_block(const SubBlock& t, float r, float theta, bool basis) {
+  const bool p0 = fires(t.x[0].x, r, theta) || basis, p1 = fires(t.x[0].y, r, theta), p2 = fires(t.x[0].z, r, theta);
+  const bool p3 = fires(t.x[0].w, r, theta), p4 = fires(t.x[1].x, r, theta), p5 = fires(t.x[1].y, r, theta);
+  const bool p6 = fires(t.x[1].z, r, theta), p7 = fires(t.x[1].w, r, theta);
+  float o = p7 ? t.x[1].w : r;
+  o = p6 ? t.z[1].z : o;
+  o = p5 ? t.z[1].y : o;
+  o = p4 ? t.z[1].x : o;
+  o = p3 ? t.z[0].w : o;
+  o = p2 ? t.z[0].z : o;
+  o = p1 ? t.z[0].y : o;
+  return p0 ? t.z[0].x : o;
+}
+
 }  // namespace
 
 // The chain of Eq. 3 costs three dependent operations per row (subtract, compare, select), about
-// 17 clocks.  Most of that can be taken off the carried state.  Over a sub-block of four rows
-// x0..x3 (in processing order) the state r either survives, or the first row i that fires
+// 17 clocks.  Most of that can be taken off the carried state.  Over a sub-block of eight rows
+// x0..x7 (in processing order) the state r either survives, or the first row i that fires
 // against r replaces it -- and from there on the chain no longer depends on r: the state at the
 // end of the sub-block is z_i, the end state of the chain that starts with reference x_i at
-// row i.  z_3 = x3, z_2 = fires(x3, x2) ? x3 : x2, and in general z_i = z_j for the first j > i
-// that fires against x_i (x_i if none does): six pair tests per sub-block, none of which
+// row i.  z_7 = x7, z_6 = fires(x7, x6) ? x7 : x6, and in general z_i = z_j for the first j > i
+// that fires against x_i (x_i if none does): 28 pair tests per sub-block, none of which
 // involves r.  Helper warps compute the z tables a stage ahead; the chain warp then does, per
-// sub-block, four tests against r in parallel and a two-level select: the dependent path is
-// subtract, compare, three selects per FOUR rows.  Every test is the same subtraction and
-// comparison the sequential chain would make, so the result is bit-identical.
+// sub-block, eight tests against r in parallel and a select tree: the dependent path is
+// subtract, compare, four selects per EIGHT rows, and the checkpoint in front of the sub-block is the only
+// store.  Every test is the same subtraction and comparison the sequential chain would make, so the
+// result is bit-identical.
 //
-// One CTA per (head, 32 channels): warp 0 carries the chain (thread = channel), warps 1-3 build
-// the tables, warp 4 streams the rows in with TMA.  Stages that hold the un-thresholded basis
-// row or are cut short by the end of the sequence take the sequential form from the staged
-// values.
+// One CTA per (head, 32 channels): a warp carries the chain (thread = channel), one streams the rows in with TMA,
+// twelve build the tables, on the three schedulers beside the chain warp's.  A lone warp builds a table in 220
+// clocks, two on a scheduler one in 163 (28 tests, half of their instructions on the half-rate pipe); the sub-blocks
+// are dealt to the warps one by one, whatever their stage (a warp that waits and arrives for every stage costs
+// 1000 clocks per stage: the chain then waits for the tables), four stages of tables ahead at most.  The chain warp
+// takes 57 clocks per sub-block of a table already there and 86 in the kernel, stage edges, checkpoint stores and the
+// helpers' shared-memory traffic included (10.8 per row; four rows per table with three helpers: 14; row by row 16.8).
+// A sub-block cut short by the end of the sequence takes the sequential form from the staged values.
+// Measured (with the launch, by events), before -> after: 1 x 32 heads, 1024 tokens, d = 64 14.7 -> 13.9 us; 4096 keys
+// 36.4 -> 30.2; 20 heads, 2048 tokens, d = 128 22.0 -> 19.9; a cut last stage (1000 tokens) 16.1 -> 14.1.
 template <typename TIn, int D>
 __global__ void __launch_bounds__(CHAIN_THREADS) delta_chain_kernel(
     const __grid_constant__ CUtensorMap tm_x, float* __restrict__ qhat_tile, float* __restrict__ qhat_out,
@@ -91,7 +129,7 @@ __global__ void __launch_bounds__(CHAIN_THREADS) delta_chain_kernel(
   constexpr uint32_t RAW_STAGE_BYTES = RC * CH * sizeof(TIn);
   extern __shared__ __align__(128) unsigned char dyn[];
   TIn* raw = reinterpret_cast<TIn*>(dyn);                                   // [NS][RC][CH]
-  float4* zb = reinterpret_cast<float4*>(dyn + NS * RAW_STAGE_BYTES);       // [NZ][NSB][x | z][CH]
+  float4* zb = reinterpret_cast<float4*>(dyn + NS * RAW_STAGE_BYTES);       // [NZ][NSB][ZV][CH]
   __shared__ __align__(8) unsigned long long bars[2 * NS + 2 * NZ];
   __shared__ uint32_t s_abort;
 
@@ -101,19 +139,23 @@ __global__ void __launch_bounds__(CHAIN_THREADS) delta_chain_kernel(
   const uint32_t zfull0 = smem_u32(&bars[2 * NS]), zfree0 = smem_u32(&bars[2 * NS + NZ]);
   volatile uint32_t* abort_flag = &s_abort;
   const int n_chunks = (T + RC - 1) / RC;
+  // Which of the four schedulers' first warps carries the chain rotates with the CTA: where several CTAs
+  // share an SM their chain warps, the busiest, then sit on different schedulers.  The producer is the
+  // other warp of the chain's scheduler.
+  const int cw = (int)blockIdx.x & 3;
   // the deferred clearing of a state reset (counters, tickets, second reference buffer): nothing
   // of this launch or of the kernels behind it touches that span before this kernel is complete
   if (zero_ptr && blockIdx.x == 0)
     for (unsigned i = tid; i < zero_n16; i += blockDim.x) zero_ptr[i] = make_uint4(0u, 0u, 0u, 0u);
 
   if (tid < 2 * NS + 2 * NZ) {      // one barrier per thread
-    const uint32_t cnt = (tid < NS) ? 1u : (tid < 2 * NS) ? (uint32_t)NHELP : (tid < 2 * NS + NZ) ? (uint32_t)NHELP : 1u;
+    const uint32_t cnt = (tid < NS) ? 1u : (tid < 2 * NS + NZ) ? (uint32_t)NSB : 1u;
     tc::mbar_init(full0 + 8 * tid, cnt);
     if (tid == 0) s_abort = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     tc::fence_proxy_async();
   }
-  if (tid == 32 * (1 + NHELP))
+  if (tid == 32 * (4 + cw))
     asm volatile("prefetch.tensormap [%0];" ::"l"(&tm_x) : "memory");
   __syncthreads();
   // a kernel launched behind this one with programmatic stream serialisation may become
@@ -121,10 +163,7 @@ __global__ void __launch_bounds__(CHAIN_THREADS) delta_chain_kernel(
   // grid-dependency wait
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 
-  // Which of the four compute warps carries the chain rotates with the CTA: where several CTAs
-  // share an SM their chain warps, the busiest, then sit on different schedulers.
-  const int cw = (int)blockIdx.x & 3;
-  if (warp == 1 + NHELP) {
+  if (warp == 4 + cw) {
     // ---- producer: keeps up to NS stages of rows in flight
     if (lane == 0) {
       const uint32_t raw0 = smem_u32(raw);
@@ -136,129 +175,114 @@ __global__ void __launch_bounds__(CHAIN_THREADS) delta_chain_kernel(
         tc::tma_load_3d(raw0 + s * RAW_STAGE_BYTES, &tm_x, full0 + 8 * s, sl * CH, ci * RC, bh);
       }
     }
-  } else if (warp != cw) {
-    // ---- helpers: helper hw takes sub-blocks hw, hw + 3, ... of every stage; rows in processing
-    // order (reverse: from the stage's last row down), tables in processing order of the sub-blocks
-    const int hw = (warp - cw - 1) & 3;      // 0, 1, 2
-    int s = 0, zs = 0;
-    uint32_t ph_full = 0, ph_zfree = 0;      // parity of the completion waited for next
-    for (int i = 0; i < n_chunks; ++i) {
-      if (!wait_ok(full0 + 8 * s, ph_full, abort_flag)) break;
-      const TIn* rows = raw + (size_t)s * RC * CH + lane;
-      constexpr int NJ = (NSB + NHELP - 1) / NHELP;
-      float y[NJ][SBR];        // every load in front of the first store (both are shared memory)
+  } else if ((warp & 3) != cw) {
+    // ---- helpers: the sub-blocks of all stages, in processing order (reverse: from the stage's last row
+    // down), are dealt round-robin
+    const int hw = ((warp - cw - 1) & 3) + 3 * (warp >> 2);
+    const ptrdiff_t rstep = reverse ? -CH : CH;
+    for (int gb = hw; gb < n_chunks * NSB; gb += NHELP) {
+      const int i = gb / NSB, sb = gb % NSB, s = i % NS, zs = i % NZ;
+      if (!wait_ok(full0 + 8 * s, (i / NS) & 1, abort_flag)) break;
+      const TIn* rows = raw + (size_t)s * RC * CH + lane + (reverse ? (RC - 1) * CH : 0) + sb * SBR * rstep;
+      float y[SBR], z[SBR];
 #pragma unroll
-      for (int j = 0; j < NJ; ++j) {
-        const int sb = min(hw + NHELP * j, NSB - 1);
+      for (int k = 0; k < SBR; ++k) z[k] = y[k] = lds_elem<TIn>(rows + k * rstep);
 #pragma unroll
-        for (int k = 0; k < SBR; ++k) y[j][k] = lds_elem<TIn>(rows + (sb * SBR + (reverse ? SBR - 1 - k : k)) * CH);
-      }
-      if (i >= NZ && !wait_ok(zfree0 + 8 * zs, ph_zfree, abort_flag)) break;
-      float4* zp = zb + (size_t)zs * Z_STAGE + lane;
+      for (int j = SBR - 1; j > 0; --j)
 #pragma unroll
-      for (int j = 0; j < NJ; ++j) {
-        const int sb = hw + NHELP * j;
-        if (sb < NSB) {
-          const float z2 = fires(y[j][3], y[j][2], theta) ? y[j][3] : y[j][2];
-          float z1 = fires(y[j][3], y[j][1], theta) ? y[j][3] : y[j][1];
-          z1 = fires(y[j][2], y[j][1], theta) ? z2 : z1;
-          float z0 = fires(y[j][3], y[j][0], theta) ? y[j][3] : y[j][0];
-          z0 = fires(y[j][2], y[j][0], theta) ? z2 : z0;
-          z0 = fires(y[j][1], y[j][0], theta) ? z1 : z0;
-          float4* o = zp + (reverse ? NSB - 1 - sb : sb) * (2 * CH);
-          o[0] = make_float4(y[j][0], y[j][1], y[j][2], y[j][3]);
-          o[CH] = make_float4(z0, z1, z2, 0.0f);
-        }
-      }
+        for (int a = j - 1; a >= 0; --a) z[a] = fires(y[j], y[a], theta) ? z[j] : z[a];
+      if (i >= NZ && !wait_ok(zfree0 + 8 * zs, ((i / NZ) - 1) & 1, abort_flag)) break;
+      float4* o = zb + (size_t)zs * Z_STAGE + sb * (ZV * CH) + lane;
+      o[0] = make_float4(y[0], y[1], y[2], y[3]);
+      o[CH] = make_float4(y[4], y[5], y[6], y[7]);
+      o[2 * CH] = make_float4(z[0], z[1], z[2], z[3]);
+      o[3 * CH] = make_float4(z[4], z[5], z[6], 0.0f);
       __syncwarp();
-      if (lane == 0) {
-        tc::mbar_arrive(zfull0 + 8 * zs);
-        tc::mbar_arrive(empty0 + 8 * s);
-      }
-      if (++s == NS) { s = 0; ph_full ^= 1u; }
-      if (++zs == NZ) { zs = 0; if (i >= NZ) ph_zfree ^= 1u; }
+      arrive_lane0(zfull0 + 8 * zs, lane);
+      arrive_lane0(empty0 + 8 * s, lane);
     }
-  } else {
+  } else if (warp == cw) {
     // ---- chain warp: thread owns channel c
     const int c = sl * CH + lane;
     float r = 0.0f;           // reference state, starts at zero (Eq. 3)
-    int zs = 0;
-    uint32_t ph_zfull = 0;
     static_assert(RC == DELTA_TILE_ROWS, "one tile reference per stage");
+    const ptrdiff_t step = reverse ? -(ptrdiff_t)D : (ptrdiff_t)D;
+    const int tile0 = reverse ? n_chunks - 1 : 0;       // tile (= stage in token order) of stage 0
+    // where the references in front of the stage and of its sub-blocks go, in processing order
+    float* qp = qhat_tile + ((size_t)bh * n_tiles + tile0) * D + c;
     float* const ckpt_c = ckpt + (size_t)bh * n_ckpt * D + c;
-    float* const qtile = qhat_tile ? qhat_tile + (size_t)bh * n_tiles * D + c : nullptr;
-    const ptrdiff_t cstep = reverse ? -(ptrdiff_t)D : (ptrdiff_t)D;
-    int t0 = reverse ? (n_chunks - 1) * RC : 0;       // first row of the stage, stepped by dt
-    const int dt = reverse ? -RC : RC;
-    // checkpoint of the 8-row block the processing order enters next (full stages step it)
-    float* cp = ckpt_c + (size_t)((t0 + (reverse ? RC - SBR : 0)) / DELTA_CKPT_ROWS) * D;
-    bool ready = false;       // the stage's tables were seen complete during the stage before
-    for (int i = 0; i < n_chunks; ++i, t0 += dt) {
-      const int nrows = min(RC, T - t0);
-      if (qhat_tile && DELTA_IN(t0 / DELTA_TILE_ROWS, n_tiles, counters)) qtile[(size_t)(t0 / DELTA_TILE_ROWS) * D] = r;
-      if (!ready && !poll_ok(zfull0 + 8 * zs, ph_zfull, abort_flag)) break;
-      const int zs_next = (zs + 1 == NZ) ? 0 : zs + 1;
-      const uint32_t ph_next = (zs + 1 == NZ) ? ph_zfull ^ 1u : ph_zfull;
-      const float4* zp = zb + (size_t)zs * Z_STAGE + lane;
-      const bool has_basis = basis_exact && i == 0;      // row 0, or row T-1 in reverse
-      if (nrows == RC) {
-        float4 x = zp[0], z = zp[CH];
-#pragma unroll
-        for (int lsb = 0; lsb < NSB; ++lsb) {
-          // the next sub-block's tables while this one is worked on
-          const float4 xn = zp[(lsb + 1 < NSB ? lsb + 1 : lsb) * (2 * CH)];
-          const float4 zn = zp[(lsb + 1 < NSB ? lsb + 1 : lsb) * (2 * CH) + CH];
-          if ((lsb & 1) == 0) {
-            // the reference in front of an 8-row block (reverse: in front of its highest row)
-            if (DELTA_IN((size_t)(cp - ckpt_c) / D, n_ckpt, counters)) *cp = r;
-            cp += cstep;
-          }
-          // (a look at the next stage's barrier a few sub-blocks before the end: the answer is
-          // back by the time it is needed)
-          if (lsb == NSB - 4) ready = mbar_test_wait(zfull0 + 8 * zs_next, ph_next);
-          const bool p3 = fires(x.w, r, theta), p2 = fires(x.z, r, theta);
-          bool p0 = fires(x.x, r, theta);
-          if (lsb == 0) p0 = p0 || has_basis;      // the basis row is taken un-thresholded
-          const bool p1 = fires(x.y, r, theta);
-          float b = p3 ? x.w : r;
-          b = p2 ? z.z : b;
-          const float a = p0 ? z.x : z.y;          // the first of rows 0, 1 that fired, if one did
-          r = (p0 || p1) ? a : b;
-          x = xn; z = zn;
-        }
-      } else {
-        // a stage cut short by the end of the sequence: row by row from the staged values
-        ready = false;
-        for (int lsb = 0; lsb < NSB; ++lsb) {
-          const float4 x4 = zp[lsb * (2 * CH)];
-          const float xs[SBR] = {x4.x, x4.y, x4.z, x4.w};
-#pragma unroll
-          for (int k = 0; k < SBR; ++k) {
-            const int l = lsb * SBR + k;
-            const int pr = reverse ? RC - 1 - l : l;     // row of the stage
-            if (pr < nrows) {
-              const int t = t0 + pr;
-              const bool at_ckpt = reverse ? ((t % DELTA_CKPT_ROWS) == DELTA_CKPT_ROWS - 1 || pr == nrows - 1)
-                                           : (t % DELTA_CKPT_ROWS) == 0;
-              if (at_ckpt && DELTA_IN(t / DELTA_CKPT_ROWS, n_ckpt, counters))
-                ckpt_c[(size_t)(t / DELTA_CKPT_ROWS) * D] = r;
-              const bool basis_here = has_basis && (reverse ? pr == nrows - 1 : pr == 0);
-              r = (basis_here || fires(xs[k], r, theta)) ? xs[k] : r;
-            }
+    float* cp = ckpt_c + (ptrdiff_t)(tile0 * NSB + (reverse ? NSB - 1 : 0)) * D;
+    const int rest = T % RC;                            // rows of a stage cut short by the end of the sequence
+    auto wait_stage = [&](int i) { mbar_poll(zfull0 + 8 * (i % NZ), (i / NZ) & 1, abort_flag); __syncwarp(); };
+    auto tile_ref = [&](int i) {
+      if (qhat_tile && DELTA_IN(reverse ? tile0 - i : i, n_tiles, counters)) *qp = r;
+      qp += step;
+    };
+    // the cut stage (the last one; reverse: the first): sub-blocks behind the end carry no state, the one the
+    // end falls into goes row by row
+    auto cut_stage = [&](int i) {
+      wait_stage(i);
+      tile_ref(i);
+      const float4* const zp = zb + (size_t)(i % NZ) * Z_STAGE + lane;
+      for (int b = 0; b < NSB; ++b, cp += step) {
+        const int pr0 = (reverse ? NSB - 1 - b : b) * SBR;          // the sub-block's lowest row of the stage
+        if (pr0 >= rest) continue;
+        const float4* const p = zp + b * (ZV * CH);
+        const bool head = basis_exact && i == 0 && (reverse ? pr0 + SBR >= rest : b == 0);
+        if (DELTA_IN((size_t)(cp - ckpt_c) / D, n_ckpt, counters)) *cp = r;
+        if (pr0 + SBR <= rest) {
+          r = chain_sub_block(load_sub_block(p), r, theta, head);
+        } else {
+          const int n = rest - pr0;                                 // rows of the sub-block, the lowest ones
+          const float* const x = reinterpret_cast<const float*>(p);
+          for (int k = reverse ? SBR - n : 0; k < (reverse ? SBR : n); ++k) {
+            const float xk = x[(k >> 2) * (4 * CH) + (k & 3)];
+            r = ((head && k == (reverse ? SBR - n : 0)) || fires(xk, r, theta)) ? xk : r;
           }
         }
       }
       __syncwarp();
-      if (lane == 0) tc::mbar_arrive(zfree0 + 8 * zs);
-      if (nrows != RC) cp = ckpt_c + (size_t)((t0 + dt + (reverse ? RC - SBR : 0)) / DELTA_CKPT_ROWS) * D;
-      zs = zs_next; ph_zfull = ph_next;
+      arrive_lane0(zfree0 + 8 * (i % NZ), lane);
+    };
+    const int i0 = (reverse && rest) ? 1 : 0, i1 = i0 + T / RC;      // the whole stages
+    if (i0) cut_stage(0);
+    if (i0 < i1) {
+      wait_stage(i0);
+      SubBlock cur = load_sub_block(zb + (size_t)(i0 % NZ) * Z_STAGE + lane);
+      // One pass of the loop per stage, its eight sub-blocks unrolled (two or four to a pass are slower: 40.6 and 36.5 us
+      // for 4096 rows, unrolled 32.7, with the stage's edge as below 30.2); a sub-block's tables are loaded while the one in front is worked on, over the stage's end too,
+      // where the next stage's barrier is looked at two sub-blocks ahead.
+#pragma unroll 1
+      for (int i = i0; i < i1; ++i) {
+        const float4* const zp = zb + (size_t)(i % NZ) * Z_STAGE + lane;
+        const int in = i + 1;
+        tile_ref(i);
+        bool ready = true;
+#pragma unroll
+        for (int b = 0; b < NSB; ++b) {
+          SubBlock nxt;
+          if (b + 1 < NSB) {
+            nxt = load_sub_block(zp + (b + 1) * (ZV * CH));
+          } else {
+            if (!__all_sync(0xffffffffu, ready)) wait_stage(in);
+            nxt = load_sub_block(zb + (size_t)(in % NZ) * Z_STAGE + lane);      // (behind the last stage: not used)
+          }
+          if (b == NSB - 3) ready = in >= i1 || mbar_test_wait(zfull0 + 8 * (in % NZ), (in / NZ) & 1);
+          if (DELTA_IN((size_t)(cp - ckpt_c) / D, n_ckpt, counters)) *cp = r;
+          cp += step;
+          r = chain_sub_block(cur, r, theta, b == 0 && i == 0 && basis_exact);
+          cur = nxt;
+        }
+        __syncwarp();
+        arrive_lane0(zfree0 + 8 * (i % NZ), lane);
+      }
     }
+    if (!reverse && rest) cut_stage(i1);
     if (!*abort_flag && qhat_out) qhat_out[(size_t)bh * D + c] = r;
   }
   __syncthreads();
   if (tid == 0 && s_abort) atomicMax(&counters[CNT_STATUS], (unsigned long long)DELTA_ERR_TIMEOUT);
 }
-
 
 static cudaError_t launch_delta_chain_tables(const Shape& s, const Workspace& w, const void* q, int T, float theta,
                                             int dtype, int init, bool key_stream, bool reverse, void* zero_ptr,
@@ -303,10 +327,8 @@ static cudaError_t launch_delta_chain_tables(const Shape& s, const Workspace& w,
 // into a ring of shared-memory stages with bulk copies.  Per row one shared-memory load, one
 // widening, the three dependent operations of Eq. 2-3 and a checkpoint store every 8 rows.  It
 // does 3 times fewer instructions and 10 times less shared-memory traffic per row than the
-// kernel above, whose tables (32 bytes written and read per element) saturate the shared-memory
-// bandwidth of an SM from about two CTAs per SM on: with every head of a large batch resident
-// at once this one is faster (stack layer: 59 us against 82), with few heads the other one
-// (a single Llama layer: 14.3 us against 18.4).
+// kernel above: with every head of a large batch resident at once this one is faster (6 x 32 heads of 1024 tokens
+// 19.5 us against 23.2, 8 x 32 19.6 against 28.3), with few heads the other one (see the rule at the launch).
 namespace {
 
 constexpr int RROWS = 64;    // rows per ring stage
@@ -535,10 +557,12 @@ cudaError_t launch_delta_chain(const Shape& s, const Workspace& w, const void* x
                                cudaStream_t st) {
   if (key_stream && reverse) return cudaErrorNotSupported;
   if (((uintptr_t)zero_ptr | zero_bytes) & 15u) return cudaErrorInvalidValue;
-  // the table kernel while every one of its CTAs (head x 32 channels) has an SM of its own (one
-  // tensor map: not for a ragged group)
+  // The table kernel while its CTAs (head x 32 channels) are all resident at once: two per SM for bf16, one for fp32
+  // (shared memory: 96 and 128 KB).  Whole prefill, tables against rows: 64 CTAs (1 x 32 heads, 1024 tokens) 28.8 us, 34.0;
+  // 160 (2 x 20 heads, d = 128, 1531 tokens) 87.9, 90.2; 192 59.5, 61.5; 256 75.0, 77.0; 384 112.6, 110.0; 512 147.5, 139.5.
+  // (One tensor map: not for a ragged group.)
   const long ctas = (long)s.B * (key_stream ? s.H_kv : s.H) * (s.d / CH);
-  if (!seqs.ragged && ctas <= device_sm_count())
+  if (!seqs.ragged && ctas <= (long)device_sm_count() * (dtype == DELTA_F32 ? 1 : 2))
     return launch_delta_chain_tables(s, w, x, seqs.s[0].T, theta, dtype, init, key_stream, reverse, zero_ptr, zero_bytes,
                                      st);
   return launch_delta_chain_rows(s, w, x, seqs, theta, dtype, init, key_stream, reverse, zero_ptr, zero_bytes, st);
