@@ -143,11 +143,6 @@ __global__ void __launch_bounds__(CHAIN_THREADS) delta_chain_kernel(
   // share an SM their chain warps, the busiest, then sit on different schedulers.  The producer is the
   // other warp of the chain's scheduler.
   const int cw = (int)blockIdx.x & 3;
-  // the deferred clearing of a state reset (counters, tickets, second reference buffer): nothing
-  // of this launch or of the kernels behind it touches that span before this kernel is complete
-  if (zero_ptr && blockIdx.x == 0)
-    for (unsigned i = tid; i < zero_n16; i += blockDim.x) zero_ptr[i] = make_uint4(0u, 0u, 0u, 0u);
-
   if (tid < 2 * NS + 2 * NZ) {      // one barrier per thread
     const uint32_t cnt = (tid < NS) ? 1u : (tid < 2 * NS + NZ) ? (uint32_t)NSB : 1u;
     tc::mbar_init(full0 + 8 * tid, cnt);
@@ -158,10 +153,18 @@ __global__ void __launch_bounds__(CHAIN_THREADS) delta_chain_kernel(
   if (tid == 32 * (4 + cw))
     asm volatile("prefetch.tensormap [%0];" ::"l"(&tm_x) : "memory");
   __syncthreads();
-  // a kernel launched behind this one with programmatic stream serialisation may become
-  // resident and run its prologue now; it sees this kernel's results only after its own
-  // grid-dependency wait
+  // Launched with programmatic stream serialisation: set up while the kernel in front runs out, then wait for it (it
+  // may have written the stream, and may still use the workspace).  Behind the wait, never ahead of it: a
+  // kernel launched behind this one in the same way may become resident now, and takes this call's
+  // inputs (queries, keys, values) for complete from its start; this kernel's results it sees after its own wait.
+  // (Whole prefills behind one another, ordinary launch -> this: 1 x 32 heads 256 tokens 12.9 -> 11.5 us, 1024 28.2 ->
+  // 26.0; d = 128, 20 heads, 2048 63.6 -> 61.5; 4 x 32 x 1024 74.9 -> 73.1; 8 x 32 x 1024 139.4 -> 137.3.)
+  asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  // the deferred clearing of a state reset (counters, tickets, second reference buffer): nothing
+  // of this launch or of the kernels behind it touches that span before this kernel is complete
+  if (zero_ptr && blockIdx.x == 0)
+    for (unsigned i = tid; i < zero_n16; i += blockDim.x) zero_ptr[i] = make_uint4(0u, 0u, 0u, 0u);
 
   if (warp == 4 + cw) {
     // ---- producer: keeps up to NS stages of rows in flight
@@ -284,6 +287,27 @@ __global__ void __launch_bounds__(CHAIN_THREADS) delta_chain_kernel(
   if (tid == 0 && s_abort) atomicMax(&counters[CNT_STATUS], (unsigned long long)DELTA_ERR_TIMEOUT);
 }
 
+// A launch on stream st with programmatic stream serialisation (grid, block and shared memory to be filled in).
+static cudaLaunchConfig_t serialised_launch(cudaLaunchAttribute (&attr)[1], cudaStream_t st) {
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.stream = st;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cfg;
+}
+
+// Shared memory to ask for so that an SM takes no more of the launch's CTAs than an even spread gives it.  A kernel in front
+// that lets this one in while it still holds most SMs (a decode step) leaves it a few SMs only: without this the CTAs
+// pile up there (one layer of 8 x 32 heads, 4096 tokens, behind decode steps: +34 us), with it they wait for their place.
+static size_t even_spread_smem(size_t need, long ctas) {
+  const long sms = device_sm_count(), per = (ctas + sms - 1) / sms;
+  const size_t even = (size_t)228 * 1024 / (size_t)(per + 1);      // one CTA more would not fit
+  return need > even ? need : even;
+}
+constexpr int kMaxChainSmem = 144 * 1024;      // (fp32 tables 128 KB; the even spread asks for 114 KB at most)
+
 static cudaError_t launch_delta_chain_tables(const Shape& s, const Workspace& w, const void* q, int T, float theta,
                                             int dtype, int init, bool key_stream, bool reverse, void* zero_ptr,
                                             size_t zero_bytes, cudaStream_t st) {
@@ -298,18 +322,23 @@ static cudaError_t launch_delta_chain_tables(const Shape& s, const Workspace& w,
                    CU_TENSOR_MAP_SWIZZLE_NONE))
     return cudaErrorInvalidValue;
   cudaError_t err = cudaSuccess;
+  cudaLaunchAttribute attr[1];
+  cudaLaunchConfig_t cfg = serialised_launch(attr, st);
 #define LAUNCH(TIN, DD)                                                                          \
   do {                                                                                           \
     auto kern = delta_chain_kernel<TIN, DD>;                                                     \
-    const size_t smem = (size_t)NS * RC * CH * sizeof(TIN) + (size_t)NZ * Z_STAGE * sizeof(float4); \
+    constexpr size_t need = (size_t)NS * RC * CH * sizeof(TIN) + (size_t)NZ * Z_STAGE * sizeof(float4); \
+    static_assert(need <= kMaxChainSmem, "shared memory");                                       \
     static std::atomic<uint64_t> ready{0};                                                       \
     if (!device_done(ready)) {                                                                   \
-      if ((err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess) return err; \
+      if ((err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxChainSmem)) != cudaSuccess) return err; \
       device_mark(ready);                                                                        \
     }                                                                                            \
-    kern<<<heads * (DD / CH), CHAIN_THREADS, smem, st>>>(tm, w.qhat_tile, w.qhat[0], w.ckpt, w.counters, T, \
-                                                         s.n_tiles, s.n_ckpt(), theta, basis, reverse ? 1 : 0, \
-                                                         (uint4*)zero_ptr, (unsigned)(zero_bytes / 16)); \
+    cfg.gridDim = dim3((unsigned)(heads * (DD / CH)));                                           \
+    cfg.blockDim = dim3(CHAIN_THREADS);                                                          \
+    cfg.dynamicSmemBytes = even_spread_smem(need, (long)heads * (DD / CH));                      \
+    err = cudaLaunchKernelEx(&cfg, kern, tm, w.qhat_tile, w.qhat[0], w.ckpt, w.counters, T, s.n_tiles, s.n_ckpt(), theta, \
+                             basis, reverse ? 1 : 0, (uint4*)zero_ptr, (unsigned)(zero_bytes / 16)); \
   } while (0)
   if (f32) {
     if (s.d == 64) LAUNCH(float, 64); else LAUNCH(float, 128);
@@ -432,10 +461,6 @@ __global__ void __launch_bounds__(D + 32) delta_chain_rows_kernel(
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const uint32_t full0 = smem_u32(&bars[0]), empty0 = smem_u32(&bars[RSTAGES]);
   const int n_chunks = (T + RROWS - 1) / RROWS;
-  // the deferred clearing of a state reset (see the table kernel)
-  if (zero_ptr && blockIdx.x == 0 && blockIdx.y == 0)
-    for (unsigned i = tid; i < zero_n16; i += blockDim.x) zero_ptr[i] = make_uint4(0u, 0u, 0u, 0u);
-
   if (tid == 0) {
     for (int s = 0; s < RSTAGES; ++s) {
       asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(full0 + 8 * s), "r"(1) : "memory");
@@ -445,10 +470,12 @@ __global__ void __launch_bounds__(D + 32) delta_chain_rows_kernel(
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   __syncthreads();
-  // a kernel launched behind this one with programmatic stream serialisation may become
-  // resident and run its prologue now; it sees this kernel's results only after its own
-  // grid-dependency wait
+  // (the order of these two: see the table kernel)
+  asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  // the deferred clearing of a state reset (see the table kernel)
+  if (zero_ptr && blockIdx.x == 0 && blockIdx.y == 0)
+    for (unsigned i = tid; i < zero_n16; i += blockDim.x) zero_ptr[i] = make_uint4(0u, 0u, 0u, 0u);
 
   if (warp == NW) {
     // ---- producer: keeps up to RSTAGES stages of query rows in flight
@@ -507,10 +534,11 @@ template <typename TIn, int D, int N>
 static cudaError_t launch_rows(const Shape& s, const Workspace& w, const void* x, const SeqBatch& seqs, float theta, int init,
                                bool key_stream, bool reverse, void* zero_ptr, size_t zero_bytes, cudaStream_t st) {
   auto kern = delta_chain_rows_kernel<TIn, D, N>;
-  constexpr size_t smem = (size_t)RSTAGES * RROWS * D * sizeof(TIn);
+  constexpr size_t need = (size_t)RSTAGES * RROWS * D * sizeof(TIn);
+  static_assert(need <= kMaxChainSmem, "shared memory");
   static std::atomic<uint64_t> ready{0};
-  if (smem > 48 * 1024 && !device_done(ready)) {
-    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (!device_done(ready)) {
+    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxChainSmem);
     if (e != cudaSuccess) return e;
     device_mark(ready);
   }
@@ -518,11 +546,17 @@ static cudaError_t launch_rows(const Shape& s, const Workspace& w, const void* x
   for (int i = 0; i < N; ++i) list.s[i] = seqs.s[i < seqs.n ? i : 0];
   const int heads = key_stream ? s.H_kv : s.H;
   const dim3 grid((unsigned)(seqs.ragged ? heads : s.B * heads), (unsigned)seqs.n);
-  kern<<<grid, D + 32, smem, st>>>((const TIn*)x, list, w.qhat_tile, w.qhat[0], w.ckpt, w.counters, s.n_tiles, s.n_ckpt(),
-                                   theta, init == DELTA_INIT_BASIS_EXACT ? 1 : 0, heads, key_stream ? s.T_max : 0,
-                                   reverse ? 1 : 0, (uint4*)zero_ptr, (unsigned)(zero_bytes / 16));
+  cudaLaunchAttribute attr[1];
+  cudaLaunchConfig_t cfg = serialised_launch(attr, st);
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(D + 32);
+  cfg.dynamicSmemBytes = even_spread_smem(need, (long)grid.x * grid.y);
+  const cudaError_t err =
+      cudaLaunchKernelEx(&cfg, kern, (const TIn*)x, list, w.qhat_tile, w.qhat[0], w.ckpt, w.counters, s.n_tiles, s.n_ckpt(),
+                         theta, init == DELTA_INIT_BASIS_EXACT ? 1 : 0, heads, key_stream ? s.T_max : 0, reverse ? 1 : 0,
+                         (uint4*)zero_ptr, (unsigned)(zero_bytes / 16));
   count_launch();
-  return cudaGetLastError();
+  return err != cudaSuccess ? err : cudaGetLastError();
 }
 
 static cudaError_t launch_delta_chain_rows(const Shape& s, const Workspace& w, const void* x, const SeqBatch& seqs,
@@ -684,10 +718,14 @@ __global__ void __launch_bounds__(256, D == 64 ? 5 : 4) delta_finish_kernel(
   // CTA of the attention kernel is resident by then, so nothing can be kept from starting.  It costs up to
   // 1.1 us where the attention kernel ends last -- three ragged sequences of up to 392 tokens, d = 128:
   // 22.9 -> 24.1 us; BitNet layer 63.8 -> 64.2 -- and nothing at the Llama layer.)
-  if (wait_front) asm volatile("griddepcontrol.wait;" ::: "memory");
-  // key deltas: the attention kernel is serialised programmatically behind this one and may set
-  // itself up meanwhile (it waits for this kernel's results itself)
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  if (wait_front) {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    // key deltas: the attention kernel is serialised programmatically behind this one and may set
+    // itself up meanwhile (it waits for this kernel's results itself).  Not where this kernel comes last: the next prefill's chain
+    // CTAs would become resident beside the attention kernel's last wave, several on each of the few SMs it leaves
+    // (1 x 32 heads, 1024 tokens 30.3 us, so 26.0; d = 128, 2048 tokens 70.0, so 61.5).
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  }
   if ((int)blockIdx.x < n_idx_blocks) {
     // ---- one block per (batch, head, 64-row tile); warp w serves rows 8w .. 8w+7
     __shared__ uint32_t s_red[3][8];

@@ -388,7 +388,9 @@ hybrid_attn_tcq_kernel(const __grid_constant__ TqMapList<N> maps, const __grid_c
       // key deltas: the ring streams reference-key rows, which the finish kernel in front of
       // this one writes (programmatic stream serialisation): wait for them.  Queries, keys and
       // values themselves are inputs.
-      if (KEY) asm volatile("griddepcontrol.wait;" ::: "memory");
+      if (KEY) {
+        asm volatile("griddepcontrol.wait;" ::: "memory");
+      }
       const CUtensorMap* tm_ring = KEY ? &tm_qh : &tm_k;
       int n_kx = 0;
       for (int t = 0; t < n; ++t) {
