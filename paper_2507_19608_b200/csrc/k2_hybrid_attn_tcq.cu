@@ -1079,15 +1079,18 @@ cudaError_t launch_hybrid_attn_tcq(const Shape& s, const Workspace& w, const voi
   if (!w.qhat_rows) return cudaErrorNotSupported;
   const bool two_heads_ok = s.d == 64 && (s.g() % 2) == 0;
   if ((form == 2 || form == 3) && !two_heads_ok) return cudaErrorNotSupported;
-  // Two heads of a KV group per CTA share every key and value tile and need no merge, but a
-  // head's key tiles are then walked by one softmax group instead of two.  That pays once
-  // there are at least two such CTAs per SM (stack layer: 0.925 of the one-head form's time).
-  // On a smaller grid that the one-head form cannot place in one wave, the heaviest query
-  // tiles of every head go one head per CTA and the rest two heads per CTA, as many of the
-  // former as one wave of SMs allows.  The forms round differently: a sequence of a ragged group takes the
-  // form of a batch of its own, so that its result does not depend on the sequences beside it.  (Two heads per
-  // CTA throughout, by the size of the group, is faster: six sequences of 99 to 1900 tokens, 32 heads, with 24
-  // steps behind them 292 us, so 305.)
+  // Two heads of a KV group per CTA share every key and value tile, need no merge and halve the CTAs (a CTA's
+  // set-up, reference-query tile, first scores and last product cost about as much as seven key tiles), but a
+  // head's key tiles are then walked by one softmax group instead of two.  So, whole prefills in us (d = 64):
+  //  - more such CTAs than one wave of SMs: two heads throughout (1 x 32 heads: 1280 tokens 32.1, one head
+  //    throughout 36.9; 2048 54.1, 63.1; 4096 144, 162; 2 x 32 x 1024 39.1, 48.2; 16 heads x 4096 85.3, 94.0);
+  //  - all one head where those and the chain kernel's CTAs, which hold SMs until the chain ends, are one wave
+  //    (16 heads x 1024 20.4, half of the query tiles two heads 21.0);
+  //  - else the heaviest query tiles of every head one head per CTA, as many as make the longest CTAs of both
+  //    kinds alike (half) and fit one wave (32 heads: 512 tokens 15.7, all one head 17.4; 640 18.5, four of five
+  //    20.0; 1024 25.9, none 26.8; 64 heads x 256 14.1, all one head 16.1).
+  // The forms round differently: a sequence of a ragged group takes the
+  // form of a batch of its own, so that its result does not depend on the sequences beside it.
   const long BH = seqs.form_heads(s), sms = device_sm_count();
   int n_one[kSeqMax];                     // query tiles of every head in the one-head form
   bool all_one = true, all_two = true;
@@ -1097,8 +1100,12 @@ cudaError_t launch_hybrid_attn_tcq(const Shape& s, const Workspace& w, const voi
     if (form == 2) n1 = 0;
     else if (form == 3) n1 = 1;
     else if (form == 0 && two_heads_ok) {
-      if (BH / 2 * nqt >= 2 * sms) n1 = 0;
-      else if (BH * nqt > sms && BH / 2 * nqt <= sms) n1 = (sms - BH / 2 * nqt) / (BH / 2);
+      const long pairs = BH / 2 * nqt;
+      if (pairs > sms) n1 = 0;
+      else if (BH * (nqt + 1) > sms) {
+        const long fit = (sms - pairs) / (BH / 2);
+        n1 = nqt / 2 < fit ? nqt / 2 : fit;
+      }
     }
     n_one[i] = (int)n1;
     all_one = all_one && n1 >= nqt;
