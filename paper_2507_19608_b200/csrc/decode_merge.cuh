@@ -226,14 +226,16 @@ __device__ __forceinline__ void merge_slices(uint32_t recs, int rank, int cs, si
   const float inv = 1.0f / l;
   store4(out + out0 + (size_t)(q / (D / 16)) * D + (q % (D / 16)) * 16 + 4 * c4, a.x * inv, a.y * inv, a.z * inv, a.w * inv);
 }
-// Slices of a step over sequences of up to L keys (the new one included).  A step takes 4 to 5 us plus,
-// for every unit a warp works through, 1.1 us (d = 64) or 1.3 us (d = 128) while a CTA has its SM for
-// itself and 1.75 us where two share one (measured from 1 to 192 KV heads, 300 to 16000 keys); the
-// slices are those that minimise that.  All slices of a KV head form one cluster, and clusters have to
-// find room in a GPC: from 1.75 CTAs per SM on (1.6 for clusters of 9 to 12, 1.35 for 13 to 16) some
-// wait for a second wave (batch 16, 2048 keys: 256 CTAs 12 us, 384 CTAs 17 us).  Very long caches of
+// Slices of a step over sequences of up to L keys (the new one included).  A step takes 3 us plus, for every
+// unit a warp works through, 0.83 us (d = 64) or 0.87 us (d = 128) while a CTA has its SM for itself, 1.15 times that
+// from half the SMs on, and 1.25 or 1.35 us where two share one (measured with 1 to 16 slices forced, 8 to 128 KV
+// heads, 300 to 4100 keys); the slices are those that minimise that.  All slices of a KV head form one cluster,
+// and clusters have to find room in a GPC: from 1.75 CTAs per SM on (1.6 for clusters of 9 to 12, 1.35 for 13 to
+// 16) some wait for a second wave (batch 16, 2048 keys: 256 CTAs 12 us, 384 CTAs 17 us).  Very long caches of
 // few heads: up to 64 slices merged through global memory (4.5 us more than a cluster).  The compressed
-// key cache: 2.5 us more per unit, for the rebuilding.
+// key cache: 1.6 us more per unit, for the rebuilding.
+// With these figures instead of those of a slower unit (1.1, 1.3, 1.75), us per step at 2048 keys, 8 KV heads: batch 2
+// 5.1 -> 4.7 (6 -> 9 slices), batch 4 6.0 -> 5.7 (4 -> 6); batch 8 at 1024 keys 5.6 -> 5.4 (2 -> 4).
 // nw: warps per CTA; us_alone, us_shared: a unit's time with the SM for itself, and shared (0: a CTA fills
 // its SM); us_more: a kernel's own extra time per unit.
 inline void decode_slices(const Shape& s, int L, int nw, float us_shared, float us_alone, float us_more, int* nsplit_out,
@@ -244,15 +246,16 @@ inline void decode_slices(const Shape& s, int L, int nw, float us_shared, float 
   int best_ns = 1;
   for (int ns = 1; ns <= kMaxDecodeSplits && (ns - 1) * nw < units; ++ns) {       // a unit per warp at least
     const long ctas = (long)bkv * ns;
-    const bool alone = ctas * 100 <= (long)sms * 92;
+    const bool alone = ctas * 100 <= (long)sms * (us_shared == 0.0f ? 92 : 98);
     if (ns > kMaxCluster && ctas > sms) break;
     if (ns > 1 && us_shared == 0.0f && !alone) continue;
     if (ns > 1 && ns <= kMaxCluster && ctas * 100 > (long)sms * (ns <= 8 ? 175 : ns <= 12 ? 160 : 135)) continue;
     const int per = (units + ns - 1) / ns;                       // units per slice; per warp mostly the longest counts
     const float rounds = 0.8f * (float)((per + nw - 1) / nw) + 0.2f * (float)per / (float)nw;
-    const float us = rounds * ((alone || us_shared == 0.0f ? us_alone : us_shared) + us_more) +
+    const float unit = us_shared == 0.0f ? us_alone : !alone ? us_shared : ctas * 2 <= sms ? us_alone : 1.15f * us_alone;
+    const float us = rounds * (unit + us_more) +
                      (ns > kMaxCluster ? 4.5f + 0.15f * (float)(ns - 24) : (ns > 8 ? 0.075f : 0.06f) * (float)ns);
-    if (us < best - 0.02f) { best = us; best_ns = ns; }
+    if (us < best) { best = us; best_ns = ns; }
   }
   const int chunk = (units + best_ns - 1) / best_ns * UK;
   *nsplit_out = (L + chunk - 1) / chunk;

@@ -819,7 +819,8 @@ cudaError_t launch_decode_step_mma(const Shape& s, const Workspace& w, const voi
   p.b0 = 0;
   const int G = s.g();
   bool cluster;
-  decode_slices(s, n + 1, s.d == 64 ? kWarps<64> : kWarps<128>, 1.75f, s.d == 64 ? 1.1f : 1.3f, packed ? 2.5f : 0.0f, &p.nsplit, &p.chunk, &cluster);
+  decode_slices(s, n + 1, s.d == 64 ? kWarps<64> : kWarps<128>, s.d == 64 ? 1.25f : 1.35f, s.d == 64 ? 0.83f : 0.87f,
+                packed ? 1.6f : 0.0f, &p.nsplit, &p.chunk, &cluster);
   if (p.nsplit > kMaxDecodeSplits) return cudaErrorInvalidValue;
   cudaError_t err = cudaSuccess;
   for (; p.b0 < s.B && err == cudaSuccess; p.b0 += kRaggedMax) {
