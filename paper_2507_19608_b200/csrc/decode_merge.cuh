@@ -3,9 +3,7 @@
 //
 // Merge.  The result of a (batch, KV head), G heads x D channels, is cut into blocks of 16 channels of one
 // head.  The slices of the (batch, KV head) are one thread-block cluster of cs CTAs; block q is finished by
-// slice q mod cs (by the CTA itself without a cluster), to whose shared memory every warp of every
-// slice sends its part: a record of 16 channels at recs + ((q / cs) * nsrc + source) * REC * 4 and a
-// (maximum, row sum) pair at mls + (..) * 8.
+// slice q mod cs (by the CTA itself without a cluster), to whose shared memory every slice sends one record.
 #pragma once
 #include "decode_common.cuh"
 #include "tc_common.cuh"
@@ -16,7 +14,6 @@ namespace {
 constexpr int UK = 32;                    // keys a warp works on at a time
 constexpr int kMaxCluster = 16;           // slices merged through distributed shared memory
 constexpr int kRaggedMax = 64;            // batch elements of one ragged launch
-constexpr int REC = 16;                   // floats of a partial result's record: 16 channels of one head
 
 __device__ __forceinline__ void async16(uint32_t dst, const void* src) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
@@ -96,56 +93,6 @@ __device__ __forceinline__ void merge_global(int ns, int bkv, size_t out0, float
     out[out0 + (size_t)hh * D + c] = from_f32<TO>(nu / de);
   }
   if (tid == 0) ticket[bkv] = 0;                          // ready for the next step
-}
-
-// The finishing half, once all records are there: combine this CTA's blocks and store them, or, where
-// a (batch, KV head) has more slices (ns) than a cluster, leave this slice's part in global memory
-// for the last CTA to arrive.  out0: first output of the group.
-template <typename TO, int D, int G, int MNW, bool CLUSTER>
-__device__ __forceinline__ void decode_merge(uint32_t recs, uint32_t mls, int rank, int cs, int nsrc, int ns, int split,
-                                             int bkv, size_t out0, float* __restrict__ partial,
-                                             uint32_t* __restrict__ ticket, TO* __restrict__ out, int* s_last) {
-  // One warp per block: lane = (4 channels, one of 8 groups of parts).
-  constexpr int NB = G * D / 16;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int c4 = lane & 3, sg = lane >> 2;
-  for (int slot = warp; slot * cs + rank < NB; slot += MNW) {
-    const int q = slot * cs + rank;
-    const uint32_t rb = recs + (uint32_t)(slot * nsrc) * (REC * 4) + 16 * c4, mb = mls + (uint32_t)(slot * nsrc) * 8;
-    float M = -INFINITY;
-#pragma unroll
-    for (int x = 0; x < (CLUSTER ? kMaxCluster : 1) * MNW; x += 32)
-      if (x + lane < nsrc) M = fmaxf(M, lds_f2(mb + 8 * (x + lane)).x);
-    M = warp_max(M);
-    float a[5] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
-#pragma unroll 4
-    for (int x = sg; x < nsrc; x += 8) {
-      const float2 ml = lds_f2(mb + 8 * x);
-      const float4 o = lds_f4(rb + x * (REC * 4));
-      const float f = tc::ex2(ml.x - M);                     // 0 for a warp without keys
-      a[0] = fmaf(f, o.x, a[0]); a[1] = fmaf(f, o.y, a[1]); a[2] = fmaf(f, o.z, a[2]); a[3] = fmaf(f, o.w, a[3]);
-      a[4] = fmaf(f, ml.y, a[4]);
-    }
-#pragma unroll
-    for (int x = 4; x < 32; x <<= 1)
-#pragma unroll
-      for (int e = 0; e < 5; ++e) a[e] += __shfl_xor_sync(0xffffffffu, a[e], x);
-    const int hh = q / (D / 16), ch = (q % (D / 16)) * 16 + 4 * c4;
-    if (sg == 0) {
-      if (CLUSTER || ns == 1) {
-        const float inv = 1.0f / a[4];
-        store4(out + out0 + (size_t)hh * D + ch, a[0] * inv, a[1] * inv, a[2] * inv, a[3] * inv);
-      } else {
-        // slices through global memory: this slice's part
-        float* const pg = partial + (((size_t)bkv * kMaxDecodeSplits + split) * G + hh) * (D + 2);
-        pg[ch] = a[0]; pg[ch + 1] = a[1]; pg[ch + 2] = a[2]; pg[ch + 3] = a[3];
-        if (ch == 0) { pg[D] = M; pg[D + 1] = a[4]; }
-      }
-    }
-  }
-  if (CLUSTER || ns == 1) return;
-
-  merge_global<TO, D, G, MNW>(ns, bkv, out0, partial, ticket, out, s_last);
 }
 
 // The merge in two steps, for kernels whose warps leave their results as fp32 rows in the CTA's shared memory:

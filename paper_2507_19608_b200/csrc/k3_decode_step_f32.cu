@@ -10,8 +10,11 @@
 //           different swizzled chunks) against references and queries broadcast from shared memory,
 //           packed fma.rn.f32x2; queries only where the unit touches the window;
 //   P.V     lane = D / 32 channels, probabilities broadcast.
-// Bound: dependent latencies at the sizes fp32 is used at (16 heads over 1000 keys move 2 MB): 10.3 us per
-// step with block barriers around every tile and a merge through global memory, 5.0 so.
+// Bound: dependent latencies at the sizes fp32 is used at (16 heads over 1000 keys move 2 MB).  The unit of the row
+// that arrives with the step comes by TMA like the others (row by row it kept its warp, the step's last, 0.4 us
+// longer) and a CTA combines its warps before one record per block of 16 channels travels (decode_merge.cuh).
+// us per step, with block barriers around every tile and a merge through global memory -> warps on their own, every
+// warp sending -> so: 16 heads at 1000 keys 10.3 -> 5.0 -> 4.4; 2 x 16 at 2000 5.4 -> 4.8; d = 128 6.8 -> 6.0.
 #include "decode_common.cuh"
 #include "decode_merge.cuh"
 
@@ -35,8 +38,11 @@ template <int D, int G> struct F32DecSmem {
   static constexpr uint32_t HALF = UK * D * 4, RING = NW * 2 * HALF;
   static constexpr int NB = G * D / 16;
   static constexpr uint32_t PROBS = NW * UK * G * 4, ROWS = 2 * G * D * 4;      // probabilities; references, queries
-  __host__ __device__ static constexpr uint32_t nrec(int cs) { return (uint32_t)((NB + cs - 1) / cs * cs) * NW; }
-  static constexpr size_t bytes(int cs) { return 1024 + RING + nrec(cs) * (REC + 2) * 4 + PROBS + ROWS; }
+  static_assert(MergePart<D, G>::BYTES <= HALF, "a warp's result fits its key slot");
+  // records of a CTA of a cluster of cs
+  __host__ __device__ static constexpr uint32_t rec_bytes(int cs) { return merge_slots<D, G>(cs) * cs * REC2 * 4; }
+  static constexpr size_t bytes(int cs) { return 1024 + RING + rec_bytes(cs) + PROBS + ROWS; }
+  static constexpr size_t bytes_max = 1024 + RING + (NB + kMaxCluster - 1) * REC2 * 4 + PROBS + ROWS;
 };
 }  // namespace
 
@@ -53,8 +59,8 @@ decode_step_f32_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_co
   const uint32_t ring = (smem_u32(dsm_raw) + 1023u) & ~1023u;
   unsigned char* const sm = dsm_raw + (ring - smem_u32(dsm_raw));
   const int cs = CLUSTER ? p.nsplit : 1;
-  const uint32_t recs = ring + SM::RING, mls = recs + SM::nrec(cs) * REC * 4;
-  float* const s_p = reinterpret_cast<float*>(sm + SM::RING + SM::nrec(cs) * (REC + 2) * 4);     // [NW][UK][G]
+  const uint32_t recs = ring + SM::RING;
+  float* const s_p = reinterpret_cast<float*>(sm + SM::RING + SM::rec_bytes(cs));     // [NW][UK][G]
   float* const s_ref = s_p + SM::PROBS / 4;  // [G][D]
   float* const s_q = s_ref + G * D;          // [G][D]
 
@@ -63,19 +69,21 @@ decode_step_f32_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_co
   const int b = bkv / H_kv, kvh = bkv - b * H_kv;
   const int n = p.ragged ? p.n_b[b - p.b0] : p.n, T_max = p.T_max, W = p.W;
   const int L = n + 1, j0 = split * p.chunk, j1 = min(j0 + p.chunk, L);
-  const int rank = CLUSTER ? split : 0, nsrc = cs * NW;
+  const int rank = CLUSTER ? split : 0;
   const uint32_t bar_m = smem_u32(&bars[2 * NW]), bar_k = smem_u32(&bars[2 * warp]), bar_v = bar_k + 8;
   if (CLUSTER) {
     if (tid == 0) {
       tc::mbar_init(bar_m, 1);
       asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-      tc::mbar_expect_tx(bar_m, (uint32_t)((SM::NB - rank + cs - 1) / cs * nsrc) * (REC + 2) * 4);
+      tc::mbar_expect_tx(bar_m, (uint32_t)((SM::NB - rank + cs - 1) / cs * cs) * (16 + 2) * 4);
     }
     __syncwarp();
     asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
   }
   if (!CLUSTER && j0 >= L) return;           // ragged batch: this sequence has fewer slices
+  const uint32_t lead = lane == 0;
   if (lane == 0) {
+    if (warp == 0) asm volatile("prefetch.tensormap [%0];" ::"l"(&tm_k) : "memory");
     tc::mbar_init(bar_k, 1);
     tc::mbar_init(bar_v, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -91,37 +99,29 @@ decode_step_f32_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_co
   unsigned char* const my = sm + (size_t)warp * 2 * SM::HALF;
   const uint32_t slot_k = ring + (uint32_t)warp * 2 * SM::HALF, slot_v = slot_k + SM::HALF;
   // row r, 16-byte chunk c of a 128-byte block: r * 128 + ((c ^ (r & 7)) << 4); values: plain rows
+  // (the unit of the row that arrives with the step too: rows behind the cached ones hold anything, that row and
+  // zeros are written over them; the values end with the cache)
   auto fetch = [&](int jg) {
-    if (lane == 0) {
-      const int rows = min(UK, n - jg);      // cached rows of the unit
-      if (rows == UK) {
-        tc::mbar_expect_tx(bar_k, SM::HALF);
+    tc::mbar_expect_tx_if(lead, bar_k, SM::HALF);
 #pragma unroll
-        for (int c = 0; c < NBLK; ++c) tc::tma_load_3d(slot_k + c * UK * 128, &tm_k, bar_k, 32 * c, jg, bkv);
-        tc::mbar_expect_tx(bar_v, SM::HALF);
-        bulk_load(slot_v, p.v_cache + (row0 + jg) * D, SM::HALF, bar_v);
-      }
-    }
-    if (jg + UK > n) {
-      // the unit of the row that arrives with the step: row by row, zeros behind it
-#pragma unroll 4
-      for (int e = lane; e < UK * D / 4; e += 32) {
-        const int r = e / (D / 4), c = e % (D / 4), j = jg + r;
-        const uint32_t dk = slot_k + (c >> 3) * (UK * 128) + r * 128 + (((c & 7) ^ (r & 7)) << 4), dv = slot_v + r * D * 4 + c * 16;
-        if (j <= n) {
-          async16(dk, (j < n ? p.k_cache + (row0 + j) * D : kn) + 4 * c);
-          async16(dv, (j < n ? p.v_cache + (row0 + j) * D : vn) + 4 * c);
-        } else {
-          sts_f4(dk, 0.0f, 0.0f, 0.0f, 0.0f);
-          sts_f4(dv, 0.0f, 0.0f, 0.0f, 0.0f);
-        }
-      }
+    for (int c = 0; c < NBLK; ++c) tc::tma_load_3d_if(lead, slot_k + c * UK * 128, &tm_k, bar_k, 32 * c, jg, bkv);
+    const uint32_t vbytes = (uint32_t)min(UK, T_max - jg) * D * 4;
+    if (lane == 0) {
+      tc::mbar_expect_tx(bar_v, vbytes);
+      bulk_load(slot_v, p.v_cache + (row0 + jg) * D, vbytes, bar_v);
     }
   };
+  // the warp that owns the row arriving with the step
+  const bool has_new = j1 == L && j0 < L && ((n - j0) / UK) % NW == warp;
   asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   int jg = j0 + UK * warp;
   if (jg < j1) fetch(jg);
+  float4 k_row = make_float4(0.0f, 0.0f, 0.0f, 0.0f), v_row = k_row;       // that row: four channels per lane
+  if (has_new && lane < D / 4) {
+    k_row = __ldcg(reinterpret_cast<const float4*>(kn) + lane);
+    v_row = __ldcg(reinterpret_cast<const float4*>(vn) + lane);
+  }
 
   // ---- threshold step (Eq. 2-3) into shared memory
   int fired = 0;
@@ -136,20 +136,6 @@ decode_step_f32_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_co
     if (split == 0) p.ref_out[o0 + e] = nq;
   }
   __syncthreads();
-  if (split == 0) {
-    const int f = warp_sum(fired);
-    if (lane == 0) {
-      const int n_in = min(L, max(W, 0));
-      if (f) atomicAdd(&p.counters[CNT_DECODE_NNZ], (unsigned long long)f);
-      if (f) atomicAdd(&p.counters[CNT_DECODE_MACS_DONE], (unsigned long long)(L - n_in) * f);
-      if (warp == 0) {
-        atomicAdd(&p.counters[CNT_DECODE_MACS_DONE], (unsigned long long)n_in * D * G);
-        atomicAdd(&p.counters[CNT_DECODE_ELEMS], (unsigned long long)G * D);
-        atomicAdd(&p.counters[CNT_DECODE_MACS_DENSE], (unsigned long long)L * D * G);
-      }
-    }
-  }
-
   float o[G][CPL], m[G], l[G];
 #pragma unroll
   for (int h = 0; h < G; ++h) {
@@ -159,7 +145,6 @@ decode_step_f32_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_co
     for (int c = 0; c < CPL; ++c) o[h][c] = 0.0f;
   }
   uint32_t ph = 0;
-  bool owns_new = false;                     // the warp owns the row that arrives with the step
   float* const pw = s_p + (size_t)warp * UK * G;
   // the lane's key against G rows of operands
   auto dots = [&](const float* rows, float (&s)[G]) {
@@ -184,10 +169,11 @@ decode_step_f32_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_co
   for (; jg < j1; jg += UK * NW) {
     const int jn = jg + UK * NW, j = jg + lane;
     const bool owner = n < jg + UK, live = j <= n;
-    if (!owner) {
-      if (!mbar_wait(bar_k, ph)) s_fail = 1;
-    } else {
-      async_wait_all();
+    if (!mbar_wait(bar_k, ph)) s_fail = 1;
+    if (owner) {                             // the new key's row (what the rows behind it hold is masked)
+      const int r = n - jg;
+      if (lane < D / 4)
+        sts_f4(slot_k + (lane >> 3) * (UK * 128) + r * 128 + (((lane & 7) ^ (r & 7)) << 4), k_row.x, k_row.y, k_row.z, k_row.w);
       __syncwarp();
     }
     float s[G];
@@ -213,7 +199,13 @@ decode_step_f32_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_co
       for (int c = 0; c < CPL; ++c) o[h][c] *= al;
       pw[lane * G + h] = pr;
     }
-    if (!owner && !mbar_wait(bar_v, ph)) s_fail = 1;
+    if (!mbar_wait(bar_v, ph)) s_fail = 1;
+    if (owner) {                             // the new value's row, zeros behind it
+      const int r = n - jg;
+      if (lane < D / 4) sts_f4(slot_v + r * D * 4 + 16 * lane, v_row.x, v_row.y, v_row.z, v_row.w);
+#pragma unroll 1
+      for (int e = (r + 1) * (D / 4) + lane; e < UK * (D / 4); e += 32) sts_f4(slot_v + 16 * e, 0.0f, 0.0f, 0.0f, 0.0f);
+    }
     __syncwarp();
     const float* const vt = reinterpret_cast<const float*>(my + SM::HALF) + CPL * lane;
 #pragma unroll 8
@@ -246,44 +238,48 @@ decode_step_f32_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_co
     __syncwarp();                            // the warp is done with the unit
     ph ^= 1u;
     if (jn < j1) fetch(jn);
-    owns_new = owner;
   }
 
-  // ---- merge: every warp sends its part to where it is finished
-#pragma unroll
-  for (int h = 0; h < G; ++h)
-#pragma unroll
-    for (int x = 16; x > 0; x >>= 1) l[h] += __shfl_xor_sync(0xffffffffu, l[h], x);
-  if (CLUSTER) asm volatile("barrier.cluster.wait.aligned;" ::: "memory");          // every slice runs
-  constexpr int LPB = 16 / CPL;              // lanes per block of 16 channels
+  // ---- merge: the warp's part into its key slot (every copy into it is complete and read)
+  using MP = MergePart<D, G>;
 #pragma unroll
   for (int h = 0; h < G; ++h) {
-    const int q = h * (D / 16) + lane / LPB, r = q % cs, rec = (q / cs) * nsrc + rank * NW + warp;
-    uint32_t dst = recs + (uint32_t)rec * (REC * 4) + (lane % LPB) * (CPL * 4), dml = mls + (uint32_t)rec * 8, rbar = bar_m;
-    if (CLUSTER) { dst = cluster_map(dst, r); dml = cluster_map(dml, r); rbar = cluster_map(bar_m, r); }
-    if constexpr (CPL == 2) {
-      if (CLUSTER) cluster_send2(dst, rbar, o[h][0], o[h][1]); else sts_f2(dst, o[h][0], o[h][1]);
-    } else {
-      if (CLUSTER) cluster_send4(dst, rbar, o[h][0], o[h][1], o[h][2], o[h][3]);
-      else sts_f4(dst, o[h][0], o[h][1], o[h][2], o[h][3]);
-    }
-    if (lane % LPB == 0) {
-      if (CLUSTER) cluster_send2(dml, rbar, m[h], l[h]); else sts_f2(dml, m[h], l[h]);
-    }
+#pragma unroll
+    for (int x = 16; x > 0; x >>= 1) l[h] += __shfl_xor_sync(0xffffffffu, l[h], x);
+    const uint32_t at = slot_k + (h * MP::LD + CPL * lane) * 4;
+    if constexpr (CPL == 2) sts_f2(at, o[h][0], o[h][1]); else sts_f4(at, o[h][0], o[h][1], o[h][2], o[h][3]);
+    if (lane == 0) sts_f2(slot_k + MP::ML + h * 8, m[h], l[h]);
   }
-  if (owns_new && lane < D / 4 && DELTA_IN(n, T_max, p.counters)) {
-    // the row that arrives with the step joins the caches while the parts travel
-    reinterpret_cast<float4*>(p.k_cache + (row0 + n) * D)[lane] = __ldcg(reinterpret_cast<const float4*>(kn) + lane);
-    reinterpret_cast<float4*>(p.v_cache + (row0 + n) * D)[lane] = __ldcg(reinterpret_cast<const float4*>(vn) + lane);
+  __syncthreads();
+  if (CLUSTER) asm volatile("barrier.cluster.wait.aligned;" ::: "memory");          // every slice runs
+  const int n_slices = (L + p.chunk - 1) / p.chunk;
+  merge_warps<float, D, G, NW, CLUSTER>(ring, 2 * SM::HALF, recs, bar_m, rank, cs, n_slices, split, bkv, o0, p.partial, p.out);
+  // ---- while the parts travel: the caches' new row, the counters
+  if (has_new && lane < D / 4 && DELTA_IN(n, T_max, p.counters)) {
+    reinterpret_cast<float4*>(p.k_cache + (row0 + n) * D)[lane] = k_row;
+    reinterpret_cast<float4*>(p.v_cache + (row0 + n) * D)[lane] = v_row;
+  }
+  if (split == 0) {
+    const int f = warp_sum(fired);
+    if (lane == 0) {
+      const int n_in = min(L, max(W, 0));
+      if (f) atomicAdd(&p.counters[CNT_DECODE_NNZ], (unsigned long long)f);
+      if (f) atomicAdd(&p.counters[CNT_DECODE_MACS_DONE], (unsigned long long)(L - n_in) * f);
+      if (warp == 0) {
+        atomicAdd(&p.counters[CNT_DECODE_MACS_DONE], (unsigned long long)n_in * D * G);
+        atomicAdd(&p.counters[CNT_DECODE_ELEMS], (unsigned long long)G * D);
+        atomicAdd(&p.counters[CNT_DECODE_MACS_DENSE], (unsigned long long)L * D * G);
+      }
+    }
   }
   if (CLUSTER) {
+    // (every slice's block records: also what keeps this CTA until the last of them has been sent to it)
     if (!mbar_wait(bar_m, 0)) s_fail = 1;
-  } else {
-    __syncthreads();
+    merge_slices<float, D, G>(recs, rank, cs, o0, p.out);
+  } else if (n_slices > 1) {
+    merge_global<float, D, G, NW>(n_slices, bkv, o0, p.partial, p.ticket, p.out, &s_last);
   }
-  if (tid == 0 && s_fail) atomicMax(&p.counters[CNT_STATUS], (unsigned long long)DELTA_ERR_TIMEOUT);
-  decode_merge<float, D, G, NW, CLUSTER>(recs, mls, rank, cs, nsrc, (L + p.chunk - 1) / p.chunk, split, bkv, o0, p.partial,
-                                         p.ticket, p.out, &s_last);
+  if (s_fail && lane == 0) atomicMax(&p.counters[CNT_STATUS], (unsigned long long)DELTA_ERR_TIMEOUT);
 }
 
 template <int D, int G, bool CLUSTER>
@@ -292,8 +288,7 @@ static cudaError_t launch_f32_step(const CUtensorMap& tk, const F32DecodeParams&
   auto kern = decode_step_f32_kernel<D, G, CLUSTER>;
   static std::atomic<uint64_t> ready{0};
   if (!device_done(ready)) {
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(SM::bytes(kMaxCluster) > SM::bytes(kMaxCluster - 1) ? SM::bytes(kMaxCluster)
-                                                                                               : SM::bytes(kMaxCluster - 1)));
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SM::bytes_max);
     if (e == cudaSuccess && CLUSTER) e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     if (e != cudaSuccess) return e;
     device_mark(ready);

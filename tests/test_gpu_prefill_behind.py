@@ -33,7 +33,8 @@ def _setup(case):
 
 @pytest.mark.parametrize("case", CASES, ids=lambda c: "-".join(map(str, c)))
 @pytest.mark.parametrize("captured", [False, True])
-def test_prefill_behind_writes_of_its_inputs(case, captured):
+@pytest.mark.parametrize("front", ["kernel", "copy"])
+def test_prefill_behind_writes_of_its_inputs(case, captured, front):
     B, st, inputs, buf, out, call = _setup(case)
     want = []
     for x in inputs:
@@ -45,9 +46,9 @@ def test_prefill_behind_writes_of_its_inputs(case, captured):
         want.append((out.clone(), B.delta_state_view(st, B.DELTA_VIEW_MASK).clone()))
     step, stage = call, [torch.empty_like(x) for x in buf]
 
-    def whole():      # kernels write the inputs, the call, a kernel reads its results
+    def whole():      # kernels (or copies) write the inputs, the call, a kernel reads its results
         for a, b in zip(buf, stage):
-            torch.mul(b, 1, out=a)
+            torch.mul(b, 1, out=a) if front == "kernel" else a.copy_(b)
         step()
         return out * 1, B.delta_state_view(st, B.DELTA_VIEW_MASK).clone()
 
