@@ -82,18 +82,17 @@ template <int D, bool PAIR> struct TqSmem {
   static constexpr uint32_t NKB = D / 64;                 // 64-element blocks per row
   static constexpr uint32_t SZ_TILE = NKB * SZ_BLK;       // one [128][D] operand tile
   static constexpr uint32_t NQ = PAIR ? 2 : 1;            // query tiles (heads) per CTA
-  static constexpr uint32_t NKS = PAIR ? 3 : (D == 64) ? 4 : 3;      // key ring stages
-  static constexpr uint32_t NVS = PAIR ? 3 : (D == 64) ? 4 : 2;      // value ring stages
+  static constexpr uint32_t NKS = (D == 64) ? 4 : 3;      // key ring stages
+  static constexpr uint32_t NVS = (D == 64) ? 4 : 2;      // value ring stages
   // original keys of mixed tiles (key deltas), from OFF_QH on: d = 64 has the scores of two mixed
   // tiles in flight at a time
   static constexpr uint32_t NKX = (D == 64) ? 2 : 1;
   static constexpr uint32_t OFF_Q = 0;                    // [NQ] query tiles
   static constexpr uint32_t OFF_QH = OFF_Q + NQ * SZ_TILE;   // [NQ] reference-query tiles
-  // d = 64, query deltas: two operand tiles mixed by row halves, [Q rows 0-63; Q_hat rows
-  // 64-127] and [Q_hat rows 0-63; Q rows 64-127] (mixed tiles of block windows whose edges
-  // fall on multiples of 64)
-  static constexpr uint32_t OFF_QM = OFF_QH + NQ * SZ_TILE;  // [NQ][2]
-  static constexpr uint32_t OFF_K = OFF_QM + ((D == 64) ? 2 * NQ * SZ_TILE : 0);
+  // d = 64, query deltas: an operand tile mixed by row halves, [Q rows 0-63; Q_hat rows 64-127]
+  // (mixed tiles of block windows whose edges fall on multiples of 64)
+  static constexpr uint32_t OFF_QM = OFF_QH + NQ * SZ_TILE;  // [NQ]
+  static constexpr uint32_t OFF_K = OFF_QM + ((D == 64) ? NQ * SZ_TILE : 0);
   static constexpr uint32_t OFF_V = OFF_K + NKS * SZ_TILE;
   static constexpr uint32_t OFF_BAR = OFF_V + NVS * SZ_TILE;
   static constexpr uint32_t OFF_MISC = OFF_BAR + 40 * 8;
@@ -169,13 +168,12 @@ __device__ __forceinline__ float chunk_max(const uint32_t (&u)[128], int lane) {
 // front of the blocks (refs; the block loop is not unrolled: this code
 // runs once per CTA and straight-line code costs more to fetch than it saves); writes the
 // reference rows into the operand tile at qh_dst and, with
-// `quarters`, the two row-mixed operand tiles at qm_dst ([Q rows 0-63; Q_hat rows 64-127] and
-// the reverse).  REV: strategy (2), rows from the top.  CHECK: the tile holds rows past the
+// `quarters`, the row-mixed operand tile at qm_dst ([Q rows 0-63; Q_hat rows 64-127]).  REV: strategy (2), rows from the top.  CHECK: the tile holds rows past the
 // end of the sequence (row0 + r >= T) or the un-thresholded basis row.
 constexpr int kMaxBlocks = 4;                // a thread's rows, 8 at a time
 template <bool REV, bool CHECK>
 __device__ __forceinline__ void build_ref_rows(const unsigned char* q_src, unsigned char* qh_dst, unsigned char* qm_dst,
-                                               uint32_t sz_tile, const uint32_t (&offs)[DELTA_CKPT_ROWS],
+                                               const uint32_t (&offs)[DELTA_CKPT_ROWS],
                                                float2 (&refs)[kMaxBlocks], int nbk, float theta, bool quarters, int seg_row0,
                                                int row0, int T, int basis_row) {
 #pragma unroll 1
@@ -184,8 +182,6 @@ __device__ __forceinline__ void build_ref_rows(const unsigned char* q_src, unsig
 #pragma unroll
     for (int i = 0; i + 1 < kMaxBlocks; ++i) refs[i] = refs[i + 1];       // (no index depends on bk: they stay in registers)
     const bool low = (seg_row0 + bk * DELTA_CKPT_ROWS) < 64;
-    unsigned char* const m_q = qm_dst + (low ? 0u : sz_tile);     // takes the query rows of this block
-    unsigned char* const m_h = qm_dst + (low ? sz_tile : 0u);     // takes the reference rows
 #pragma unroll
     for (int rr = 0; rr < DELTA_CKPT_ROWS; ++rr) {
       const int r8 = REV ? DELTA_CKPT_ROWS - 1 - rr : rr;
@@ -205,10 +201,7 @@ __device__ __forceinline__ void build_ref_rows(const unsigned char* q_src, unsig
       // exact: the reference is a copy of an input element (or the zero it starts from)
       const uint32_t hw = __byte_perm(__float_as_uint(cur0), __float_as_uint(cur1), 0x7632);
       *reinterpret_cast<uint32_t*>(qh_dst + off) = hw;
-      if (quarters) {
-        *reinterpret_cast<uint32_t*>(m_q + off) = xw;
-        *reinterpret_cast<uint32_t*>(m_h + off) = hw;
-      }
+      if (quarters) *reinterpret_cast<uint32_t*>(qm_dst + off) = low ? xw : hw;
     }
   }
 }
@@ -461,14 +454,14 @@ hybrid_attn_tcq_kernel(const __grid_constant__ TqMapList<N> maps, const __grid_c
         const uint32_t ring = base + OFF_K + ((uint32_t)t % NKS) * SZ_TILE;
         if (cls == 3) {
           // each half of 64 keys against the operand tile whose row halves are Q where the
-          // quarter lies inside the window and Q_hat where it does not
+          // quarter lies inside the window and Q_hat where it does not.  (Keys inside the window of rows
+          // 64-127 alone begin a window block behind rows 0-63, which the causal mask takes: Q.)
           const int rb0 = i0 / W, rb1 = (i0 + 64) / W;
 #pragma unroll
           for (int hf = 0; hf < 2; ++hf) {
             const int jb = (t * BN + 64 * hf) / W;
             const bool in0 = rb0 == jb, in1 = rb1 == jb;
-            const uint32_t a = base + (in0 ? (in1 ? OFF_Q + qsel : OFF_QM + 2 * qsel)
-                                           : (in1 ? OFF_QM + 2 * qsel + SZ_TILE : OFF_QH + qsel));
+            const uint32_t a = base + (in1 ? OFF_Q : in0 ? OFF_QM : OFF_QH) + qsel;
 #pragma unroll
             for (int ks = 0; ks < D / 16; ++ks)
               tc_mma_if(lead, tmem + TMEM_S + 128u * X + 64u * hf, make_desc(a + (ks >> 2) * SZ_BLK + (ks & 3) * 32, 16, 1024),
@@ -624,10 +617,10 @@ hybrid_attn_tcq_kernel(const __grid_constant__ TqMapList<N> maps, const __grid_c
       mbar_wait(BAR(BAR_Q), 0, abort_flag);      // the query tile has landed
       const unsigned char* const q_src = sm + OFF_Q + qsel + thr_off;
       unsigned char* const qh_dst = sm + OFF_QH + qsel + thr_off;
-      unsigned char* const qm_dst = sm + OFF_QM + 2 * qsel + thr_off;
+      unsigned char* const qm_dst = sm + OFF_QM + qsel + thr_off;
       const bool check = (i0 + BM > T) || (basis_row >= i0 && basis_row < i0 + BM);
 #define BUILD(REV, CHECK)                                                                              \
-  build_ref_rows<REV, CHECK>(q_src, qh_dst, qm_dst, SZ_TILE, offs, refs, nbk, p.theta, quarters, seg * SEG, i0, T, \
+  build_ref_rows<REV, CHECK>(q_src, qh_dst, qm_dst, offs, refs, nbk, p.theta, quarters, seg * SEG, i0, T, \
                              basis_row)
       if (p.reverse) { if (check) BUILD(true, true); else BUILD(true, false); }
       else { if (check) BUILD(false, true); else BUILD(false, false); }
