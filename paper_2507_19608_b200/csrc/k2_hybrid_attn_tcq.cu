@@ -145,24 +145,6 @@ template <> struct TqMapList<1> { TqMaps m[1]; };
 // make the compiler reserve all sixteen hardware barriers).
 __device__ __forceinline__ void softmax_groups_sync() { asm volatile("bar.sync 1, 256;" ::: "memory"); }
 
-// Maximum of the 32-column chunk Q of a score row; MASKED: only the columns up to `lane`.
-template <int Q, bool MASKED>
-__device__ __forceinline__ float chunk_max(const uint32_t (&u)[128], int lane) {
-  float m0 = __uint_as_float(u[32 * Q]), m1 = -INFINITY;
-#pragma unroll
-  for (int c = 1; c < 32; c += 2) {
-    const float a0 = __uint_as_float(u[32 * Q + c]);
-    const float a1 = (c + 1 < 32) ? __uint_as_float(u[32 * Q + c + 1]) : -INFINITY;
-    if (!MASKED) {
-      m0 = fmax3(m0, a0, a1);
-    } else {
-      m0 = fmaxf(m0, c <= lane ? a0 : -INFINITY);
-      m1 = fmaxf(m1, c + 1 <= lane ? a1 : -INFINITY);
-    }
-  }
-  return fmaxf(m0, m1);
-}
-
 // Eq. 2-3 re-run over nbk 8-row blocks of two neighbouring channels of a query tile in shared
 // memory (128-byte swizzle, offs[rr] = offset of row rr of a block), from the references in
 // front of the blocks (refs; the block loop is not unrolled: this code
@@ -299,6 +281,8 @@ hybrid_attn_tcq_kernel(const __grid_constant__ TqMapList<N> maps, const __grid_c
   // scores: the next score product is issued as soon as the group has read the buffer, by a
   // warp of its own, while another one issues the P.V products.
   constexpr bool ALIAS = (D == 128);
+  // d = 128 with mixed tiles: no room for a row's scores beside the mixed tiles' code, they are read twice
+  constexpr bool REREAD = ALIAS && MIXED;
 
   if (warp == 0) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
@@ -485,7 +469,13 @@ hybrid_attn_tcq_kernel(const __grid_constant__ TqMapList<N> maps, const __grid_c
       if (!KEY) poll(BAR(BAR_QH), 0, abort_flag);   // the softmax warps have built Q_hat
       tc_fence_after();
       first_scores(0);
-      if (U > 1) first_scores(1);
+      if (U > 1) {
+        // d = 64: the second group starts when the first has its first tile's maximum.  Started together, the groups
+        // reach their exponentials together too and share the unit that the rest of their tiles leaves idle (16 x 32
+        // heads x 2048 tokens 549 -> 512 us with the scores read once).  (Held to strict turns they are slower, 554.)
+        if (!ALIAS && !(MIXED && tile_class(0) == 1)) poll(BAR(BAR_SCONS0), 0, abort_flag);
+        first_scores(1);
+      }
       for (int u = 0; u < U; ++u) {
         const int t = tile_of(u);
         const uint32_t X = (uint32_t)u & 1u;
@@ -750,70 +740,56 @@ hybrid_attn_tcq_kernel(const __grid_constant__ TqMapList<N> maps, const __grid_c
       const bool diag = (t == qt);
       pv_waited = false;
       if (!MIXED || tile_class(t) != 1) {
-        // ---- the common tile: two passes over the score buffer, the row maximum first, then the
-        // exponentials in halves of 64 columns
+        // ---- the common tile: the scores stay in registers from the one read on, the row maximum first, then
+        // the exponentials in halves of 64 columns.  (Each half read again for its exponentials: 16 x 32 heads x
+        // 2048 tokens 531 us, so 512.)
+        uint32_t sr[128];
+        tc_ld128(t_s, sr);
+        // causal mask on the diagonal tile.  The warp's rows are 32 w4 .. 32 w4 + 31 of the
+        // tile: the 32-column chunks in front of chunk w4 are unmasked for all of them, chunk
+        // w4 is masked behind each thread's own column, the chunks after it entirely
+        auto mask_chunk = [&](uint32_t* x, int q) {
+#pragma unroll
+          for (int c = 0; c < 32; ++c) x[c] = (q > w4 || (q == w4 && c > lane)) ? 0xff800000u : x[c];      // -inf
+        };
+        const int live = diag ? w4 + 1 : 4;        // 32-column chunks that hold anything but masked scores
+        if (diag)
+#pragma unroll
+          for (int q = 0; q < 4; ++q) mask_chunk(sr + 32 * q, q);
         float mx;
         {
-          uint32_t u[128];
-          tc_ld128(t_s, u);
-          if (!diag) {
-            float m0 = fmax3(__uint_as_float(u[0]), __uint_as_float(u[1]), __uint_as_float(u[2]));
-            float m1 = fmax3(__uint_as_float(u[3]), __uint_as_float(u[4]), __uint_as_float(u[5]));
-            float m2 = fmax3(__uint_as_float(u[6]), __uint_as_float(u[7]), __uint_as_float(u[8]));
-            float m3 = fmax3(__uint_as_float(u[9]), __uint_as_float(u[10]), __uint_as_float(u[11]));
+          float m0 = fmax3(__uint_as_float(sr[0]), __uint_as_float(sr[1]), __uint_as_float(sr[2]));
+          float m1 = fmax3(__uint_as_float(sr[3]), __uint_as_float(sr[4]), __uint_as_float(sr[5]));
+          float m2 = fmax3(__uint_as_float(sr[6]), __uint_as_float(sr[7]), __uint_as_float(sr[8]));
+          float m3 = fmax3(__uint_as_float(sr[9]), __uint_as_float(sr[10]), __uint_as_float(sr[11]));
 #pragma unroll
-            for (int c = 12; c < 124; c += 8) {
-              m0 = fmax3(m0, __uint_as_float(u[c]), __uint_as_float(u[c + 1]));
-              m1 = fmax3(m1, __uint_as_float(u[c + 2]), __uint_as_float(u[c + 3]));
-              m2 = fmax3(m2, __uint_as_float(u[c + 4]), __uint_as_float(u[c + 5]));
-              m3 = fmax3(m3, __uint_as_float(u[c + 6]), __uint_as_float(u[c + 7]));
-            }
-            m0 = fmax3(m0, __uint_as_float(u[124]), __uint_as_float(u[125]));
-            m1 = fmax3(m1, __uint_as_float(u[126]), __uint_as_float(u[127]));
-            mx = fmaxf(fmaxf(m0, m1), fmaxf(m2, m3));
-          } else {
-            // causal mask on the diagonal tile.  The warp's rows are 32 w4 .. 32 w4 + 31 of the
-            // tile: the 32-column chunks in front of chunk w4 are unmasked for all of them, chunk
-            // w4 is masked behind each thread's own column, the chunks after it entirely
-            mx = (w4 == 0) ? chunk_max<0, true>(u, lane) : chunk_max<0, false>(u, lane);
-            if (w4 >= 1) mx = fmaxf(mx, (w4 == 1) ? chunk_max<1, true>(u, lane) : chunk_max<1, false>(u, lane));
-            if (w4 >= 2) mx = fmaxf(mx, (w4 == 2) ? chunk_max<2, true>(u, lane) : chunk_max<2, false>(u, lane));
-            if (w4 >= 3) mx = fmaxf(mx, chunk_max<3, true>(u, lane));
+          for (int c = 12; c < 124; c += 8) {
+            m0 = fmax3(m0, __uint_as_float(sr[c]), __uint_as_float(sr[c + 1]));
+            m1 = fmax3(m1, __uint_as_float(sr[c + 2]), __uint_as_float(sr[c + 3]));
+            m2 = fmax3(m2, __uint_as_float(sr[c + 4]), __uint_as_float(sr[c + 5]));
+            m3 = fmax3(m3, __uint_as_float(sr[c + 6]), __uint_as_float(sr[c + 7]));
           }
+          m0 = fmax3(m0, __uint_as_float(sr[124]), __uint_as_float(sr[125]));
+          m1 = fmax3(m1, __uint_as_float(sr[126]), __uint_as_float(sr[127]));
+          mx = fmaxf(fmaxf(m0, m1), fmaxf(m2, m3));
         }
         settle_scale(u, mx, u >= 2, false);
-        // the exponentials, one half of 64 columns at a time
-        auto exp_half = [&](int hf) {
+        s_consumed();
+#pragma unroll
+        for (int hf = 0; hf < 2; ++hf) {
+          if constexpr (REREAD) {
+            uint32_t x[64];
+            tc_ld64(t_s + 64u * hf, x);
+#pragma unroll
+            for (int c = 0; c < 64; ++c) sr[64 * hf + c] = x[c];
+            if (diag)
+#pragma unroll
+              for (int q = 2 * hf; q < 2 * hf + 2; ++q) mask_chunk(sr + 32 * q, q);
+          }
           float v[64];
-          {
-            uint32_t u[64];
-            tc_ld64(t_s + 64u * hf, u);
 #pragma unroll
-            for (int c = 0; c < 64; ++c) v[c] = __uint_as_float(u[c]);
-          }
-          if (hf == 1) s_consumed();
-          int live = 2;
-          if (diag) {
-            live = min(max(w4 + 1 - 2 * hf, 0), 2);
-            // chunk w4 of the tile, if it lies in this half: masked behind the thread's own column
-            // (selects on every element of the half: no index may depend on w4)
-#pragma unroll
-            for (int qq = 0; qq < 2; ++qq) {
-              const bool part = w4 == 2 * hf + qq;
-#pragma unroll
-              for (int c = 1; c < 32; ++c) v[32 * qq + c] = (part && c > lane) ? -INFINITY : v[32 * qq + c];
-            }
-          }
-          exp_store(v, hf, u, live);
-        };
-        if (D == 64) {
-          // (two copies of the code: 8 % faster in the steady state than a loop)
-          exp_half(0);
-          exp_half(1);
-        } else {
-          // (d = 128: the two-copy form spills)
-#pragma unroll 1
-          for (int hf = 0; hf < 2; ++hf) exp_half(hf);
+          for (int c = 0; c < 64; ++c) v[c] = __uint_as_float(sr[64 * hf + c]);
+          exp_store(v, hf, u, min(max(live - 2 * hf, 0), 2));
         }
       } else {
         // ---- a mixed tile (Section III-B hybrid select), one half of 64 keys at a time.  d = 64: the
