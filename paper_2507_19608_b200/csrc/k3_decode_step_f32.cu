@@ -274,8 +274,7 @@ decode_step_f32_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_co
   }
   if (CLUSTER) {
     // (every slice's block records: also what keeps this CTA until the last of them has been sent to it)
-    if (!mbar_wait(bar_m, 0)) s_fail = 1;
-    merge_slices<float, D, G>(recs, rank, cs, o0, p.out);
+    if (!merge_slices<float, D, G, NW>(recs, bar_m, rank, cs, o0, p.out)) s_fail = 1;
   } else if (n_slices > 1) {
     merge_global<float, D, G, NW>(n_slices, bkv, o0, p.partial, p.ticket, p.out, &s_last);
   }

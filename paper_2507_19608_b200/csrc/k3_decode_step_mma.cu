@@ -735,8 +735,7 @@ decode_step_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_co
   }
   if (CLUSTER) {
     // (every slice's block records: also what keeps this CTA until the last of them has been sent to it)
-    if (!mbar_wait(bar_m, 0)) s_fail = 1;
-    merge_slices<TC, D, G>(recs, rank, cs, out0, p.out);
+    if (!merge_slices<TC, D, G, MNW>(recs, bar_m, rank, cs, out0, p.out)) s_fail = 1;
   } else if (n_slices > 1) {
     merge_global<TC, D, G, MNW>(n_slices, bkv, out0, p.partial, p.ticket, p.out, &s_last);
   }

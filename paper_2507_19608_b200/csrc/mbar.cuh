@@ -67,4 +67,14 @@ __device__ __forceinline__ void mbar_poll(uint32_t bar, uint32_t parity, volatil
   }
 }
 
+// ... for a warp at the end of a kernel that waits for the last bytes.
+__device__ __forceinline__ bool mbar_spin(uint32_t bar, uint32_t parity) {
+  if (mbar_test_wait(bar, parity)) return true;
+  const long long t0 = clock64();
+  unsigned spins = 0;
+  while (!mbar_test_wait(bar, parity))
+    if ((++spins & 255u) == 0 && clock64() - t0 > kWaitBudgetClocks) return false;
+  return true;
+}
+
 }  // namespace delta
