@@ -343,12 +343,9 @@ decode_step_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_co
     uint4 q4[NC];
 #pragma unroll
     for (int c = 0; c < NC; ++c) q4[c] = __ldcg(reinterpret_cast<const uint4*>(p.q_new + o0 + hd * D + 32 * c + 8 * t));
-    // (behind those loads: they are what the warp waits for next)
-    if (jg < j1) {
-      if (!early_k) fetch_k(jg, 0);
-      fetch_v(jg, 1);
-      if (NS == 3 && jg + UK * MNW < j1) fetch_k(jg + UK * MNW, 2);
-    }
+    // (behind those loads: they are what the warp waits for next; the values, needed last, behind their arrival: a
+    // unit's rows of every warp at once take the SM half a microsecond, which the loads would wait for)
+    if (jg < j1 && !early_k) fetch_k(jg, 0);
     if (has_new) {
 #pragma unroll
       for (int e = 0; e < 2 * (D / 8); e += 32)
@@ -356,6 +353,11 @@ decode_step_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_co
           const int ch = (e + lane) % (D / 8);
           async16(new_s + 16 * (e + lane), (e + lane < D / 8 ? kn : vn) + 8 * ch);
         }
+    }
+    if (mine) asm volatile("" : "+f"(x[0]), "+f"(ref[0])::"memory");          // (they have arrived)
+    if (jg < j1) {
+      fetch_v(jg, 1);
+      if (NS == 3 && jg + UK * MNW < j1) fetch_k(jg + UK * MNW, 2);
     }
     int fired = 0;
     if (mine) {
