@@ -303,6 +303,62 @@ decode_step_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_co
 #pragma unroll
     for (int c = 0; c < NV; ++c) tc::tma_load_3d_if(lead, slot_v + c * UK * 128, &tm_v, bar_v, 64 * c, jg, bkv);
   };
+  // Rows jg .. jg + 31 of the reference-key stream from their encoding, into the key slot: lane = two
+  // channels (of a 64-channel block), walking the rows; the window's rows and the new one are keys.
+  // Issue-bound, so what a row needs is laid out first, lane = row: for either half of the block's channels where the
+  // row's values of that half start and its mask word.  (Every lane counting for itself, and a row's loads behind the
+  // store of the one before: 147 clocks per row, a unit 2.5 us.)
+  auto rebuild = [&](int jg, uint32_t slot_k) {
+    constexpr int NWD = D / 32;
+    const int last = min(UK, min(n, wl) - jg);             // rows that are cached references
+    const int hi = lane >> 4, sh = 2 * (lane & 15);        // this lane's channels: bits sh, sh + 1 of word 2 c + hi
+    const uint32_t lt = (1u << sh) - 1u;
+    const uint32_t table = pack_s + SM::VALS + SM::MASKS + D * 2;
+    uint32_t w[NWD], total = 0;
+    lds_words(pack_s + SM::VALS + 4 * NWD * lane, w);
+#pragma unroll
+    for (int k = 0; k < NWD; ++k) total += __popc(w[k]);
+    uint32_t at = total;                                   // values up to this row, then in front of it
+#pragma unroll
+    for (int x = 1; x < 32; x <<= 1) {
+      const uint32_t up = __shfl_up_sync(0xffffffffu, at, x);
+      at += lane >= x ? up : 0u;
+    }
+    at = pack_s + 2 * (at - total);
+#pragma unroll
+    for (int c = 0; c < NV; ++c) {
+      const uint32_t at1 = at + 2 * __popc(w[2 * c]);
+      sts_u4(table + 16 * lane, make_uint4(at, w[2 * c], at1, w[2 * c + 1]));
+      at = at1 + 2 * __popc(w[2 * c + 1]);
+      __syncwarp();
+      uint32_t cur = lds_u32(pack_s + SM::VALS + SM::MASKS + 128 * c + 4 * lane);
+      const uint32_t dst = slot_k + c * UK * 128 + 4 * (lane & 3);
+#pragma unroll 1
+      for (int r0 = 0; r0 < last; r0 += 8) {
+        uint32_t f[8], a[8], x0[8], x1[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+          uint32_t e[2];
+          lds_words(table + 16 * (r0 + i) + 8 * hi, e);
+          a[i] = e[0] + 2 * __popc(e[1] & lt);
+          f[i] = e[1] >> sh;
+        }
+        // (a channel that has not fired reads some value of the pool and drops it: no branch)
+#pragma unroll
+        for (int i = 0; i < 8; ++i) { x0[i] = lds_u16(a[i]); x1[i] = lds_u16(a[i] + 2 * (f[i] & 1u)); }
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+          const int r = r0 + i;
+          cur = (f[i] & 1u) ? __byte_perm(cur, x0[i], 0x3254) : cur;
+          cur = (f[i] & 2u) ? __byte_perm(cur, x1[i], 0x5410) : cur;
+          if (r < last) sts_u32(dst + r * 128 + (((lane >> 2) ^ (r & 7)) << 4), cur);
+        }
+      }
+      __syncwarp();
+    }
+    async_wait_all();                                      // the rows that are not cached references (fetch_k)
+    __syncwarp();
+  };
   // the warp that owns the row arriving with the step, and that row in shared memory (keys, values)
   const bool has_new = j1 == L && j0 < L && ((n - j0) / UK) % MNW == warp;
   const uint32_t new_s = packs + MNW * SM::PACK;
@@ -314,6 +370,12 @@ decode_step_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_co
   int jg = j0 + UK * warp;
   const bool early_k = KEY && p.early && jg < j1 && jg + UK <= min(n - 1, wl);
   if (early_k) fetch_k(jg, 0);
+  // The first unit's rows from such an encoding are rebuilt ahead of the wait too, under the end of the step in front.
+  bool built = early_k && from_pack(jg), late = false;
+  if (built) {
+    late = !mbar_wait(bars0, 0);
+    rebuild(jg, slots);
+  }
   // the step in front (or the prefill) has written the reference, row n - 1 of the caches, the tickets
   asm volatile("griddepcontrol.wait;" ::: "memory");
   // The next step's CTAs may become resident from here on.  (Released at the kernel's start they
@@ -404,7 +466,8 @@ decode_step_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_co
     for (int e = 0; e < 4; ++e) o_acc[i][e] = 0.0f;
   float m = -INFINITY, l = 0.0f;
   unsigned done = 0;
-  uint32_t phases = 0;                       // of the slots' barriers, a bit each
+  uint32_t phases = built ? 1u : 0u;         // of the slots' barriers, a bit each
+  if (late) s_fail = 1;
   int sk = 0, sv = 1;                        // the slots of the unit's keys and values
   // Column x of a score block stands for key x ^ (4 (x & 1)) of its 8 keys: with the swizzle, the
   // eight lanes of a shared-memory phase then touch eight different chunks, for keys and values alike.
@@ -416,62 +479,6 @@ decode_step_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_co
   const int vr_ = (lane & 7) ^ (4 * (lane & 1));
   const uint32_t v_off = (lane >> 3) * 1024 + vr_ * 128 + (vr_ << 4);
   float* const Rg = KEY ? nullptr : p.R + ((size_t)b * p.H + kvh * G + hd) * T_max;
-  // Rows jg .. jg + 31 of the reference-key stream from their encoding, into the key slot: lane = two
-  // channels (of a 64-channel block), walking the rows; the window's rows and the new one are keys.
-  // Issue-bound, so what a row needs is laid out first, lane = row: for either half of the block's channels where the
-  // row's values of that half start and its mask word.  (Every lane counting for itself, and a row's loads behind the
-  // store of the one before: 147 clocks per row, a unit 2.5 us.)
-  auto rebuild = [&](int jg, uint32_t slot_k) {
-    constexpr int NWD = D / 32;
-    const int last = min(UK, min(n, wl) - jg);             // rows that are cached references
-    const int hi = lane >> 4, sh = 2 * (lane & 15);        // this lane's channels: bits sh, sh + 1 of word 2 c + hi
-    const uint32_t lt = (1u << sh) - 1u;
-    const uint32_t table = pack_s + SM::VALS + SM::MASKS + D * 2;
-    uint32_t w[NWD], total = 0;
-    lds_words(pack_s + SM::VALS + 4 * NWD * lane, w);
-#pragma unroll
-    for (int k = 0; k < NWD; ++k) total += __popc(w[k]);
-    uint32_t at = total;                                   // values up to this row, then in front of it
-#pragma unroll
-    for (int x = 1; x < 32; x <<= 1) {
-      const uint32_t up = __shfl_up_sync(0xffffffffu, at, x);
-      at += lane >= x ? up : 0u;
-    }
-    at = pack_s + 2 * (at - total);
-#pragma unroll
-    for (int c = 0; c < NV; ++c) {
-      const uint32_t at1 = at + 2 * __popc(w[2 * c]);
-      sts_u4(table + 16 * lane, make_uint4(at, w[2 * c], at1, w[2 * c + 1]));
-      at = at1 + 2 * __popc(w[2 * c + 1]);
-      __syncwarp();
-      uint32_t cur = lds_u32(pack_s + SM::VALS + SM::MASKS + 128 * c + 4 * lane);
-      const uint32_t dst = slot_k + c * UK * 128 + 4 * (lane & 3);
-#pragma unroll 1
-      for (int r0 = 0; r0 < last; r0 += 8) {
-        uint32_t f[8], a[8], x0[8], x1[8];
-#pragma unroll
-        for (int i = 0; i < 8; ++i) {
-          uint32_t e[2];
-          lds_words(table + 16 * (r0 + i) + 8 * hi, e);
-          a[i] = e[0] + 2 * __popc(e[1] & lt);
-          f[i] = e[1] >> sh;
-        }
-        // (a channel that has not fired reads some value of the pool and drops it: no branch)
-#pragma unroll
-        for (int i = 0; i < 8; ++i) { x0[i] = lds_u16(a[i]); x1[i] = lds_u16(a[i] + 2 * (f[i] & 1u)); }
-#pragma unroll
-        for (int i = 0; i < 8; ++i) {
-          const int r = r0 + i;
-          cur = (f[i] & 1u) ? __byte_perm(cur, x0[i], 0x3254) : cur;
-          cur = (f[i] & 2u) ? __byte_perm(cur, x1[i], 0x5410) : cur;
-          if (r < last) sts_u32(dst + r * 128 + (((lane >> 2) ^ (r & 7)) << 4), cur);
-        }
-      }
-      __syncwarp();
-    }
-    async_wait_all();                                      // the rows that are not cached references (fetch_k)
-    __syncwarp();
-  };
   // The new row joins the encoding (the warp that owns its unit): values behind the pool's end (on a
   // multiple of 8 where it opens a segment), mask words, count, offsets, the segment's base.
   auto append = [&](int nz) {
@@ -546,9 +553,12 @@ decode_step_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_co
     const bool owner = n < jg + UK;          // of the row that arrives with the step
     const bool packed = from_pack(jg), tma_k = !packed && k_plain(jg);
     if (packed) {
-      if (!mbar_wait(bar_k, (phases >> sk) & 1u)) s_fail = 1;
-      phases ^= 1u << sk;
-      rebuild(jg, slot_k);
+      if (!built) {
+        if (!mbar_wait(bar_k, (phases >> sk) & 1u)) s_fail = 1;
+        phases ^= 1u << sk;
+        rebuild(jg, slot_k);
+      }
+      built = false;
     } else if (tma_k) {
       if (!mbar_wait(bar_k, (phases >> sk) & 1u)) s_fail = 1;
       phases ^= 1u << sk;
