@@ -13,7 +13,7 @@ if not torch.cuda.is_available():
     (1, 32, 8, 384, "query", 64), (1, 32, 8, 385, "query", 64),          # all one head | half of the query tiles
     (1, 16, 4, 1024, "query", 100), (1, 16, 4, 1025, "query", 100),
     (1, 32, 8, 1000, "key", 64),                                         # as many as fit one wave
-    (1, 32, 8, 1152, "query", 64), (1, 32, 8, 1153, "query", 64),        # the last such size | all two heads
+    (1, 32, 8, 1024, "query", 64), (1, 32, 8, 1025, "query", 64),        # the last such size | all two heads
     (1, 32, 8, 1153, "key", 100), (3, 16, 8, 800, "query", 0), (2, 32, 8, 640, "query", 0)])
 def test_forms_agree(Bn, H, Hk, T, source, W):
     from paper_2507_19608_b200 import binding as B

@@ -95,9 +95,11 @@ def test_ragged_batches(B, source, Bn, d):
 
 
 @pytest.mark.parametrize("source", ["query", "key"])
-@pytest.mark.parametrize("d", [64, 128])
-@pytest.mark.parametrize("ramp", [0.004, -0.004])
+@pytest.mark.parametrize("d,ramp", [(64, 0.004), (64, -0.004), (128, 0.006), (128, -0.006)])
 def test_scores_that_run_away(B, source, d, ramp):
-    # one CTA, several units per warp: a row's maximum moves by more than the 2^8 up to which the scale is kept
-    # (ramp 0.004 over the 256 keys between a warp's units: scores double from unit to unit, up to hundreds), or only falls
-    _compare(B, source, 40, 4, 1, d, [1100] * 40, 64, 2, ramp=ramp)
+    # Several units per warp: a row's maximum moves by more than the 2^8 up to which the scale is kept (a warp's units
+    # are 256 keys apart, 128 at d = 128: scores grow by 2 and 1.7 from unit to unit, up to hundreds), or only falls.
+    # 160 KV heads take one slice each, since clusters of two have no room (320 CTAs, 1.75 per SM at most): 35 units on
+    # a CTA's 8 or 4 warps.
+    assert 2 * 160 > 1.75 * torch.cuda.get_device_properties(0).multi_processor_count
+    _compare(B, source, 40, 16, 4, d, [1100] * 40, 64, 2, ramp=ramp)

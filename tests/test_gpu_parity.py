@@ -565,7 +565,8 @@ def test_key_delta_prefill_matches_oracle(B, case, form):
     (1, 1, 1, 1, 64, 0.1, 2, 4),
     (2, 4, 2, 700, 64, 0.2, 100, 3),       # the window's edge inside a tile, several slices
     (3, 4, 4, 1500, 64, 0.2, 300, 2),      # window over three tiles: key-cache tiles, one mixed tile
-    (40, 4, 4, 1100, 64, 0.2, 64, 2),      # 160 KV heads: one slice of 9 tiles per head
+    (40, 4, 4, 1100, 64, 0.2, 64, 2),      # 160 KV heads: one slice of 35 units per head
+    (40, 4, 4, 1100, 128, 0.2, 64, 2),     # the same: nine units per warp of a CTA's four
 ])
 @pytest.mark.parametrize("decode_kernel", [0, 1, 2], ids=["fp32_pipes", "tc_scores", "packed_cache"])
 def test_key_delta_decode_steps_match_oracle(B, Bn, H, Hk, T, d, theta, W, steps, decode_kernel):
@@ -645,7 +646,7 @@ BOTTOM_UP_CASES = [
     (1, 8, 2, 384, 128, 0.25, 128, "block", "basis_exact"),
     (1, 2, 1, 1000, 64, 0.29, 64, "block", "zero_state"),
     (1, 2, 1, 1, 64, 0.1, 4, "block", "basis_exact"),
-    (1, 96, 96, 150, 64, 0.2, 64, "block", "basis_exact"),      # more heads than SMs: the row-by-row chain kernel
+    (1, 150, 150, 150, 64, 0.2, 64, "block", "basis_exact"),    # 300 CTAs of the table kernel on 148 SMs: row by row
 ]
 
 
