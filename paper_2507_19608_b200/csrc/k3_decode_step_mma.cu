@@ -10,7 +10,7 @@
 // Bound: one pass over the key and value cache (HBM, or L2 for a layer stepped in a loop); for a few
 // sequences the chain of dependent latencies in front of and behind that pass.  So a warp works alone:
 // it owns units of 32 keys, brings their key and value rows in by TMA (one box each, 128-byte swizzle,
-// a ring of three halves), multiplies on mma.sync (m16n8k16) straight from the swizzled rows and keeps
+// a ring of three halves, two for the compressed key cache), multiplies on mma.sync (m16n8k16) straight from the swizzled rows and keeps
 // its own running softmax; warps meet once, at the end.  Staging by per-thread cp.async instead of TMA
 // was bound by the SM's load path at half the rate (batch 16, 2048 keys: 18.9 us per step, TMA 12.2).
 // With the copies ahead of their use, a unit's time is its instructions (two CTAs per SM: 3060 clocks a
@@ -23,8 +23,8 @@
 // scores of a (head, key) pair in registers.
 //   scores  A = [references; queries] (16 x D), B = 8 keys: the contraction index may be permuted
 //           freely as long as both operands agree, so a thread takes 16-byte pieces of its key's row;
-//   P.V     A = P with the score accumulator's layout, B = 16 keys x 8 channels: output columns may
-//           be permuted, so a thread takes 16-byte pieces of four value rows and zips pairs of rows.
+//   P.V     A = P with the score accumulator's layout, B = 16 keys x 8 channels: one ldmatrix.trans
+//           brings a unit's four 8-key tiles of 8 channels (keys in the order of A's columns).
 //           P keeps fp32 precision as a sum of three bf16 parts: rows 0-7 of A carry the first part,
 //           rows 8-15 the second (the same thread holds both), the third goes to rows G .. 2G-1,
 //           whose lanes duplicate the scores of rows 0 .. G-1 (G <= 4), or to a second product (G = 8).
