@@ -16,10 +16,11 @@
 // sparse delta sums on the FP32 pipes, at 6.  Relative error against fp64 dense attention at 1000
 // tokens: 1.8e-7 (FP32-pipe kernel 3.7e-7).  mma.sync and not tcgen05: accumulators in registers make the
 // separate small-product sums and the per-tile fresh output sums free to join in fp32, and no key tile waits
-// for a hand-over through tensor memory; whether tcgen05 at the same precision would pay has not been measured.  Measured, whole prefill: 24 heads x 1425 tokens, d = 64:
-// 212 us = 29 TFLOP/s; 16 heads x 1000: 350 -> 95 us; one head x 128: 54 -> 13 us (the kernel 42 -> 6).
+// for a hand-over through tensor memory; whether tcgen05 at the same precision would pay has not been measured.
+// Measured, whole prefill, before this kernel, with head after head, with the longest walks first: 24 heads x 1425 tokens
+// -, 190, 136 us (46 TFLOP/s); 16 heads x 1000 350, 86, 66; one head x 128 54, 13, 13 (the kernel 42 -> 6).
 //
-// Bound: mma.sync issue (m16n8k16 every 8 clocks per scheduler) once the chip is full, the walk of the
+// Bound: mma.sync issue (m16n8k16 every 8 clocks per scheduler) once the chip is full (KS = 1: 60 % of it), the walk of the
 // last query tile where it is not.  A CTA of four warps owns 64 / KS query rows of one head and walks
 // the 64-key tiles up to the diagonal; KS warps share 16 rows and deal a tile's keys among themselves
 // (KS = 1: most work per byte staged; KS = 4: the shortest walk, with four times as many CTAs; the
@@ -432,21 +433,22 @@ __device__ __forceinline__ void attn_f32_tile(const F32Args<TIn>& p, const Seq& 
 
 }  // namespace
 
-// A uniform batch.
+// A uniform batch.  Heads are the fastest index: the longest walks of every head start first.  (Head after head, the
+// last head's longest walk started last: 16 heads x 1000 86.5 us, so 66.8; 32 x 2000 384, 314; d = 128 924, 819.)
 template <typename TIn, int D, int KS>
 __global__ void __launch_bounds__(NT, D == 64 ? 2 : 1)
 hybrid_attn_f32_kernel(const __grid_constant__ F32Args<TIn> p, const __grid_constant__ SeqList<1> seqs) {
-  attn_f32_tile<TIn, D, KS>(p, seqs.s[0], (int)blockIdx.x, (int)blockIdx.y);
+  attn_f32_tile<TIn, D, KS>(p, seqs.s[0], (int)blockIdx.y, (int)blockIdx.x);
 }
 // A ragged group: every sequence in the form of a batch of its own.
 template <typename TIn, int D>
 __global__ void __launch_bounds__(NT, D == 64 ? 2 : 1)
 hybrid_attn_f32_ragged_kernel(const __grid_constant__ F32Args<TIn> p, const __grid_constant__ SeqList<kSeqMax> seqs,
                               const __grid_constant__ F32Forms forms) {
-  const int i = (int)blockIdx.z, ks = forms.ks[i];
-  if (ks == 1) attn_f32_tile<TIn, D, 1>(p, seqs.s[i], (int)blockIdx.x, (int)blockIdx.y);
-  else if (ks == 2) attn_f32_tile<TIn, D, 2>(p, seqs.s[i], (int)blockIdx.x, (int)blockIdx.y);
-  else attn_f32_tile<TIn, D, 4>(p, seqs.s[i], (int)blockIdx.x, (int)blockIdx.y);
+  const int i = (int)blockIdx.y, ks = forms.ks[i];
+  if (ks == 1) attn_f32_tile<TIn, D, 1>(p, seqs.s[i], (int)blockIdx.z, (int)blockIdx.x);
+  else if (ks == 2) attn_f32_tile<TIn, D, 2>(p, seqs.s[i], (int)blockIdx.z, (int)blockIdx.x);
+  else attn_f32_tile<TIn, D, 4>(p, seqs.s[i], (int)blockIdx.z, (int)blockIdx.x);
 }
 
 template <typename K, typename... A>
@@ -471,25 +473,27 @@ static cudaError_t launch_f32(K kern, std::atomic<uint64_t>& ready, size_t smem,
   return e != cudaSuccess ? e : cudaGetLastError();
 }
 
-// Warps per row group for `heads` heads of T tokens.  A key tile of 64 costs 3.3 / 2.2 / 1.4 us where a CTA
-// walks alone and takes 4.0 / 2.2 / 1.6 us of an SM where the chip is full (KS = 1 / 2 / 4; d = 64, 1 to
-// 256 heads of 128 to 4000 tokens); every halving of the rows doubles the tiles.  The longest walk bounds a
-// small grid, the sum of all tiles, with half a walk for the uneven end, a large one.  Only the ratios count,
-// and they carry over to d = 128 (one CTA per SM, two to three times the time) and to bf16 inputs: with each
-// form timed at 1 to 128 heads of 128 to 4000 tokens (30 shapes per type and d) the chosen one is the
-// fastest or, fp32, within 6 % of it (64 or 128 heads of 128 tokens: 10 to 15 %); bf16, which runs here only
-// when kernel 0 is forced, within 16 % (there: 23 %).  16 heads x 1000, d = 64 / 128, KS = 1, 2, 4: 82, 81, 92 us
-// / 185, 170, 207; 32 x 2000: 375, 408, 521 / 930, 988, 1306.  A sequence of a
+// Warps per row group for `heads` heads of T tokens.  A key tile of 64 costs 3.5 / 2.2 / 1.4 us where a CTA
+// walks alone (its set-up about as much as a tile) and takes 2.7 / 1.6 / 1.1 us of an SM where the chip is full (KS = 1 /
+// 2 / 4, d = 64, two CTAs per SM; d = 128, one: 7.0 / 4.4 / 3.1 and 7.0 / 4.2 / 2.9); every halving of the rows doubles
+// the tiles.  The longest walk bounds a small grid; a large one the sum of all tiles and set-ups, and a part of a walk
+// for the uneven end, less of it the more CTAs a place gets.  With each form timed at 16 shapes per d (1 to 128 heads of
+// 64 to 2500 tokens, fp32) the chosen one is the fastest or within 1.1 % of it; KS = 1, 2, 4 in us: 16 heads x 1000
+// 75, 65, 80 / d = 128 125, 148, 196; 16 x 1800 147, 165, 217; 32 x 600 56, 49, 66 / 109, 120, 165; 8 x 700 44, 34, 31 /
+// 90, 58, 65.  bf16 inputs, which run here only when kernel 0 is forced, take the same form.  A sequence of a
 // ragged group takes the form of a batch of its own (the forms round differently: its result does not
 // depend on the sequences beside it).
-static int f32_form(long heads, int T) {
+static int f32_form(long heads, int T, int d) {
+  constexpr float alone[2][3] = {{3.5f, 2.2f, 1.4f}, {7.0f, 4.4f, 3.1f}}, full[2][3] = {{2.7f, 1.6f, 1.1f}, {7.0f, 4.2f, 2.9f}};
+  constexpr float set_up[2] = {0.8f, 4.0f};        // us of an SM per CTA
+  const int x = d == 64 ? 0 : 1;
+  const float sms = (float)device_sm_count(), t = (float)((T + BN - 1) / BN), pairs = 0.5f * t * (t + 1.0f) * (float)heads;
   int ks = 1;
   float best = 3.4e38f;
-  const float t = (float)((T + BN - 1) / BN), pairs = 0.5f * t * (t + 1.0f) * (float)heads;
   for (int c = 0; c < 3; ++c) {
-    constexpr float alone[3] = {3.3f, 2.2f, 1.4f}, full[3] = {4.0f, 2.2f, 1.6f};
-    const float walk = t * alone[c];
-    const float us = fmaxf(walk, pairs * (float)(1 << c) / (float)device_sm_count() * full[c] + 0.5f * walk);
+    const float walk = (t + 1.0f) * alone[x][c], ctas = (float)heads * (float)((T * (1l << c) + BN - 1) / BN);
+    const float r = fmaxf(1.0f, ctas / (sms * (float)(2 - x)));
+    const float us = fmaxf(walk, (pairs * (float)(1 << c) * full[x][c] + ctas * set_up[x]) / sms + 0.3f * walk / (r * r));
     if (us < best) { best = us; ks = 1 << c; }
   }
   return ks;
@@ -509,21 +513,21 @@ static cudaError_t launch_f32_form(const Shape& s, const Workspace& w, const voi
     unsigned tiles = 0;
     for (int i = 0; i < kSeqMax; ++i) {
       list.s[i] = seqs.s[i < seqs.n ? i : 0];
-      forms.ks[i] = f32_form(heads, list.s[i].T);
+      forms.ks[i] = f32_form(heads, list.s[i].T, D);
       const unsigned bm = 64u / (unsigned)forms.ks[i], n = ((unsigned)list.s[i].T + bm - 1) / bm;
       tiles = n > tiles ? n : tiles;
     }
     return launch_f32(hybrid_attn_f32_ragged_kernel<TIn, D>, ready[3],
                       std::max({F32Smem<D, 1, NP>::bytes, F32Smem<D, 2, NP>::bytes, F32Smem<D, 4, NP>::bytes}),
-                      dim3(tiles, (unsigned)s.H, (unsigned)seqs.n), st, p, list, forms);
+                      dim3((unsigned)s.H, (unsigned)seqs.n, tiles), st, p, list, forms);
   }
   SeqList<1> list;
   list.s[0] = seqs.s[0];
   const unsigned T = (unsigned)list.s[0].T, bh = (unsigned)(s.B * s.H);
-  const int ks = f32_form(heads, (int)T);
+  const int ks = f32_form(heads, (int)T, D);
 #define GO(KS)                                                                                               \
   return launch_f32(hybrid_attn_f32_kernel<TIn, D, KS>, ready[KS / 2], F32Smem<D, KS, NP>::bytes,            \
-                    dim3((T + 64 / KS - 1) / (64 / KS), bh), st, p, list)
+                    dim3(bh, (T + 64 / KS - 1) / (64 / KS)), st, p, list)
   if (ks == 4) GO(4);
   if (ks == 2) GO(2);
   GO(1);
