@@ -20,6 +20,8 @@
 // Eq. 6 -- plus, for query deltas, two passes over the keys that prefill needs anyway: the
 // hand-off row R(T-1)[j] = q_hat(T-1).k_j for decode and, for the tensor-core attention kernel
 // with the FP32 delta path, the channel-major fp32 copy of the keys.
+#include <algorithm>
+
 #include "delta_internal.cuh"
 #include "tc_common.cuh"
 
@@ -94,6 +96,13 @@ __device__ __forceinline__ float chain_sub_block(const SubBlock& t, float r, flo
   return p0 ? t.z[0].x : o;
 }
 
+// The streams of a launch, each as a map [heads][rows 0..T-1][D] with boxes of [64 rows][32 channels]: one over all
+// heads of a batch, or one per sequence of a ragged group; b: batch element of the workspace arrays that head 0 belongs to.
+template <int N> struct ChainSeqs {
+  CUtensorMap map[N];
+  int T[N], b[N];
+};
+
 }  // namespace
 
 // The chain of Eq. 3 costs three dependent operations per row (subtract, compare, select), about
@@ -104,9 +113,8 @@ __device__ __forceinline__ float chain_sub_block(const SubBlock& t, float r, flo
 // row i.  z_7 = x7, z_6 = fires(x7, x6) ? x7 : x6, and in general z_i = z_j for the first j > i
 // that fires against x_i (x_i if none does): 28 pair tests per sub-block, none of which
 // involves r.  Helper warps compute the z tables a stage ahead; the chain warp then does, per
-// sub-block, eight tests against r in parallel and a select tree: the dependent path is
-// subtract, compare, four selects per EIGHT rows, and the checkpoint in front of the sub-block is the only
-// store.  Every test is the same subtraction and comparison the sequential chain would make, so the
+// sub-block, eight tests against r in parallel and a chain of eight selects (a tree of them made no
+// difference), and the checkpoint in front of the sub-block is the only store.  Every test is the same subtraction and comparison the sequential chain would make, so the
 // result is bit-identical.
 //
 // One CTA per (head, 32 channels): a warp carries the chain (thread = channel), one streams the rows in with TMA,
@@ -119,12 +127,15 @@ __device__ __forceinline__ float chain_sub_block(const SubBlock& t, float r, flo
 // A sub-block cut short by the end of the sequence takes the sequential form from the staged values.
 // Measured (with the launch, by events), before -> after: 1 x 32 heads, 1024 tokens, d = 64 14.7 -> 13.9 us; 4096 keys
 // 36.4 -> 30.2; 20 heads, 2048 tokens, d = 128 22.0 -> 19.9; a cut last stage (1000 tokens) 16.1 -> 14.1.
-template <typename TIn, int D>
+template <typename TIn, int D, int N>
 __global__ void __launch_bounds__(CHAIN_THREADS) delta_chain_kernel(
-    const __grid_constant__ CUtensorMap tm_x, float* __restrict__ qhat_tile, float* __restrict__ qhat_out,
-    float* __restrict__ ckpt, unsigned long long* __restrict__ counters, int T, int n_tiles, int n_ckpt,
-    float theta, int basis_exact, int reverse, uint4* zero_ptr, unsigned zero_n16) {
-  // tm_x: the stream that becomes the delta matrix as [heads][rows 0..T-1][D]; box = [64 rows][32 channels]
+    const __grid_constant__ ChainSeqs<N> seqs, float* __restrict__ qhat_tile, float* __restrict__ qhat_out,
+    float* __restrict__ ckpt, unsigned long long* __restrict__ counters, int n_tiles, int n_ckpt,
+    float theta, int basis_exact, int reverse, int heads, uint4* zero_ptr, unsigned zero_n16) {
+  // blockIdx.x: (head, 32 channels) of the batch, or of sequence blockIdx.y of a ragged group
+  const int si = N == 1 ? 0 : (int)blockIdx.y;
+  const CUtensorMap& tm_x = seqs.map[si];
+  const int T = seqs.T[si];
   constexpr int NSL = D / CH;                      // channel slices (CTAs) per head
   constexpr uint32_t RAW_STAGE_BYTES = RC * CH * sizeof(TIn);
   extern __shared__ __align__(128) unsigned char dyn[];
@@ -133,7 +144,8 @@ __global__ void __launch_bounds__(CHAIN_THREADS) delta_chain_kernel(
   __shared__ __align__(8) unsigned long long bars[2 * NS + 2 * NZ];
   __shared__ uint32_t s_abort;
 
-  const int bh = blockIdx.x / NSL, sl = blockIdx.x - bh * NSL;
+  const int head = blockIdx.x / NSL, sl = blockIdx.x - head * NSL;       // head of the map
+  const int bh = seqs.b[si] * heads + head;                               // head of the workspace arrays
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const uint32_t full0 = smem_u32(&bars[0]), empty0 = smem_u32(&bars[NS]);
   const uint32_t zfull0 = smem_u32(&bars[2 * NS]), zfree0 = smem_u32(&bars[2 * NS + NZ]);
@@ -163,7 +175,7 @@ __global__ void __launch_bounds__(CHAIN_THREADS) delta_chain_kernel(
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   // the deferred clearing of a state reset (counters, tickets, second reference buffer): nothing
   // of this launch or of the kernels behind it touches that span before this kernel is complete
-  if (zero_ptr && blockIdx.x == 0)
+  if (zero_ptr && blockIdx.x == 0 && blockIdx.y == 0)
     for (unsigned i = tid; i < zero_n16; i += blockDim.x) zero_ptr[i] = make_uint4(0u, 0u, 0u, 0u);
 
   if (warp == 4 + cw) {
@@ -175,7 +187,7 @@ __global__ void __launch_bounds__(CHAIN_THREADS) delta_chain_kernel(
         if (i >= NS) mbar_wait(empty0 + 8 * s, ((i / NS) - 1) & 1, abort_flag);
         const int ci = reverse ? n_chunks - 1 - i : i;      // stage of the head in token order
         tc::mbar_expect_tx(full0 + 8 * s, RAW_STAGE_BYTES); // rows past T arrive as zeros
-        tc::tma_load_3d(raw0 + s * RAW_STAGE_BYTES, &tm_x, full0 + 8 * s, sl * CH, ci * RC, bh);
+        tc::tma_load_3d(raw0 + s * RAW_STAGE_BYTES, &tm_x, full0 + 8 * s, sl * CH, ci * RC, head);
       }
     }
   } else if ((warp & 3) != cw) {
@@ -308,46 +320,59 @@ static size_t even_spread_smem(size_t need, long ctas) {
 }
 constexpr int kMaxChainSmem = 144 * 1024;      // (fp32 tables 128 KB; the even spread asks for 114 KB at most)
 
-static cudaError_t launch_delta_chain_tables(const Shape& s, const Workspace& w, const void* q, int T, float theta,
-                                            int dtype, int init, bool key_stream, bool reverse, void* zero_ptr,
-                                            size_t zero_bytes, cudaStream_t st) {
-  const int heads = s.B * (key_stream ? s.H_kv : s.H);
-  const int src_rows = key_stream ? s.T_max : T;
-  const int basis = (init == DELTA_INIT_BASIS_EXACT) ? 1 : 0;
-  const bool f32 = dtype == DELTA_F32;
-  const size_t esz = f32 ? sizeof(float) : sizeof(__nv_bfloat16);
-  CUtensorMap tm;
-  if (!tc::encode3(&tm, f32 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, q, (uint64_t)s.d,
-                   (uint64_t)T, (uint64_t)heads, (uint64_t)s.d * esz, (uint64_t)src_rows * s.d * esz, CH, RC,
-                   CU_TENSOR_MAP_SWIZZLE_NONE))
-    return cudaErrorInvalidValue;
-  cudaError_t err = cudaSuccess;
+template <typename TIn, int D, int N>
+static cudaError_t launch_tables(const Shape& s, const Workspace& w, const void* x, const SeqBatch& seqs, float theta, int init,
+                                 bool key_stream, bool reverse, void* zero_ptr, size_t zero_bytes, cudaStream_t st) {
+  auto kern = delta_chain_kernel<TIn, D, N>;
+  constexpr size_t need = (size_t)NS * RC * CH * sizeof(TIn) + (size_t)NZ * Z_STAGE * sizeof(float4);
+  static_assert(need <= kMaxChainSmem, "shared memory");
+  static std::atomic<uint64_t> ready{0};
+  if (!device_done(ready)) {
+    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxChainSmem);
+    if (e != cudaSuccess) return e;
+    device_mark(ready);
+  }
+  const int heads = key_stream ? s.H_kv : s.H, map_heads = seqs.ragged ? heads : s.B * heads;
+  ChainSeqs<N> list;
+  int order[N];
+  for (int i = 0; i < seqs.n; ++i) order[i] = i;
+  std::sort(order, order + seqs.n, [&](int a, int b) { return seqs.s[a].T > seqs.s[b].T; });       // longest first
+  for (int i = 0; i < seqs.n; ++i) {
+    const Seq& sq = seqs.s[order[i]];
+    const size_t rows = key_stream ? (size_t)s.T_max : (size_t)sq.T;       // of a head in memory
+    const TIn* const from = (const TIn*)x + (key_stream ? (size_t)(seqs.ragged ? sq.b : 0) * heads * rows * D : sq.q_off);
+    if (!tc::encode3(&list.map[i], sizeof(TIn) == 4 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, from,
+                     (uint64_t)D, (uint64_t)sq.T, (uint64_t)map_heads, (uint64_t)D * sizeof(TIn), rows * D * sizeof(TIn), CH, RC,
+                     CU_TENSOR_MAP_SWIZZLE_NONE))
+      return cudaErrorInvalidValue;
+    list.T[i] = sq.T;
+    list.b[i] = seqs.ragged ? sq.b : 0;
+  }
   cudaLaunchAttribute attr[1];
   cudaLaunchConfig_t cfg = serialised_launch(attr, st);
-#define LAUNCH(TIN, DD)                                                                          \
-  do {                                                                                           \
-    auto kern = delta_chain_kernel<TIN, DD>;                                                     \
-    constexpr size_t need = (size_t)NS * RC * CH * sizeof(TIN) + (size_t)NZ * Z_STAGE * sizeof(float4); \
-    static_assert(need <= kMaxChainSmem, "shared memory");                                       \
-    static std::atomic<uint64_t> ready{0};                                                       \
-    if (!device_done(ready)) {                                                                   \
-      if ((err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxChainSmem)) != cudaSuccess) return err; \
-      device_mark(ready);                                                                        \
-    }                                                                                            \
-    cfg.gridDim = dim3((unsigned)(heads * (DD / CH)));                                           \
-    cfg.blockDim = dim3(CHAIN_THREADS);                                                          \
-    cfg.dynamicSmemBytes = even_spread_smem(need, (long)heads * (DD / CH));                      \
-    err = cudaLaunchKernelEx(&cfg, kern, tm, w.qhat_tile, w.qhat[0], w.ckpt, w.counters, T, s.n_tiles, s.n_ckpt(), theta, \
-                             basis, reverse ? 1 : 0, (uint4*)zero_ptr, (unsigned)(zero_bytes / 16)); \
-  } while (0)
-  if (f32) {
-    if (s.d == 64) LAUNCH(float, 64); else LAUNCH(float, 128);
-  } else {
-    if (s.d == 64) LAUNCH(__nv_bfloat16, 64); else LAUNCH(__nv_bfloat16, 128);
-  }
-#undef LAUNCH
+  cfg.gridDim = dim3((unsigned)(map_heads * (D / CH)), (unsigned)seqs.n);
+  cfg.blockDim = dim3(CHAIN_THREADS);
+  cfg.dynamicSmemBytes = even_spread_smem(need, (long)cfg.gridDim.x * seqs.n);
+  const cudaError_t err =
+      cudaLaunchKernelEx(&cfg, kern, list, w.qhat_tile, w.qhat[0], w.ckpt, w.counters, s.n_tiles, s.n_ckpt(), theta,
+                         init == DELTA_INIT_BASIS_EXACT ? 1 : 0, reverse ? 1 : 0, heads, (uint4*)zero_ptr, (unsigned)(zero_bytes / 16));
   count_launch();
   return err != cudaSuccess ? err : cudaGetLastError();
+}
+
+static cudaError_t launch_delta_chain_tables(const Shape& s, const Workspace& w, const void* x, const SeqBatch& seqs,
+                                             float theta, int dtype, int init, bool key_stream, bool reverse,
+                                             void* zero_ptr, size_t zero_bytes, cudaStream_t st) {
+#define GO(TIN, DD)                                                                                                 \
+  return seqs.ragged                                                                                                \
+             ? launch_tables<TIN, DD, kSeqMax>(s, w, x, seqs, theta, init, key_stream, reverse, zero_ptr, zero_bytes, st) \
+             : launch_tables<TIN, DD, 1>(s, w, x, seqs, theta, init, key_stream, reverse, zero_ptr, zero_bytes, st)
+  if (dtype == DELTA_F32) {
+    if (s.d == 64) { GO(float, 64); } else { GO(float, 128); }
+  } else {
+    if (s.d == 64) { GO(__nv_bfloat16, 64); } else { GO(__nv_bfloat16, 128); }
+  }
+#undef GO
 }
 
 // ---------------------------------------------------------------------------------------
@@ -586,19 +611,26 @@ int device_sm_count() {
   return cached[dev];
 }
 
+static bool chain_by_tables(const Shape& s, const SeqBatch& seqs, int dtype, bool key_stream) {
+  // The table kernel while its CTAs (head x 32 channels) are all resident at once: two per SM for bf16, one for fp32
+  // (shared memory: 96 and 128 KB).  Whole prefill, tables against rows: 64 CTAs (1 x 32 heads, 1024 tokens) 28.8 us, 34.0;
+  // 160 (2 x 20 heads, d = 128, 1531 tokens) 87.9, 90.2; 192 59.5, 61.5; 256 75.0, 77.0; 384 112.6, 110.0; 512 147.5, 139.5.
+  // In a ragged group, whose longest sequences come first, the CTAs count by their rows: six sequences of 99 to 1900 tokens,
+  // 32 heads, rows 121.8 us, tables 116.2; eight of 200 to 4000 264, 243; four of 90 to 900, key deltas 33.4, 28.4; four
+  // of 300 to 1500, 20 heads, d = 128 142.2, 143.1.
+  const long seq_ctas = (long)(seqs.ragged ? 1 : s.B) * (key_stream ? s.H_kv : s.H) * (s.d / CH);
+  long rows = 0;
+  for (int i = 0; i < seqs.n; ++i) rows += seqs.s[i].T;
+  return seq_ctas * rows <= (long)device_sm_count() * (dtype == DELTA_F32 ? 1 : 2) * seqs.T_longest;
+}
+
 cudaError_t launch_delta_chain(const Shape& s, const Workspace& w, const void* x, const SeqBatch& seqs, float theta,
                                int dtype, int init, bool key_stream, bool reverse, void* zero_ptr, size_t zero_bytes,
                                cudaStream_t st) {
   if (key_stream && reverse) return cudaErrorNotSupported;
   if (((uintptr_t)zero_ptr | zero_bytes) & 15u) return cudaErrorInvalidValue;
-  // The table kernel while its CTAs (head x 32 channels) are all resident at once: two per SM for bf16, one for fp32
-  // (shared memory: 96 and 128 KB).  Whole prefill, tables against rows: 64 CTAs (1 x 32 heads, 1024 tokens) 28.8 us, 34.0;
-  // 160 (2 x 20 heads, d = 128, 1531 tokens) 87.9, 90.2; 192 59.5, 61.5; 256 75.0, 77.0; 384 112.6, 110.0; 512 147.5, 139.5.
-  // (One tensor map: not for a ragged group.)
-  const long ctas = (long)s.B * (key_stream ? s.H_kv : s.H) * (s.d / CH);
-  if (!seqs.ragged && ctas <= (long)device_sm_count() * (dtype == DELTA_F32 ? 1 : 2))
-    return launch_delta_chain_tables(s, w, x, seqs.s[0].T, theta, dtype, init, key_stream, reverse, zero_ptr, zero_bytes,
-                                     st);
+  if (chain_by_tables(s, seqs, dtype, key_stream))
+    return launch_delta_chain_tables(s, w, x, seqs, theta, dtype, init, key_stream, reverse, zero_ptr, zero_bytes, st);
   return launch_delta_chain_rows(s, w, x, seqs, theta, dtype, init, key_stream, reverse, zero_ptr, zero_bytes, st);
 }
 

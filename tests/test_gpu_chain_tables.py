@@ -62,3 +62,37 @@ def _check(B, H, T, d, dtype, theta, init, order):
             nt = (T + 63) // 64
             assert np.array_equal(got_tile[0, h, :nt].view(np.uint32), r["ahat_tile"].view(np.uint32)), h
     assert B.delta_sparsity_stats(st)["device_status"] == 0
+
+
+@pytest.mark.parametrize("source", ["query", "key", "bottom_up"])
+@pytest.mark.parametrize("d,lens", [(64, (300, 261, 299, 300)), (64, (300, 295, 300, 299, 280)), (64, (777, 8, 513, 64, 1, 505)),
+                                    (128, (300, 300)), (128, (300, 299, 300)), (64, (100,) * 17 + (600,))])
+def test_ragged_groups(B, source, d, lens):
+    """Query deltas: 4 and 5, 2 and 3 sequences of a length lie on either side of the line between tables and rows."""
+    H, Hk, T_max = 32, 8, max(lens) + 2
+    gen = torch.Generator("cuda").manual_seed(len(lens))
+    rnd = lambda *s: (torch.randn(*s, generator=gen, device="cuda").cumsum(-2) * 0.1).bfloat16()      # noqa: E731
+    src = {"query": B.DELTA_SRC_QUERY, "key": B.DELTA_SRC_KEY, "bottom_up": B.DELTA_SRC_QUERY_BOTTOM_UP}[source]
+    kc = torch.full((len(lens), Hk, T_max, d), float("nan"), dtype=torch.bfloat16, device="cuda")
+    qs = [rnd(H, n, d) for n in lens]
+    for b, n in enumerate(lens):
+        kc[b, :, :n] = rnd(Hk, n, d)
+    st = B.delta_state_init(B.make_config(len(lens), H, Hk, d, T_max, "bf16", source=src))
+    out = torch.empty(sum(q.numel() for q in qs), dtype=torch.bfloat16, device="cuda")
+    B.delta_attn_prefill_varlen(st, torch.cat([q.reshape(-1) for q in qs]), kc, kc, out, list(lens), [16] * len(lens), 0.25)
+    Hs = Hk if source == "key" else H
+    dq = B.delta_state_view(st, B.DELTA_VIEW_DQ).reshape(-1)[:len(lens) * Hs * T_max * d].view(len(lens), Hs, T_max, d)
+    ref = B.delta_state_view(st, B.DELTA_VIEW_QHAT).reshape(-1)[:len(lens) * Hs * d].view(len(lens), Hs, d)
+    for b, n in enumerate(lens):
+        x = (kc[b, :, :n] if source == "key" else qs[b]).float()
+        order = range(n - 1, -1, -1) if source == "bottom_up" else range(n)
+        r, want = None, []
+        for i in order:                                    # Eq. 2-3 row by row: one subtraction, a strict comparison
+            diff = x[:, i] if r is None else x[:, i] - r
+            fire = torch.ones_like(diff, dtype=torch.bool) if r is None else diff.abs() > 0.25
+            r = torch.where(fire, x[:, i], r if r is not None else diff)
+            want.append(torch.where(fire, diff, torch.zeros_like(diff)))
+        if source == "bottom_up":
+            want.reverse()
+        assert torch.equal(dq[b, :, :n], torch.stack(want, 1)) and torch.equal(ref[b], r), b
+    assert B.delta_sparsity_stats(st)["device_status"] == 0
