@@ -359,7 +359,7 @@ static bool finish_comes_last(const delta_state* st) {
   return st->cfg.source != DELTA_SRC_KEY && delta_state_prefill_kernel(st) != 1;
 }
 static delta_status_t prefill_launch(delta_state* st, const Shape& shape, const Workspace& ws, const void* q,
-                                     const void* k, const void* v, void* out, const SeqBatch& seqs, float theta,
+                                     const void* k, const void* v, void* out, const SeqBatch& batch, float theta,
                                      cudaStream_t cs, bool prof, int parts = PREFILL_ALL) {
   const delta_config_t& c = st->cfg;
   cudaError_t e;
@@ -387,6 +387,10 @@ static delta_status_t prefill_launch(delta_state* st, const Shape& shape, const 
   // the finish kernel's launch overlaps the end of the attention kernel.  With per-kernel
   // timing on, the kernels run in their natural order with events between them.
   const bool chained = !use_tc && !prof;
+  // (query deltas: the attention kernel may even begin on the first query tiles while the chain goes on)
+  const int form = which == 3 ? 1 : which == 4 ? 2 : which == 5 ? 3 : 0;
+  SeqBatch seqs = batch;
+  if (chained && tcq && !key) seqs.beside = form;
   if (parts == PREFILL_FINISH)
     return (e = launch_delta_finish(shape, ws, q, k, seqs, theta, c.prefill_window, c.dtype, c.init, false, key, rev, 1,
                                     cs)) == cudaSuccess ? DELTA_OK : cuda_fail(e);
@@ -398,7 +402,7 @@ static delta_status_t prefill_launch(delta_state* st, const Shape& shape, const 
     if (use_tc) return launch_hybrid_attn_tc(shape, ws, q, k, v, out, seqs.s[0].T, seqs.s[0].W, c.prefill_window, cs);
     if (tcq)
       return launch_hybrid_attn_tcq(shape, ws, q, k, v, out, seqs, theta, c.init, c.prefill_window, key,
-                                    rev, /*form=*/which == 3 ? 1 : which == 4 ? 2 : which == 5 ? 3 : 0, cs);
+                                    rev, form, cs);
     return launch_hybrid_attn_f32(shape, ws, q, k, v, out, seqs, theta, c.init, c.prefill_window, c.dtype, cs);
   };
   if (chained && !key) {

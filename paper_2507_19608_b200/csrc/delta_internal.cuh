@@ -77,6 +77,7 @@ struct SeqBatch {
   int n, T_longest;
   bool ragged;
   int grid_heads = 0;
+  int beside = -1;      // >= 0: the telescoped attention kernel comes next, with this form, and may begin beside the chain
   Seq s[kSeqMax];
   // query heads of the grid that chooses the form (ragged: of every sequence's grid)
   long form_heads(const Shape& sh) const { return grid_heads ? grid_heads : (long)(ragged ? 1 : sh.B) * sh.H; }
@@ -111,6 +112,12 @@ delta_status_t cuda_fail(cudaError_t e);
 cudaError_t launch_delta_chain(const Shape& s, const Workspace& w, const void* x, const SeqBatch& seqs, float theta,
                                int dtype, int init, bool key_stream, bool reverse, void* zero_ptr, size_t zero_bytes,
                                cudaStream_t st);
+// Does it go by the table kernel?  That one also tells, at chain_progress where that is not null, a word per (head, 32
+// channels), kProgressStride apart (a line each), how many 64-row stages' references are in memory, in processing order;
+// never the last one, which a kernel behind takes from that kernel's end.
+constexpr int kProgressStride = 32;
+bool chain_by_tables(const Shape& s, const SeqBatch& seqs, int dtype, bool key_stream);
+unsigned* chain_progress(const Shape& s, const Workspace& w, const SeqBatch& seqs, int dtype, bool key_stream);
 // K1b: row-parallel finish: delta values, mask words and (key stream) reference rows from the
 // 8-row checkpoints; counts, compacted indices, Eq. 6 counters, the decode hand-off row
 // R(T-1)[j] = q_hat . k_j and (want_kt) the channel-major fp32 key copy.

@@ -23,6 +23,7 @@
 #include <algorithm>
 
 #include "delta_internal.cuh"
+#include "k2_tc.cuh"
 #include "tc_common.cuh"
 
 namespace delta {
@@ -131,7 +132,7 @@ template <typename TIn, int D, int N>
 __global__ void __launch_bounds__(CHAIN_THREADS) delta_chain_kernel(
     const __grid_constant__ ChainSeqs<N> seqs, float* __restrict__ qhat_tile, float* __restrict__ qhat_out,
     float* __restrict__ ckpt, unsigned long long* __restrict__ counters, int n_tiles, int n_ckpt,
-    float theta, int basis_exact, int reverse, int heads, uint4* zero_ptr, unsigned zero_n16) {
+    float theta, int basis_exact, int reverse, int heads, unsigned* __restrict__ progress, uint4* zero_ptr, unsigned zero_n16) {
   // blockIdx.x: (head, 32 channels) of the batch, or of sequence blockIdx.y of a ragged group
   const int si = N == 1 ? 0 : (int)blockIdx.y;
   const CUtensorMap& tm_x = seqs.map[si];
@@ -142,7 +143,7 @@ __global__ void __launch_bounds__(CHAIN_THREADS) delta_chain_kernel(
   TIn* raw = reinterpret_cast<TIn*>(dyn);                                   // [NS][RC][CH]
   float4* zb = reinterpret_cast<float4*>(dyn + NS * RAW_STAGE_BYTES);       // [NZ][NSB][ZV][CH]
   __shared__ __align__(8) unsigned long long bars[2 * NS + 2 * NZ];
-  __shared__ uint32_t s_abort;
+  __shared__ uint32_t s_abort, s_done;             // s_done: stages the chain warp is through with
 
   const int head = blockIdx.x / NSL, sl = blockIdx.x - head * NSL;       // head of the map
   const int bh = seqs.b[si] * heads + head;                               // head of the workspace arrays
@@ -158,7 +159,7 @@ __global__ void __launch_bounds__(CHAIN_THREADS) delta_chain_kernel(
   if (tid < 2 * NS + 2 * NZ) {      // one barrier per thread
     const uint32_t cnt = (tid < NS) ? 1u : (tid < 2 * NS + NZ) ? (uint32_t)NSB : 1u;
     tc::mbar_init(full0 + 8 * tid, cnt);
-    if (tid == 0) s_abort = 0;
+    if (tid == 0) s_abort = s_done = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     tc::fence_proxy_async();
   }
@@ -172,7 +173,15 @@ __global__ void __launch_bounds__(CHAIN_THREADS) delta_chain_kernel(
   // (Whole prefills behind one another, ordinary launch -> this: 1 x 32 heads 256 tokens 12.9 -> 11.5 us, 1024 28.2 ->
   // 26.0; d = 128, 20 heads, 2048 63.6 -> 61.5; 4 x 32 x 1024 74.9 -> 73.1; 8 x 32 x 1024 139.4 -> 137.3.)
   asm volatile("griddepcontrol.wait;" ::: "memory");
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  unsigned* const my_progress = progress ? progress + ((size_t)bh * NSL + sl) * kProgressStride : nullptr;
+  if (!progress) {
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  } else if (tid == 32 * (8 + cw)) {
+    // (cleared before anything behind this kernel can look at it)
+    *my_progress = 0;
+    __threadfence();
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  }
   // the deferred clearing of a state reset (counters, tickets, second reference buffer): nothing
   // of this launch or of the kernels behind it touches that span before this kernel is complete
   if (zero_ptr && blockIdx.x == 0 && blockIdx.y == 0)
@@ -188,6 +197,23 @@ __global__ void __launch_bounds__(CHAIN_THREADS) delta_chain_kernel(
         const int ci = reverse ? n_chunks - 1 - i : i;      // stage of the head in token order
         tc::mbar_expect_tx(full0 + 8 * s, RAW_STAGE_BYTES); // rows past T arrive as zeros
         tc::tma_load_3d(raw0 + s * RAW_STAGE_BYTES, &tm_x, full0 + 8 * s, sl * CH, ci * RC, head);
+      }
+    }
+  } else if (warp == 8 + cw) {
+    // ---- progress: how many stages' references are in memory, for a kernel behind that starts on the first ones while
+    // the chain goes on.  (Not by the chain warp, which a fence would hold up for a trip to memory per stage.)
+    if (progress && lane == 0) {
+      for (int seen = 0; seen + 1 < n_chunks && !*abort_flag;) {
+        // (s_done says which stage's barrier to look at, the barrier orders what the chain warp stored; where the chain
+        // has gone round the ring since, the look fails and the next one is at a later stage)
+        const int now = (int)*(volatile uint32_t*)&s_done;
+        if (now > seen && mbar_test_wait(zfree0 + 8 * ((now - 1) % NZ), ((now - 1) / NZ) & 1)) {
+          seen = now;
+          __threadfence();
+          *(volatile unsigned*)my_progress = (unsigned)seen;
+        } else {
+          __nanosleep(64);
+        }
       }
     }
   } else if ((warp & 3) != cw) {
@@ -229,6 +255,11 @@ __global__ void __launch_bounds__(CHAIN_THREADS) delta_chain_kernel(
     float* cp = ckpt_c + (ptrdiff_t)(tile0 * NSB + (reverse ? NSB - 1 : 0)) * D;
     const int rest = T % RC;                            // rows of a stage cut short by the end of the sequence
     auto wait_stage = [&](int i) { mbar_poll(zfull0 + 8 * (i % NZ), (i / NZ) & 1, abort_flag); __syncwarp(); };
+    auto stage_done = [&](int i) {
+      __syncwarp();
+      arrive_lane0(zfree0 + 8 * (i % NZ), lane);
+      if (lane == 0) *(volatile uint32_t*)&s_done = (uint32_t)(i + 1);
+    };
     auto tile_ref = [&](int i) {
       if (qhat_tile && DELTA_IN(reverse ? tile0 - i : i, n_tiles, counters)) *qp = r;
       qp += step;
@@ -256,8 +287,7 @@ __global__ void __launch_bounds__(CHAIN_THREADS) delta_chain_kernel(
           }
         }
       }
-      __syncwarp();
-      arrive_lane0(zfree0 + 8 * (i % NZ), lane);
+      stage_done(i);
     };
     const int i0 = (reverse && rest) ? 1 : 0, i1 = i0 + T / RC;      // the whole stages
     if (i0) cut_stage(0);
@@ -288,8 +318,7 @@ __global__ void __launch_bounds__(CHAIN_THREADS) delta_chain_kernel(
           r = chain_sub_block(cur, r, theta, b == 0 && i == 0 && basis_exact);
           cur = nxt;
         }
-        __syncwarp();
-        arrive_lane0(zfree0 + 8 * (i % NZ), lane);
+        stage_done(i);
       }
     }
     if (!reverse && rest) cut_stage(i1);
@@ -322,7 +351,8 @@ constexpr int kMaxChainSmem = 144 * 1024;      // (fp32 tables 128 KB; the even 
 
 template <typename TIn, int D, int N>
 static cudaError_t launch_tables(const Shape& s, const Workspace& w, const void* x, const SeqBatch& seqs, float theta, int init,
-                                 bool key_stream, bool reverse, void* zero_ptr, size_t zero_bytes, cudaStream_t st) {
+                                 bool key_stream, bool reverse, unsigned* progress, void* zero_ptr, size_t zero_bytes,
+                                 cudaStream_t st) {
   auto kern = delta_chain_kernel<TIn, D, N>;
   constexpr size_t need = (size_t)NS * RC * CH * sizeof(TIn) + (size_t)NZ * Z_STAGE * sizeof(float4);
   static_assert(need <= kMaxChainSmem, "shared memory");
@@ -355,18 +385,19 @@ static cudaError_t launch_tables(const Shape& s, const Workspace& w, const void*
   cfg.dynamicSmemBytes = even_spread_smem(need, (long)cfg.gridDim.x * seqs.n);
   const cudaError_t err =
       cudaLaunchKernelEx(&cfg, kern, list, w.qhat_tile, w.qhat[0], w.ckpt, w.counters, s.n_tiles, s.n_ckpt(), theta,
-                         init == DELTA_INIT_BASIS_EXACT ? 1 : 0, reverse ? 1 : 0, heads, (uint4*)zero_ptr, (unsigned)(zero_bytes / 16));
+                         init == DELTA_INIT_BASIS_EXACT ? 1 : 0, reverse ? 1 : 0, heads, progress, (uint4*)zero_ptr,
+                         (unsigned)(zero_bytes / 16));
   count_launch();
   return err != cudaSuccess ? err : cudaGetLastError();
 }
 
 static cudaError_t launch_delta_chain_tables(const Shape& s, const Workspace& w, const void* x, const SeqBatch& seqs,
                                              float theta, int dtype, int init, bool key_stream, bool reverse,
-                                             void* zero_ptr, size_t zero_bytes, cudaStream_t st) {
+                                             unsigned* progress, void* zero_ptr, size_t zero_bytes, cudaStream_t st) {
 #define GO(TIN, DD)                                                                                                 \
   return seqs.ragged                                                                                                \
-             ? launch_tables<TIN, DD, kSeqMax>(s, w, x, seqs, theta, init, key_stream, reverse, zero_ptr, zero_bytes, st) \
-             : launch_tables<TIN, DD, 1>(s, w, x, seqs, theta, init, key_stream, reverse, zero_ptr, zero_bytes, st)
+             ? launch_tables<TIN, DD, kSeqMax>(s, w, x, seqs, theta, init, key_stream, reverse, progress, zero_ptr, zero_bytes, st) \
+             : launch_tables<TIN, DD, 1>(s, w, x, seqs, theta, init, key_stream, reverse, progress, zero_ptr, zero_bytes, st)
   if (dtype == DELTA_F32) {
     if (s.d == 64) { GO(float, 64); } else { GO(float, 128); }
   } else {
@@ -611,7 +642,7 @@ int device_sm_count() {
   return cached[dev];
 }
 
-static bool chain_by_tables(const Shape& s, const SeqBatch& seqs, int dtype, bool key_stream) {
+bool chain_by_tables(const Shape& s, const SeqBatch& seqs, int dtype, bool key_stream) {
   // The table kernel while its CTAs (head x 32 channels) are all resident at once: two per SM for bf16, one for fp32
   // (shared memory: 96 and 128 KB).  Whole prefill, tables against rows: 64 CTAs (1 x 32 heads, 1024 tokens) 28.8 us, 34.0;
   // 160 (2 x 20 heads, d = 128, 1531 tokens) 87.9, 90.2; 192 59.5, 61.5; 256 75.0, 77.0; 384 112.6, 110.0; 512 147.5, 139.5.
@@ -624,13 +655,20 @@ static bool chain_by_tables(const Shape& s, const SeqBatch& seqs, int dtype, boo
   return seq_ctas * rows <= (long)device_sm_count() * (dtype == DELTA_F32 ? 1 : 2) * seqs.T_longest;
 }
 
+// (In the decode steps' scratch, which nothing in flight uses during a prefill; it holds 256 (d + 2) bytes per head.)
+unsigned* chain_progress(const Shape& s, const Workspace& w, const SeqBatch& seqs, int dtype, bool key_stream) {
+  return seqs.beside >= 0 && chain_by_tables(s, seqs, dtype, key_stream) && tcq_begins_beside_chain(s, seqs, seqs.beside)
+             ? reinterpret_cast<unsigned*>(w.dec_partial) : nullptr;
+}
+
 cudaError_t launch_delta_chain(const Shape& s, const Workspace& w, const void* x, const SeqBatch& seqs, float theta,
                                int dtype, int init, bool key_stream, bool reverse, void* zero_ptr, size_t zero_bytes,
                                cudaStream_t st) {
   if (key_stream && reverse) return cudaErrorNotSupported;
   if (((uintptr_t)zero_ptr | zero_bytes) & 15u) return cudaErrorInvalidValue;
   if (chain_by_tables(s, seqs, dtype, key_stream))
-    return launch_delta_chain_tables(s, w, x, seqs, theta, dtype, init, key_stream, reverse, zero_ptr, zero_bytes, st);
+    return launch_delta_chain_tables(s, w, x, seqs, theta, dtype, init, key_stream, reverse,
+                                     chain_progress(s, w, seqs, dtype, key_stream), zero_ptr, zero_bytes, st);
   return launch_delta_chain_rows(s, w, x, seqs, theta, dtype, init, key_stream, reverse, zero_ptr, zero_bytes, st);
 }
 

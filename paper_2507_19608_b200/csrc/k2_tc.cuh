@@ -21,4 +21,6 @@ bool tcq_kernel_shape(int d);
 cudaError_t launch_hybrid_attn_tcq(const Shape& s, const Workspace& w, const void* q, const void* k,
                                    const void* v, void* out, const SeqBatch& seqs, float theta, int init,
                                    int shape, bool key_deltas, bool reverse, int form, cudaStream_t st);
+// Should the kernel above begin while the chain goes on (chain_progress)?
+bool tcq_begins_beside_chain(const Shape& s, const SeqBatch& seqs, int form);
 }  // namespace delta
