@@ -201,6 +201,32 @@ __device__ __forceinline__ bool merge_slices(uint32_t recs, uint32_t bar, int ra
   store4(out + out0 + (size_t)(q / (D / 16)) * D + (q % (D / 16)) * 16 + 4 * c4, a.x * inv, a.y * inv, a.z * inv, a.w * inv);
   return ok;
 }
+// The same by the CTA's first threads, one record after the other, behind a suspended wait of every warp: key deltas, whose
+// warps all have counters to update in front of the merge (us per step, shared by idle warps | so: batch 4 at 1777 keys 5.17,
+// 4.99; batch 1 3.78, 3.75; compressed key cache, batch 4 at 1024 keys 6.40, 6.25; batch 16 at 1777 keys 8.04, 8.09).
+template <typename TO, int D, int G>
+__device__ __forceinline__ bool merge_slices_in_turn(uint32_t recs, uint32_t bar, int rank, int cs, size_t out0, TO* __restrict__ out) {
+  constexpr int NB = G * D / 16;
+  const int slot = threadIdx.x >> 2, c4 = threadIdx.x & 3, q = slot * cs + rank;
+  const bool ok = mbar_wait(bar, 0);
+  if (q >= NB) return ok;
+  const uint32_t rb = recs + (uint32_t)(slot * cs) * (REC2 * 4);
+  float M = -INFINITY, l = 0.0f;
+#pragma unroll 8
+  for (int x = 0; x < cs; ++x) M = fmaxf(M, lds_f2(rb + x * (REC2 * 4) + 64).x);
+  float4 a = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+#pragma unroll 8
+  for (int x = 0; x < cs; ++x) {
+    const float2 ml = lds_f2(rb + x * (REC2 * 4) + 64);
+    const float4 o = lds_f4(rb + x * (REC2 * 4) + 16 * c4);
+    const float f = tc::ex2(ml.x - M);                       // 0 for a slice without keys
+    a.x = fmaf(f, o.x, a.x); a.y = fmaf(f, o.y, a.y); a.z = fmaf(f, o.z, a.z); a.w = fmaf(f, o.w, a.w);
+    l = fmaf(f, ml.y, l);
+  }
+  const float inv = 1.0f / l;
+  store4(out + out0 + (size_t)(q / (D / 16)) * D + (q % (D / 16)) * 16 + 4 * c4, a.x * inv, a.y * inv, a.z * inv, a.w * inv);
+  return ok;
+}
 // Slices of a step over sequences of up to L keys (the new one included).  A step takes 3 us plus, for every
 // unit a warp works through, 0.83 us (d = 64) or 0.87 us (d = 128) while a CTA has its SM for itself, 1.15 times that
 // from half the SMs on, and 1.25 or 1.35 us where two share one (measured with 1 to 16 slices forced, 8 to 128 KV

@@ -747,7 +747,10 @@ decode_step_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_co
   }
   if (CLUSTER) {
     // (every slice's block records: also what keeps this CTA until the last of them has been sent to it)
-    if (!merge_slices<TC, D, G, MNW>(recs, bar_m, rank, cs, out0, p.out)) s_fail = 1;
+    bool ok;
+    if constexpr (KEY) ok = merge_slices_in_turn<TC, D, G>(recs, bar_m, rank, cs, out0, p.out);
+    else ok = merge_slices<TC, D, G, MNW>(recs, bar_m, rank, cs, out0, p.out);
+    if (!ok) s_fail = 1;
   } else if (n_slices > 1) {
     merge_global<TC, D, G, MNW>(n_slices, bkv, out0, p.partial, p.ticket, p.out, &s_last);
   }
