@@ -473,28 +473,33 @@ static cudaError_t launch_f32(K kern, std::atomic<uint64_t>& ready, size_t smem,
   return e != cudaSuccess ? e : cudaGetLastError();
 }
 
-// Warps per row group for `heads` heads of T tokens.  A key tile of 64 costs 3.5 / 2.2 / 1.4 us where a CTA
-// walks alone (its set-up about as much as a tile) and takes 2.7 / 1.6 / 1.1 us of an SM where the chip is full (KS = 1 /
-// 2 / 4, d = 64, two CTAs per SM; d = 128, one: 7.0 / 4.4 / 3.1 and 7.0 / 4.2 / 2.9); every halving of the rows doubles
-// the tiles.  The longest walk bounds a small grid; a large one the sum of all tiles and set-ups, and a part of a walk
-// for the uneven end, less of it the more CTAs a place gets.  With each form timed at 16 shapes per d (1 to 128 heads of
-// 64 to 2500 tokens, fp32) the chosen one is the fastest or within 1.1 % of it; KS = 1, 2, 4 in us: 16 heads x 1000
-// 75, 65, 80 / d = 128 125, 148, 196; 16 x 1800 147, 165, 217; 32 x 600 56, 49, 66 / 109, 120, 165; 8 x 700 44, 34, 31 /
-// 90, 58, 65.  bf16 inputs, which run here only when kernel 0 is forced, take the same form.  A sequence of a
-// ragged group takes the form of a batch of its own (the forms round differently: its result does not
-// depend on the sequences beside it).
+// Warps per row group for `heads` heads of T tokens.  Every halving of the rows doubles the tiles; the longest walk bounds
+// a small grid; a large one the sum of all tiles, and a part of a walk for the uneven end.  d = 64: a key tile of 64 costs
+// 3.3 / 2.2 / 1.4 us where a CTA walks alone and counts 4.0 / 2.2 / 1.6 us of an SM (KS = 1 / 2 / 4).  d = 128 (one CTA per SM): 7.0 /
+// 4.4 / 3.1 and 7.0 / 4.2 / 2.9, a CTA's set-up about a tile of its walk and 4 us of an SM, and the end shorter the more CTAs an
+// SM gets; KS = 4 only where it is clearly ahead.  A sequence of a ragged group takes the form of a batch of its own (the forms
+// round differently: its result does not depend on the sequences beside it), so a form that is a little faster alone and
+// does more work in all is not taken: five sequences of up to 404 tokens, 20 heads, d = 64, 59.5 us, with the rule of d = 128 69.1.
+// With each form timed at 16 shapes per d (1 to 128 heads of 64 to 2500 tokens, fp32) the chosen one is the fastest or within
+// 2 % of it but for 32 heads x 128 (5 %), 8 x 700 (9 %), 128 x 128 (6 %) and, d = 128, 16 x 200 (12 %); KS = 1, 2, 4 in us: 16 heads x 1000 75, 65, 80 / d = 128
+// 125, 148, 196; 16 x 1800 147, 165, 217 / 355, 407, 551; 32 x 600 56, 49, 66 / 109, 120, 165.  bf16 inputs, which run here only
+// when kernel 0 is forced, take the same form.
 static int f32_form(long heads, int T, int d) {
-  constexpr float alone[2][3] = {{3.5f, 2.2f, 1.4f}, {7.0f, 4.4f, 3.1f}}, full[2][3] = {{2.7f, 1.6f, 1.1f}, {7.0f, 4.2f, 2.9f}};
-  constexpr float set_up[2] = {0.8f, 4.0f};        // us of an SM per CTA
+  constexpr float alone[2][3] = {{3.3f, 2.2f, 1.4f}, {7.0f, 4.4f, 3.1f}}, full[2][3] = {{4.0f, 2.2f, 1.6f}, {7.0f, 4.2f, 2.9f}};
   const int x = d == 64 ? 0 : 1;
   const float sms = (float)device_sm_count(), t = (float)((T + BN - 1) / BN), pairs = 0.5f * t * (t + 1.0f) * (float)heads;
   int ks = 1;
   float best = 3.4e38f;
   for (int c = 0; c < 3; ++c) {
-    const float walk = (t + 1.0f) * alone[x][c], ctas = (float)heads * (float)((T * (1l << c) + BN - 1) / BN);
-    const float r = fmaxf(1.0f, ctas / (sms * (float)(2 - x)));
-    const float us = fmaxf(walk, (pairs * (float)(1 << c) * full[x][c] + ctas * set_up[x]) / sms + 0.3f * walk / (r * r));
-    if (us < best) { best = us; ks = 1 << c; }
+    float walk = t * alone[x][c], sum = pairs * (float)(1 << c) * full[x][c] / sms, end = 0.5f;
+    if (x) {
+      const float ctas = (float)heads * (float)((T * (1l << c) + BN - 1) / BN), r = fmaxf(1.0f, ctas / sms);
+      walk += alone[x][c];
+      sum += 4.0f * ctas / sms;
+      end = 0.3f / (r * r);
+    }
+    const float us = fmaxf(walk, sum + end * walk);
+    if (us < (x && c == 2 ? 0.85f : 1.0f) * best) { best = us; ks = 1 << c; }
   }
   return ks;
 }
