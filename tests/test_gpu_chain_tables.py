@@ -65,10 +65,11 @@ def _check(B, H, T, d, dtype, theta, init, order):
 
 
 @pytest.mark.parametrize("source", ["query", "key", "bottom_up"])
-@pytest.mark.parametrize("d,lens", [(64, (300, 261, 299, 300)), (64, (300, 295, 300, 299, 280)), (64, (777, 8, 513, 64, 1, 505)),
-                                    (128, (300, 300)), (128, (300, 299, 300)), (64, (100,) * 17 + (600,))])
+@pytest.mark.parametrize("d,lens", [(64, (600, 561, 599, 600)), (64, (600, 595, 600, 599, 580)), (64, (777, 8, 513, 64, 1, 505)),
+                                    (64, (240, 9, 100)), (64, (239, 9, 100)), (128, (400, 400)), (128, (400, 399, 400)), (64, (100,) * 17 + (600,))])
 def test_ragged_groups(B, source, d, lens):
-    """Query deltas: 4 and 5, 2 and 3 sequences of a length lie on either side of the line between tables and rows."""
+    """Query deltas: 4 and 5, 2 and 3 sequences of a length lie on either side of one line between tables and rows, the longest
+    sequence of 240 or 239 tokens among three on either side of the other."""
     H, Hk, T_max = 32, 8, max(lens) + 2
     gen = torch.Generator("cuda").manual_seed(len(lens))
     rnd = lambda *s: (torch.randn(*s, generator=gen, device="cuda").cumsum(-2) * 0.1).bfloat16()      # noqa: E731
