@@ -228,7 +228,9 @@ __device__ __forceinline__ void build_ref_rows(const unsigned char* q_src, unsig
 // follows its place in the grid (see below).
 // N: entries of the sequence list: 1 (a uniform batch), or kSeqMax (a ragged group: the CTAs of the
 // sequences one behind the other, the longest sequence first, each as in a batch of its own).
-template <int D, bool KEY, int FORM, bool MIXED, int N>
+// BESIDE (query deltas): p.progress says how far the chain is; without it the launch waits for the chain kernel's end, in code
+// of its own (with both in one, 8 x 32 heads x 4096 tokens and 128 steps 2192 us a pass, so 2176).
+template <int D, bool KEY, int FORM, bool MIXED, int N, bool BESIDE>
 __global__ void __launch_bounds__(NTHR, 1)
 hybrid_attn_tcq_kernel(const __grid_constant__ TqMapList<N> maps, const __grid_constant__ SeqList<N> seqs,
                        const __grid_constant__ TqParams p) {
@@ -267,9 +269,9 @@ hybrid_attn_tcq_kernel(const __grid_constant__ TqMapList<N> maps, const __grid_c
     idx -= maps.first[si];
   }
   if (PAIR) {
-    const int n1 = (FORM == 1) ? 0 : p.BH * n_one, nl = (N == 1 && !KEY) ? p.light * (p.BH / 2) : 0;
+    const int n1 = (FORM == 1) ? 0 : p.BH * n_one, nl = (N == 1 && BESIDE) ? p.light * (p.BH / 2) : 0;
     idx -= nl;
-    if (N == 1 && !KEY && idx < 0) {
+    if (N == 1 && BESIDE && idx < 0) {
       const int j = idx + nl, hp = p.BH / 2;
       pr = true;
       qt = j / hp;
@@ -287,8 +289,8 @@ hybrid_attn_tcq_kernel(const __grid_constant__ TqMapList<N> maps, const __grid_c
     qt = nqt - 1 - idx / p.BH;
     bh = idx % p.BH;
   } else {
-    const int y = (int)blockIdx.y - (KEY ? 0 : p.light);
-    qt = y < 0 ? (int)blockIdx.y : (int)gridDim.y - 1 - y;
+    const int y = (int)blockIdx.y - (BESIDE ? p.light : 0);
+    qt = y < 0 ? (int)blockIdx.y : p.nqt - 1 - y;
     bh = (int)blockIdx.x;
   }
   // (bh, bkv: head and KV head within the entry of the sequence list; g_bh: of the workspace arrays)
@@ -319,10 +321,10 @@ hybrid_attn_tcq_kernel(const __grid_constant__ TqMapList<N> maps, const __grid_c
   // How far the chain has to be for this tile, in stages of 64 rows (all of them: this kernel waits for that one's end), and
   // a first look whether it is, under the set-up.
   const unsigned stages = (unsigned)(T + DELTA_TILE_ROWS - 1) / DELTA_TILE_ROWS;
-  const unsigned need = KEY || !p.progress ? stages : p.reverse ? stages - 2u * (unsigned)qt : 2u * (unsigned)qt + 2u;
+  const unsigned need = !BESIDE ? stages : p.reverse ? stages - 2u * (unsigned)qt : 2u * (unsigned)qt + 2u;
   const unsigned* const words = p.progress + (size_t)(g_bh + bh) * (D / 32) * kProgressStride;
   const int n_words = (pr ? 2 : 1) * (D / 32);
-  if (need < stages && warp == 1) {
+  if (BESIDE && need < stages && warp == 1) {
     const bool there = lane >= n_words || chain_stages(words + lane * kProgressStride) >= need;
     const bool all = __all_sync(0xffffffffu, there);
     if (lane == 0) sMisc[2] = all ? 1u : 0u;
@@ -634,7 +636,7 @@ hybrid_attn_tcq_kernel(const __grid_constant__ TqMapList<N> maps, const __grid_c
         offs[rr] = (uint32_t)rr * 128u + ((((uint32_t)(c & 63) >> 3) ^ (uint32_t)rr) << 4) + ((uint32_t)c & 7u) * 2u;
       const uint32_t thr_off = (uint32_t)(c >> 6) * SZ_BLK + (uint32_t)(seg * SEG) * 128u;
       // the chain kernel's checkpoints: that kernel's end, or its word that this tile's are there
-      if (need >= stages) {
+      if (!BESIDE || need >= stages) {
         asm volatile("griddepcontrol.wait;" ::: "memory");
       } else if (!sMisc[2]) {
         // (one warp looks, a lane per word: with every warp looking the chain's own loads queue behind, +5 us)
@@ -658,7 +660,8 @@ hybrid_attn_tcq_kernel(const __grid_constant__ TqMapList<N> maps, const __grid_c
       for (int bk = 0; bk < kMaxBlocks; ++bk)
         refs[bk] = (bk < nbk && r00 + bk * DELTA_CKPT_ROWS < T &&
                     DELTA_IN(r00 / DELTA_CKPT_ROWS + bk, p.n_ckpt, p.counters))
-                       ? __ldcg(reinterpret_cast<const float2*>(ck + bk * D)) : make_float2(0.0f, 0.0f);
+                       ? (BESIDE ? __ldcg(reinterpret_cast<const float2*>(ck + bk * D)) : *reinterpret_cast<const float2*>(ck + bk * D))
+                       : make_float2(0.0f, 0.0f);
       mbar_wait(BAR(BAR_Q), 0, abort_flag);      // the query tile has landed
       const unsigned char* const q_src = sm + OFF_Q + qsel + thr_off;
       unsigned char* const qh_dst = sm + OFF_QH + qsel + thr_off;
@@ -998,12 +1001,12 @@ hybrid_attn_tcq_kernel(const __grid_constant__ TqMapList<N> maps, const __grid_c
 #undef BAR
 }
 
-template <int D, bool KEY, int FORM, bool MIXED, int N>
+template <int D, bool KEY, int FORM, bool MIXED, int N, bool BESIDE = false>
 static cudaError_t launch_tcq_m(const Shape& s, const Workspace& w, const void* q, const void* k, const void* v,
                                 void* out, const SeqBatch& seqs, const int (&n_one)[kSeqMax], int light, const unsigned* progress,
                                 float theta, int init, int shape, bool reverse, cudaStream_t st) {
   constexpr bool PAIR = FORM != 0;
-  auto kern = hybrid_attn_tcq_kernel<D, KEY, FORM, MIXED, N>;
+  auto kern = hybrid_attn_tcq_kernel<D, KEY, FORM, MIXED, N, BESIDE>;
   using TC = __nv_bfloat16;
   const int nb = seqs.ragged ? 1 : s.B;
   const uint64_t BH = (uint64_t)nb * s.H, BKV = (uint64_t)nb * s.H_kv;     // heads of one entry
@@ -1092,9 +1095,22 @@ template <int D, bool KEY, int FORM>
 static cudaError_t launch_tcq(const Shape& s, const Workspace& w, const void* q, const void* k, const void* v,
                               void* out, const SeqBatch& seqs, const int (&n_one)[kSeqMax], int light, const unsigned* progress,
                               float theta, int init, int shape, bool reverse, cudaStream_t st) {
+  if constexpr (!KEY) {
+    if (progress && seqs.ragged)
+      return launch_tcq_m<D, KEY, FORM == 0 ? 0 : 2, true, kSeqMax, true>(s, w, q, k, v, out, seqs, n_one, light, progress, theta,
+                                                                                 init, shape, reverse, st);
+  }
   if (seqs.ragged)       // (windows differ: with the mixed tiles' code; the form is each sequence's)
     return launch_tcq_m<D, KEY, FORM == 0 ? 0 : 2, true, kSeqMax>(s, w, q, k, v, out, seqs, n_one, light, progress, theta, init, shape,
                                                                  reverse, st);
+  if constexpr (!KEY) {
+    if (progress)
+      return mixed_tiles_possible<D, KEY>(seqs.s[0].W, shape)
+                 ? launch_tcq_m<D, KEY, FORM, true, 1, true>(s, w, q, k, v, out, seqs, n_one, light, progress, theta, init, shape,
+                                                                    reverse, st)
+                 : launch_tcq_m<D, KEY, FORM, false, 1, true>(s, w, q, k, v, out, seqs, n_one, light, progress, theta, init, shape,
+                                                                     reverse, st);
+  }
   return mixed_tiles_possible<D, KEY>(seqs.s[0].W, shape)
              ? launch_tcq_m<D, KEY, FORM, true, 1>(s, w, q, k, v, out, seqs, n_one, light, progress, theta, init, shape, reverse, st)
              : launch_tcq_m<D, KEY, FORM, false, 1>(s, w, q, k, v, out, seqs, n_one, light, progress, theta, init, shape, reverse, st);
