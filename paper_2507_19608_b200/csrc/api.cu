@@ -391,6 +391,8 @@ static delta_status_t prefill_launch(delta_state* st, const Shape& shape, const 
   const int form = which == 3 ? 1 : which == 4 ? 2 : which == 5 ? 3 : 0;
   SeqBatch seqs = batch;
   if (chained && tcq && !key) seqs.beside = form;
+  bool finished = false;
+  if (chained && !key && parts == PREFILL_ALL) seqs.with_finish = &finished;
   if (parts == PREFILL_FINISH)
     return (e = launch_delta_finish(shape, ws, q, k, seqs, theta, c.prefill_window, c.dtype, c.init, false, key, rev, 1,
                                     cs)) == cudaSuccess ? DELTA_OK : cuda_fail(e);
@@ -408,7 +410,7 @@ static delta_status_t prefill_launch(delta_state* st, const Shape& shape, const 
   if (chained && !key) {
     if ((e = attention()) != cudaSuccess) return cuda_fail(e);
     // (released by the attention CTAs once the chain is complete: it runs beside their last wave)
-    if (parts == PREFILL_ALL && (e = launch_delta_finish(shape, ws, q, k, seqs, theta, c.prefill_window, c.dtype, c.init,
+    if (parts == PREFILL_ALL && !finished && (e = launch_delta_finish(shape, ws, q, k, seqs, theta, c.prefill_window, c.dtype, c.init,
                                  use_tc, key, rev, 2, cs)) != cudaSuccess)
       return cuda_fail(e);
   } else if (chained) {

@@ -78,6 +78,7 @@ struct SeqBatch {
   bool ragged;
   int grid_heads = 0;
   int beside = -1;      // >= 0: the telescoped attention kernel comes next, with this form, and may begin beside the chain
+  bool* with_finish = nullptr;      // the attention launch may do the finish kernel's work too, and says here that it does
   Seq s[kSeqMax];
   // query heads of the grid that chooses the form (ragged: of every sequence's grid)
   long form_heads(const Shape& sh) const { return grid_heads ? grid_heads : (long)(ragged ? 1 : sh.B) * sh.H; }

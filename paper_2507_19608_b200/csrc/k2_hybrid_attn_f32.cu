@@ -32,6 +32,7 @@
 #include <algorithm>
 
 #include "delta_internal.cuh"
+#include "k1_finish.cuh"
 #include "tc_common.cuh"
 
 namespace delta {
@@ -435,9 +436,20 @@ __device__ __forceinline__ void attn_f32_tile(const F32Args<TIn>& p, const Seq& 
 
 // A uniform batch.  Heads are the fastest index: the longest walks of every head start first.  (Head after head, the
 // last head's longest walk started last: 16 heads x 1000 86.5 us, so 66.8; 32 x 2000 384, 314; d = 128 924, 819.)
-template <typename TIn, int D, int KS>
+// FIN: the CTAs from tile fin_y on do the finish kernel's work, one of its blocks each.
+template <typename TIn, int D, int KS, bool FIN>
 __global__ void __launch_bounds__(NT, D == 64 ? 2 : 1)
-hybrid_attn_f32_kernel(const __grid_constant__ F32Args<TIn> p, const __grid_constant__ SeqList<1> seqs) {
+hybrid_attn_f32_kernel(const __grid_constant__ F32Args<TIn> p, const __grid_constant__ SeqList<1> seqs,
+                       const __grid_constant__ FinishWork<TIn> fin, int fin_y) {
+  if (FIN && (int)blockIdx.y >= fin_y) {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    const int block = ((int)blockIdx.y - fin_y) * (int)gridDim.x + (int)blockIdx.x;
+    extern __shared__ unsigned char smem_raw[];
+    if (block < fin.blocks)
+      finish_block<TIn, D, NT / 32>(fin, seqs.s[0], block, smem_raw + (-(int)smem_u32(smem_raw) & 15));
+    return;
+  }
   attn_f32_tile<TIn, D, KS>(p, seqs.s[0], (int)blockIdx.y, (int)blockIdx.x);
 }
 // A ragged group: every sequence in the form of a batch of its own.
@@ -511,7 +523,7 @@ static cudaError_t launch_f32_form(const Shape& s, const Workspace& w, const voi
   const F32Args<TIn> p{(const TIn*)q, (const TIn*)k, (const TIn*)v, (TIn*)out, w.ckpt, w.counters, s.T_max, s.n_ckpt(), s.H,
                        s.g(), shape, theta, init == DELTA_INIT_BASIS_EXACT ? 0 : -1, 1.4426950408889634f / sqrtf((float)s.d)};
   const long heads = seqs.form_heads(s);
-  static std::atomic<uint64_t> ready[4] = {};
+  static std::atomic<uint64_t> ready[4] = {}, ready_fin[3] = {};
   if (seqs.ragged) {
     SeqList<kSeqMax> list;
     F32Forms forms;
@@ -530,9 +542,25 @@ static cudaError_t launch_f32_form(const Shape& s, const Workspace& w, const voi
   list.s[0] = seqs.s[0];
   const unsigned T = (unsigned)list.s[0].T, bh = (unsigned)(s.B * s.H);
   const int ks = f32_form(heads, (int)T, D);
-#define GO(KS)                                                                                               \
-  return launch_f32(hybrid_attn_f32_kernel<TIn, D, KS>, ready[KS / 2], F32Smem<D, KS, NP>::bytes,            \
-                    dim3(bh, (T + 64 / KS - 1) / (64 / KS)), st, p, list)
+  // (a small call does the finish kernel's work in the same launch)
+  const unsigned tiles = (T + 64 / ks - 1) / (64 / ks);
+  FinishWork<TIn> fin{};
+  if constexpr (NP == 3) {
+    if (seqs.with_finish) {
+      fin = finish_work<TIn>(s, w, q, k, (int)T, theta, shape, init, false);
+      if (finish_beside((int)T, (long)bh * tiles, fin.blocks)) *seqs.with_finish = true;
+      else fin.blocks = 0;
+    }
+  }
+  const unsigned more = ((unsigned)fin.blocks + bh - 1) / bh;
+#define GO(KS)                                                                                                        \
+  do {                                                                                                                \
+    if (NP == 3 && fin.blocks)                                                                                        \
+      return launch_f32(hybrid_attn_f32_kernel<TIn, D, KS, NP == 3>, ready_fin[KS / 2], F32Smem<D, KS, NP>::bytes,    \
+                        dim3(bh, tiles + more), st, p, list, fin, (int)tiles);                                        \
+    return launch_f32(hybrid_attn_f32_kernel<TIn, D, KS, false>, ready[KS / 2], F32Smem<D, KS, NP>::bytes,            \
+                      dim3(bh, tiles), st, p, list, fin, (int)tiles);                                                 \
+  } while (0)
   if (ks == 4) GO(4);
   if (ks == 2) GO(2);
   GO(1);

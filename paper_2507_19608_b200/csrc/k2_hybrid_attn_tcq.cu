@@ -49,7 +49,9 @@
 
 #include <algorithm>
 #include <climits>
+#include <type_traits>
 
+#include "k1_finish.cuh"
 #include "k2_tc.cuh"
 #include "tc_common.cuh"
 
@@ -228,14 +230,28 @@ __device__ __forceinline__ void build_ref_rows(const unsigned char* q_src, unsig
 // follows its place in the grid (see below).
 // N: entries of the sequence list: 1 (a uniform batch), or kSeqMax (a ragged group: the CTAs of the
 // sequences one behind the other, the longest sequence first, each as in a batch of its own).
+// FIN (FORM 0, uniform batch, query deltas): the CTAs behind the query tiles do the finish kernel's work, a block each.
+struct NoFinish { int blocks; };
+template <bool FIN> using FinishArg = std::conditional_t<FIN, FinishWork<__nv_bfloat16>, NoFinish>;
 // BESIDE (query deltas): p.progress says how far the chain is; without it the launch waits for the chain kernel's end, in code
 // of its own (with both in one, 8 x 32 heads x 4096 tokens and 128 steps 2192 us a pass, so 2176).
-template <int D, bool KEY, int FORM, bool MIXED, int N, bool BESIDE>
+template <int D, bool KEY, int FORM, bool MIXED, int N, bool FIN, bool BESIDE>
 __global__ void __launch_bounds__(NTHR, 1)
 hybrid_attn_tcq_kernel(const __grid_constant__ TqMapList<N> maps, const __grid_constant__ SeqList<N> seqs,
-                       const __grid_constant__ TqParams p) {
+                       const __grid_constant__ TqParams p, const __grid_constant__ FinishArg<FIN> fin) {
   extern __shared__ unsigned char smem_raw[];
   const uint32_t raw = smem_u32(smem_raw);
+  if constexpr (FIN) {
+    static_assert(FORM == 0 && N == 1 && !KEY, "where the finish kernel's work is done too");
+    if ((int)blockIdx.y >= p.nqt) {
+      if (threadIdx.x >= 256) return;
+      asm volatile("griddepcontrol.wait;" ::: "memory");
+      asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+      const int block = ((int)blockIdx.y - p.nqt) * (int)gridDim.x + (int)blockIdx.x;
+      if (block < fin.blocks) finish_block<__nv_bfloat16, D, 8>(fin, seqs.s[0], block, smem_raw + (-(int)raw & 15));
+      return;
+    }
+  }
   const uint32_t base = (raw + 1023u) & ~1023u;
   unsigned char* sm = smem_raw + (base - raw);
   constexpr bool PAIR = FORM != 0;       // the layout holds two query tiles
@@ -1001,12 +1017,13 @@ hybrid_attn_tcq_kernel(const __grid_constant__ TqMapList<N> maps, const __grid_c
 #undef BAR
 }
 
-template <int D, bool KEY, int FORM, bool MIXED, int N, bool BESIDE = false>
+template <int D, bool KEY, int FORM, bool MIXED, int N, bool FIN = false, bool BESIDE = false>
 static cudaError_t launch_tcq_m(const Shape& s, const Workspace& w, const void* q, const void* k, const void* v,
                                 void* out, const SeqBatch& seqs, const int (&n_one)[kSeqMax], int light, const unsigned* progress,
-                                float theta, int init, int shape, bool reverse, cudaStream_t st) {
+                                float theta, int init, int shape, bool reverse, cudaStream_t st,
+                                FinishArg<FIN> fin = FinishArg<FIN>{}) {
   constexpr bool PAIR = FORM != 0;
-  auto kern = hybrid_attn_tcq_kernel<D, KEY, FORM, MIXED, N, BESIDE>;
+  auto kern = hybrid_attn_tcq_kernel<D, KEY, FORM, MIXED, N, FIN, BESIDE>;
   using TC = __nv_bfloat16;
   const int nb = seqs.ragged ? 1 : s.B;
   const uint64_t BH = (uint64_t)nb * s.H, BKV = (uint64_t)nb * s.H_kv;     // heads of one entry
@@ -1066,7 +1083,8 @@ static cudaError_t launch_tcq_m(const Shape& s, const Workspace& w, const void* 
   // griddepcontrol.wait.
   cudaLaunchConfig_t cfg = {};
   p.BH = (int)BH;
-  cfg.gridDim = (PAIR || N > 1) ? dim3((unsigned)ctas) : dim3((unsigned)BH, (unsigned)p.nqt);
+  const unsigned more = FIN ? ((unsigned)fin.blocks + (unsigned)BH - 1) / (unsigned)BH : 0u;
+  cfg.gridDim = (PAIR || N > 1) ? dim3((unsigned)ctas) : dim3((unsigned)BH, (unsigned)p.nqt + more);
   cfg.blockDim = dim3(NTHR);
   cfg.dynamicSmemBytes = TqSmem<D, PAIR>::BYTES;
   cfg.stream = st;
@@ -1075,7 +1093,7 @@ static cudaError_t launch_tcq_m(const Shape& s, const Workspace& w, const void* 
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  const cudaError_t err = cudaLaunchKernelEx(&cfg, kern, maps, list, p);
+  const cudaError_t err = cudaLaunchKernelEx(&cfg, kern, maps, list, p, fin);
   count_launch();
   return err != cudaSuccess ? err : cudaGetLastError();
 }
@@ -1097,18 +1115,33 @@ static cudaError_t launch_tcq(const Shape& s, const Workspace& w, const void* q,
                               float theta, int init, int shape, bool reverse, cudaStream_t st) {
   if constexpr (!KEY) {
     if (progress && seqs.ragged)
-      return launch_tcq_m<D, KEY, FORM == 0 ? 0 : 2, true, kSeqMax, true>(s, w, q, k, v, out, seqs, n_one, light, progress, theta,
+      return launch_tcq_m<D, KEY, FORM == 0 ? 0 : 2, true, kSeqMax, false, true>(s, w, q, k, v, out, seqs, n_one, light, progress, theta,
                                                                                  init, shape, reverse, st);
   }
   if (seqs.ragged)       // (windows differ: with the mixed tiles' code; the form is each sequence's)
     return launch_tcq_m<D, KEY, FORM == 0 ? 0 : 2, true, kSeqMax>(s, w, q, k, v, out, seqs, n_one, light, progress, theta, init, shape,
                                                                  reverse, st);
+  // (a small call does the finish kernel's work in the same launch)
+  if constexpr (FORM == 0 && !KEY) {
+    if (seqs.with_finish) {
+      const int T = seqs.s[0].T;
+      const FinishWork<__nv_bfloat16> fin = finish_work<__nv_bfloat16>(s, w, q, k, T, theta, shape, init, reverse);
+      if (finish_beside(T, (long)s.B * s.H * ((T + BM - 1) / BM), fin.blocks)) {
+        *seqs.with_finish = true;
+        return mixed_tiles_possible<D, KEY>(seqs.s[0].W, shape)
+                   ? launch_tcq_m<D, KEY, FORM, true, 1, true>(s, w, q, k, v, out, seqs, n_one, light, progress, theta, init, shape,
+                                                               reverse, st, fin)
+                   : launch_tcq_m<D, KEY, FORM, false, 1, true>(s, w, q, k, v, out, seqs, n_one, light, progress, theta, init, shape,
+                                                                reverse, st, fin);
+      }
+    }
+  }
   if constexpr (!KEY) {
     if (progress)
       return mixed_tiles_possible<D, KEY>(seqs.s[0].W, shape)
-                 ? launch_tcq_m<D, KEY, FORM, true, 1, true>(s, w, q, k, v, out, seqs, n_one, light, progress, theta, init, shape,
+                 ? launch_tcq_m<D, KEY, FORM, true, 1, false, true>(s, w, q, k, v, out, seqs, n_one, light, progress, theta, init, shape,
                                                                     reverse, st)
-                 : launch_tcq_m<D, KEY, FORM, false, 1, true>(s, w, q, k, v, out, seqs, n_one, light, progress, theta, init, shape,
+                 : launch_tcq_m<D, KEY, FORM, false, 1, false, true>(s, w, q, k, v, out, seqs, n_one, light, progress, theta, init, shape,
                                                                      reverse, st);
   }
   return mixed_tiles_possible<D, KEY>(seqs.s[0].W, shape)
