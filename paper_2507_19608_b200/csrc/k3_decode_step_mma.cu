@@ -172,7 +172,7 @@ template <int D, int G, bool PACKED> struct MmaSmem {
 // MODE 0: query deltas; 1: key deltas, dense reference-key rows; 2: key deltas from the compressed
 // key-delta cache (k1_pack_keys.cu has its layout): a unit is one segment of the
 // encoding, whose rows the warp rebuilds into its key slot.
-template <int D, int G, int MODE, bool CLUSTER>
+template <int D, int G, int MODE, bool CLUSTER, bool LATE>
 __global__ void __launch_bounds__(32 * kWarps<D>, 2)
 decode_step_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ CUtensorMap tm_v,
                        const __grid_constant__ CUtensorMap tm_h, const __grid_constant__ MmaDecodeParams p) {
@@ -378,9 +378,9 @@ decode_step_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_co
   }
   // the step in front (or the prefill) has written the reference, row n - 1 of the caches, the tickets
   asm volatile("griddepcontrol.wait;" ::: "memory");
-  // The next step's CTAs may become resident from here on.  (Released at the kernel's start they
-  // take the places of this step's own late CTAs: 30 us per step for 18 at batch 16.)
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  // The next step's CTAs may become resident from here on, LATE: from the merge on.  (Released at the kernel's start
+  // they take the places of this step's own late CTAs: 30 us per step for 18 at batch 16.)
+  if constexpr (!LATE) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 
   // ---- threshold step (Eq. 2-3), a few elements per thread; the references meet in shared memory, from
   // where every warp takes its operand rows (each warp on its own: 150 instructions more per warp, 0.2 us
@@ -699,6 +699,7 @@ decode_step_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_co
       o_acc[i][1] += __shfl_down_sync(0xffffffffu, o_acc[i][1], 4 * G);
     }
   }
+  if constexpr (LATE) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   // ---- merge: the warp's part into its first slot (every copy into it is complete and read)
   if (part == 0) {
     using MP = MergePart<D, G>;
@@ -757,10 +758,10 @@ decode_step_mma_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_co
   if (s_fail && lane == 0) atomicMax(&p.counters[CNT_STATUS], (unsigned long long)DELTA_ERR_TIMEOUT);
 }
 
-template <int D, int G, int MODE, bool CLUSTER>
+template <int D, int G, int MODE, bool CLUSTER, bool LATE>
 static cudaError_t launch_mma(const CUtensorMap& tk, const CUtensorMap& tv, const CUtensorMap& th,
                               const MmaDecodeParams& p, int bkv, cudaStream_t st) {
-  auto kern = decode_step_mma_kernel<D, G, MODE, CLUSTER>;
+  auto kern = decode_step_mma_kernel<D, G, MODE, CLUSTER, LATE>;
   using SM = MmaSmem<D, G, MODE == 2>;
   const size_t smem = SM::bytes(CLUSTER ? p.nsplit : 1);
   static std::atomic<uint64_t> ready{0};
@@ -836,16 +837,26 @@ cudaError_t launch_decode_step_mma(const Shape& s, const Workspace& w, const voi
   decode_slices(s, n + 1, s.d == 64 ? kWarps<64> : kWarps<128>, s.d == 64 ? 1.25f : 1.35f, s.d == 64 ? 0.83f : 0.87f,
                 packed ? 1.6f : 0.0f, &p.nsplit, &p.chunk, &cluster);
   if (p.nsplit > kMaxDecodeSplits) return cudaErrorInvalidValue;
+  // When the next step's CTAs may come (query deltas): from the merge on where two CTAs share an SM (from 1.6 per SM on) and,
+  // d = 128, where a warp has two units at most; else behind the wait.  us per step, behind the wait | at the merge: 16 x 32 heads
+  // at 2048 keys 9.48, 9.27; 8 x 32 at 4096 9.56, 9.41; 30 x 8 at 700 7.34, 7.05; d = 128, 20 heads, batch 1 at 1000 3.98, 3.90, 2 at
+  // 1531 4.78, 4.70, 8 at 2000 7.56, 7.44; but 2 x 8 at 3500 7.67, 7.76; d = 64, batch 2 at 2048 4.71, 4.88.  Key deltas fetch ahead
+  // of the wait and want their place early: batch 4 at 1777 keys 5.17, 5.46.
+  const bool late = (long)s.B * s.H_kv * p.nsplit * 10 > 16l * device_sm_count() ||
+                    (s.d == 128 && p.chunk <= 2 * UK * kWarps<128>);
   cudaError_t err = cudaSuccess;
   for (; p.b0 < s.B && err == cudaSuccess; p.b0 += kRaggedMax) {
     const int nb = n_b ? (s.B - p.b0 < kRaggedMax ? s.B - p.b0 : kRaggedMax) : s.B;
     if (n_b)
       for (int i = 0; i < nb; ++i) p.n_b[i] = n_b[p.b0 + i];
-#define GO_M(DD, GG, M)                                                                                      \
-    err = cluster ? launch_mma<DD, GG, M, true>(*tk, *tv, *th, p, nb * s.H_kv, st)                           \
-                  : launch_mma<DD, GG, M, false>(*tk, *tv, *th, p, nb * s.H_kv, st)
+#define GO_M(DD, GG, M, L)                                                                                   \
+    err = cluster ? launch_mma<DD, GG, M, true, L>(*tk, *tv, *th, p, nb * s.H_kv, st)                        \
+                  : launch_mma<DD, GG, M, false, L>(*tk, *tv, *th, p, nb * s.H_kv, st)
 #define GO(DD, GG)                                                                                           \
-    if (packed) { GO_M(DD, GG, 2); } else if (key) { GO_M(DD, GG, 1); } else { GO_M(DD, GG, 0); }
+    if (packed) { GO_M(DD, GG, 2, false); }                                                                  \
+    else if (key) { GO_M(DD, GG, 1, false); }                                                                \
+    else if (late) { GO_M(DD, GG, 0, true); }                                                                \
+    else { GO_M(DD, GG, 0, false); }
 #define GO_G(DD)                                                                                             \
     switch (G) {                                                                                             \
       case 1: GO(DD, 1); break;                                                                              \
